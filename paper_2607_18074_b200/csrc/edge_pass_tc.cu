@@ -395,51 +395,49 @@ __global__ void __launch_bounds__((NCW + NLW + 1) * 32, MINB) k_edge_tc(const Et
         }
     } else if (warp == NCW + NLW) {
         // =========================== MMA warp ===========================
-        if (lane == 0) {
-            uint32_t it = 0, zi = 0, ai = 0;
-            const uint32_t sZ_u = smem_u32(sZ);
-            for (int64_t v = blockIdx.x; v < a.n_nodes; v += gridDim.x) {
-                int64_t seg0, seg1;
-                et_bounds(a, v, nullptr, seg0, seg1);
-                if (!any_op) seg1 = seg0;
-                if (seg1 <= seg0) continue;
-                for (int64_t b0 = seg0; b0 < seg1; b0 += tb)
-                for (int sb = 0; sb < nsub; ++sb, ++it) {
-                    const bool first = b0 == seg0 && sb == 0, last = b0 + tb >= seg1 && sb == nsub - 1;
-                    const int st = (int)(it % NS);
-                    mbar_wait(bar_full + 8 * st, (it / NS) & 1, a.status);
+        // the whole warp waits; one elected lane issues
+        uint32_t it = 0, zi = 0, ai = 0;
+        const uint64_t dK = make_desc(0, 16, 1024);                 // K-major, 128-byte swizzle; addresses are added in 16-byte units
+        const uint32_t z16 = smem_u32(sZ) >> 4, ring16 = smem_u32(sRing) >> 4;
+        const uint32_t xlo16 = (uint32_t)a.x_cap >> 4, zlo16 = (uint32_t)a.z_cap >> 4;
+        for (int64_t v = blockIdx.x; v < a.n_nodes; v += gridDim.x) {
+            int64_t seg0, seg1;
+            et_bounds(a, v, nullptr, seg0, seg1);
+            if (!any_op) seg1 = seg0;
+            if (seg1 <= seg0) continue;
+            for (int64_t b0 = seg0; b0 < seg1; b0 += tb)
+            for (int sb = 0; sb < nsub; ++sb, ++it) {
+                const bool first = b0 == seg0 && sb == 0, last = b0 + tb >= seg1 && sb == nsub - 1;
+                const int st = (int)(it % NS);
+                mbar_wait(bar_full + 8 * st, (it / NS) & 1, a.status);
+                fence_async_smem();
+                tc_fence_after();
+                const uint32_t x16 = ring16 + (((uint32_t)st * stage_bytes) >> 4);
+                for (int ui = 0; ui < S.nunit; ++ui, ++ai) {
+                    const UInfo U = sU[ui];
+                    const uint32_t buf = ai & 1;
+                    if (first) mbar_wait(bar_zfull + 8 * ui, zi & 1, a.status);
+                    if (ai >= 2) mbar_wait(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
                     fence_async_smem();
                     tc_fence_after();
-                    const uint32_t sX_u = smem_u32(sRing + (size_t)st * stage_bytes);
-                    for (int ui = 0; ui < S.nunit; ++ui, ++ai) {
-                        const UInfo U = sU[ui];
-                        const uint32_t buf = ai & 1;
-                        if (first) mbar_wait(bar_zfull + 8 * ui, zi & 1, a.status);
-                        if (ai >= 2) mbar_wait(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
-                        fence_async_smem();
-                        tc_fence_after();
-                        for (uint32_t mt = 0; mt < U.nmt; ++mt) {
-                            const uint32_t d_tmem = tmem_base + buf * (uint32_t)a.acc_cols + mt * U.npad;
+                    const uint32_t xu = x16 + (U.x_off >> 4), zu = z16 + (U.z_off >> 4), d_tmem = tmem_base + buf * (uint32_t)a.acc_cols;
+                    if (elect_one()) {
+                        for (uint32_t mt = 0; mt < U.nmt; ++mt)
+#pragma unroll 4
                             for (uint32_t ks = 0; ks < U.ksteps; ++ks) {
-                                const uint32_t kb = ks >> 2, kk = ks & 3;
-                                const uint32_t xh = sX_u + U.x_off + kb * U.x_kb + mt * (128u * 128u) + 32u * kk;
-                                const uint32_t xl = xh + a.x_cap;
-                                const uint32_t zh = sZ_u + U.z_off + kb * U.z_kb + 32u * kk;
-                                const uint32_t zl = zh + a.z_cap;
-                                const uint64_t dXh = make_desc(xh, 16, 1024), dXl = make_desc(xl, 16, 1024);
-                                const uint64_t dZh = make_desc(zh, 16, 1024), dZl = make_desc(zl, 16, 1024);
-                                tc_mma_bf16(d_tmem, dXh, dZh, U.idesc, ks > 0 ? 1u : 0u);
-                                tc_mma_bf16(d_tmem, dXl, dZh, U.idesc, 1u);
-                                tc_mma_bf16(d_tmem, dXh, dZl, U.idesc, 1u);
+                                const uint32_t kb = ks >> 2, kk = 2u * (ks & 3);
+                                const uint64_t dXh = dK + (xu + kb * (U.x_kb >> 4) + mt * (128u * 128u / 16u) + kk);
+                                const uint64_t dZh = dK + (zu + kb * (U.z_kb >> 4) + kk);
+                                tc_mma_bf16_x3(d_tmem + mt * U.npad, dXh, dXh + xlo16, dZh, dZh + zlo16, U.idesc, ks > 0 ? 1u : 0u);
                             }
-                        }
                         tc_commit(bar_accfull + 8 * buf);
                         if (last) tc_commit(bar_zfree + 8 * ui);
+                        if (ui + 1 == S.nunit) tc_commit(bar_free + 8 * st);
                     }
-                    tc_commit(bar_free + 8 * st);
+                    __syncwarp();
                 }
-                ++zi;
             }
+            ++zi;
         }
     } else {
         // =========================== compute warps ===========================

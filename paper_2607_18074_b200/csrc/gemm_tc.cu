@@ -146,40 +146,37 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            // instruction descriptor: D = F32, A = B = BF16, M = 128, N = BN
-            uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
-            if (g.mn_major) idesc |= (1u << 15) | (1u << 16);
-            for (int kb = 0; kb < num_kb; ++kb) {
-                const int s = kb % S;
-                const uint32_t ph = (kb / S) & 1;
-                mbar_wait(bar0 + 8 * s, ph, g.status);                  // operands landed
-                tc_fence_after();
-                const uint32_t sa = sbase + s * stage_bytes;
-                const uint32_t ah = sa, al = sa + a_bytes, bh = sa + 2 * a_bytes, bl = bh + b_bytes;
+        // the whole warp waits; one elected lane issues
+        // instruction descriptor: D = F32, A = B = BF16, M = 128, N = BN
+        uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(g.BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
+        if (g.mn_major) idesc |= (1u << 15) | (1u << 16);
+        // K-major: rows of 128 B, 8-row groups 1024 B apart; 16 k-elements = 32 B.
+        // MN-major: 64 MN-elements per 128-B row, 8 k-rows per 1024-B group (stride), next 64 MN-elements one box further
+        // (leading); 16 k = two groups
+        const uint32_t kstep16 = g.mn_major ? 2048 >> 4 : 32 >> 4;
+        const uint64_t d0 = g.mn_major ? make_desc(sbase, 64 * BK * 2, 1024) : make_desc(sbase, 16, 1024);
+        for (int kb = 0; kb < num_kb; ++kb) {
+            const int s = kb % S;
+            const uint32_t ph = (kb / S) & 1;
+            mbar_wait(bar0 + 8 * s, ph, g.status);                  // operands landed
+            tc_fence_after();
+            const uint64_t dAh = d0 + ((uint32_t)s * stage_bytes >> 4), dAl = dAh + (a_bytes >> 4), dBh = dAl + (a_bytes >> 4),
+                           dBl = dBh + (b_bytes >> 4);
+            if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k) {
-                    uint64_t dAh, dAl, dBh, dBl;
-                    if (!g.mn_major) {
-                        // K-major: rows of 128 B, 8-row groups 1024 B apart; 16 k-elements = 32 B
-                        dAh = make_desc(ah + 32 * k, 16, 1024); dAl = make_desc(al + 32 * k, 16, 1024);
-                        dBh = make_desc(bh + 32 * k, 16, 1024); dBl = make_desc(bl + 32 * k, 16, 1024);
-                    } else {
-                        // MN-major: 64 MN-elements per 128-B row, 8 k-rows per 1024-B group (stride),
-                        // next 64 MN-elements one box further (leading); 16 k = two groups
-                        dAh = make_desc(ah + 2048 * k, 64 * BK * 2, 1024); dAl = make_desc(al + 2048 * k, 64 * BK * 2, 1024);
-                        dBh = make_desc(bh + 2048 * k, 64 * BK * 2, 1024); dBl = make_desc(bl + 2048 * k, 64 * BK * 2, 1024);
-                    }
-                    const uint32_t first = (kb > 0 || k > 0) ? 1u : 0u;
-                    tc_mma_bf16(tmem_base, dAh, dBh, idesc, first);
-                    if (g.passes != 1) {
-                        tc_mma_bf16(tmem_base, dAl, dBh, idesc, 1u);
-                        tc_mma_bf16(tmem_base, dAh, dBl, idesc, 1u);
-                    }
+                for (uint32_t k = 0; k < BK / 16; ++k) {
+                    const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u, o = k * kstep16;
+                    if (g.passes != 1) tc_mma_bf16_x3(tmem_base, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
+                    else tc_mma_bf16(tmem_base, dAh + o, dBh + o, idesc, acc);
                 }
-                tc_commit(bar0 + 8 * (S + s));                           // frees the slot when the MMAs retire
+                tc_commit(bar0 + 8 * (S + s));                       // frees the slot when the MMAs retire
+                if (kb + 1 == num_kb) tc_commit(bar0 + 8 * 2 * S);   // accumulator complete
             }
-            tc_commit(bar0 + 8 * 2 * S);                                 // accumulator complete
+            __syncwarp();
+        }
+        if (num_kb == 0) {
+            if (elect_one()) tc_commit(bar0 + 8 * 2 * S);
+            __syncwarp();
         }
     } else {
         // epilogue: warp w may touch TMEM lanes 32*(w%4) .. +31

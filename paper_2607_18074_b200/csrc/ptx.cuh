@@ -75,6 +75,28 @@ __device__ __forceinline__ void tc_mma_bf16_ts(uint32_t tmem_d, uint32_t tmem_a,
         "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
         ::"r"(tmem_d), "r"(tmem_a), "l"(db), "r"(idesc), "r"(acc) : "memory");
 }
+// True in one lane of a converged warp.  A tcgen05.mma issued under `if (elect_one())` takes its operands through the
+// uniform registers without a per-instruction hand-over: under `if (lane == 0)` one thread got an instruction accepted
+// every 127 - 138 cycles whatever its shape, under elect_one() every 10 + N/2 (A in tensor memory) and N/2 (A in shared
+// memory, with the collector below; at least 41), measured with dependence-free bursts on all SMs.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\tselp.u32 %0, 1, 0, q;\n\t}" : "=r"(p)::"memory");
+    return p != 0;
+}
+// D (+)= A_hi B_hi + A_hi B_lo + A_lo B_hi of one k-step, A and B in shared memory.  The first two share their A operand:
+// it is kept in the collector buffer and read from shared memory once.
+__device__ __forceinline__ void tc_mma_bf16_x3(uint32_t tmem_d, uint64_t da_hi, uint64_t da_lo, uint64_t db_hi, uint64_t db_lo,
+                                               uint32_t idesc, uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p, t;\n\t"
+        "setp.ne.b32 p, %6, 0;\n\t"
+        "setp.eq.u32 t, 0, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %3, %5, p;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %4, %5, t;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %3, %5, t;\n\t}"
+        ::"r"(tmem_d), "l"(da_hi), "l"(da_lo), "l"(db_hi), "l"(db_lo), "r"(idesc), "r"(acc) : "memory");
+}
 // eight consecutive 32-bit columns of this thread's TMEM lane (lane = 32 * (warp % 4) + lane id)
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* r) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"

@@ -510,7 +510,8 @@ __global__ void __launch_bounds__(TT, 1) k_stream_tc(const TcArgs a) {
         }
     } else if (warp >= W_MMA && warp < W_MMA + NMW) {
         // =========================== MMA warps ===========================
-        if (lane == 0) {
+        // the whole warp waits; one elected lane issues
+        {
             const uint32_t me = (uint32_t)(warp - W_MMA);
             uint32_t mi = 0;
             uint32_t uses[NSLOT];            // how often every slot has been used before the current batch
@@ -552,17 +553,23 @@ __global__ void __launch_bounds__(TT, 1) k_stream_tc(const TcArgs a) {
                             count_wait(fill0 + 4 * slot, 4u * (before + use + 1u), a.status);
                             tc_fence_after();
                             const uint32_t a_h = tmem_base + (uint32_t)RING0 + slot * 16u, a_l = a_h + 8u;
-                            tc_mma_bf16_ts(d_tmem, a_h, dBh, idesc, (first && sl == 0) ? 0u : 1u);
-                            tc_mma_bf16_ts(d_tmem, a_l, dBh, idesc, 1u);
-                            tc_mma_bf16_ts(d_tmem, a_h, dBh + bcap16, idesc, 1u);
-                            tc_commit(bar_slotfree + 8 * slot);
+                            if (elect_one()) {
+                                tc_mma_bf16_ts(d_tmem, a_h, dBh, idesc, (first && sl == 0) ? 0u : 1u);
+                                tc_mma_bf16_ts(d_tmem, a_l, dBh, idesc, 1u);
+                                tc_mma_bf16_ts(d_tmem, a_h, dBh + bcap16, idesc, 1u);
+                                tc_commit(bar_slotfree + 8 * slot);
+                            }
+                            __syncwarp();
                             j = (mw >> 16) & 255u;
                         }
 #pragma unroll
                         for (int s = 0; s < NSLOT; ++s) uses[s] += (uint32_t)(S.nslab + NSLOT - 1 - s) / NSLOT;
                         // (a commit with nothing outstanding arrives at once: every MMA thread takes part)
-                        tc_commit(bar_sfree + 8 * st);
-                        if (b0 + TB >= seg1 && sb == nsub - 1) tc_commit(bar_accfull + 8 * buf);
+                        if (elect_one()) {
+                            tc_commit(bar_sfree + 8 * st);
+                            if (b0 + TB >= seg1 && sb == nsub - 1) tc_commit(bar_accfull + 8 * buf);
+                        }
+                        __syncwarp();
                         if (++st == NS) { st = 0; ++round; }
                     }
                 }
