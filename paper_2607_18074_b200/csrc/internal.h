@@ -163,6 +163,50 @@ struct TcSets {
     int32_t smem_bytes = 0, ctas_per_sm = 1;
 };
 
+// --- moment-form edge stream (moment_stream.cu) --------------------------------------------
+struct MSet {          // a run of source blocks whose gathered rows share the slots of the shared-memory ring
+    int32_t unit_begin, nunit, blk_begin, nblk;
+};
+struct MBlk {          // (part of) a source block: at most 128 multiplicities
+    int32_t src_off, c;       // first element inside a source feature row, multiplicities
+    int32_t c_row, d_src;     // elements between consecutive components, components
+    int32_t slab0, nch;       // first slab of the block in a slot, slabs (64 multiplicities each) per component
+    int32_t pad[2];
+};
+struct MUnit {         // one accumulator: a block x radial indices q0.. x a run of harmonic orders
+    int32_t slab0, d_src;     // first slab of the block, components
+    int32_t halves;           // 2: M = 64 products, even / odd radial indices in the lane halves; 1: M = 128
+    int32_t N, nq, q0;        // columns of one product; radial indices per lane half; first of them
+    int32_t nb, b0;           // harmonics of the run and the first one's offset in the block's list
+    int32_t c, c_row;         // multiplicities, those of the whole source block
+    int32_t row_begin;        // first entry of the column table
+    int32_t task_begin, ntask, pad;
+};
+struct MTask {         // read-out of one (source order, harmonic order, parity of the destination order)
+    int32_t fn, boff;         // (l_src * 5 + l_sh) * 2 + parity; offset of the order in the block's list of harmonics
+    int32_t act;              // bit j: the j-th destination order is wanted
+    int32_t out_ptr[4];       // its paths: outs[out_ptr[j] .. out_ptr[j + 1])
+    int32_t pad;
+};
+struct MOut {          // where a path's state goes
+    int64_t zoff;             // state offset per node of the destination group
+    int32_t ld, koff;         // row pitch, offset in the contraction axis
+    float scale;              // the path's tensor over the unit-norm tensor of its orders
+    int32_t pad;
+};
+struct MomentSets {
+    bool ok = false;
+    std::vector<MSet> sets;
+    std::vector<MBlk> blks;
+    std::vector<MUnit> units;
+    std::vector<MTask> tasks;
+    std::vector<MOut> outs;
+    std::vector<uint16_t> rows;      // per column of a unit: radial index inside the unit | harmonic << 8; 0xffff: padding
+    MSet* d_sets = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MTask* d_tasks = nullptr; MOut* d_outs = nullptr;
+    uint16_t* d_rows = nullptr;
+    int32_t x_cap = 0, slot_bytes = 0, ns = 0, w_bytes = 0, smem_bytes = 0;
+};
+
 struct FStage {        // one 256-column stage of the fused kernel's contraction axis
     int32_t path;
     int32_t u0;        // first multiplicity of the block (256/KP wide)
@@ -193,6 +237,7 @@ struct Direction {
     STask* d_stasks = nullptr;
     SComp* d_scomps = nullptr;
     TcSets tc[2];                     // tensor-core stream: [0] plain, [1] dual
+    MomentSets ms[2];                 // moment-form stream: [0] plain, [1] dual
     TcSets etc[2];                    // tensor-core edge pass: [0] plain, [1] dual
     // receiver-owned edge pass: source-major tasks over all multiplicities
     std::vector<STask> etasks;
@@ -374,6 +419,13 @@ void build_tc_sets(const sobek_plan* p, Direction& dir);
 cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
                              int64_t n_nodes, const SplitSrc& ss, const float* Y, const float* vY, const float* phi,
                              const float* vphi, int dual, void* zh, void* zl, int* status, cudaStream_t s);
+
+// --- moment_stream.cu -------------------------------------------------------------------
+bool cg_scale(const sobek_plan* p, const DPath& P, int ls, int lb, int ld, float& scale);
+void build_moment_sets(const sobek_plan* p, Direction& dir);
+cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
+                                 const SplitSrc& ss, const float* Y, const float* vY, const float* phi, const float* vphi, int dual,
+                                 void* zh, void* zl, int* status, cudaStream_t s);
 
 cudaError_t stream_launch_k8(const void* args, int cls, int t_begin, int t_count, cudaStream_t s);
 cudaError_t stream_launch_k16(const void* args, int cls, int t_begin, int t_count, cudaStream_t s);

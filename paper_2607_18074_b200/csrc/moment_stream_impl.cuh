@@ -1,0 +1,639 @@
+// Edge stream in moment form (sm_100a, tcgen05 / TMEM), warp-specialised.
+//
+// The receiver state (Eqs. angular_path_contraction, receiver_state)
+//     Z_i[path, o, q, u] = sum_e phi_e[q] sum_{s,b} c[s,b,o] Y_e[b] x_{src(e)}[s,u]
+// is linear in the edge's outer product, so the Clebsch-Gordan coefficients come out of the sum over the edges:
+//     P_i[q,b,s,u] = sum_e (phi_e[q] Y_e[b]) x_{src(e)}[s,u]          (moments of the neighbourhood, no coupling in them)
+//     Z_i[path, o, q, u] = sum_{s,b} c[s,b,o] P_i[q,b,s,u]            (once per node)
+// The first line is a dense contraction over the edges: per component s of a source block
+//     D_s[u, (q,b)] = sum_e x_e[s,u] W_e[(q,b)],    W_e[(q,b)] = phi_e[q] Y_e[b],
+// whose first operand is the gathered sender rows as they lie in memory and whose second is K x (harmonics) values per edge,
+// whatever the multiplicity, the number of paths or their order.  The second line is a sparse sum (1.9 terms per moment at order 4)
+// over the node's moments, independent of its degree.  Building the contraction's operand with the coupling folded in
+// (phi_e[q] M_e[s,o]) takes K sum d_src d_dst values per edge instead: 1,840 against 144 at 64 x (0..2), K = 16, 20,832 against
+// 400 at 64 x (0..4), and that build bound the kernel.  fp32 parity comes from the split-bf16 product
+// a*b ~= a_hi*b_hi + a_hi*b_lo + a_lo*b_hi with fp32 accumulation in TMEM; the coupling sums run in fp32.
+//
+// Work items are (set, node): a set is a run of source blocks (128 multiplicities at most each, wider ones are cut) whose gathered
+// rows of 16 edges fit one slot of the shared-memory ring.  An item's accumulators are produced unit after unit: a unit is one
+// block x a range of radial indices x some harmonic orders, at most 256 TMEM columns, so that the two TMEM halves alternate
+// between products and read-out.  Blocks of at most 64 multiplicities use M = 64 products, whose 64 rows take 16 lanes of each
+// 32-lane quarter: the even radial indices go to the lower 16, the odd ones to the upper 16, and every lane has work in the
+// read-out.  When the slots of a node's edges all fit the ring they stay there for all units; longer segments are gathered again
+// for every unit.
+//   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
+//   builder warps  W of one (unit, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
+//   MMA warp       one elected lane issues the three products per component (and lane half);
+//   drain warps    two groups, one per TMEM half, of two teams of four warps that share the unit's radial indices: a lane holds one
+//                  multiplicity, sums the coupling terms (unrolled, coefficients as immediates) and writes bf16 hi / lo.
+// With DUAL the kernel produces the directional state of the double backward (Eq. receiver_double_adjoint)
+//     dP = sum_e (vphi Y + phi vY)[q,b] x[s,u] + (phi Y)[q,b] vx[s,u]
+// as two slots per batch of edges.  The same kernel runs the sender-owned transposed traversal.  Every wait is bounded.
+#pragma once
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "cg_apply.cuh"
+#include "geometry.cuh"
+#include "guard.cuh"
+#include "moment_stream.h"
+#include "ptx.cuh"
+
+namespace sobek {
+namespace {
+
+using namespace ptx;
+
+__device__ __forceinline__ int64_t owner_of(const int64_t* __restrict__ row_ptr, int64_t N, int64_t e) {
+    int64_t lo = 0, hi = N;   // row_ptr[lo] <= e < row_ptr[hi]
+    while (hi - lo > 1) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (__ldg(row_ptr + mid) <= e) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+// (hi, lo) bf16 split of two floats: hi pair, lo pair (element 0 in the low half)
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const float ra = a - __uint_as_float(hi << 16);
+    const float rb = b - __uint_as_float(hi & 0xffff0000u);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(ra, rb);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// ---- read-out: n columns of this thread's TMEM lane, exactly (no load reaches past the accumulator) ----------------
+__device__ __forceinline__ void tm_ld1(uint32_t t, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(v[0]) : "r"(t) : "memory");
+}
+__device__ __forceinline__ void tm_ld2(uint32_t t, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(t) : "memory");
+}
+__device__ __forceinline__ void tm_ld4(uint32_t t, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
+}
+__device__ __forceinline__ void tm_ld8(uint32_t t, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(t) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void tm_ld(uint32_t t, float* v) {
+    if constexpr (N >= 8) { tm_ld8(t, v); if constexpr (N > 8) tm_ld<N - 8>(t + 8, v + 8); }
+    else if constexpr (N >= 4) { tm_ld4(t, v); if constexpr (N > 4) tm_ld<N - 4>(t + 4, v + 4); }
+    else if constexpr (N >= 2) { tm_ld2(t, v); if constexpr (N > 2) tm_ld<N - 2>(t + 2, v + 2); }
+    else if constexpr (N == 1) tm_ld1(t, v);
+}
+// the wait for the loads in flight; the loaded registers pass through it so that nothing that reads them is scheduled ahead
+template <int N>
+__device__ __forceinline__ void tm_wait(float* v) {
+    tc_wait_ld();
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
+}
+
+template <int LS, int LB, int LD, int O0, int I>
+__device__ __forceinline__ void cg_term(const float* p, float* acc) {
+    using T = CGTerms<LS, LB, LD>;
+    constexpr int id = T::id[I];
+    constexpr float c = T::c[I];
+    acc[O0 + (id & 15)] = fmaf(c, p[(id >> 4) & 15], acc[O0 + (id & 15)]);
+}
+template <int LS, int LB, int LD, int O0, int I0, int... I>
+__device__ __forceinline__ void cg_terms(const float* p, float* acc, std::integer_sequence<int, I...>) {
+    (cg_term<LS, LB, LD, O0, I0 + I>(p, acc), ...);
+}
+// the terms of component S for every destination order of the task
+template <int LS, int LB, int PAR, int S, int J>
+__device__ __forceinline__ void cg_row(const float* p, float* acc, uint32_t act) {
+    using Sp = CGSpan<LS, LB, PAR>;
+    if constexpr (J < Sp::n) {
+        using R = CGRange<LS, LB, Sp::ld(J), S>;
+        if constexpr (R::count > 0)
+            if ((act >> J) & 1u) cg_terms<LS, LB, Sp::ld(J), Sp::off(J), R::first>(p, acc, std::make_integer_sequence<int, R::count>());
+        cg_row<LS, LB, PAR, S, J + 1>(p, acc, act);
+    }
+}
+
+// Coupling sums of one radial index: moments in the columns t + s * pitch + b.
+template <int LS, int LB, int PAR>
+struct Coupling {
+    using Sp = CGSpan<LS, LB, PAR>;
+    static constexpr int DB = 2 * LB + 1, DS = 2 * LS + 1;
+    static constexpr int CS = DB >= 7 ? 2 : (DB == 5 ? 3 : (DB == 3 ? 5 : 9));     // components per chunk of loads
+    static constexpr int NC = (DS + CS - 1) / CS;
+    template <int I>      // I: component
+    static __device__ __forceinline__ void load(uint32_t t, uint32_t pitch, float* p) {
+        if constexpr (I < DS) tm_ld<DB>(t + I * pitch, p + (I % CS) * DB);
+        if constexpr ((I + 1) % CS != 0) load<I + 1>(t, pitch, p);
+    }
+    template <int I>
+    static __device__ __forceinline__ void use(const float* p, float* acc, uint32_t act) {
+        if constexpr (I < DS) cg_row<LS, LB, PAR, I, 0>(p + (I % CS) * DB, acc, act);
+        if constexpr ((I + 1) % CS != 0) use<I + 1>(p, acc, act);
+    }
+    template <int C>
+    static __device__ __forceinline__ void step(uint32_t t, uint32_t pitch, float* acc, uint32_t act) {
+        float p[CS * DB];
+#pragma unroll
+        for (int i = 0; i < CS * DB; ++i) p[i] = 0.f;
+        load<C * CS>(t, pitch, p);
+        tm_wait<CS * DB>(p);
+        use<C * CS>(p, acc, act);
+        if constexpr (C + 1 < NC) step<C + 1>(t, pitch, acc, act);
+    }
+};
+
+// the unit that a drain warp reads out
+struct DrainCtx {
+    uint32_t pitch, nb;      // columns between components / between radial indices
+    int ql0, nql;            // radial indices of this warp's team: ql0, ql0 + MS_NDT, ... < nql (counted per lane half)
+    int q0, qs, K;           // this lane's radial index is q0 + ql * qs
+    int c_row;               // multiplicities of the whole source block
+    const MOut* outs;
+    bool full, ok;           // the node has edges; this lane owns a multiplicity
+    int64_t n_nodes, nl;
+    int u;
+    __nv_bfloat16* zh;
+    int64_t lo;              // elements from the hi to the lo array
+};
+
+// where the components of one destination order go: component 0 of radial index 0 of this lane, row pitch
+struct DrainDst { __nv_bfloat16* h; uint32_t ld; float scale; };
+
+template <int DD>
+__device__ __forceinline__ DrainDst drain_dst(const DrainCtx& d, const MOut& o) {
+    const int64_t a = d.n_nodes * o.zoff + d.nl * DD * (int64_t)o.ld + o.koff + d.u;
+    return DrainDst{d.zh + a, (uint32_t)o.ld, o.scale};
+}
+template <int DD>
+__device__ __forceinline__ void drain_write(const DrainCtx& d, const DrainDst& t, uint32_t off, const float* acc) {
+    __nv_bfloat16* l = t.h + d.lo;
+#pragma unroll
+    for (int i = 0; i < DD; ++i, off += t.ld) {
+        const float v = acc[i] * t.scale;
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        t.h[off] = h;
+        l[off] = __float2bfloat16_rn(v - __bfloat162float(h));
+    }
+}
+// f(j, first component, components) for every wanted destination order j
+template <int LS, int LB, int PAR, int J = 0, class F>
+__device__ __forceinline__ void each_dst(uint32_t act, F&& f) {
+    using Sp = CGSpan<LS, LB, PAR>;
+    if constexpr (J < Sp::n) {
+        if ((act >> J) & 1u) f(std::integral_constant<int, J>(), std::integral_constant<int, Sp::off(J)>(), std::integral_constant<int, 2 * Sp::ld(J) + 1>());
+        each_dst<LS, LB, PAR, J + 1>(act, f);
+    }
+}
+
+template <int LS, int LB, int PAR>
+__device__ __forceinline__ void drain_task(const DrainCtx& d, const MTask& task, uint32_t t) {
+    using Sp = CGSpan<LS, LB, PAR>;
+    if constexpr (Sp::n > 0) {
+        const uint32_t act = (uint32_t)task.act;
+        DrainDst dst[Sp::n];
+        each_dst<LS, LB, PAR>(act, [&](auto j, auto, auto dd) { dst[decltype(j)::value] = drain_dst<decltype(dd)::value>(d, d.outs[task.out_ptr[decltype(j)::value]]); });
+#pragma unroll 1
+        for (int ql = d.ql0; ql < d.nql; ql += MS_NDT) {
+            float acc[Sp::NO];
+#pragma unroll
+            for (int i = 0; i < Sp::NO; ++i) acc[i] = 0.f;
+            if (d.full) Coupling<LS, LB, PAR>::template step<0>(t + (uint32_t)ql * d.nb, d.pitch, acc, act);
+            const int q = d.q0 + ql * d.qs;
+            if (d.ok && q < d.K) {
+                const uint32_t off = (uint32_t)(q * d.c_row);
+                each_dst<LS, LB, PAR>(act, [&](auto j, auto o0, auto dd) {
+                    constexpr int DD = decltype(dd)::value, J = decltype(j)::value;
+                    drain_write<DD>(d, dst[J], off, acc + decltype(o0)::value);
+                    for (int k = task.out_ptr[J] + 1; k < task.out_ptr[J + 1]; ++k)      // further destinations of the same order
+                        drain_write<DD>(d, drain_dst<DD>(d, d.outs[k]), off, acc + decltype(o0)::value);
+                });
+            }
+        }
+    }
+}
+__device__ __forceinline__ void drain_pick(const DrainCtx& d, const MTask& task, uint32_t t) {
+#define SOBEK_FN(ls, lb)                                                        \
+    case (ls * 5 + lb) * 2: drain_task<ls, lb, 0>(d, task, t); break;           \
+    case (ls * 5 + lb) * 2 + 1: drain_task<ls, lb, 1>(d, task, t); break;
+#define SOBEK_FN5(ls) SOBEK_FN(ls, 0) SOBEK_FN(ls, 1) SOBEK_FN(ls, 2) SOBEK_FN(ls, 3) SOBEK_FN(ls, 4)
+    switch (task.fn) { SOBEK_FN5(0) SOBEK_FN5(1) SOBEK_FN5(2) SOBEK_FN5(3) SOBEK_FN5(4) default: break; }
+#undef SOBEK_FN5
+#undef SOBEK_FN
+}
+
+// Every role walks the same items; the next item's bounds are requested one item ahead.
+struct MsItem { int set; int64_t nl, seg0; int len, nslot; bool resident; };
+struct MsWalk {
+    const MsArgs& a;
+    int64_t v, nl, s0, s1;
+    int set, nsub, ns;
+    int* st;
+    __device__ MsWalk(const MsArgs& a_, int nsub_, int ns_, int* st_) : a(a_), nl(0), s0(0), s1(0), nsub(nsub_), ns(ns_), st(st_) {
+        v = blockIdx.x % a.n_nodes; set = (int)(blockIdx.x / a.n_nodes);
+        fetch();
+    }
+    __device__ void fetch() {
+        if (set >= a.nsets) return;
+        if (a.oseg) { const int4 q = __ldg(a.oseg + v); nl = q.x; s0 = q.y; s1 = q.z; return; }
+        seg_bounds(a.ev.ptr, a.node0 + v, a.ev.E, st, s0, s1);
+        nl = v;
+    }
+    __device__ bool next(MsItem& it) {
+        if (set >= a.nsets) return false;
+        it.set = set; it.nl = nl; it.seg0 = s0; it.len = nsub ? (int)(s1 - s0) : 0;
+        it.nslot = ((it.len + MS_TB - 1) / MS_TB) * nsub;
+        it.resident = it.nslot <= ns;
+        v += gridDim.x;
+        while (v >= a.n_nodes && set < a.nsets) { v -= a.n_nodes; ++set; }
+        fetch();
+        return true;
+    }
+};
+
+template <bool DUAL>
+__global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    constexpr int TB = MS_TB, PS = MS_PS, NW = MS_NW, SLAB = MS_SLAB, HALF = MS_HALF;
+    constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_GEO = W_MMA + 1;
+    const int NS = a.ns;
+    uint8_t* sRing = smem;                                            // slots: x hi, x lo, raw phi / Y (+ directions)
+    uint8_t* sW = sRing + (size_t)NS * a.slot_bytes;                  // W ring: hi rows, lo rows
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sW + (size_t)NW * a.w_bytes);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + MS_NBAR);
+    MOut* sOut = reinterpret_cast<MOut*>(tmem_holder + 4);
+    MSet* sSet = reinterpret_cast<MSet*>(sOut + a.n_outs);
+    MBlk* sBlk = reinterpret_cast<MBlk*>(sSet + a.nsets);
+    MUnit* sUnit = reinterpret_cast<MUnit*>(sBlk + a.n_blks);
+    MTask* sTask = reinterpret_cast<MTask*>(sUnit + a.n_units);
+    uint16_t* sRow = reinterpret_cast<uint16_t*>(sTask + a.n_tasks);
+    const uint32_t bar0 = smem_u32(bars);
+    const uint32_t bar_full = bar0, bar_sfree = bar0 + 8 * MS_MAXNS, bar_wfull = bar0 + 16 * MS_MAXNS, bar_wfree = bar_wfull + 8 * NW,
+                   bar_accfull = bar_wfree + 8 * NW, bar_accfree = bar_accfull + 16;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool has_vx = DUAL && a.vsh != nullptr, has_vY = DUAL && (a.rvec ? a.vrvec != nullptr : a.vY != nullptr),
+               has_vphi = DUAL && (a.rvec ? a.vrvec != nullptr : a.vphi != nullptr);
+    const bool has_a1 = !DUAL || has_vY || has_vphi;   // operand 1: phi Y (plain) or vphi Y + phi vY (dual), times x
+    const bool has_a2 = has_vx;                        // operand 2 (dual): phi Y, times vx
+    const int nsub = (has_a1 ? 1 : 0) + (has_a2 ? 1 : 0);
+
+    if (tid == 0) {
+        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, NLW * 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 1); }
+        for (int s = 0; s < NW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 1); }
+        for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, 4 * MS_NDT); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    {   // raw rows of absent directions stay zero for ever
+        const int words = a.slot_bytes / 4, x_words = 2 * a.x_cap / 4;
+        for (int s = 0; s < NS; ++s)
+            for (int i = x_words + tid; i < words; i += MS_TT) reinterpret_cast<uint32_t*>(sRing + (size_t)s * a.slot_bytes)[i] = 0u;
+    }
+    auto table = [&](void* dst, const void* src, int bytes) {
+        for (int i = tid; i < bytes / 2; i += MS_TT) reinterpret_cast<uint16_t*>(dst)[i] = reinterpret_cast<const uint16_t*>(src)[i];
+    };
+    table(sOut, a.outs, a.n_outs * (int)sizeof(MOut)); table(sSet, a.sets, a.nsets * (int)sizeof(MSet));
+    table(sBlk, a.blks, a.n_blks * (int)sizeof(MBlk)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit));
+    table(sTask, a.tasks, a.n_tasks * (int)sizeof(MTask)); table(sRow, a.rows, a.n_rows * 2);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+
+    if (warp >= W_LOAD && warp < W_LOAD + NLW) {
+        // =========================== loader warps ===========================
+        const int lt = (warp - W_LOAD) * 32 + lane;
+        const int le = lane & (TB - 1);
+        MsWalk walk(a, nsub, NS, a.status);
+        MsItem it{};
+        int rep = 0, nrep = 0, b0 = 0, sub = 0;
+        // position of the next slot's batch; false at the end
+        auto advance = [&](bool first) -> bool {
+            if (!first) {
+                if (++sub < nsub) return true;
+                sub = 0; b0 += TB;
+                if (b0 < it.len) return true;
+                b0 = 0;
+                if (++rep < nrep) return true;
+            }
+            for (;;) {
+                if (!walk.next(it)) return false;
+                if (it.len == 0) continue;
+                rep = 0; b0 = 0; sub = 0; nrep = it.resident ? 1 : sSet[it.set].nunit;
+                return true;
+            }
+        };
+        // lane e < 16 holds edge e of the batch; bit e of msk says that the edge exists and that its ids are in range (an id
+        // that is not turns the edge's copies into zero fills and is reported in the status word)
+        auto load_ids = [&](int64_t& eid, int32_t& sn, uint32_t& msk) {
+            eid = 0; sn = 0;
+            bool ok = false;
+            if (b0 + lane < it.len && lane < TB) {
+                const int64_t pos = it.seg0 + b0 + lane;
+                eid = a.ev.perm ? (int64_t)a.ev.perm[pos] : pos;
+                ok = id_ok(eid, a.ev.E, a.status);
+                if (ok) {
+                    const int64_t v = a.ev.transposed ? (a.ev.recv ? (int64_t)a.ev.recv[pos] : owner_of(a.ev.row_ptr, a.ev.N, eid))
+                                                      : (int64_t)a.ev.col[eid];
+                    ok = id_ok(v, a.ev.N, a.status);
+                    sn = ok ? (int32_t)v : 0;
+                } else {
+                    eid = 0;
+                }
+            }
+            msk = __ballot_sync(0xffffffffu, ok);
+        };
+        bool have = advance(true);
+        int64_t eid = 0; int32_t sn = 0; uint32_t msk = 0;
+        if (have) load_ids(eid, sn, msk);
+        int st = 0; uint32_t round = 0;
+        while (have) {
+            const MSet S = sSet[it.set];
+            const int op = has_a1 ? sub : 1;
+            have = advance(false);
+            int64_t eid_n = 0; int32_t sn_n = 0; uint32_t msk_n = 0;
+            if (have) load_ids(eid_n, sn_n, msk_n);
+            if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
+            const uint32_t slot_u = smem_u32(sRing + (size_t)st * a.slot_bytes);
+            const uint32_t raw_u = slot_u + (uint32_t)(2 * a.x_cap);
+            if (!a.rvec) {
+                // phi and Y, transposed: thread <-> (edge le, every fourth radial index / harmonic)
+                const int64_t ee = __shfl_sync(0xffffffffu, eid, le);
+                const uint32_t ok = ((msk >> le) & 1u) * 4u;
+                for (int q = lt >> 4; q < a.K; q += NLW * 32 / TB) {
+                    cp_async4_zfill(raw_u + (uint32_t)(q * PS + le) * 4, a.phi + ee * a.K + q, ok);
+                    if (has_vphi) cp_async4_zfill(raw_u + (uint32_t)((a.K + a.dsh + q) * PS + le) * 4, a.vphi + ee * a.K + q, ok);
+                }
+                for (int b = lt >> 4; b < a.dsh; b += NLW * 32 / TB) {
+                    cp_async4_zfill(raw_u + (uint32_t)((a.K + b) * PS + le) * 4, a.Y + ee * a.dsh + b, ok);
+                    if (has_vY) cp_async4_zfill(raw_u + (uint32_t)((2 * a.K + a.dsh + b) * PS + le) * 4, a.vY + ee * a.dsh + b, ok);
+                }
+            }
+            // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: up to sixteen consecutive threads per row
+            const __nv_bfloat16* baseh = op == 0 ? a.sh : a.vsh;
+            const __nv_bfloat16* basel = op == 0 ? a.sl : a.vsl;
+            for (int bi = 0; bi < S.nblk; ++bi) {
+                const MBlk B = sBlk[S.blk_begin + bi];
+                const int cpr = (B.c + 7) >> 3;
+                const int lgp = cpr > 8 ? 4 : (cpr > 4 ? 3 : (cpr > 2 ? 2 : 1));
+                const int j = lt & ((1 << lgp) - 1), rows = (NLW * 32) >> lgp, nsg = rows > TB ? rows / TB : 1, sg = (lt >> lgp) / TB;
+#pragma unroll 1
+                for (int re0 = 0; re0 < TB; re0 += rows) {
+                    const int re = re0 + ((lt >> lgp) & (TB - 1));
+                    const int32_t sne = __shfl_sync(0xffffffffu, sn, re);
+                    if (j < cpr) {
+                        const uint32_t ok = ((msk >> re) & 1u) * 16u;
+                        const int64_t g = (int64_t)sne * a.C_src + B.src_off + 8 * j;
+                        const int step = nsg * B.nch * SLAB;
+                        uint32_t dst = slot_u + (uint32_t)((B.slab0 + sg * B.nch + (j >> 3)) * SLAB + re * 128 + (((j & 7) ^ (re & 7)) << 4));
+                        const __nv_bfloat16* ph = baseh + g + sg * B.c_row;
+                        const __nv_bfloat16* pl = basel + g + sg * B.c_row;
+                        for (int s = sg; s < B.d_src; s += nsg) {
+                            cp_async16_zfill(dst, ph, ok);
+                            cp_async16_zfill(dst + (uint32_t)a.x_cap, pl, ok);
+                            dst += (uint32_t)step; ph += nsg * B.c_row; pl += nsg * B.c_row;
+                        }
+                    }
+                }
+            }
+            // this thread's arrival on the slot's barrier fires when all its copies above have landed
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st) : "memory");
+            eid = eid_n; sn = sn_n; msk = msk_n;
+            if (++st == NS) { st = 0; ++round; }
+        }
+    } else if (warp == W_GEO) {
+        // =========================== geometry warp ===========================
+        // Walks the same slots as the loaders and fills their phi and Y rows from the edge vectors (lane <-> edge lane & 15, half
+        // of the radial indices / components each).
+        if (a.rvec != nullptr) {
+            MsWalk walk(a, nsub, NS, nullptr);
+            MsItem it{};
+            const int le = lane & (TB - 1), hf = lane >> 4;
+            int st = 0; uint32_t round = 0;
+            while (walk.next(it)) {
+                if (it.len == 0) continue;
+                const int nrep = it.resident ? 1 : sSet[it.set].nunit;
+                for (int rep = 0; rep < nrep; ++rep)
+                for (int b0 = 0; b0 < it.len; b0 += TB) {
+                    bool okb = b0 + le < it.len;
+                    int64_t ee = 0;
+                    if (okb) { const int64_t pos = it.seg0 + b0 + le; ee = a.ev.perm ? (int64_t)a.ev.perm[pos] : pos; okb = ee >= 0 && ee < a.ev.E; }
+                    float rx = 0.f, ry = 0.f, rz = 1.f;
+                    if (okb) { const float* rp = a.rvec + ee * 3; rx = __ldg(rp); ry = __ldg(rp + 1); rz = __ldg(rp + 2); }
+                    const float r = sqrtf(rx * rx + ry * ry + rz * rz), ir = 1.f / r;
+                    const float ux = rx * ir, uy = ry * ir, uz = rz * ir;
+                    // DUAL: the directions vphi = phi'(r) (u . v) and vY = grad F . (v - u (u . v)) / r of the edge-vector direction v
+                    float uv = 0.f, tx = 0.f, ty = 0.f, tz = 0.f;
+                    const bool dirs = DUAL && a.vrvec != nullptr;
+                    if (dirs && okb) {
+                        const float* vp = a.vrvec + ee * 3;
+                        const float vx_ = __ldg(vp), vy_ = __ldg(vp + 1), vz_ = __ldg(vp + 2);
+                        uv = ux * vx_ + uy * vy_ + uz * vz_;
+                        tx = (vx_ - ux * uv) * ir; ty = (vy_ - uy * uv) * ir; tz = (vz_ - uz * uv) * ir;
+                    }
+                    for (int sub = 0; sub < nsub; ++sub) {       // the slots of the operand pairs need the same rows
+                        if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
+                        float* F = reinterpret_cast<float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
+                        float* Yt = F + a.K * PS;
+                        const int dv = (a.K + a.dsh) * PS, dsh = a.dsh;
+                        geo_radial(r, a.K, a.geo_rc, a.geo_basis, a.geo_p, [&](int q, float f, float df) {
+                            if ((q & 1) == hf) {
+                                F[q * PS + le] = okb ? f : 0.f;
+                                if (dirs) F[dv + q * PS + le] = okb ? df * uv : 0.f;
+                            }
+                        });
+                        geo_sh(ux, uy, uz, [&](int b, float yb, float fx, float fy, float fz) {
+                            if (b < dsh && (b & 1) == hf) {
+                                Yt[b * PS + le] = okb ? yb : 0.f;
+                                if (dirs) Yt[dv + b * PS + le] = okb ? fx * tx + fy * ty + fz * tz : 0.f;
+                            }
+                        });
+                        mbar_arrive(bar_full + 8 * st);      // release: the stores above are visible to whoever sees the slot full
+                        if (++st == NS) { st = 0; ++round; }
+                    }
+                }
+            }
+        }
+    } else if (warp >= W_BUILD && warp < W_BUILD + NBW) {
+        // =========================== builder warps ===========================
+        const int bt = (warp - W_BUILD) * 32 + lane;
+        MsWalk walk(a, nsub, NS, nullptr);
+        MsItem it{};
+        int st0 = 0; uint32_t r0 = 0;          // slot and round of the item's first slot
+        int ws = 0; uint32_t wr = 0;
+        while (walk.next(it)) {
+            if (it.len == 0) continue;
+            const MSet S = sSet[it.set];
+            int st = st0; uint32_t rd = r0;
+            for (int ui = 0; ui < S.nunit; ++ui) {
+                if (it.resident) { st = st0; rd = r0; }
+                const MUnit U = sUnit[S.unit_begin + ui];
+                const uint16_t* rt = sRow + U.row_begin;
+                const int rows = U.N * U.halves;
+                for (int j = 0; j < it.nslot; ++j) {
+                    const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
+                    mbar_wait(bar_full + 8 * st, rd & 1, a.status);
+                    if (wr > 0) mbar_wait(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
+                    const float* F = reinterpret_cast<const float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
+                    const float* Yt = F + a.K * PS;
+                    const int dv = (a.K + a.dsh) * PS;
+                    uint8_t* w = sW + (size_t)ws * a.w_bytes;
+                    for (int i = bt; i < 2 * rows; i += NBW * 32) {       // (row, eight edges)
+                        const int n = ((i >> 4) << 3) | (i & 7), h = (i >> 3) & 1;
+                        const uint32_t qb = rt[n];
+                        const int q = U.q0 + (int)(qb & 255u), b = (int)(qb >> 8);
+                        if (qb == 0xffffu || q >= a.K) continue;      // a column that no sum reads
+                        float f[8], y[8], v[8];
+                        *reinterpret_cast<float4*>(f) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h);
+                        *reinterpret_cast<float4*>(f + 4) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h + 4);
+                        *reinterpret_cast<float4*>(y) = *reinterpret_cast<const float4*>(Yt + b * PS + 8 * h);
+                        *reinterpret_cast<float4*>(y + 4) = *reinterpret_cast<const float4*>(Yt + b * PS + 8 * h + 4);
+                        if (DUAL && op == 0) {
+                            float vf[8], vy[8];
+                            *reinterpret_cast<float4*>(vf) = *reinterpret_cast<const float4*>(F + dv + q * PS + 8 * h);
+                            *reinterpret_cast<float4*>(vf + 4) = *reinterpret_cast<const float4*>(F + dv + q * PS + 8 * h + 4);
+                            *reinterpret_cast<float4*>(vy) = *reinterpret_cast<const float4*>(Yt + dv + b * PS + 8 * h);
+                            *reinterpret_cast<float4*>(vy + 4) = *reinterpret_cast<const float4*>(Yt + dv + b * PS + 8 * h + 4);
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) v[e] = fmaf(vf[e], y[e], f[e] * vy[e]);
+                        } else {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) v[e] = f[e] * y[e];
+                        }
+                        uint4 hi, lo;
+                        split2(v[0], v[1], hi.x, lo.x); split2(v[2], v[3], hi.y, lo.y);
+                        split2(v[4], v[5], hi.z, lo.z); split2(v[6], v[7], hi.w, lo.w);
+                        uint8_t* d = w + (n >> 3) * 256 + h * 128 + (n & 7) * 16;
+                        *reinterpret_cast<uint4*>(d) = hi;
+                        *reinterpret_cast<uint4*>(d + rows * 32) = lo;
+                    }
+                    fence_async_smem();
+                    mbar_arrive(bar_wfull + 8 * ws);
+                    if (++ws == NW) { ws = 0; ++wr; }
+                    if (++st == NS) { st = 0; ++rd; }
+                }
+            }
+            st0 = st; r0 = rd;
+        }
+    } else if (warp == W_MMA) {
+        // =========================== MMA warp ===========================
+        MsWalk walk(a, nsub, NS, nullptr);
+        MsItem it{};
+        int st0 = 0; uint32_t r0 = 0;
+        int ws = 0; uint32_t wr = 0, ai = 0;
+        const uint64_t dX0 = make_desc(smem_u32(sRing), SLAB, 1024);          // 64 multiplicities per row, the next 64 a slab on
+        const uint64_t dW0 = make_desc_plain(smem_u32(sW), 128, 256);
+        const uint32_t slot16 = (uint32_t)a.slot_bytes >> 4, w16 = (uint32_t)a.w_bytes >> 4, xlo16 = (uint32_t)a.x_cap >> 4;
+        while (walk.next(it)) {
+            if (it.len == 0) continue;
+            const MSet S = sSet[it.set];
+            int st = st0; uint32_t rd = r0;
+            for (int ui = 0; ui < S.nunit; ++ui, ++ai) {
+                if (it.resident) { st = st0; rd = r0; }
+                const MUnit U = sUnit[S.unit_begin + ui];
+                const uint32_t buf = ai & 1;
+                // D = F32, A = B = BF16, A MN-major, B K-major, M = 128 / halves
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(U.N >> 3) << 17) | ((8u / (uint32_t)U.halves) << 24);
+                if (ai >= 2) mbar_wait(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
+                tc_fence_after();
+                const uint32_t d0 = tmem_base + buf * HALF, wlo16 = (uint32_t)(U.N * U.halves * 2), sl16 = (uint32_t)((U.halves == 1 ? 2 : 1) * (SLAB >> 4));
+                const bool release = ui + 1 == S.nunit || !it.resident;
+                for (int j = 0; j < it.nslot; ++j) {
+                    mbar_wait(bar_full + 8 * st, rd & 1, a.status);
+                    mbar_wait(bar_wfull + 8 * ws, wr & 1, a.status);
+                    fence_async_smem();      // the gathered rows were written through the generic proxy
+                    tc_fence_after();
+                    const uint64_t dX = dX0 + ((uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4)), dW = dW0 + (uint32_t)ws * w16;
+                    if (elect_one()) {
+                        for (int h = 0; h < U.halves; ++h) {
+                            const uint64_t dWh = dW + (uint32_t)(h * U.N * 2);
+                            const uint32_t dh = d0 + ((uint32_t)(16 * h) << 16);
+#pragma unroll 3
+                            for (int s = 0; s < U.d_src; ++s)
+                                tc_mma_bf16_x3(dh + (uint32_t)(s * U.N), dX + (uint32_t)s * sl16, dX + (uint32_t)s * sl16 + xlo16, dWh, dWh + wlo16, idesc, j > 0 ? 1u : 0u);
+                        }
+                        tc_commit(bar_wfree + 8 * ws);
+                        if (release) tc_commit(bar_sfree + 8 * st);
+                        if (j + 1 == it.nslot) tc_commit(bar_accfull + 8 * buf);
+                    }
+                    __syncwarp();
+                    if (++ws == NW) { ws = 0; ++wr; }
+                    if (++st == NS) { st = 0; ++rd; }
+                }
+            }
+            st0 = st; r0 = rd;
+        }
+    } else if (warp < NDW) {
+        // =========================== drain warps ===========================
+        const int grp = warp / (4 * MS_NDT), quarter = warp & 3;
+        MsWalk walk(a, nsub, NS, nullptr);
+        MsItem it{};
+        uint32_t ai = 0;
+        DrainCtx d;
+        d.n_nodes = a.n_nodes; d.zh = a.zh; d.lo = a.zl - a.zh; d.outs = sOut; d.K = a.K; d.ql0 = (warp >> 2) % MS_NDT;
+        while (walk.next(it)) {
+            const MSet S = sSet[it.set];
+            d.nl = it.nl; d.full = it.len > 0;
+            for (int ui = 0; ui < S.nunit; ++ui) {
+                const uint32_t buf = d.full ? (ai & 1) : (uint32_t)(ui & 1);
+                const uint32_t par = (ai >> 1) & 1;
+                if (d.full) ++ai;
+                if (buf != (uint32_t)grp) continue;
+                const MUnit U = sUnit[S.unit_begin + ui];
+                if (d.full) {
+                    mbar_wait(bar_accfull + 8 * buf, par, a.status);
+                    tc_fence_after();
+                }
+                const int uw = U.halves == 2 ? 16 : 32;          // multiplicities of a quarter
+                if (quarter * uw < U.c) {
+                    d.u = quarter * uw + (lane & (uw - 1));
+                    d.ok = d.u < U.c;
+                    d.q0 = U.q0 + (U.halves == 2 ? lane >> 4 : 0); d.qs = U.halves; d.nql = U.nq;
+                    d.pitch = (uint32_t)U.N; d.nb = (uint32_t)U.nb; d.c_row = U.c_row;
+                    const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF - (uint32_t)U.b0;
+                    for (int ti = 0; ti < U.ntask; ++ti) {
+                        const MTask& T = sTask[U.task_begin + ti];
+                        drain_pick(d, T, t0 + (uint32_t)T.boff);
+                    }
+                }
+                if (d.full) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_accfree + 8 * buf);
+                }
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    }
+}
+
+template <bool DUAL>
+cudaError_t moment_stream_launch(const MsArgs& a, int grid, int smem, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_moment_stream<DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    k_moment_stream<DUAL><<<grid, MS_TT, smem, s>>>(a);
+    return cudaGetLastError();
+}
+
+}  // namespace
+}  // namespace sobek

@@ -512,6 +512,15 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
         if (e == cudaSuccess) e = upload(d->fs_begin, &d->d_fs_begin);
         if (e == cudaSuccess) e = upload(d->fs_count, &d->d_fs_count);
         if (e == cudaSuccess) e = upload(d->fk_off, &d->d_fk_off);
+        for (MomentSets& t : d->ms) {
+            if (!t.ok) continue;
+            if (e == cudaSuccess) e = upload(t.sets, &t.d_sets);
+            if (e == cudaSuccess) e = upload(t.blks, &t.d_blks);
+            if (e == cudaSuccess) e = upload(t.units, &t.d_units);
+            if (e == cudaSuccess) e = upload(t.tasks, &t.d_tasks);
+            if (e == cudaSuccess) e = upload(t.outs, &t.d_outs);
+            if (e == cudaSuccess) e = upload(t.rows, &t.d_rows);
+        }
         for (TcSets* tp : {&d->tc[0], &d->tc[1], &d->etc[0], &d->etc[1]}) {
             TcSets& t = *tp;
             if (!t.ok) continue;
@@ -562,6 +571,9 @@ extern "C" void sobek_plan_destroy(sobek_plan* p) {
         cudaFree(d->d_kn_off); cudaFree(d->d_nk_off); cudaFree(d->d_kn_ld); cudaFree(d->d_nk_ld); cudaFree(d->d_path_group);
         cudaFree(d->d_stasks); cudaFree(d->d_scomps); cudaFree(d->d_etasks); cudaFree(d->d_ecomps); cudaFree(d->d_zb_off);
         cudaFree(d->d_fstages); cudaFree(d->d_fs_begin); cudaFree(d->d_fs_count); cudaFree(d->d_fk_off);
+        for (MomentSets& t : d->ms) {
+            cudaFree(t.d_sets); cudaFree(t.d_blks); cudaFree(t.d_units); cudaFree(t.d_tasks); cudaFree(t.d_outs); cudaFree(t.d_rows);
+        }
         for (TcSets* tp : {&d->tc[0], &d->tc[1], &d->etc[0], &d->etc[1]}) {
             TcSets& t = *tp;
             cudaFree(t.d_inv_ptr); cudaFree(t.d_inv);

@@ -144,6 +144,11 @@ __device__ __forceinline__ uint64_t make_desc(uint32_t saddr, uint32_t lbo_bytes
     d |= (uint64_t)2 << 61;   // SWIZZLE_128B
     return d;
 }
+// the same without swizzle, K-major: core matrices of 8 rows x 16 bytes, lbo apart along k, sbo along the rows
+__device__ __forceinline__ uint64_t make_desc_plain(uint32_t saddr, uint32_t lbo_bytes, uint32_t sbo_bytes) {
+    return (uint64_t)((saddr >> 4) & 0x3FFF) | (uint64_t)((lbo_bytes >> 4) & 0x3FFF) << 16 |
+           (uint64_t)((sbo_bytes >> 4) & 0x3FFF) << 32 | (uint64_t)1 << 46;
+}
 
 
 // host side: tensor-map encoder fetched from the driver at run time (no link-time dependency)
