@@ -236,7 +236,6 @@ struct Direction {
     std::vector<SClass> sclasses;
     STask* d_stasks = nullptr;
     SComp* d_scomps = nullptr;
-    TcSets tc[2];                     // tensor-core stream: [0] plain, [1] dual
     MomentSets ms[2];                 // moment-form stream: [0] plain, [1] dual
     TcSets etc[2];                    // tensor-core edge pass: [0] plain, [1] dual
     // receiver-owned edge pass: source-major tasks over all multiplicities
@@ -414,12 +413,6 @@ cudaError_t launch_edge_pass_tc(const sobek_plan* p, const Direction& dir, const
                                 int64_t n_nodes, const SplitSrc& ss, const float* Y, const float* vY, const float* phi,
                                 const float* vphi, int dual, const void* zqh, const void* zql, float* gphi, float* gY,
                                 int phi_mode, int Y_mode, int* status, cudaStream_t s);
-// --- stream_tc.cu ---------------------------------------------------------------------
-void build_tc_sets(const sobek_plan* p, Direction& dir);
-cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
-                             int64_t n_nodes, const SplitSrc& ss, const float* Y, const float* vY, const float* phi,
-                             const float* vphi, int dual, void* zh, void* zl, int* status, cudaStream_t s);
-
 // --- moment_stream.cu -------------------------------------------------------------------
 bool cg_scale(const sobek_plan* p, const DPath& P, int ls, int lb, int ld, float& scale);
 void build_moment_sets(const sobek_plan* p, Direction& dir);
