@@ -143,7 +143,7 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
         T.w_bytes = max_rows * 64;
         const int tables = (int)(T.outs.size() * sizeof(MOut) + parts.size() * (sizeof(MSet) + sizeof(MBlk)) + n_units * sizeof(MUnit) +
                                  T.tasks.size() * sizeof(MTask) + T.rows.size() * 2 + 64);
-        const int fixed = 1024 + MS_NW * T.w_bytes + MS_NBAR * 8 + 16 + tables;
+        const int fixed = 1024 + MS_NW * T.w_bytes + MS_NBAR * 8 + 16 + MS_NDW * MS_CTX + tables;
         // Sets: consecutive parts whose rows of 16 edges leave room for four slots (a node of 32 edges and the next one's
         // first rows); a wider part is a set of its own with the slots it leaves, at least two.
         const int slot4 = ((kSmem - fixed) / 4) & ~1023;

@@ -152,37 +152,39 @@ struct Coupling {
     }
 };
 
-// the unit that a drain warp reads out
+// What a drain warp needs to read out a unit, in shared memory (written by the warp itself): the read-out functions below are
+// not inlined, so that their registers do not compete with the state of the walk (inlined, the spills of it made up half of
+// the kernel's time: with the shared memory taken, next to no L1 is left to serve them).
 struct DrainCtx {
-    uint32_t pitch, nb;      // columns between components / between radial indices
-    int ql0, nql;            // radial indices of this warp's team: ql0, ql0 + MS_NDT, ... < nql (counted per lane half)
-    int q0, qs, K;           // this lane's radial index is q0 + ql * qs
-    int c_row;               // multiplicities of the whole source block
-    const MOut* outs;
-    bool full, ok;           // the node has edges; this lane owns a multiplicity
+    __nv_bfloat16 *zh, *zl;
     int64_t n_nodes, nl;
-    int u;
-    __nv_bfloat16* zh;
-    int64_t lo;              // elements from the hi to the lo array
+    const MOut* outs;
+    uint32_t t0;             // TMEM address of the unit's first column in this warp's lanes
+    uint32_t pitch, nb;      // columns between components / between radial indices
+    int32_t ql0, nql;        // radial indices of this warp's team: ql0, ql0 + MS_NDT, ... < nql (counted per lane half)
+    int32_t q0, halves, K;
+    int32_t c, c_row;        // multiplicities of the block, of the whole source block
+    int32_t quarter, full;   // TMEM lane quarter of the warp; the node has edges
 };
 
+static_assert(sizeof(DrainCtx) == MS_CTX, "context size");
+
 // where the components of one destination order go: component 0 of radial index 0 of this lane, row pitch
-struct DrainDst { __nv_bfloat16* h; uint32_t ld; float scale; };
+struct DrainDst { int64_t a; uint32_t ld; float scale; };
 
 template <int DD>
-__device__ __forceinline__ DrainDst drain_dst(const DrainCtx& d, const MOut& o) {
-    const int64_t a = d.n_nodes * o.zoff + d.nl * DD * (int64_t)o.ld + o.koff + d.u;
-    return DrainDst{d.zh + a, (uint32_t)o.ld, o.scale};
+__device__ __forceinline__ DrainDst drain_dst(const DrainCtx& d, const MOut& o, int u) {
+    return DrainDst{d.n_nodes * o.zoff + d.nl * DD * (int64_t)o.ld + o.koff + u, (uint32_t)o.ld, o.scale};
 }
 template <int DD>
-__device__ __forceinline__ void drain_write(const DrainCtx& d, const DrainDst& t, uint32_t off, const float* acc) {
-    __nv_bfloat16* l = t.h + d.lo;
+__device__ __forceinline__ void drain_write(__nv_bfloat16* zh, __nv_bfloat16* zl, const DrainDst& t, uint32_t off, const float* acc) {
+    __nv_bfloat16 *h = zh + t.a, *l = zl + t.a;
 #pragma unroll
     for (int i = 0; i < DD; ++i, off += t.ld) {
         const float v = acc[i] * t.scale;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        t.h[off] = h;
-        l[off] = __float2bfloat16_rn(v - __bfloat162float(h));
+        const __nv_bfloat16 b = __float2bfloat16_rn(v);
+        h[off] = b;
+        l[off] = __float2bfloat16_rn(v - __bfloat162float(b));
     }
 }
 // f(j, first component, components) for every wanted destination order j
@@ -195,40 +197,54 @@ __device__ __forceinline__ void each_dst(uint32_t act, F&& f) {
     }
 }
 
+// ctx, task: shared-memory addresses
 template <int LS, int LB, int PAR>
-__device__ __forceinline__ void drain_task(const DrainCtx& d, const MTask& task, uint32_t t) {
+__device__ __noinline__ void drain_task(uint32_t ctx_u, uint32_t task_u) {
     using Sp = CGSpan<LS, LB, PAR>;
-    if constexpr (Sp::n > 0) {
-        const uint32_t act = (uint32_t)task.act;
-        DrainDst dst[Sp::n];
-        each_dst<LS, LB, PAR>(act, [&](auto j, auto, auto dd) { dst[decltype(j)::value] = drain_dst<decltype(dd)::value>(d, d.outs[task.out_ptr[decltype(j)::value]]); });
+    const DrainCtx& d = *reinterpret_cast<const DrainCtx*>(__cvta_shared_to_generic(ctx_u));
+    const MTask& task = *reinterpret_cast<const MTask*>(__cvta_shared_to_generic(task_u));
+    const uint32_t act = (uint32_t)task.act, t = d.t0 + (uint32_t)task.boff, pitch = d.pitch, nb = d.nb;
+    const int lane = threadIdx.x & 31, uw = 32 / d.halves, u = d.quarter * uw + (lane & (uw - 1));
+    const bool ok = u < d.c, full = d.full != 0;
+    const int K = d.K, nql = d.nql, qs = d.halves, c_row = d.c_row;
+    __nv_bfloat16 *zh = d.zh, *zl = d.zl;
+    DrainDst dst[Sp::n];
+    bool more = false;                     // an order with several destinations
+    each_dst<LS, LB, PAR>(act, [&](auto j, auto, auto dd) {
+        constexpr int J = decltype(j)::value;
+        dst[J] = drain_dst<decltype(dd)::value>(d, d.outs[task.out_ptr[J]], u);
+        more |= task.out_ptr[J + 1] > task.out_ptr[J] + 1;
+    });
+    int q = d.q0 + (lane >= uw ? 1 : 0) + d.ql0 * qs;
 #pragma unroll 1
-        for (int ql = d.ql0; ql < d.nql; ql += MS_NDT) {
-            float acc[Sp::NO];
+    for (int ql = d.ql0; ql < nql; ql += MS_NDT, q += MS_NDT * qs) {
+        float acc[Sp::NO];
 #pragma unroll
-            for (int i = 0; i < Sp::NO; ++i) acc[i] = 0.f;
-            if (d.full) Coupling<LS, LB, PAR>::template step<0>(t + (uint32_t)ql * d.nb, d.pitch, acc, act);
-            const int q = d.q0 + ql * d.qs;
-            if (d.ok && q < d.K) {
-                const uint32_t off = (uint32_t)(q * d.c_row);
+        for (int i = 0; i < Sp::NO; ++i) acc[i] = 0.f;
+        if (full) Coupling<LS, LB, PAR>::template step<0>(t + (uint32_t)ql * nb, pitch, acc, act);
+        if (ok && q < K) {
+            const uint32_t off = (uint32_t)(q * c_row);
+            each_dst<LS, LB, PAR>(act, [&](auto j, auto o0, auto dd) {
+                drain_write<decltype(dd)::value>(zh, zl, dst[decltype(j)::value], off, acc + decltype(o0)::value);
+            });
+            if (more)
                 each_dst<LS, LB, PAR>(act, [&](auto j, auto o0, auto dd) {
                     constexpr int DD = decltype(dd)::value, J = decltype(j)::value;
-                    drain_write<DD>(d, dst[J], off, acc + decltype(o0)::value);
-                    for (int k = task.out_ptr[J] + 1; k < task.out_ptr[J + 1]; ++k)      // further destinations of the same order
-                        drain_write<DD>(d, drain_dst<DD>(d, d.outs[k]), off, acc + decltype(o0)::value);
+                    for (int k = task.out_ptr[J] + 1; k < task.out_ptr[J + 1]; ++k)
+                        drain_write<DD>(zh, zl, drain_dst<DD>(d, d.outs[k], u), off, acc + decltype(o0)::value);
                 });
-            }
         }
     }
 }
-__device__ __forceinline__ void drain_pick(const DrainCtx& d, const MTask& task, uint32_t t) {
-#define SOBEK_FN(ls, lb)                                                        \
-    case (ls * 5 + lb) * 2: drain_task<ls, lb, 0>(d, task, t); break;           \
-    case (ls * 5 + lb) * 2 + 1: drain_task<ls, lb, 1>(d, task, t); break;
+__device__ __forceinline__ void drain_pick(int fn, uint32_t ctx, uint32_t task) {
+#define SOBEK_FN1(ls, lb, par) \
+    case (ls * 5 + lb) * 2 + par: if constexpr (CGSpan<ls, lb, par>::n > 0) drain_task<ls, lb, par>(ctx, task); break;
+#define SOBEK_FN(ls, lb) SOBEK_FN1(ls, lb, 0) SOBEK_FN1(ls, lb, 1)
 #define SOBEK_FN5(ls) SOBEK_FN(ls, 0) SOBEK_FN(ls, 1) SOBEK_FN(ls, 2) SOBEK_FN(ls, 3) SOBEK_FN(ls, 4)
-    switch (task.fn) { SOBEK_FN5(0) SOBEK_FN5(1) SOBEK_FN5(2) SOBEK_FN5(3) SOBEK_FN5(4) default: break; }
+    switch (fn) { SOBEK_FN5(0) SOBEK_FN5(1) SOBEK_FN5(2) SOBEK_FN5(3) SOBEK_FN5(4) default: break; }
 #undef SOBEK_FN5
 #undef SOBEK_FN
+#undef SOBEK_FN1
 }
 
 // Every role walks the same items; the next item's bounds are requested one item ahead.
@@ -263,7 +279,7 @@ struct MsWalk {
 template <bool DUAL>
 __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);       // (keeps the pointer in the shared address space)
     constexpr int TB = MS_TB, PS = MS_PS, NW = MS_NW, SLAB = MS_SLAB, HALF = MS_HALF;
     constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_GEO = W_MMA + 1;
     const int NS = a.ns;
@@ -271,7 +287,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     uint8_t* sW = sRing + (size_t)NS * a.slot_bytes;                  // W ring: hi rows, lo rows
     uint64_t* bars = reinterpret_cast<uint64_t*>(sW + (size_t)NW * a.w_bytes);
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + MS_NBAR);
-    MOut* sOut = reinterpret_cast<MOut*>(tmem_holder + 4);
+    DrainCtx* sCtx = reinterpret_cast<DrainCtx*>(tmem_holder + 4);    // one per drain warp
+    MOut* sOut = reinterpret_cast<MOut*>(sCtx + MS_NDW);
     MSet* sSet = reinterpret_cast<MSet*>(sOut + a.n_outs);
     MBlk* sBlk = reinterpret_cast<MBlk*>(sSet + a.nsets);
     MUnit* sUnit = reinterpret_cast<MUnit*>(sBlk + a.n_blks);
@@ -583,34 +600,37 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         MsWalk walk(a, nsub, NS, nullptr);
         MsItem it{};
         uint32_t ai = 0;
-        DrainCtx d;
-        d.n_nodes = a.n_nodes; d.zh = a.zh; d.lo = a.zl - a.zh; d.outs = sOut; d.K = a.K; d.ql0 = (warp >> 2) % MS_NDT;
+        DrainCtx& d = sCtx[warp];
+        if (lane == 0) {
+            d.n_nodes = a.n_nodes; d.zh = a.zh; d.zl = a.zl; d.outs = sOut; d.K = a.K; d.ql0 = (warp >> 2) % MS_NDT; d.quarter = quarter;
+        }
         while (walk.next(it)) {
-            const MSet S = sSet[it.set];
-            d.nl = it.nl; d.full = it.len > 0;
-            for (int ui = 0; ui < S.nunit; ++ui) {
-                const uint32_t buf = d.full ? (ai & 1) : (uint32_t)(ui & 1);
+            const int u_begin = sSet[it.set].unit_begin, nunit = sSet[it.set].nunit;
+            const bool full = it.len > 0;
+            __syncwarp();
+            if (lane == 0) { d.nl = it.nl; d.full = full; }
+            for (int ui = 0; ui < nunit; ++ui) {
+                const uint32_t buf = full ? (ai & 1) : (uint32_t)(ui & 1);
                 const uint32_t par = (ai >> 1) & 1;
-                if (d.full) ++ai;
+                if (full) ++ai;
                 if (buf != (uint32_t)grp) continue;
-                const MUnit U = sUnit[S.unit_begin + ui];
-                if (d.full) {
+                const MUnit& U = sUnit[u_begin + ui];
+                __syncwarp();
+                if (lane == 0) {
+                    d.halves = U.halves; d.c = U.c; d.c_row = U.c_row; d.q0 = U.q0; d.nql = U.nq; d.pitch = (uint32_t)U.N; d.nb = (uint32_t)U.nb;
+                    d.t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF - (uint32_t)U.b0;
+                }
+                __syncwarp();
+                if (full) {
                     mbar_wait(bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
-                const int uw = U.halves == 2 ? 16 : 32;          // multiplicities of a quarter
-                if (quarter * uw < U.c) {
-                    d.u = quarter * uw + (lane & (uw - 1));
-                    d.ok = d.u < U.c;
-                    d.q0 = U.q0 + (U.halves == 2 ? lane >> 4 : 0); d.qs = U.halves; d.nql = U.nq;
-                    d.pitch = (uint32_t)U.N; d.nb = (uint32_t)U.nb; d.c_row = U.c_row;
-                    const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF - (uint32_t)U.b0;
+                if (quarter * (32 / U.halves) < U.c)
                     for (int ti = 0; ti < U.ntask; ++ti) {
                         const MTask& T = sTask[U.task_begin + ti];
-                        drain_pick(d, T, t0 + (uint32_t)T.boff);
+                        drain_pick(T.fn, smem_u32(&d), smem_u32(&T));
                     }
-                }
-                if (d.full) {
+                if (full) {
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar_accfree + 8 * buf);
