@@ -92,14 +92,6 @@ __device__ __forceinline__ void tm_ld(uint32_t t, float* v) {
     else if constexpr (N >= 2) { tm_ld2(t, v); if constexpr (N > 2) tm_ld<N - 2>(t + 2, v + 2); }
     else if constexpr (N == 1) tm_ld1(t, v);
 }
-// the wait for the loads in flight; the loaded registers pass through it so that nothing that reads them is scheduled ahead
-template <int N>
-__device__ __forceinline__ void tm_wait(float* v) {
-    tc_wait_ld();
-#pragma unroll
-    for (int i = 0; i < N; ++i) asm volatile("" : "+f"(v[i]));
-}
-
 template <int LS, int LB, int LD, int O0, int I>
 __device__ __forceinline__ void cg_term(const float* p, float* acc) {
     using T = CGTerms<LS, LB, LD>;
@@ -111,22 +103,14 @@ template <int LS, int LB, int LD, int O0, int I0, int... I>
 __device__ __forceinline__ void cg_terms(const float* p, float* acc, std::integer_sequence<int, I...>) {
     (cg_term<LS, LB, LD, O0, I0 + I>(p, acc), ...);
 }
-// the terms of component S for every destination order of the task
-template <int LS, int LB, int PAR, int S, int J>
-__device__ __forceinline__ void cg_row(const float* p, float* acc, uint32_t act) {
-    using Sp = CGSpan<LS, LB, PAR>;
-    if constexpr (J < Sp::n) {
-        using R = CGRange<LS, LB, Sp::ld(J), S>;
-        if constexpr (R::count > 0)
-            if ((act >> J) & 1u) cg_terms<LS, LB, Sp::ld(J), Sp::off(J), R::first>(p, acc, std::make_integer_sequence<int, R::count>());
-        cg_row<LS, LB, PAR, S, J + 1>(p, acc, act);
-    }
-}
 
-// Coupling sums of one radial index: moments in the columns t + s * pitch + b.
-template <int LS, int LB, int PAR>
+// Coupling sums for the wanted destination orders (bits of MASK) of R radial indices side by side: moments in the columns
+// t[r] + s * pitch + b, sums in acc[r].
+template <int LS, int LB, int PAR, int MASK>
 struct Coupling {
     using Sp = CGSpan<LS, LB, PAR>;
+    static __host__ __device__ constexpr int off(int j) { int o = 0; for (int i = 0; i < j; ++i) if ((MASK >> i) & 1) o += 2 * Sp::ld(i) + 1; return o; }
+    static constexpr int NO = off(Sp::n);
     static constexpr int DB = 2 * LB + 1, DS = 2 * LS + 1;
     static constexpr int CS = DB >= 7 ? 2 : (DB == 5 ? 3 : (DB == 3 ? 5 : 9));     // components per chunk of loads
     static constexpr int NC = (DS + CS - 1) / CS;
@@ -135,20 +119,37 @@ struct Coupling {
         if constexpr (I < DS) tm_ld<DB>(t + I * pitch, p + (I % CS) * DB);
         if constexpr ((I + 1) % CS != 0) load<I + 1>(t, pitch, p);
     }
-    template <int I>
-    static __device__ __forceinline__ void use(const float* p, float* acc, uint32_t act) {
-        if constexpr (I < DS) cg_row<LS, LB, PAR, I, 0>(p + (I % CS) * DB, acc, act);
-        if constexpr ((I + 1) % CS != 0) use<I + 1>(p, acc, act);
+    template <int S, int J>
+    static __device__ __forceinline__ void row(const float* p, float* acc) {
+        if constexpr (J < Sp::n) {
+            using G = CGRange<LS, LB, Sp::ld(J), S>;
+            if constexpr (((MASK >> J) & 1) && G::count > 0)
+                cg_terms<LS, LB, Sp::ld(J), off(J), G::first>(p, acc, std::make_integer_sequence<int, G::count>());
+            row<S, J + 1>(p, acc);
+        }
     }
-    template <int C>
-    static __device__ __forceinline__ void step(uint32_t t, uint32_t pitch, float* acc, uint32_t act) {
-        float p[CS * DB];
+    template <int I>
+    static __device__ __forceinline__ void use(const float* p, float* acc) {
+        if constexpr (I < DS) row<I, 0>(p + (I % CS) * DB, acc);
+        if constexpr ((I + 1) % CS != 0) use<I + 1>(p, acc);
+    }
+    template <int R, int C = 0>
+    static __device__ __forceinline__ void run(const uint32_t* t, uint32_t pitch, float (*acc)[NO]) {
+        float p[R][CS * DB];
 #pragma unroll
-        for (int i = 0; i < CS * DB; ++i) p[i] = 0.f;
-        load<C * CS>(t, pitch, p);
-        tm_wait<CS * DB>(p);
-        use<C * CS>(p, acc, act);
-        if constexpr (C + 1 < NC) step<C + 1>(t, pitch, acc, act);
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int i = 0; i < CS * DB; ++i) p[r][i] = 0.f;
+            load<C * CS>(t[r], pitch, p[r]);
+        }
+        tc_wait_ld();
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int i = 0; i < CS * DB; ++i) asm volatile("" : "+f"(p[r][i]));      // nothing that reads them is scheduled ahead of the wait
+#pragma unroll
+        for (int r = 0; r < R; ++r) use<C * CS>(p[r], acc[r]);
+        if constexpr (C + 1 < NC) run<R, C + 1>(t, pitch, acc);
     }
 };
 
@@ -176,74 +177,97 @@ template <int DD>
 __device__ __forceinline__ DrainDst drain_dst(const DrainCtx& d, const MOut& o, int u) {
     return DrainDst{d.n_nodes * o.zoff + d.nl * DD * (int64_t)o.ld + o.koff + u, (uint32_t)o.ld, o.scale};
 }
+__device__ __forceinline__ void st_b16_if(bool ok, __nv_bfloat16* p, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tcvt.u16.u32 h, %1;\n\t@p st.global.b16 [%0], h;\n\t}" ::"l"(p), "r"(v), "r"((uint32_t)ok) : "memory");
+}
 template <int DD>
-__device__ __forceinline__ void drain_write(__nv_bfloat16* zh, __nv_bfloat16* zl, const DrainDst& t, uint32_t off, const float* acc) {
+__device__ __forceinline__ void drain_write(__nv_bfloat16* zh, __nv_bfloat16* zl, const DrainDst& t, uint32_t off, const float* acc, bool ok) {
     __nv_bfloat16 *h = zh + t.a, *l = zl + t.a;
 #pragma unroll
     for (int i = 0; i < DD; ++i, off += t.ld) {
         const float v = acc[i] * t.scale;
-        const __nv_bfloat16 b = __float2bfloat16_rn(v);
-        h[off] = b;
-        l[off] = __float2bfloat16_rn(v - __bfloat162float(b));
+        uint32_t w, x;                 // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v), "f"(0.f));
+        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(v), "f"(v - __uint_as_float(w)));
+        st_b16_if(ok, h + off, x >> 16);
+        st_b16_if(ok, l + off, x);
     }
 }
 // f(j, first component, components) for every wanted destination order j
-template <int LS, int LB, int PAR, int J = 0, class F>
-__device__ __forceinline__ void each_dst(uint32_t act, F&& f) {
+template <int LS, int LB, int PAR, int MASK, int J = 0, class F>
+__device__ __forceinline__ void each_dst(F&& f) {
     using Sp = CGSpan<LS, LB, PAR>;
     if constexpr (J < Sp::n) {
-        if ((act >> J) & 1u) f(std::integral_constant<int, J>(), std::integral_constant<int, Sp::off(J)>(), std::integral_constant<int, 2 * Sp::ld(J) + 1>());
-        each_dst<LS, LB, PAR, J + 1>(act, f);
+        if constexpr ((MASK >> J) & 1)
+            f(std::integral_constant<int, J>(), std::integral_constant<int, Coupling<LS, LB, PAR, MASK>::off(J)>(), std::integral_constant<int, 2 * Sp::ld(J) + 1>());
+        each_dst<LS, LB, PAR, MASK, J + 1>(f);
     }
 }
 
 // ctx, task: shared-memory addresses
-template <int LS, int LB, int PAR>
+template <int LS, int LB, int PAR, int MASK>
 __device__ __noinline__ void drain_task(uint32_t ctx_u, uint32_t task_u) {
     using Sp = CGSpan<LS, LB, PAR>;
+    using Cp = Coupling<LS, LB, PAR, MASK>;
     const DrainCtx& d = *reinterpret_cast<const DrainCtx*>(__cvta_shared_to_generic(ctx_u));
     const MTask& task = *reinterpret_cast<const MTask*>(__cvta_shared_to_generic(task_u));
-    const uint32_t act = (uint32_t)task.act, t = d.t0 + (uint32_t)task.boff, pitch = d.pitch, nb = d.nb;
+    const uint32_t t0 = d.t0 + (uint32_t)task.boff, pitch = d.pitch, nb = d.nb;
     const int lane = threadIdx.x & 31, uw = 32 / d.halves, u = d.quarter * uw + (lane & (uw - 1));
-    const bool ok = u < d.c, full = d.full != 0;
-    const int K = d.K, nql = d.nql, qs = d.halves, c_row = d.c_row;
+    const bool full = d.full != 0;
+    const int K = u < d.c ? d.K : 0, nql = d.nql, qs = d.halves, c_row = d.c_row;       // lanes without a multiplicity write nothing
     __nv_bfloat16 *zh = d.zh, *zl = d.zl;
     DrainDst dst[Sp::n];
     bool more = false;                     // an order with several destinations
-    each_dst<LS, LB, PAR>(act, [&](auto j, auto, auto dd) {
+    each_dst<LS, LB, PAR, MASK>([&](auto j, auto, auto dd) {
         constexpr int J = decltype(j)::value;
         dst[J] = drain_dst<decltype(dd)::value>(d, d.outs[task.out_ptr[J]], u);
         more |= task.out_ptr[J + 1] > task.out_ptr[J] + 1;
     });
-    int q = d.q0 + (lane >= uw ? 1 : 0) + d.ql0 * qs;
+    constexpr int R = 2;                   // radial indices at a time: independent chains for the scheduler
+    const int qb = d.q0 + (lane >= uw ? 1 : 0);
 #pragma unroll 1
-    for (int ql = d.ql0; ql < nql; ql += MS_NDT, q += MS_NDT * qs) {
-        float acc[Sp::NO];
+    for (int ql = d.ql0; ql < nql; ql += R * MS_NDT) {
+        float acc[R][Cp::NO];
+        uint32_t t[R];
+        int q[R];
 #pragma unroll
-        for (int i = 0; i < Sp::NO; ++i) acc[i] = 0.f;
-        if (full) Coupling<LS, LB, PAR>::template step<0>(t + (uint32_t)ql * nb, pitch, acc, act);
-        if (ok && q < K) {
-            const uint32_t off = (uint32_t)(q * c_row);
-            each_dst<LS, LB, PAR>(act, [&](auto j, auto o0, auto dd) {
-                drain_write<decltype(dd)::value>(zh, zl, dst[decltype(j)::value], off, acc + decltype(o0)::value);
+        for (int r = 0; r < R; ++r) {
+#pragma unroll
+            for (int i = 0; i < Cp::NO; ++i) acc[r][i] = 0.f;
+            const int qr = min(ql + r * MS_NDT, nql - 1);
+            t[r] = t0 + (uint32_t)qr * nb;
+            q[r] = ql + r * MS_NDT < nql ? qb + qr * qs : K;
+        }
+        if (full) Cp::template run<R>(t, pitch, acc);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const uint32_t off = (uint32_t)(q[r] * c_row);
+            each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto dd) {
+                drain_write<decltype(dd)::value>(zh, zl, dst[decltype(j)::value], off, acc[r] + decltype(o0)::value, q[r] < K);
             });
-            if (more)
-                each_dst<LS, LB, PAR>(act, [&](auto j, auto o0, auto dd) {
+        }
+        if (more) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+                each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto dd) {
                     constexpr int DD = decltype(dd)::value, J = decltype(j)::value;
                     for (int k = task.out_ptr[J] + 1; k < task.out_ptr[J + 1]; ++k)
-                        drain_write<DD>(zh, zl, drain_dst<DD>(d, d.outs[k], u), off, acc + decltype(o0)::value);
+                        drain_write<DD>(zh, zl, drain_dst<DD>(d, d.outs[k], u), (uint32_t)(q[r] * c_row), acc[r] + decltype(o0)::value, q[r] < K);
                 });
         }
     }
 }
 __device__ __forceinline__ void drain_pick(int fn, uint32_t ctx, uint32_t task) {
-#define SOBEK_FN1(ls, lb, par) \
-    case (ls * 5 + lb) * 2 + par: if constexpr (CGSpan<ls, lb, par>::n > 0) drain_task<ls, lb, par>(ctx, task); break;
-#define SOBEK_FN(ls, lb) SOBEK_FN1(ls, lb, 0) SOBEK_FN1(ls, lb, 1)
+#define SOBEK_FN1(ls, lb, par, m) \
+    case ((ls * 5 + lb) * 2 + par) * 8 + m: if constexpr (m < (1 << CGSpan<ls, lb, par>::n)) drain_task<ls, lb, par, m>(ctx, task); break;
+#define SOBEK_FN2(ls, lb, par) SOBEK_FN1(ls, lb, par, 1) SOBEK_FN1(ls, lb, par, 2) SOBEK_FN1(ls, lb, par, 3) SOBEK_FN1(ls, lb, par, 4) \
+    SOBEK_FN1(ls, lb, par, 5) SOBEK_FN1(ls, lb, par, 6) SOBEK_FN1(ls, lb, par, 7)
+#define SOBEK_FN(ls, lb) SOBEK_FN2(ls, lb, 0) SOBEK_FN2(ls, lb, 1)
 #define SOBEK_FN5(ls) SOBEK_FN(ls, 0) SOBEK_FN(ls, 1) SOBEK_FN(ls, 2) SOBEK_FN(ls, 3) SOBEK_FN(ls, 4)
     switch (fn) { SOBEK_FN5(0) SOBEK_FN5(1) SOBEK_FN5(2) SOBEK_FN5(3) SOBEK_FN5(4) default: break; }
 #undef SOBEK_FN5
 #undef SOBEK_FN
+#undef SOBEK_FN2
 #undef SOBEK_FN1
 }
 
@@ -628,7 +652,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (quarter * (32 / U.halves) < U.c)
                     for (int ti = 0; ti < U.ntask; ++ti) {
                         const MTask& T = sTask[U.task_begin + ti];
-                        drain_pick(T.fn, smem_u32(&d), smem_u32(&T));
+                        drain_pick(T.fn * 8 + T.act, smem_u32(&d), smem_u32(&T));
                     }
                 if (full) {
                     tc_fence_before();
