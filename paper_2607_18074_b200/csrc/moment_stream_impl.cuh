@@ -300,6 +300,20 @@ struct MsWalk {
     }
 };
 
+// The products of one slot: per component x_hi W_hi, x_hi W_lo, x_lo W_hi, and with M = 64 both lane halves, so that the collector
+// serves four and two of them with one read of x.  Unrolled: a loop over runtime counts issues M = 64, N = 40 products every 38
+// cycles, this every 23 (N = 24 / 48 / 72: 18 / 26 / 36; M = 128, N = 48 / 80: 37 / 46).
+template <int D, int HALVES>
+__device__ __forceinline__ void ms_issue(uint32_t d0, uint64_t dX, uint32_t xlo16, uint64_t dW, uint32_t wlo16, uint32_t N, uint32_t idesc, uint32_t acc) {
+#pragma unroll
+    for (int s = 0; s < D; ++s) {
+        const uint64_t x = dX + (uint32_t)(s * (HALVES == 2 ? 1 : 2) * (MS_SLAB >> 4));
+        const uint32_t d = d0 + (uint32_t)s * N;
+        if (HALVES == 2) tc_mma_bf16_x6(d, d + (16u << 16), x, x + xlo16, dW, dW + wlo16, 2u * N, idesc, acc);
+        else tc_mma_bf16_x3(d, x, x + xlo16, dW, dW + wlo16, idesc, acc);
+    }
+}
+
 template <bool DUAL>
 __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -591,7 +605,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(U.N >> 3) << 17) | ((8u / (uint32_t)U.halves) << 24);
                 if (ai >= 2) mbar_wait(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
                 tc_fence_after();
-                const uint32_t d0 = tmem_base + buf * HALF, wlo16 = (uint32_t)(U.N * U.halves * 2), sl16 = (uint32_t)((U.halves == 1 ? 2 : 1) * (SLAB >> 4));
+                const uint32_t d0 = tmem_base + buf * HALF, wlo16 = (uint32_t)(U.N * U.halves * 2);
                 const bool release = ui + 1 == S.nunit || !it.resident;
                 for (int j = 0; j < it.nslot; ++j) {
                     mbar_wait(bar_full + 8 * st, rd & 1, a.status);
@@ -600,12 +614,13 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     tc_fence_after();
                     const uint64_t dX = dX0 + ((uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4)), dW = dW0 + (uint32_t)ws * w16;
                     if (elect_one()) {
-                        for (int h = 0; h < U.halves; ++h) {
-                            const uint64_t dWh = dW + (uint32_t)(h * U.N * 2);
-                            const uint32_t dh = d0 + ((uint32_t)(16 * h) << 16);
-#pragma unroll 3
-                            for (int s = 0; s < U.d_src; ++s)
-                                tc_mma_bf16_x3(dh + (uint32_t)(s * U.N), dX + (uint32_t)s * sl16, dX + (uint32_t)s * sl16 + xlo16, dWh, dWh + wlo16, idesc, j > 0 ? 1u : 0u);
+                        const uint32_t acc = j > 0 ? 1u : 0u;
+                        switch (U.d_src * 2 + U.halves) {
+#define SOBEK_MMA(d) case 2 * d + 1: ms_issue<d, 1>(d0, dX, xlo16, dW, wlo16, (uint32_t)U.N, idesc, acc); break; \
+                     case 2 * d + 2: ms_issue<d, 2>(d0, dX, xlo16, dW, wlo16, (uint32_t)U.N, idesc, acc); break;
+                            SOBEK_MMA(1) SOBEK_MMA(3) SOBEK_MMA(5) SOBEK_MMA(7) SOBEK_MMA(9)
+#undef SOBEK_MMA
+                            default: break;
                         }
                         tc_commit(bar_wfree + 8 * ws);
                         if (release) tc_commit(bar_sfree + 8 * st);
