@@ -88,10 +88,10 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
             }
             lboff.push_back(off);
             // Harmonic orders that share a unit, and how many radial indices it takes: the partition with the fewest MMA cycles.
-            // (see the rates at ms_issue: M = 64 takes about max(N/2, 10 + 0.32 N) cycles, M = 128 max(N/2, 27 + 0.23 N))
+            // (see the rates at ms_issue: M = 64 takes about max(N/2, 16 + 0.24 N) cycles, M = 128 max(N/2, 27 + 0.23 N))
             const int nl = (int)lbs.size(), teams = MS_NDT;
             const int cap = std::min(MS_NMAX, MS_HALF / B.d & ~(gran - 1));
-            auto cycles = [&](int n) { return halves == 2 ? 2.0 * std::max(0.5 * n, 10.0 + 0.32 * n) : std::max(0.5 * n, 27.0 + 0.23 * n); };
+            auto cycles = [&](int n) { return halves == 2 ? 2.0 * std::max(0.5 * n, 16.0 + 0.24 * n) : std::max(0.5 * n, 27.0 + 0.23 * n); };
             double best = 1e30; int best_mask = 0; std::vector<int> best_nq;
             for (int mask = 0; mask < (1 << (nl - 1)); ++mask) {      // bit i: cut after order i
                 double cost = 0; std::vector<int> nqs; bool good = true;

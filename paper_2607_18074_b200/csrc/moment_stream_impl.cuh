@@ -300,18 +300,18 @@ struct MsWalk {
     }
 };
 
-// The products of one slot: per component x_hi W_hi, x_hi W_lo, x_lo W_hi, and with M = 64 both lane halves, so that the collector
-// serves four and two of them with one read of x.  Unrolled: a loop over runtime counts issues M = 64, N = 40 products every 38
-// cycles, this every 23 (N = 24 / 48 / 72: 18 / 26 / 36; M = 128, N = 48 / 80: 37 / 46).
+// The products of one slot: x_hi W_hi, x_hi W_lo, x_lo W_hi per component and lane half.  Unrolled: a loop over runtime counts
+// issues M = 64, N = 40 products every 38 cycles, this every 26 (N = 24 / 48 / 72: 22 / 28 / 36; M = 128, N = 48 / 80: 37 / 46).
+// (x_hi stays in the collector for two products of one lane half; a product into the other half does not find it there.)
 template <int D, int HALVES>
 __device__ __forceinline__ void ms_issue(uint32_t d0, uint64_t dX, uint32_t xlo16, uint64_t dW, uint32_t wlo16, uint32_t N, uint32_t idesc, uint32_t acc) {
 #pragma unroll
-    for (int s = 0; s < D; ++s) {
-        const uint64_t x = dX + (uint32_t)(s * (HALVES == 2 ? 1 : 2) * (MS_SLAB >> 4));
-        const uint32_t d = d0 + (uint32_t)s * N;
-        if (HALVES == 2) tc_mma_bf16_x6(d, d + (16u << 16), x, x + xlo16, dW, dW + wlo16, 2u * N, idesc, acc);
-        else tc_mma_bf16_x3(d, x, x + xlo16, dW, dW + wlo16, idesc, acc);
-    }
+    for (int s = 0; s < D; ++s)
+#pragma unroll
+        for (int h = 0; h < HALVES; ++h) {
+            const uint64_t x = dX + (uint32_t)(s * (HALVES == 2 ? 1 : 2) * (MS_SLAB >> 4)), w = dW + (uint32_t)h * 2u * N;
+            tc_mma_bf16_x3(d0 + (uint32_t)s * N + (uint32_t)(h * 16 << 16), x, x + xlo16, w, w + wlo16, idesc, acc);
+        }
 }
 
 template <bool DUAL>

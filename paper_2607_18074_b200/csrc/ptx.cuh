@@ -97,23 +97,6 @@ __device__ __forceinline__ void tc_mma_bf16_x3(uint32_t tmem_d, uint64_t da_hi, 
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %3, %5, t;\n\t}"
         ::"r"(tmem_d), "l"(da_hi), "l"(da_lo), "l"(db_hi), "l"(db_lo), "r"(idesc), "r"(acc) : "memory");
 }
-// The same for two accumulators d0, d1 that share the A operand (two halves of the B rows, `b_half` 16-byte units apart): A_hi is
-// read once for four products, A_lo once for two.
-__device__ __forceinline__ void tc_mma_bf16_x6(uint32_t d0, uint32_t d1, uint64_t da_hi, uint64_t da_lo, uint64_t db_hi, uint64_t db_lo,
-                                               uint32_t b_half, uint32_t idesc, uint32_t acc) {
-    const uint64_t db_hi1 = db_hi + b_half, db_lo1 = db_lo + b_half;
-    asm volatile(
-        "{\n\t.reg .pred p, t;\n\t"
-        "setp.ne.b32 p, %9, 0;\n\t"
-        "setp.eq.u32 t, 0, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %2, %4, %8, p;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%1], %2, %5, %8, p;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %2, %6, %8, t;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], %2, %7, %8, t;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %3, %4, %8, t;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], %3, %5, %8, t;\n\t}"
-        ::"r"(d0), "r"(d1), "l"(da_hi), "l"(da_lo), "l"(db_hi), "l"(db_hi1), "l"(db_lo), "l"(db_lo1), "r"(idesc), "r"(acc) : "memory");
-}
 // eight consecutive 32-bit columns of this thread's TMEM lane (lane = 32 * (warp % 4) + lane id)
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* r) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
