@@ -18,7 +18,8 @@ constexpr int MS_HALF = 256;            // columns of one TMEM half
 constexpr int MS_NMAX = 80;             // columns of one product at most
 constexpr int MS_PS = 20;               // pitch (floats) of the transposed phi / Y rows: 16 values + 4 (bank spread)
 constexpr int MS_SLAB = MS_TB * 128;    // bytes of 64 multiplicities of one component: 16 edges x 64 bf16
-constexpr int MS_CTX = 88;               // bytes of a drain warp's context
+constexpr int MS_STAGE = 16;            // components that a drain warp stages before it writes them
+constexpr int MS_CTX = 96 + MS_STAGE * (8 + 128);      // bytes of a drain warp's context
 constexpr int MS_NBAR = 2 * MS_MAXNS + 2 * MS_NW + 4;
 
 struct MsArgs {

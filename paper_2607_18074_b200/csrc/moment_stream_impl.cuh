@@ -104,8 +104,7 @@ __device__ __forceinline__ void cg_terms(const float* p, float* acc, std::intege
     (cg_term<LS, LB, LD, O0, I0 + I>(p, acc), ...);
 }
 
-// Coupling sums for the wanted destination orders (bits of MASK) of R radial indices side by side: moments in the columns
-// t[r] + s * pitch + b, sums in acc[r].
+// Coupling sums of one radial index for the wanted destination orders (bits of MASK): moments in the columns t + s * pitch + b.
 template <int LS, int LB, int PAR, int MASK>
 struct Coupling {
     using Sp = CGSpan<LS, LB, PAR>;
@@ -133,29 +132,23 @@ struct Coupling {
         if constexpr (I < DS) row<I, 0>(p + (I % CS) * DB, acc);
         if constexpr ((I + 1) % CS != 0) use<I + 1>(p, acc);
     }
-    template <int R, int C = 0>
-    static __device__ __forceinline__ void run(const uint32_t* t, uint32_t pitch, float (*acc)[NO]) {
-        float p[R][CS * DB];
+    template <int C = 0>
+    static __device__ __forceinline__ void run(uint32_t t, uint32_t pitch, float* acc) {
+        float p[CS * DB];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-#pragma unroll
-            for (int i = 0; i < CS * DB; ++i) p[r][i] = 0.f;
-            load<C * CS>(t[r], pitch, p[r]);
-        }
+        for (int i = 0; i < CS * DB; ++i) p[i] = 0.f;
+        load<C * CS>(t, pitch, p);
         tc_wait_ld();
 #pragma unroll
-        for (int r = 0; r < R; ++r)
-#pragma unroll
-            for (int i = 0; i < CS * DB; ++i) asm volatile("" : "+f"(p[r][i]));      // nothing that reads them is scheduled ahead of the wait
-#pragma unroll
-        for (int r = 0; r < R; ++r) use<C * CS>(p[r], acc[r]);
-        if constexpr (C + 1 < NC) run<R, C + 1>(t, pitch, acc);
+        for (int i = 0; i < CS * DB; ++i) asm volatile("" : "+f"(p[i]));      // nothing that reads them is scheduled ahead of the wait
+        use<C * CS>(p, acc);
+        if constexpr (C + 1 < NC) run<C + 1>(t, pitch, acc);
     }
 };
 
-// What a drain warp needs to read out a unit, in shared memory (written by the warp itself): the read-out functions below are
-// not inlined, so that their registers do not compete with the state of the walk (inlined, the spills of it made up half of
-// the kernel's time: with the shared memory taken, next to no L1 is left to serve them).
+// What a drain warp needs to read out a unit, in shared memory (written by the warp itself).  The read-out functions are not
+// inlined, so that their registers do not compete with the state of the walk (inlined, its spills cost half of the kernel's
+// time: the shared memory leaves next to no L1 to serve them).
 struct DrainCtx {
     __nv_bfloat16 *zh, *zl;
     int64_t n_nodes, nl;
@@ -166,32 +159,32 @@ struct DrainCtx {
     int32_t q0, halves, K;
     int32_t c, c_row;        // multiplicities of the block, of the whole source block
     int32_t quarter, full;   // TMEM lane quarter of the warp; the node has edges
+    int32_t pad[2];
+    int64_t off[MS_STAGE];   // state offset of every staged component (-1: none): radial index 0, multiplicity 0 of the block
+    uint32_t stage[MS_STAGE][32];      // staged values, one per lane: bf16 hi << 16 | lo
 };
 
-static_assert(sizeof(DrainCtx) == MS_CTX, "context size");
+static_assert(sizeof(DrainCtx) == MS_CTX && MS_CTX % 16 == 0 && MS_NBAR * 8 % 16 == 0, "context size and alignment");
 
-// where the components of one destination order go: component 0 of radial index 0 of this lane, row pitch
-struct DrainDst { int64_t a; uint32_t ld; float scale; };
-
-template <int DD>
-__device__ __forceinline__ DrainDst drain_dst(const DrainCtx& d, const MOut& o, int u) {
-    return DrainDst{d.n_nodes * o.zoff + d.nl * DD * (int64_t)o.ld + o.koff + u, (uint32_t)o.ld, o.scale};
-}
-__device__ __forceinline__ void st_b16_if(bool ok, __nv_bfloat16* p, uint32_t v) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tcvt.u16.u32 h, %1;\n\t@p st.global.b16 [%0], h;\n\t}" ::"l"(p), "r"(v), "r"((uint32_t)ok) : "memory");
-}
-template <int DD>
-__device__ __forceinline__ void drain_write(__nv_bfloat16* zh, __nv_bfloat16* zl, const DrainDst& t, uint32_t off, const float* acc, bool ok) {
-    __nv_bfloat16 *h = zh + t.a, *l = zl + t.a;
-#pragma unroll
-    for (int i = 0; i < DD; ++i, off += t.ld) {
-        const float v = acc[i] * t.scale;
-        uint32_t w, x;                 // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v), "f"(0.f));
-        asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(v), "f"(v - __uint_as_float(w)));
-        st_b16_if(ok, h + off, x >> 16);
-        st_b16_if(ok, l + off, x);
+// Writes `cnt` staged radial indices (the first of them is `ql`) of `no` components each: a thread takes eight multiplicities of
+// one (index, component) and stores 16 bytes to each array.  2-byte stores straight from the lanes cost 12 cycles an instruction,
+// a third of the kernel.  inv = 65536 / no + 1.
+__device__ __noinline__ void drain_flush(DrainCtx* dp, int no, uint32_t inv, int cnt, int ql) {
+    const DrainCtx& d = *dp;
+    __syncwarp();
+    const int lane = threadIdx.x & 31, n = 4 * no * cnt, half = d.halves == 2;
+    for (int j = lane; j < n; j += 32) {
+        const int row = j >> 2, seg = j & 3, r = (int)(((uint32_t)row * inv) >> 16);
+        const uint4 a = *reinterpret_cast<const uint4*>(&d.stage[row][8 * seg]), b = *reinterpret_cast<const uint4*>(&d.stage[row][8 * seg + 4]);
+        const int u = d.quarter * (32 >> half) + 8 * (half ? seg & 1 : seg);
+        const int q = d.q0 + (ql + r * MS_NDT) * d.halves + (half ? seg >> 1 : 0);
+        const int64_t off = d.off[row - r * no];
+        if (u >= d.c || q >= d.K || off < 0) continue;
+        const int64_t e = off + (int64_t)(q * d.c_row + u);
+        *reinterpret_cast<uint4*>(d.zh + e) = make_uint4(__byte_perm(a.x, a.y, 0x7632), __byte_perm(a.z, a.w, 0x7632), __byte_perm(b.x, b.y, 0x7632), __byte_perm(b.z, b.w, 0x7632));
+        *reinterpret_cast<uint4*>(d.zl + e) = make_uint4(__byte_perm(a.x, a.y, 0x5410), __byte_perm(a.z, a.w, 0x5410), __byte_perm(b.x, b.y, 0x5410), __byte_perm(b.z, b.w, 0x5410));
     }
+    __syncwarp();
 }
 // f(j, first component, components) for every wanted destination order j
 template <int LS, int LB, int PAR, int MASK, int J = 0, class F>
@@ -204,60 +197,68 @@ __device__ __forceinline__ void each_dst(F&& f) {
     }
 }
 
-// ctx, task: shared-memory addresses
 template <int LS, int LB, int PAR, int MASK>
-__device__ __noinline__ void drain_task(uint32_t ctx_u, uint32_t task_u) {
-    using Sp = CGSpan<LS, LB, PAR>;
+__device__ __noinline__ void drain_task(DrainCtx* dp, const MTask* tp) {
     using Cp = Coupling<LS, LB, PAR, MASK>;
-    const DrainCtx& d = *reinterpret_cast<const DrainCtx*>(__cvta_shared_to_generic(ctx_u));
-    const MTask& task = *reinterpret_cast<const MTask*>(__cvta_shared_to_generic(task_u));
-    const uint32_t t0 = d.t0 + (uint32_t)task.boff, pitch = d.pitch, nb = d.nb;
-    const int lane = threadIdx.x & 31, uw = 32 / d.halves, u = d.quarter * uw + (lane & (uw - 1));
-    const bool full = d.full != 0;
-    const int K = u < d.c ? d.K : 0, nql = d.nql, qs = d.halves, c_row = d.c_row;       // lanes without a multiplicity write nothing
-    __nv_bfloat16 *zh = d.zh, *zl = d.zl;
-    DrainDst dst[Sp::n];
-    bool more = false;                     // an order with several destinations
-    each_dst<LS, LB, PAR, MASK>([&](auto j, auto, auto dd) {
+    constexpr int NO = Cp::NO, RF = NO >= 8 ? 1 : MS_STAGE / NO;       // radial indices staged between two flushes
+    DrainCtx& d = *dp;
+    const MTask& task = *tp;
+    const int lane = threadIdx.x & 31;
+    int rounds = 1;                        // destinations of an order (several paths with the same orders)
+    float scale[CGSpan<LS, LB, PAR>::n];
+    each_dst<LS, LB, PAR, MASK>([&](auto j, auto, auto) {
         constexpr int J = decltype(j)::value;
-        dst[J] = drain_dst<decltype(dd)::value>(d, d.outs[task.out_ptr[J]], u);
-        more |= task.out_ptr[J + 1] > task.out_ptr[J] + 1;
+        scale[J] = d.outs[task.out_ptr[J]].scale;
+        rounds = max(rounds, task.out_ptr[J + 1] - task.out_ptr[J]);
     });
-    constexpr int R = 2;                   // radial indices at a time: independent chains for the scheduler
-    const int qb = d.q0 + (lane >= uw ? 1 : 0);
+    // lane o: where component o of the task goes
+    auto fill = [&](int k) {
+        int o = -1, out = 0, dd = 1;
+        each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto ddc) {
+            constexpr int J = decltype(j)::value, O0 = decltype(o0)::value, DD = decltype(ddc)::value;
+            if (lane >= O0 && lane < O0 + DD && task.out_ptr[J] + k < task.out_ptr[J + 1]) { o = lane - O0; out = task.out_ptr[J] + k; dd = DD; }
+        });
+        __syncwarp();
+        if (lane < NO) {
+            const MOut m = d.outs[out];
+            d.off[lane] = o < 0 ? -1 : d.n_nodes * m.zoff + (d.nl * dd + o) * (int64_t)m.ld + m.koff;
+        }
+    };
+    fill(0);
+    const uint32_t t0 = d.t0 + (uint32_t)task.boff, pitch = d.pitch, nb = d.nb;
+    const bool full = d.full != 0;
+    const int nql = d.nql;
+    uint32_t* stage = &d.stage[0][lane];
+    int r = 0, first = d.ql0;
 #pragma unroll 1
-    for (int ql = d.ql0; ql < nql; ql += R * MS_NDT) {
-        float acc[R][Cp::NO];
-        uint32_t t[R];
-        int q[R];
+    for (int ql = d.ql0; ql < nql; ql += MS_NDT) {
+        float acc[NO];
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
+        for (int i = 0; i < NO; ++i) acc[i] = 0.f;
+        if (full) Cp::run(t0 + (uint32_t)ql * nb, pitch, acc);
+        uint32_t* st = stage + r * NO * 32;
+        each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto ddc) {
 #pragma unroll
-            for (int i = 0; i < Cp::NO; ++i) acc[r][i] = 0.f;
-            const int qr = min(ql + r * MS_NDT, nql - 1);
-            t[r] = t0 + (uint32_t)qr * nb;
-            q[r] = ql + r * MS_NDT < nql ? qb + qr * qs : K;
-        }
-        if (full) Cp::template run<R>(t, pitch, acc);
-#pragma unroll
-        for (int r = 0; r < R; ++r) {
-            const uint32_t off = (uint32_t)(q[r] * c_row);
-            each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto dd) {
-                drain_write<decltype(dd)::value>(zh, zl, dst[decltype(j)::value], off, acc[r] + decltype(o0)::value, q[r] < K);
-            });
-        }
-        if (more) {
-#pragma unroll
-            for (int r = 0; r < R; ++r)
-                each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto dd) {
-                    constexpr int DD = decltype(dd)::value, J = decltype(j)::value;
-                    for (int k = task.out_ptr[J] + 1; k < task.out_ptr[J + 1]; ++k)
-                        drain_write<DD>(zh, zl, drain_dst<DD>(d, d.outs[k], u), (uint32_t)(q[r] * c_row), acc[r] + decltype(o0)::value, q[r] < K);
-                });
+            for (int i = decltype(o0)::value; i < decltype(o0)::value + decltype(ddc)::value; ++i) {
+                const float v = acc[i] * scale[decltype(j)::value];
+                uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v), "f"(0.f));
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(v), "f"(v - __uint_as_float(w)));
+                st[i * 32] = x;
+            }
+        });
+        if (++r == RF || ql + MS_NDT >= nql) {
+            drain_flush(dp, NO, 65536u / NO + 1u, r, first);
+            for (int k = 1; k < rounds; ++k) {
+                fill(k);
+                drain_flush(dp, NO, 65536u / NO + 1u, r, first);
+                if (k + 1 == rounds) fill(0);
+            }
+            r = 0; first = ql + MS_NDT;
         }
     }
 }
-__device__ __forceinline__ void drain_pick(int fn, uint32_t ctx, uint32_t task) {
+__device__ __forceinline__ void drain_pick(int fn, DrainCtx* ctx, const MTask* task) {
 #define SOBEK_FN1(ls, lb, par, m) \
     case ((ls * 5 + lb) * 2 + par) * 8 + m: if constexpr (m < (1 << CGSpan<ls, lb, par>::n)) drain_task<ls, lb, par, m>(ctx, task); break;
 #define SOBEK_FN2(ls, lb, par) SOBEK_FN1(ls, lb, par, 1) SOBEK_FN1(ls, lb, par, 2) SOBEK_FN1(ls, lb, par, 3) SOBEK_FN1(ls, lb, par, 4) \
@@ -667,7 +668,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (quarter * (32 / U.halves) < U.c)
                     for (int ti = 0; ti < U.ntask; ++ti) {
                         const MTask& T = sTask[U.task_begin + ti];
-                        drain_pick(T.fn * 8 + T.act, smem_u32(&d), smem_u32(&T));
+                        drain_pick(T.fn * 8 + T.act, &d, &T);
                     }
                 if (full) {
                     tc_fence_before();
