@@ -177,32 +177,27 @@ struct MUnit {         // one accumulator: a block x radial indices q0.. x a run
     int32_t slab0, d_src;     // first slab of the block, components
     int32_t halves;           // 2: M = 64 products, even / odd radial indices in the lane halves; 1: M = 128
     int32_t N, nq, q0;        // columns of one product; radial indices per lane half; first of them
-    int32_t nb, b0;           // harmonics of the run and the first one's offset in the block's list
     int32_t c, c_row;         // multiplicities, those of the whole source block
     int32_t row_begin;        // first entry of the column table
-    int32_t task_begin, ntask, pad;
-};
-struct MTask {         // read-out of one (source order, harmonic order, parity of the destination order)
-    int32_t fn, boff;         // (l_src * 5 + l_sh) * 2 + parity; offset of the order in the block's list of harmonics
-    int32_t act;              // bit j: the j-th destination order is wanted
-    int32_t out_ptr[4];       // its paths: outs[out_ptr[j] .. out_ptr[j + 1])
+    int32_t out_begin, n_out; // state components
     int32_t pad;
 };
-struct MOut {          // where a path's state goes
+struct MOut {          // a state component (path, o) and its coupling terms
+    int64_t a;                // state offset of radial index 0, multiplicity 0 for node 0, without the group's share:
     int64_t zoff;             // state offset per node of the destination group
-    int32_t ld, koff;         // row pitch, offset in the contraction axis
-    float scale;              // the path's tensor over the unit-norm tensor of its orders
-    int32_t pad;
+    int32_t b;                // state elements from one node to the next
+    int32_t term, n, pad;     // first term, terms (even)
 };
+struct MTerm { uint32_t col; float coef; };      // column of the term's moment (radial index 0 of the unit), coefficient
 struct MomentSets {
     bool ok = false;
     std::vector<MSet> sets;
     std::vector<MBlk> blks;
     std::vector<MUnit> units;
-    std::vector<MTask> tasks;
     std::vector<MOut> outs;
+    std::vector<MTerm> terms;
     std::vector<uint16_t> rows;      // per column of a unit: radial index inside the unit | harmonic << 8; 0xffff: padding
-    MSet* d_sets = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MTask* d_tasks = nullptr; MOut* d_outs = nullptr;
+    MSet* d_sets = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
     uint16_t* d_rows = nullptr;
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, w_bytes = 0, smem_bytes = 0;
 };
@@ -414,7 +409,6 @@ cudaError_t launch_edge_pass_tc(const sobek_plan* p, const Direction& dir, const
                                 const float* vphi, int dual, const void* zqh, const void* zql, float* gphi, float* gY,
                                 int phi_mode, int Y_mode, int* status, cudaStream_t s);
 // --- moment_stream.cu -------------------------------------------------------------------
-bool cg_scale(const sobek_plan* p, const DPath& P, int ls, int lb, int ld, float& scale);
 void build_moment_sets(const sobek_plan* p, Direction& dir);
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
                                  const SplitSrc& ss, const float* Y, const float* vY, const float* phi, const float* vphi, int dual,

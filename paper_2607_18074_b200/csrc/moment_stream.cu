@@ -1,38 +1,19 @@
-// Host side of the moment-form edge stream: sets, units and read-out tasks of a direction, and the launch.
+// Host side of the moment-form edge stream: sets, units and read-out tables of a direction, and the launch.
 #include <algorithm>
 
-#include "cg_apply.cuh"
 #include "moment_stream.h"
 
 namespace sobek {
 
-// the factor by which the path's tensor c'[s][b][o] is the unit-norm tensor of its orders; false if it is no multiple of it
-bool cg_scale(const sobek_plan* p, const DPath& P, int ls, int lb, int ld, float& scale) {
-    const CGHost h = cg_host(ls, lb, ld);
-    if (!h.n) return false;
-    std::vector<double> ref((size_t)P.d_src * P.d_sh * P.d_dst, 0.0), got(ref.size(), 0.0);
-    for (int i = 0; i < h.n; ++i) ref[((size_t)(h.id[i] >> 8) * P.d_sh + ((h.id[i] >> 4) & 15)) * P.d_dst + (h.id[i] & 15)] = h.c[i];
-    for (int s = 0; s < P.d_src; ++s)
-        for (int o = 0; o < P.d_dst; ++o)
-            for (int k = p->tab_ptr[P.tabM + s * P.d_dst + o]; k < p->tab_ptr[P.tabM + s * P.d_dst + o + 1]; ++k)
-                got[((size_t)s * P.d_sh + p->tab_idx[k]) * P.d_dst + o] = p->tab_coef[k];
-    double dot = 0;
-    for (size_t i = 0; i < ref.size(); ++i) dot += ref[i] * got[i];
-    for (size_t i = 0; i < ref.size(); ++i)
-        if (fabs(got[i] - dot * ref[i]) > 1e-6 * fabs(dot)) return false;
-    scale = (float)dot;
-    return true;
-}
-
-// Sets, units and tasks of one direction for the plain ([0]) and the dual ([1]) stream.
+// Sets, units and read-out tables of one direction for the plain ([0]) and the dual ([1]) stream.
 void build_moment_sets(const sobek_plan* p, Direction& dir) {
     constexpr int kSmem = 227 * 1024;
     for (int dual = 0; dual < 2; ++dual) {
         MomentSets& T = dir.ms[dual];
         T = MomentSets{};
-        if (p->K > 16 || p->l_max > CG_LMAX || (dir.C_src & 7) || dir.paths.empty()) continue;
+        if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) continue;
         bool ok = true;
-        struct Pth { const DPath* P; int lb, ld, group; float scale; };
+        struct Pth { const DPath* P; int lb, group; };
         struct Blk { int so, c, d; std::vector<Pth> paths; };
         std::vector<Blk> blocks;
         for (size_t gi = 0; gi < dir.groups.size(); ++gi)
@@ -41,9 +22,7 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
                 if ((P.c_src & 7) || (P.src_off & 7)) ok = false;
                 auto it = std::find_if(blocks.begin(), blocks.end(), [&](const Blk& b) { return b.so == P.src_off; });
                 if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
-                Pth t{&P, (P.d_sh - 1) / 2, (P.d_dst - 1) / 2, (int)gi, 0.f};
-                if (!cg_scale(p, P, (P.d_src - 1) / 2, t.lb, t.ld, t.scale)) ok = false;
-                it->paths.push_back(t);
+                it->paths.push_back(Pth{&P, (P.d_sh - 1) / 2, (int)gi});
             }
         if (!ok) continue;
         std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
@@ -59,53 +38,38 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
         std::vector<std::vector<MUnit>> units(parts.size());
         for (size_t pi = 0; pi < parts.size() && ok; ++pi) {
             const Blk& B = blocks[parts[pi].blk];
-            const int ls = (B.d - 1) / 2, halves = parts[pi].c > 64 ? 1 : 2, gran = halves == 2 ? 8 : 16;
-            std::vector<int> lbs, lboff;
-            for (int lb = 0; lb <= CG_LMAX; ++lb)
-                if (std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb == lb; })) lbs.push_back(lb);
-            // tasks: one per (harmonic order, parity of the destination order)
-            struct Tk { int lb, id; };
-            std::vector<Tk> tk;
-            int off = 0;
-            for (int lb : lbs) {
-                lboff.push_back(off);
-                for (int par = 0; par < 2; ++par) {
-                    MTask t{};
-                    const int lo = std::abs(ls - lb), ld0 = lo + ((lo + ls + lb + par) & 1);
-                    t.fn = (ls * 5 + lb) * 2 + par; t.boff = off; t.act = 0;
-                    for (int j = 0; j < 3; ++j) {
-                        t.out_ptr[j] = (int)T.outs.size();
-                        for (const Pth& q : B.paths)
-                            if (q.lb == lb && q.ld == ld0 + 2 * j) {
-                                T.outs.push_back(MOut{dir.zb_off[q.group], dir.nk_ld[q.group], q.P->koff + parts[pi].u0, q.scale, 0});
-                                t.act |= 1 << j;
-                            }
-                    }
-                    t.out_ptr[3] = (int)T.outs.size();
-                    if (t.act) { tk.push_back(Tk{lb, (int)T.tasks.size()}); T.tasks.push_back(t); }
-                }
-                off += 2 * lb + 1;
-            }
-            lboff.push_back(off);
+            const int halves = parts[pi].c > 64 ? 1 : 2, gran = halves == 2 ? 8 : 16;
+            std::vector<int> lbs, lboff(1, 0);
+            for (int lb = 0; lb <= p->l_max; ++lb)
+                if (std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb == lb; })) { lbs.push_back(lb); lboff.push_back(lboff.back() + 2 * lb + 1); }
             // Harmonic orders that share a unit, and how many radial indices it takes: the partition with the fewest MMA cycles.
             // (see the rates at ms_issue: M = 64 takes about max(N/2, 16 + 0.24 N) cycles, M = 128 max(N/2, 27 + 0.23 N))
-            const int nl = (int)lbs.size(), teams = MS_NDT;
+            const int nl = (int)lbs.size(), KH = (p->K + halves - 1) / halves;     // radial indices per lane half
             const int cap = std::min(MS_NMAX, MS_HALF / B.d & ~(gran - 1));
             auto cycles = [&](int n) { return halves == 2 ? 2.0 * std::max(0.5 * n, 16.0 + 0.24 * n) : std::max(0.5 * n, 27.0 + 0.23 * n); };
+            // columns of nb harmonics x nq radial indices: the read-out takes four indices at a time from three on, and its last
+            // read may reach past them
+            auto width = [&](int nb, int nq) { return (nb * nq + (nq > 2 ? (4 - nq % 4) % 4 : 0) + gran - 1) & ~(gran - 1); };
             double best = 1e30; int best_mask = 0; std::vector<int> best_nq;
             for (int mask = 0; mask < (1 << (nl - 1)); ++mask) {      // bit i: cut after order i
                 double cost = 0; std::vector<int> nqs; bool good = true;
                 for (int i = 0; i < nl && good;) {
                     int j = i;
                     while (j + 1 < nl && !((mask >> j) & 1)) ++j;
-                    const int nb = lboff[j + 1] - lboff[i], KH = (p->K + halves - 1) / halves;     // radial indices per lane half
-                    const int most = std::min(cap / nb, KH);
-                    if (most < 1) { good = false; break; }
-                    const int nu = (KH + most - 1) / most;
-                    int nq = (KH + nu - 1) / nu;
-                    if (nq % teams && nq < most) ++nq;                // both drain teams busy
-                    const int n = (nb * nq + gran - 1) & ~(gran - 1);
-                    cost += ((KH + nq - 1) / nq) * B.d * cycles(n);
+                    const int nb = lboff[j + 1] - lboff[i];
+                    int nout = 0;
+                    for (const Pth& t : B.paths) if (t.lb >= lbs[i] && t.lb <= lbs[j]) nout += t.P->d_dst;
+                    // as many radial indices as fit, in equal units; then the cheapest count by products and read-out steps (about
+                    // 12 cycles per component and step)
+                    double c_best = 1e30; int nq = 0;
+                    for (int t = 1; t <= KH; ++t) {
+                        if (width(nb, t) > cap) break;
+                        const int nu = (KH + t - 1) / t;
+                        const double c = nu * (B.d * 3.0 * cycles(width(nb, t)) + 12.0 * nout * ((t > 2 ? (t + 3) / 4 : 1) + 0.5));
+                        if (c <= c_best) { c_best = c; nq = t; }
+                    }
+                    if (!nq) { good = false; break; }
+                    cost += c_best;
                     nqs.push_back(nq);
                     i = j + 1;
                 }
@@ -117,19 +81,33 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
                 while (j + 1 < nl && !((best_mask >> j) & 1)) ++j;
                 const int nb = lboff[j + 1] - lboff[i], nq = best_nq[gi];
                 MUnit U{};
-                U.d_src = B.d; U.halves = halves; U.N = (nb * nq + gran - 1) & ~(gran - 1); U.nq = nq; U.nb = nb; U.b0 = lboff[i];
-                U.c = parts[pi].c; U.c_row = B.c;
+                U.d_src = B.d; U.halves = halves; U.N = width(nb, nq); U.nq = nq; U.c = parts[pi].c; U.c_row = B.c;
+                // columns: radial index fastest, so that one read-out instruction takes several of them
                 U.row_begin = (int)T.rows.size();
                 for (int h = 0; h < halves; ++h)
                     for (int n = 0; n < U.N; ++n) {
                         if (n >= nb * nq) { T.rows.push_back(0xffff); continue; }
-                        int r = n % nb, b = 0;
+                        int r = n / nq, b = 0;
                         for (int k = i; k <= j; ++k) { const int db = 2 * lbs[k] + 1; if (r < db) { b = lbs[k] * lbs[k] + r; break; } r -= db; }
-                        T.rows.push_back((uint16_t)(((n / nb) * halves + h) | (b << 8)));
+                        T.rows.push_back((uint16_t)(((n % nq) * halves + h) | (b << 8)));
                     }
-                U.task_begin = -1;
-                for (const Tk& t : tk)
-                    if (t.lb >= lbs[i] && t.lb <= lbs[j]) { if (U.task_begin < 0) U.task_begin = t.id; ++U.ntask; }
+                U.out_begin = (int)T.outs.size();
+                for (int k = i; k <= j; ++k)
+                    for (const Pth& t : B.paths) {
+                        if (t.lb != lbs[k]) continue;
+                        for (int o = 0; o < t.P->d_dst; ++o) {
+                            const int ld = dir.nk_ld[t.group];
+                            MOut e{(int64_t)o * ld + t.P->koff + parts[pi].u0, dir.zb_off[t.group], t.P->d_dst * ld, (int)T.terms.size(), 0, 0};
+                            for (int sc = 0; sc < B.d; ++sc)
+                                for (int z = p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o]; z < p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o + 1]; ++z)
+                                    T.terms.push_back(MTerm{(uint32_t)(sc * U.N + (lboff[k] - lboff[i] + p->tab_idx[z]) * nq), p->tab_coef[z]});
+                            if ((int)T.terms.size() == e.term) T.terms.push_back(MTerm{0, 0.f});
+                            if ((T.terms.size() - e.term) & 1) T.terms.push_back(MTerm{T.terms.back().col, 0.f});
+                            e.n = (int)T.terms.size() - e.term;
+                            T.outs.push_back(e);
+                        }
+                    }
+                U.n_out = (int)T.outs.size() - U.out_begin;
                 max_rows = std::max(max_rows, U.N * halves);
                 for (int q0 = 0; q0 < p->K; q0 += nq * halves) { U.q0 = q0; units[pi].push_back(U); }
                 i = j + 1;
@@ -139,9 +117,9 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
         size_t n_units = 0;
         for (const auto& u : units) n_units += u.size();
         T.w_bytes = max_rows * 64;
-        const int tables = (int)(T.outs.size() * sizeof(MOut) + parts.size() * (sizeof(MSet) + sizeof(MBlk)) + n_units * sizeof(MUnit) +
-                                 T.tasks.size() * sizeof(MTask) + T.rows.size() * 2 + 64);
-        const int fixed = 1024 + MS_NW * T.w_bytes + MS_NBAR * 8 + 16 + MS_NDW * MS_CTX + tables;
+        const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + parts.size() * (sizeof(MSet) + sizeof(MBlk)) + n_units * sizeof(MUnit) +
+                                 T.rows.size() * 2 + 64);
+        const int fixed = 1024 + MS_NW * T.w_bytes + MS_NBAR * 8 + 16 + tables;
         // Sets: consecutive parts whose rows of 16 edges leave room for four slots (a node of 32 edges and the next one's
         // first rows); a wider part is a set of its own with the slots it leaves, at least two.
         const int slot4 = ((kSmem - fixed) / 4) & ~1023;
@@ -179,8 +157,8 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
     if (!T.ok || !ss.h || !ss.l) return cudaErrorInvalidValue;
     if (n_nodes <= 0) return cudaSuccess;
     MsArgs a{};
-    a.sets = T.d_sets; a.blks = T.d_blks; a.units = T.d_units; a.tasks = T.d_tasks; a.outs = T.d_outs; a.rows = T.d_rows;
-    a.nsets = (int)T.sets.size(); a.n_blks = (int)T.blks.size(); a.n_units = (int)T.units.size(); a.n_tasks = (int)T.tasks.size();
+    a.sets = T.d_sets; a.blks = T.d_blks; a.units = T.d_units; a.outs = T.d_outs; a.terms = T.d_terms; a.rows = T.d_rows;
+    a.nsets = (int)T.sets.size(); a.n_blks = (int)T.blks.size(); a.n_units = (int)T.units.size(); a.n_terms = (int)T.terms.size();
     a.n_outs = (int)T.outs.size(); a.n_rows = (int)T.rows.size();
     a.ev = ev; a.node0 = node0; a.n_nodes = n_nodes;
     a.oseg = ss.oseg ? ss.oseg + node0 : nullptr;

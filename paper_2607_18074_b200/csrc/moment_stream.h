@@ -7,7 +7,7 @@
 namespace sobek {
 
 constexpr int MS_TB = 16;               // edges per slot = k extent of one MMA
-constexpr int MS_NDT = 1;               // teams (four warps each) of a drain group; one group per TMEM half
+constexpr int MS_NDT = 2;               // teams (four warps each) of a drain group; one group per TMEM half
 constexpr int MS_NDW = 2 * 4 * MS_NDT;
 constexpr int MS_NLW = 2;               // loader warps
 constexpr int MS_NBW = 4;               // builder warps
@@ -18,18 +18,16 @@ constexpr int MS_HALF = 256;            // columns of one TMEM half
 constexpr int MS_NMAX = 80;             // columns of one product at most
 constexpr int MS_PS = 20;               // pitch (floats) of the transposed phi / Y rows: 16 values + 4 (bank spread)
 constexpr int MS_SLAB = MS_TB * 128;    // bytes of 64 multiplicities of one component: 16 edges x 64 bf16
-constexpr int MS_STAGE = 16;            // components that a drain warp stages before it writes them
-constexpr int MS_CTX = 96 + MS_STAGE * (8 + 128);      // bytes of a drain warp's context
 constexpr int MS_NBAR = 2 * MS_MAXNS + 2 * MS_NW + 4;
 
 struct MsArgs {
     const MSet* sets;
     const MBlk* blks;
     const MUnit* units;
-    const MTask* tasks;
     const MOut* outs;
+    const MTerm* terms;
     const uint16_t* rows;
-    int32_t nsets, n_blks, n_units, n_tasks, n_outs, n_rows;
+    int32_t nsets, n_blks, n_units, n_outs, n_terms, n_rows;
     EdgeView ev;
     int64_t node0, n_nodes;
     const int4* oseg;           // the chunk's nodes in processing order {local node, segment begin, end} or NULL

@@ -24,8 +24,8 @@
 //   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
 //   builder warps  W of one (unit, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
 //   MMA warp       one elected lane issues the three products per component (and lane half);
-//   drain warps    two groups, one per TMEM half, of two teams of four warps that share the unit's radial indices: a lane holds one
-//                  multiplicity, sums the coupling terms (unrolled, coefficients as immediates) and writes bf16 hi / lo.
+//   drain warps    two groups, one per TMEM half, of two teams of four warps that share the unit's state components: a lane holds one
+//                  multiplicity, sums the coupling terms and writes bf16 hi / lo.
 // With DUAL the kernel produces the directional state of the double backward (Eq. receiver_double_adjoint)
 //     dP = sum_e (vphi Y + phi vY)[q,b] x[s,u] + (phi Y)[q,b] vx[s,u]
 // as two slots per batch of edges.  The same kernel runs the sender-owned transposed traversal.  Every wait is bounded.
@@ -34,7 +34,6 @@
 
 #include <algorithm>
 
-#include "cg_apply.cuh"
 #include "geometry.cuh"
 #include "guard.cuh"
 #include "moment_stream.h"
@@ -81,195 +80,83 @@ __device__ __forceinline__ void tm_ld4(uint32_t t, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
 }
-__device__ __forceinline__ void tm_ld8(uint32_t t, float* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(t) : "memory");
-}
-template <int N>
+template <int R>
 __device__ __forceinline__ void tm_ld(uint32_t t, float* v) {
-    if constexpr (N >= 8) { tm_ld8(t, v); if constexpr (N > 8) tm_ld<N - 8>(t + 8, v + 8); }
-    else if constexpr (N >= 4) { tm_ld4(t, v); if constexpr (N > 4) tm_ld<N - 4>(t + 4, v + 4); }
-    else if constexpr (N >= 2) { tm_ld2(t, v); if constexpr (N > 2) tm_ld<N - 2>(t + 2, v + 2); }
-    else if constexpr (N == 1) tm_ld1(t, v);
+    if constexpr (R == 4) tm_ld4(t, v);
+    else if constexpr (R == 2) tm_ld2(t, v);
+    else tm_ld1(t, v);
 }
-template <int LS, int LB, int LD, int O0, int I>
-__device__ __forceinline__ void cg_term(const float* p, float* acc) {
-    using T = CGTerms<LS, LB, LD>;
-    constexpr int id = T::id[I];
-    constexpr float c = T::c[I];
-    acc[O0 + (id & 15)] = fmaf(c, p[(id >> 4) & 15], acc[O0 + (id & 15)]);
-}
-template <int LS, int LB, int LD, int O0, int I0, int... I>
-__device__ __forceinline__ void cg_terms(const float* p, float* acc, std::integer_sequence<int, I...>) {
-    (cg_term<LS, LB, LD, O0, I0 + I>(p, acc), ...);
-}
-
-// Coupling sums of one radial index for the wanted destination orders (bits of MASK): moments in the columns t + s * pitch + b.
-template <int LS, int LB, int PAR, int MASK>
-struct Coupling {
-    using Sp = CGSpan<LS, LB, PAR>;
-    static __host__ __device__ constexpr int off(int j) { int o = 0; for (int i = 0; i < j; ++i) if ((MASK >> i) & 1) o += 2 * Sp::ld(i) + 1; return o; }
-    static constexpr int NO = off(Sp::n);
-    static constexpr int DB = 2 * LB + 1, DS = 2 * LS + 1;
-    static constexpr int CS = DB >= 7 ? 2 : (DB == 5 ? 3 : (DB == 3 ? 5 : 9));     // components per chunk of loads
-    static constexpr int NC = (DS + CS - 1) / CS;
-    template <int I>      // I: component
-    static __device__ __forceinline__ void load(uint32_t t, uint32_t pitch, float* p) {
-        if constexpr (I < DS) tm_ld<DB>(t + I * pitch, p + (I % CS) * DB);
-        if constexpr ((I + 1) % CS != 0) load<I + 1>(t, pitch, p);
-    }
-    template <int S, int J>
-    static __device__ __forceinline__ void row(const float* p, float* acc) {
-        if constexpr (J < Sp::n) {
-            using G = CGRange<LS, LB, Sp::ld(J), S>;
-            if constexpr (((MASK >> J) & 1) && G::count > 0)
-                cg_terms<LS, LB, Sp::ld(J), off(J), G::first>(p, acc, std::make_integer_sequence<int, G::count>());
-            row<S, J + 1>(p, acc);
-        }
-    }
-    template <int I>
-    static __device__ __forceinline__ void use(const float* p, float* acc) {
-        if constexpr (I < DS) row<I, 0>(p + (I % CS) * DB, acc);
-        if constexpr ((I + 1) % CS != 0) use<I + 1>(p, acc);
-    }
-    template <int C = 0>
-    static __device__ __forceinline__ void run(uint32_t t, uint32_t pitch, float* acc) {
-        float p[CS * DB];
+template <int R>
+__device__ __forceinline__ void tm_pin(float* v) {      // after the wait: nothing that reads the registers is scheduled ahead of it
 #pragma unroll
-        for (int i = 0; i < CS * DB; ++i) p[i] = 0.f;
-        load<C * CS>(t, pitch, p);
-        tc_wait_ld();
-#pragma unroll
-        for (int i = 0; i < CS * DB; ++i) asm volatile("" : "+f"(p[i]));      // nothing that reads them is scheduled ahead of the wait
-        use<C * CS>(p, acc);
-        if constexpr (C + 1 < NC) run<C + 1>(t, pitch, acc);
-    }
-};
-
-// What a drain warp needs to read out a unit, in shared memory (written by the warp itself).  The read-out functions are not
-// inlined, so that their registers do not compete with the state of the walk (inlined, its spills cost half of the kernel's
-// time: the shared memory leaves next to no L1 to serve them).
-struct DrainCtx {
-    __nv_bfloat16 *zh, *zl;
-    int64_t n_nodes, nl;
-    const MOut* outs;
-    uint32_t t0;             // TMEM address of the unit's first column in this warp's lanes
-    uint32_t pitch, nb;      // columns between components / between radial indices
-    int32_t ql0, nql;        // radial indices of this warp's team: ql0, ql0 + MS_NDT, ... < nql (counted per lane half)
-    int32_t q0, halves, K;
-    int32_t c, c_row;        // multiplicities of the block, of the whole source block
-    int32_t quarter, full;   // TMEM lane quarter of the warp; the node has edges
-    int32_t pad[2];
-    int64_t off[MS_STAGE];   // state offset of every staged component (-1: none): radial index 0, multiplicity 0 of the block
-    uint32_t stage[MS_STAGE][32];      // staged values, one per lane: bf16 hi << 16 | lo
-};
-
-static_assert(sizeof(DrainCtx) == MS_CTX && MS_CTX % 16 == 0 && MS_NBAR * 8 % 16 == 0, "context size and alignment");
-
-// Writes `cnt` staged radial indices (the first of them is `ql`) of `no` components each: a thread takes eight multiplicities of
-// one (index, component) and stores 16 bytes to each array.  2-byte stores straight from the lanes cost 12 cycles an instruction,
-// a third of the kernel.  inv = 65536 / no + 1.
-__device__ __noinline__ void drain_flush(DrainCtx* dp, int no, uint32_t inv, int cnt, int ql) {
-    const DrainCtx& d = *dp;
-    __syncwarp();
-    const int lane = threadIdx.x & 31, n = 4 * no * cnt, half = d.halves == 2;
-    for (int j = lane; j < n; j += 32) {
-        const int row = j >> 2, seg = j & 3, r = (int)(((uint32_t)row * inv) >> 16);
-        const uint4 a = *reinterpret_cast<const uint4*>(&d.stage[row][8 * seg]), b = *reinterpret_cast<const uint4*>(&d.stage[row][8 * seg + 4]);
-        const int u = d.quarter * (32 >> half) + 8 * (half ? seg & 1 : seg);
-        const int q = d.q0 + (ql + r * MS_NDT) * d.halves + (half ? seg >> 1 : 0);
-        const int64_t off = d.off[row - r * no];
-        if (u >= d.c || q >= d.K || off < 0) continue;
-        const int64_t e = off + (int64_t)(q * d.c_row + u);
-        *reinterpret_cast<uint4*>(d.zh + e) = make_uint4(__byte_perm(a.x, a.y, 0x7632), __byte_perm(a.z, a.w, 0x7632), __byte_perm(b.x, b.y, 0x7632), __byte_perm(b.z, b.w, 0x7632));
-        *reinterpret_cast<uint4*>(d.zl + e) = make_uint4(__byte_perm(a.x, a.y, 0x5410), __byte_perm(a.z, a.w, 0x5410), __byte_perm(b.x, b.y, 0x5410), __byte_perm(b.z, b.w, 0x5410));
-    }
-    __syncwarp();
+    for (int r = 0; r < R; ++r) asm volatile("" : "+f"(v[r]));
 }
-// f(j, first component, components) for every wanted destination order j
-template <int LS, int LB, int PAR, int MASK, int J = 0, class F>
-__device__ __forceinline__ void each_dst(F&& f) {
-    using Sp = CGSpan<LS, LB, PAR>;
-    if constexpr (J < Sp::n) {
-        if constexpr ((MASK >> J) & 1)
-            f(std::integral_constant<int, J>(), std::integral_constant<int, Coupling<LS, LB, PAR, MASK>::off(J)>(), std::integral_constant<int, 2 * Sp::ld(J) + 1>());
-        each_dst<LS, LB, PAR, MASK, J + 1>(f);
-    }
+__device__ __forceinline__ void st_b16_if(bool ok, __nv_bfloat16* p, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tcvt.u16.u32 h, %1;\n\t@p st.global.b16 [%0], h;\n\t}" ::"l"(p), "r"(v), "r"((uint32_t)ok) : "memory");
 }
 
-template <int LS, int LB, int PAR, int MASK>
-__device__ __noinline__ void drain_task(DrainCtx* dp, const MTask* tp) {
-    using Cp = Coupling<LS, LB, PAR, MASK>;
-    constexpr int NO = Cp::NO, RF = NO >= 8 ? 1 : MS_STAGE / NO;       // radial indices staged between two flushes
-    DrainCtx& d = *dp;
-    const MTask& task = *tp;
-    const int lane = threadIdx.x & 31;
-    int rounds = 1;                        // destinations of an order (several paths with the same orders)
-    float scale[CGSpan<LS, LB, PAR>::n];
-    each_dst<LS, LB, PAR, MASK>([&](auto j, auto, auto) {
-        constexpr int J = decltype(j)::value;
-        scale[J] = d.outs[task.out_ptr[J]].scale;
-        rounds = max(rounds, task.out_ptr[J + 1] - task.out_ptr[J]);
-    });
-    // lane o: where component o of the task goes
-    auto fill = [&](int k) {
-        int o = -1, out = 0, dd = 1;
-        each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto ddc) {
-            constexpr int J = decltype(j)::value, O0 = decltype(o0)::value, DD = decltype(ddc)::value;
-            if (lane >= O0 && lane < O0 + DD && task.out_ptr[J] + k < task.out_ptr[J + 1]) { o = lane - O0; out = task.out_ptr[J] + k; dd = DD; }
-        });
-        __syncwarp();
-        if (lane < NO) {
-            const MOut m = d.outs[out];
-            d.off[lane] = o < 0 ? -1 : d.n_nodes * m.zoff + (d.nl * dd + o) * (int64_t)m.ld + m.koff;
-        }
-    };
-    fill(0);
-    const uint32_t t0 = d.t0 + (uint32_t)task.boff, pitch = d.pitch, nb = d.nb;
-    const bool full = d.full != 0;
-    const int nql = d.nql;
-    uint32_t* stage = &d.stage[0][lane];
-    int r = 0, first = d.ql0;
+// Read-out of a unit by one warp: every MS_NDT-th component of the state, R radial indices (columns) at a time.  The coupling
+// terms come from a table {column, coefficient} and are summed straight out of TMEM, which serves the repeated reads at a few
+// cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients the same sums ran at
+// 8 - 10 cycles an instruction, however many warps and independent chains there were: every warp streamed kilobytes of code
+// through the instruction cache for each radial index.)
+template <int R>
+__device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
+                                         int team, int u, int qh) {
+    const bool uok = u < U.c;
+    const int nq = U.nq, q0 = U.q0 + qh, qs = U.halves, n_out = U.n_out, c_row = U.c_row;
+    outs += U.out_begin;
 #pragma unroll 1
-    for (int ql = d.ql0; ql < nql; ql += MS_NDT) {
-        float acc[NO];
+    for (int o = team; o < n_out; o += MS_NDT) {
+        const MOut e = outs[o];
+        const int64_t base = e.a + nl * e.b + u;
+        const uint4* tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
+#pragma unroll 1
+        for (int qc = 0; qc < nq; qc += R) {
+            float acc[R];
 #pragma unroll
-        for (int i = 0; i < NO; ++i) acc[i] = 0.f;
-        if (full) Cp::run(t0 + (uint32_t)ql * nb, pitch, acc);
-        uint32_t* st = stage + r * NO * 32;
-        each_dst<LS, LB, PAR, MASK>([&](auto j, auto o0, auto ddc) {
+            for (int r = 0; r < R; ++r) acc[r] = 0.f;
+            if (full) {
+                const uint32_t t = t0 + (uint32_t)qc;
+#pragma unroll 1
+                for (int k = 0; k < e.n; k += 4) {
+                    float p[4][R];
+                    const uint4 c01 = tp[k >> 1];
+                    tm_ld<R>(t + c01.x, p[0]);
+                    tm_ld<R>(t + c01.z, p[1]);
+                    uint4 c23 = make_uint4(0u, 0u, 0u, 0u);
+                    const bool more = k + 2 < e.n;
+                    if (more) {
+                        c23 = tp[(k >> 1) + 1];
+                        tm_ld<R>(t + c23.x, p[2]);
+                        tm_ld<R>(t + c23.z, p[3]);
+                    }
+                    tc_wait_ld();
+                    tm_pin<R>(p[0]);
+                    tm_pin<R>(p[1]);
 #pragma unroll
-            for (int i = decltype(o0)::value; i < decltype(o0)::value + decltype(ddc)::value; ++i) {
-                const float v = acc[i] * scale[decltype(j)::value];
+                    for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c01.w), p[1][r], fmaf(__uint_as_float(c01.y), p[0][r], acc[r]));
+                    if (more) {
+                        tm_pin<R>(p[2]);
+                        tm_pin<R>(p[3]);
+#pragma unroll
+                        for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c23.w), p[3][r], fmaf(__uint_as_float(c23.y), p[2][r], acc[r]));
+                    }
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int q = q0 + (qc + r) * qs;
+                const bool ok = uok && q < a.K && qc + r < nq;
                 uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(v), "f"(0.f));
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(v), "f"(v - __uint_as_float(w)));
-                st[i * 32] = x;
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
+                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
+                const int64_t p = base + (int64_t)(q * c_row);
+                st_b16_if(ok, a.zh + p, x >> 16);
+                st_b16_if(ok, a.zl + p, x);
             }
-        });
-        if (++r == RF || ql + MS_NDT >= nql) {
-            drain_flush(dp, NO, 65536u / NO + 1u, r, first);
-            for (int k = 1; k < rounds; ++k) {
-                fill(k);
-                drain_flush(dp, NO, 65536u / NO + 1u, r, first);
-                if (k + 1 == rounds) fill(0);
-            }
-            r = 0; first = ql + MS_NDT;
         }
     }
-}
-__device__ __forceinline__ void drain_pick(int fn, DrainCtx* ctx, const MTask* task) {
-#define SOBEK_FN1(ls, lb, par, m) \
-    case ((ls * 5 + lb) * 2 + par) * 8 + m: if constexpr (m < (1 << CGSpan<ls, lb, par>::n)) drain_task<ls, lb, par, m>(ctx, task); break;
-#define SOBEK_FN2(ls, lb, par) SOBEK_FN1(ls, lb, par, 1) SOBEK_FN1(ls, lb, par, 2) SOBEK_FN1(ls, lb, par, 3) SOBEK_FN1(ls, lb, par, 4) \
-    SOBEK_FN1(ls, lb, par, 5) SOBEK_FN1(ls, lb, par, 6) SOBEK_FN1(ls, lb, par, 7)
-#define SOBEK_FN(ls, lb) SOBEK_FN2(ls, lb, 0) SOBEK_FN2(ls, lb, 1)
-#define SOBEK_FN5(ls) SOBEK_FN(ls, 0) SOBEK_FN(ls, 1) SOBEK_FN(ls, 2) SOBEK_FN(ls, 3) SOBEK_FN(ls, 4)
-    switch (fn) { SOBEK_FN5(0) SOBEK_FN5(1) SOBEK_FN5(2) SOBEK_FN5(3) SOBEK_FN5(4) default: break; }
-#undef SOBEK_FN5
-#undef SOBEK_FN
-#undef SOBEK_FN2
-#undef SOBEK_FN1
 }
 
 // Every role walks the same items; the next item's bounds are requested one item ahead.
@@ -326,13 +213,12 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     uint8_t* sW = sRing + (size_t)NS * a.slot_bytes;                  // W ring: hi rows, lo rows
     uint64_t* bars = reinterpret_cast<uint64_t*>(sW + (size_t)NW * a.w_bytes);
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + MS_NBAR);
-    DrainCtx* sCtx = reinterpret_cast<DrainCtx*>(tmem_holder + 4);    // one per drain warp
-    MOut* sOut = reinterpret_cast<MOut*>(sCtx + MS_NDW);
+    MTerm* sTerm = reinterpret_cast<MTerm*>(tmem_holder + 4);
+    MOut* sOut = reinterpret_cast<MOut*>(sTerm + a.n_terms);
     MSet* sSet = reinterpret_cast<MSet*>(sOut + a.n_outs);
     MBlk* sBlk = reinterpret_cast<MBlk*>(sSet + a.nsets);
     MUnit* sUnit = reinterpret_cast<MUnit*>(sBlk + a.n_blks);
-    MTask* sTask = reinterpret_cast<MTask*>(sUnit + a.n_units);
-    uint16_t* sRow = reinterpret_cast<uint16_t*>(sTask + a.n_tasks);
+    uint16_t* sRow = reinterpret_cast<uint16_t*>(sUnit + a.n_units);
     const uint32_t bar0 = smem_u32(bars);
     const uint32_t bar_full = bar0, bar_sfree = bar0 + 8 * MS_MAXNS, bar_wfull = bar0 + 16 * MS_MAXNS, bar_wfree = bar_wfull + 8 * NW,
                    bar_accfull = bar_wfree + 8 * NW, bar_accfree = bar_accfull + 16;
@@ -358,9 +244,13 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     auto table = [&](void* dst, const void* src, int bytes) {
         for (int i = tid; i < bytes / 2; i += MS_TT) reinterpret_cast<uint16_t*>(dst)[i] = reinterpret_cast<const uint16_t*>(src)[i];
     };
-    table(sOut, a.outs, a.n_outs * (int)sizeof(MOut)); table(sSet, a.sets, a.nsets * (int)sizeof(MSet));
-    table(sBlk, a.blks, a.n_blks * (int)sizeof(MBlk)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit));
-    table(sTask, a.tasks, a.n_tasks * (int)sizeof(MTask)); table(sRow, a.rows, a.n_rows * 2);
+    table(sTerm, a.terms, a.n_terms * (int)sizeof(MTerm)); table(sSet, a.sets, a.nsets * (int)sizeof(MSet));
+    table(sBlk, a.blks, a.n_blks * (int)sizeof(MBlk)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit)); table(sRow, a.rows, a.n_rows * 2);
+    for (int i = tid; i < a.n_outs; i += MS_TT) {
+        MOut e = a.outs[i];
+        e.a += a.n_nodes * e.zoff;         // the groups of a chunk's state lie one after another
+        sOut[i] = e;
+    }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -640,36 +530,28 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         MsWalk walk(a, nsub, NS, nullptr);
         MsItem it{};
         uint32_t ai = 0;
-        DrainCtx& d = sCtx[warp];
-        if (lane == 0) {
-            d.n_nodes = a.n_nodes; d.zh = a.zh; d.zl = a.zl; d.outs = sOut; d.K = a.K; d.ql0 = (warp >> 2) % MS_NDT; d.quarter = quarter;
-        }
+        const int team = (warp >> 2) % MS_NDT;
         while (walk.next(it)) {
             const int u_begin = sSet[it.set].unit_begin, nunit = sSet[it.set].nunit;
             const bool full = it.len > 0;
-            __syncwarp();
-            if (lane == 0) { d.nl = it.nl; d.full = full; }
             for (int ui = 0; ui < nunit; ++ui) {
                 const uint32_t buf = full ? (ai & 1) : (uint32_t)(ui & 1);
                 const uint32_t par = (ai >> 1) & 1;
                 if (full) ++ai;
                 if (buf != (uint32_t)grp) continue;
                 const MUnit& U = sUnit[u_begin + ui];
-                __syncwarp();
-                if (lane == 0) {
-                    d.halves = U.halves; d.c = U.c; d.c_row = U.c_row; d.q0 = U.q0; d.nql = U.nq; d.pitch = (uint32_t)U.N; d.nb = (uint32_t)U.nb;
-                    d.t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF - (uint32_t)U.b0;
-                }
-                __syncwarp();
                 if (full) {
                     mbar_wait(bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
-                if (quarter * (32 / U.halves) < U.c)
-                    for (int ti = 0; ti < U.ntask; ++ti) {
-                        const MTask& T = sTask[U.task_begin + ti];
-                        drain_pick(T.fn * 8 + T.act, &d, &T);
-                    }
+                const int uw = 32 / U.halves;          // multiplicities of a quarter
+                if (quarter * uw < U.c) {
+                    const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
+                    const int u = quarter * uw + (lane & (uw - 1)), qh = lane >= uw ? 1 : 0;
+                    if (U.nq > 2) read_out<4>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    else if (U.nq == 2) read_out<2>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    else read_out<1>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                }
                 if (full) {
                     tc_fence_before();
                     __syncwarp();
