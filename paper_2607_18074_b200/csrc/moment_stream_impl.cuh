@@ -91,10 +91,6 @@ __device__ __forceinline__ void tm_pin(float* v) {      // after the wait: nothi
 #pragma unroll
     for (int r = 0; r < R; ++r) asm volatile("" : "+f"(v[r]));
 }
-__device__ __forceinline__ void st_b16_if(bool ok, __nv_bfloat16* p, uint32_t v) {
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b16 h;\n\tsetp.ne.u32 p, %2, 0;\n\tcvt.u16.u32 h, %1;\n\t@p st.global.b16 [%0], h;\n\t}" ::"l"(p), "r"(v), "r"((uint32_t)ok) : "memory");
-}
-
 // Read-out of a unit by one warp: every MS_NDT-th component of the state, R radial indices (columns) at a time.  The coupling
 // terms come from a table {column, coefficient} and are summed straight out of TMEM, which serves the repeated reads at a few
 // cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients the same sums ran at
@@ -104,12 +100,14 @@ template <int R>
 __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
                                          int team, int u, int qh) {
     const bool uok = u < U.c;
-    const int nq = U.nq, q0 = U.q0 + qh, qs = U.halves, n_out = U.n_out, c_row = U.c_row;
+    const int nq = U.nq, q0 = U.q0 + qh, qs = U.halves, n_out = U.n_out, c_row = U.c_row, Kq = min(a.K, U.q0 + nq * qs);
+    const uint32_t q_step = (uint32_t)(qs * c_row), sel = u & 1 ? 0x1054u : 0x7632u;
+    __nv_bfloat16* const z0 = u & 1 ? a.zl + u - 1 : a.zh + u;
     outs += U.out_begin;
 #pragma unroll 1
     for (int o = team; o < n_out; o += MS_NDT) {
         const MOut e = outs[o];
-        const int64_t base = e.a + nl * e.b + u;
+        __nv_bfloat16* const z = z0 + (e.a + nl * e.b);
         const uint4* tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
 #pragma unroll 1
         for (int qc = 0; qc < nq; qc += R) {
@@ -144,19 +142,25 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
                     }
                 }
             }
+            // Two neighbouring lanes swap halves: the even one writes the hi, the odd one the lo parts of both multiplicities.
+            const uint32_t off = (uint32_t)((q0 + qc * qs) * c_row);
 #pragma unroll
             for (int r = 0; r < R; ++r) {
-                const int q = q0 + (qc + r) * qs;
-                const bool ok = uok && q < a.K && qc + r < nq;
                 uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
-                const int64_t p = base + (int64_t)(q * c_row);
-                st_b16_if(ok, a.zh + p, x >> 16);
-                st_b16_if(ok, a.zl + p, x);
+                const uint32_t y = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel);
+                if (uok && q0 + (qc + r) * qs < Kq) *reinterpret_cast<uint32_t*>(z + (off + (uint32_t)r * q_step)) = y;
             }
         }
     }
+}
+
+// Wait of a role of several warps: its first warp polls, the others sleep at the role's barrier (25 polling warps took half of
+// the issue slots).
+__device__ __forceinline__ void role_wait(bool leader, int id, int threads, uint32_t bar, uint32_t parity, int* status) {
+    if (leader) mbar_wait(bar, parity, status);
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
 // Every role walks the same items; the next item's bounds are requested one item ahead.
@@ -283,41 +287,46 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 return true;
             }
         };
-        // lane e < 16 holds edge e of the batch; bit e of msk says that the edge exists and that its ids are in range (an id
-        // that is not turns the edge's copies into zero fills and is reported in the status word)
-        auto load_ids = [&](int64_t& eid, int32_t& sn, uint32_t& msk) {
-            eid = 0; sn = 0;
-            bool ok = false;
-            if (b0 + lane < it.len && lane < TB) {
+        // Lane e < 16 holds edge e of the batch.  The ids of the next batch are requested one batch ahead and not looked at before
+        // their turn: bit e of msk then says that the edge exists and that its ids are in range (an id that is not turns the
+        // edge's copies into zero fills and is reported in the status word).
+        struct Ids { int64_t eid; int64_t v; bool in; };
+        auto request = [&]() -> Ids {
+            Ids d{0, 0, b0 + lane < it.len && lane < TB};
+            if (d.in) {
                 const int64_t pos = it.seg0 + b0 + lane;
-                eid = a.ev.perm ? (int64_t)a.ev.perm[pos] : pos;
-                ok = id_ok(eid, a.ev.E, a.status);
-                if (ok) {
-                    const int64_t v = a.ev.transposed ? (a.ev.recv ? (int64_t)a.ev.recv[pos] : owner_of(a.ev.row_ptr, a.ev.N, eid))
-                                                      : (int64_t)a.ev.col[eid];
-                    ok = id_ok(v, a.ev.N, a.status);
-                    sn = ok ? (int32_t)v : 0;
-                } else {
-                    eid = 0;
-                }
+                d.eid = a.ev.perm ? (int64_t)a.ev.perm[pos] : pos;
+                if (!a.ev.transposed) d.v = (int64_t)a.ev.col[pos];
+                else if (a.ev.recv) d.v = (int64_t)a.ev.recv[pos];
             }
-            msk = __ballot_sync(0xffffffffu, ok);
+            return d;
+        };
+        auto settle = [&](const Ids& d, int64_t& eid, int32_t& sn) -> uint32_t {
+            bool ok = d.in && id_ok(d.eid, a.ev.E, a.status);
+            eid = ok ? d.eid : 0; sn = 0;
+            if (ok) {
+                const int64_t v = a.ev.transposed && !a.ev.recv ? owner_of(a.ev.row_ptr, a.ev.N, eid) : d.v;
+                ok = id_ok(v, a.ev.N, a.status);
+                sn = ok ? (int32_t)v : 0;
+            }
+            return __ballot_sync(0xffffffffu, ok);
         };
         bool have = advance(true);
-        int64_t eid = 0; int32_t sn = 0; uint32_t msk = 0;
-        if (have) load_ids(eid, sn, msk);
+        Ids ids{0, 0, false};
+        if (have) ids = request();
         int st = 0; uint32_t round = 0;
         while (have) {
             const MSet S = sSet[it.set];
             const int op = has_a1 ? sub : 1;
+            int64_t eid; int32_t sn;
+            const uint32_t msk = settle(ids, eid, sn);
             have = advance(false);
-            int64_t eid_n = 0; int32_t sn_n = 0; uint32_t msk_n = 0;
-            if (have) load_ids(eid_n, sn_n, msk_n);
-            if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
+            if (have) ids = request();
+            if (round > 0) role_wait(warp == W_LOAD, 4, NLW * 32, bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
             const uint32_t slot_u = smem_u32(sRing + (size_t)st * a.slot_bytes);
             const uint32_t raw_u = slot_u + (uint32_t)(2 * a.x_cap);
             if (!a.rvec) {
-                // phi and Y, transposed: thread <-> (edge le, every fourth radial index / harmonic)
+                // phi and Y, transposed: thread <-> (edge le, every eighth radial index / harmonic)
                 const int64_t ee = __shfl_sync(0xffffffffu, eid, le);
                 const uint32_t ok = ((msk >> le) & 1u) * 4u;
                 for (int q = lt >> 4; q < a.K; q += NLW * 32 / TB) {
@@ -358,7 +367,6 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             }
             // this thread's arrival on the slot's barrier fires when all its copies above have landed
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st) : "memory");
-            eid = eid_n; sn = sn_n; msk = msk_n;
             if (++st == NS) { st = 0; ++round; }
         }
     } else if (warp == W_GEO) {
@@ -432,8 +440,11 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 const int rows = U.N * U.halves;
                 for (int j = 0; j < it.nslot; ++j) {
                     const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
-                    mbar_wait(bar_full + 8 * st, rd & 1, a.status);
-                    if (wr > 0) mbar_wait(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
+                    if (warp == W_BUILD) {
+                        mbar_wait(bar_full + 8 * st, rd & 1, a.status);
+                        if (wr > 0) mbar_wait(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
+                    }
+                    asm volatile("bar.sync 3, %0;" ::"n"(MS_NBW * 32) : "memory");
                     const float* F = reinterpret_cast<const float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
                     const float* Yt = F + a.K * PS;
                     const int dv = (a.K + a.dsh) * PS;
@@ -541,7 +552,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (buf != (uint32_t)grp) continue;
                 const MUnit& U = sUnit[u_begin + ui];
                 if (full) {
-                    mbar_wait(bar_accfull + 8 * buf, par, a.status);
+                    role_wait(warp % (4 * MS_NDT) == 0, 1 + grp, 4 * MS_NDT * 32, bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
                 const int uw = 32 / U.halves;          // multiplicities of a quarter
