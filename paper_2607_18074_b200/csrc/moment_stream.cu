@@ -47,9 +47,9 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
             const int nl = (int)lbs.size(), KH = (p->K + halves - 1) / halves;     // radial indices per lane half
             const int cap = std::min(MS_NMAX, MS_HALF / B.d & ~(gran - 1));
             auto cycles = [&](int n) { return halves == 2 ? 2.0 * std::max(0.5 * n, 16.0 + 0.24 * n) : std::max(0.5 * n, 27.0 + 0.23 * n); };
-            // columns of nb harmonics x nq radial indices: the read-out takes four indices at a time from three on, and its last
-            // read may reach past them
-            auto width = [&](int nb, int nq) { return (nb * nq + (nq > 2 ? (4 - nq % 4) % 4 : 0) + gran - 1) & ~(gran - 1); };
+            // columns of nb harmonics x nq radial indices: the read-out takes four or eight indices at a time from three or five
+            // on, and its last read may reach past them
+            auto width = [&](int nb, int nq) { return (nb * nq + (nq > 4 ? (8 - nq % 8) % 8 : nq == 3 ? 1 : 0) + gran - 1) & ~(gran - 1); };
             double best = 1e30; int best_mask = 0; std::vector<int> best_nq;
             for (int mask = 0; mask < (1 << (nl - 1)); ++mask) {      // bit i: cut after order i
                 double cost = 0; std::vector<int> nqs; bool good = true;
@@ -59,13 +59,13 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
                     const int nb = lboff[j + 1] - lboff[i];
                     int nout = 0;
                     for (const Pth& t : B.paths) if (t.lb >= lbs[i] && t.lb <= lbs[j]) nout += t.P->d_dst;
-                    // as many radial indices as fit, in equal units; then the cheapest count by products and read-out steps (about
-                    // 12 cycles per component and step)
+                    // as many radial indices as fit, in equal units; then the cheapest count by products and read-out steps (some
+                    // 8 + 4 R cycles per component)
                     double c_best = 1e30; int nq = 0;
                     for (int t = 1; t <= KH; ++t) {
                         if (width(nb, t) > cap) break;
                         const int nu = (KH + t - 1) / t;
-                        const double c = nu * (B.d * 3.0 * cycles(width(nb, t)) + 12.0 * nout * ((t > 2 ? (t + 3) / 4 : 1) + 0.5));
+                        const double c = nu * (B.d * 3.0 * cycles(width(nb, t)) + nout * (8.0 + 4.0 * (t > 4 ? 8 : (t > 2 ? 4 : t))));
                         if (c <= c_best) { c_best = c; nq = t; }
                     }
                     if (!nq) { good = false; break; }

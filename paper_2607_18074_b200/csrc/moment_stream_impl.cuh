@@ -69,7 +69,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// ---- read-out: n columns of this thread's TMEM lane, exactly (no load reaches past the accumulator) ----------------
+// ---- read-out: n consecutive columns of this thread's TMEM lane ----------------
 __device__ __forceinline__ void tm_ld1(uint32_t t, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(v[0]) : "r"(t) : "memory");
 }
@@ -80,9 +80,14 @@ __device__ __forceinline__ void tm_ld4(uint32_t t, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
 }
+__device__ __forceinline__ void tm_ld8(uint32_t t, float* v) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(t) : "memory");
+}
 template <int R>
 __device__ __forceinline__ void tm_ld(uint32_t t, float* v) {
-    if constexpr (R == 4) tm_ld4(t, v);
+    if constexpr (R == 8) tm_ld8(t, v);
+    else if constexpr (R == 4) tm_ld4(t, v);
     else if constexpr (R == 2) tm_ld2(t, v);
     else tm_ld1(t, v);
 }
@@ -91,6 +96,10 @@ __device__ __forceinline__ void tm_pin(float* v) {      // after the wait: nothi
 #pragma unroll
     for (int r = 0; r < R; ++r) asm volatile("" : "+f"(v[r]));
 }
+__device__ __forceinline__ void st_b32_if(uint32_t ok, void* p, uint32_t v) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(p), "r"(v), "r"(ok) : "memory");
+}
+
 // Read-out of a unit by one warp: every MS_NDT-th component of the state, R radial indices (columns) at a time.  The coupling
 // terms come from a table {column, coefficient} and are summed straight out of TMEM, which serves the repeated reads at a few
 // cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients the same sums ran at
@@ -99,58 +108,59 @@ __device__ __forceinline__ void tm_pin(float* v) {      // after the wait: nothi
 template <int R>
 __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
                                          int team, int u, int qh) {
-    const bool uok = u < U.c;
-    const int nq = U.nq, q0 = U.q0 + qh, qs = U.halves, n_out = U.n_out, c_row = U.c_row, Kq = min(a.K, U.q0 + nq * qs);
+    constexpr int G = R == 8 ? 1 : 2;      // pairs of terms per wait
+    const int nq = U.nq, q0 = U.q0 + qh, qs = U.halves, n_out = U.n_out, c_row = U.c_row, Kq = u < U.c ? min(a.K, U.q0 + nq * qs) : 0;
     const uint32_t q_step = (uint32_t)(qs * c_row), sel = u & 1 ? 0x1054u : 0x7632u;
     __nv_bfloat16* const z0 = u & 1 ? a.zl + u - 1 : a.zh + u;
     outs += U.out_begin;
+    MOut e = outs[team < n_out ? team : 0];
 #pragma unroll 1
     for (int o = team; o < n_out; o += MS_NDT) {
-        const MOut e = outs[o];
         __nv_bfloat16* const z = z0 + (e.a + nl * e.b);
         const uint4* tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
+        const int n = full ? e.n : 0;
+        e = outs[min(o + MS_NDT, n_out - 1)];
 #pragma unroll 1
         for (int qc = 0; qc < nq; qc += R) {
             float acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = 0.f;
-            if (full) {
-                const uint32_t t = t0 + (uint32_t)qc;
+            const uint32_t t = t0 + (uint32_t)qc;
 #pragma unroll 1
-                for (int k = 0; k < e.n; k += 4) {
-                    float p[4][R];
-                    const uint4 c01 = tp[k >> 1];
-                    tm_ld<R>(t + c01.x, p[0]);
-                    tm_ld<R>(t + c01.z, p[1]);
-                    uint4 c23 = make_uint4(0u, 0u, 0u, 0u);
-                    const bool more = k + 2 < e.n;
-                    if (more) {
-                        c23 = tp[(k >> 1) + 1];
-                        tm_ld<R>(t + c23.x, p[2]);
-                        tm_ld<R>(t + c23.z, p[3]);
-                    }
-                    tc_wait_ld();
-                    tm_pin<R>(p[0]);
-                    tm_pin<R>(p[1]);
+            for (int k = 0; k < n; k += 2 * G) {
+                float p[2 * G][R];
+                uint4 c[G];
+                c[0] = tp[k >> 1];
+                tm_ld<R>(t + c[0].x, p[0]);
+                tm_ld<R>(t + c[0].z, p[1]);
+                const bool more = G > 1 && k + 2 < n;
+                if (more) {
+                    c[G - 1] = tp[(k >> 1) + G - 1];
+                    tm_ld<R>(t + c[G - 1].x, p[2 * G - 2]);
+                    tm_ld<R>(t + c[G - 1].z, p[2 * G - 1]);
+                }
+                tc_wait_ld();
+                tm_pin<R>(p[0]);
+                tm_pin<R>(p[1]);
 #pragma unroll
-                    for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c01.w), p[1][r], fmaf(__uint_as_float(c01.y), p[0][r], acc[r]));
-                    if (more) {
-                        tm_pin<R>(p[2]);
-                        tm_pin<R>(p[3]);
+                for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c[0].w), p[1][r], fmaf(__uint_as_float(c[0].y), p[0][r], acc[r]));
+                if (more) {
+                    tm_pin<R>(p[2 * G - 2]);
+                    tm_pin<R>(p[2 * G - 1]);
 #pragma unroll
-                        for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c23.w), p[3][r], fmaf(__uint_as_float(c23.y), p[2][r], acc[r]));
-                    }
+                    for (int r = 0; r < R; ++r)
+                        acc[r] = fmaf(__uint_as_float(c[G - 1].w), p[2 * G - 1][r], fmaf(__uint_as_float(c[G - 1].y), p[2 * G - 2][r], acc[r]));
                 }
             }
             // Two neighbouring lanes swap halves: the even one writes the hi, the odd one the lo parts of both multiplicities.
-            const uint32_t off = (uint32_t)((q0 + qc * qs) * c_row);
+            const int q = q0 + qc * qs;
+            uint32_t off = (uint32_t)(q * c_row);
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
+            for (int r = 0; r < R; ++r, off += q_step) {
                 uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
-                const uint32_t y = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel);
-                if (uok && q0 + (qc + r) * qs < Kq) *reinterpret_cast<uint32_t*>(z + (off + (uint32_t)r * q_step)) = y;
+                st_b32_if(q + r * qs < Kq, z + off, __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel));
             }
         }
     }
@@ -512,7 +522,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 for (int j = 0; j < it.nslot; ++j) {
                     mbar_wait(bar_full + 8 * st, rd & 1, a.status);
                     mbar_wait(bar_wfull + 8 * ws, wr & 1, a.status);
-                    fence_async_smem();      // the gathered rows were written through the generic proxy
+                    if (ui == 0 || !it.resident) fence_async_smem();      // the gathered rows were written through the generic proxy
                     tc_fence_after();
                     const uint64_t dX = dX0 + ((uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4)), dW = dW0 + (uint32_t)ws * w16;
                     if (elect_one()) {
@@ -559,7 +569,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (quarter * uw < U.c) {
                     const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
                     const int u = quarter * uw + (lane & (uw - 1)), qh = lane >= uw ? 1 : 0;
-                    if (U.nq > 2) read_out<4>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    if (U.nq > 4) read_out<8>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    else if (U.nq > 2) read_out<4>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
                     else if (U.nq == 2) read_out<2>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
                     else read_out<1>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
                 }
