@@ -169,7 +169,7 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
 // Wait of a role of several warps: its first warp polls, the others sleep at the role's barrier (25 polling warps took half of
 // the issue slots).
 __device__ __forceinline__ void role_wait(bool leader, int id, int threads, uint32_t bar, uint32_t parity, int* status) {
-    if (leader) mbar_wait(bar, parity, status);
+    if (leader) mbar_spin(bar, parity, status);
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                         tx = (vx_ - ux * uv) * ir; ty = (vy_ - uy * uv) * ir; tz = (vz_ - uz * uv) * ir;
                     }
                     for (int sub = 0; sub < nsub; ++sub) {       // the slots of the operand pairs need the same rows
-                        if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
+                        if (round > 0) mbar_spin(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
                         float* F = reinterpret_cast<float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
                         float* Yt = F + a.K * PS;
                         const int dv = (a.K + a.dsh) * PS, dsh = a.dsh;
@@ -451,8 +451,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 for (int j = 0; j < it.nslot; ++j) {
                     const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
                     if (warp == W_BUILD) {
-                        mbar_wait(bar_full + 8 * st, rd & 1, a.status);
-                        if (wr > 0) mbar_wait(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
+                        mbar_spin(bar_full + 8 * st, rd & 1, a.status);
+                        if (wr > 0) mbar_spin(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
                     }
                     asm volatile("bar.sync 3, %0;" ::"n"(MS_NBW * 32) : "memory");
                     const float* F = reinterpret_cast<const float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
@@ -515,13 +515,13 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 const uint32_t buf = ai & 1;
                 // D = F32, A = B = BF16, A MN-major, B K-major, M = 128 / halves
                 const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(U.N >> 3) << 17) | ((8u / (uint32_t)U.halves) << 24);
-                if (ai >= 2) mbar_wait(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
+                if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
                 tc_fence_after();
                 const uint32_t d0 = tmem_base + buf * HALF, wlo16 = (uint32_t)(U.N * U.halves * 2);
                 const bool release = ui + 1 == S.nunit || !it.resident;
                 for (int j = 0; j < it.nslot; ++j) {
-                    mbar_wait(bar_full + 8 * st, rd & 1, a.status);
-                    mbar_wait(bar_wfull + 8 * ws, wr & 1, a.status);
+                    mbar_spin(bar_full + 8 * st, rd & 1, a.status);
+                    mbar_spin(bar_wfull + 8 * ws, wr & 1, a.status);
                     if (ui == 0 || !it.resident) fence_async_smem();      // the gathered rows were written through the generic proxy
                     tc_fence_after();
                     const uint64_t dX = dX0 + ((uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4)), dW = dW0 + (uint32_t)ws * w16;

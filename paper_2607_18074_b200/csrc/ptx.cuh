@@ -50,6 +50,26 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int* st
     }
     atomicExch(status, (int)SOBEK_ERR_DEVICE_TIMEOUT);
 }
+// The same without suspending the thread between polls: for roles whose single polling warp is on the critical path.
+__device__ __forceinline__ void mbar_spin(uint32_t bar, uint32_t parity, int* status, uint64_t limit_ns = 2000000000ull) {
+    uint64_t t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n\t.reg .pred p;\n\t"
+            "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+            "selp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        if (ok) return;
+        if ((it & 255u) == 255u) {
+            uint64_t t1;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+            if (t0 == 0) t0 = t1;
+            else if (t1 - t0 > limit_ns) break;
+        }
+    }
+    atomicExch(status, (int)SOBEK_ERR_DEVICE_TIMEOUT);
+}
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
