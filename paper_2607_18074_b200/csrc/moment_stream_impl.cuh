@@ -459,11 +459,10 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     const float* Yt = F + a.K * PS;
                     const int dv = (a.K + a.dsh) * PS;
                     uint8_t* w = sW + (size_t)ws * a.w_bytes;
-                    for (int i = bt; i < 2 * rows; i += NBW * 32) {       // (row, eight edges)
+                    auto build = [&](int i) {                  // (row, eight edges)
                         const int n = ((i >> 4) << 3) | (i & 7), h = (i >> 3) & 1;
                         const uint32_t qb = rt[n];
-                        const int q = U.q0 + (int)(qb & 255u), b = (int)(qb >> 8);
-                        if (qb == 0xffffu || q >= a.K) continue;      // a column that no sum reads
+                        const int q = min(U.q0 + (int)(qb & 255u), a.K - 1), b = min((int)(qb >> 8), a.dsh - 1);   // (padding: any value)
                         float f[8], y[8], v[8];
                         *reinterpret_cast<float4*>(f) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h);
                         *reinterpret_cast<float4*>(f + 4) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h + 4);
@@ -487,7 +486,11 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                         uint8_t* d = w + (n >> 3) * 256 + h * 128 + (n & 7) * 16;
                         *reinterpret_cast<uint4*>(d) = hi;
                         *reinterpret_cast<uint4*>(d + rows * 32) = lo;
-                    }
+                    };
+                    int i = bt;
+#pragma unroll 1
+                    for (; i + NBW * 32 < 2 * rows; i += 2 * NBW * 32) { build(i); build(i + NBW * 32); }
+                    if (i < 2 * rows) build(i);
                     fence_async_smem();
                     mbar_arrive(bar_wfull + 8 * ws);
                     if (++ws == NW) { ws = 0; ++wr; }
@@ -502,6 +505,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         MsItem it{};
         int st0 = 0; uint32_t r0 = 0;
         int ws = 0; uint32_t wr = 0, ai = 0;
+        const uint32_t tm_u = __shfl_sync(0xffffffffu, tmem_base, 0);
         const uint64_t dX0 = make_desc(smem_u32(sRing), SLAB, 1024);          // 64 multiplicities per row, the next 64 a slab on
         const uint64_t dW0 = make_desc_plain(smem_u32(sW), 128, 256);
         const uint32_t slot16 = (uint32_t)a.slot_bytes >> 4, w16 = (uint32_t)a.w_bytes >> 4, xlo16 = (uint32_t)a.x_cap >> 4;
@@ -512,24 +516,27 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             for (int ui = 0; ui < S.nunit; ++ui, ++ai) {
                 if (it.resident) { st = st0; rd = r0; }
                 const MUnit U = sUnit[S.unit_begin + ui];
-                const uint32_t buf = ai & 1;
+                const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0);
                 // D = F32, A = B = BF16, A MN-major, B K-major, M = 128 / halves
-                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(U.N >> 3) << 17) | ((8u / (uint32_t)U.halves) << 24);
+                const uint32_t uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0);
+                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | (__shfl_sync(0xffffffffu, 8u / (uint32_t)U.halves, 0) << 24);
                 if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
                 tc_fence_after();
-                const uint32_t d0 = tmem_base + buf * HALF, wlo16 = (uint32_t)(U.N * U.halves * 2);
+                const uint32_t d0 = tm_u + buf * HALF;
                 const bool release = ui + 1 == S.nunit || !it.resident;
                 for (int j = 0; j < it.nslot; ++j) {
                     mbar_spin(bar_full + 8 * st, rd & 1, a.status);
                     mbar_spin(bar_wfull + 8 * ws, wr & 1, a.status);
                     if (ui == 0 || !it.resident) fence_async_smem();      // the gathered rows were written through the generic proxy
                     tc_fence_after();
-                    const uint64_t dX = dX0 + ((uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4)), dW = dW0 + (uint32_t)ws * w16;
+                    // (broadcasts: operands that the compiler knows to be uniform take no transfer per instruction)
+                    const uint64_t dX = dX0 + __shfl_sync(0xffffffffu, (uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4), 0),
+                                   dW = dW0 + __shfl_sync(0xffffffffu, (uint32_t)ws * w16, 0);
                     if (elect_one()) {
                         const uint32_t acc = j > 0 ? 1u : 0u;
                         switch (U.d_src * 2 + U.halves) {
-#define SOBEK_MMA(d) case 2 * d + 1: ms_issue<d, 1>(d0, dX, xlo16, dW, wlo16, (uint32_t)U.N, idesc, acc); break; \
-                     case 2 * d + 2: ms_issue<d, 2>(d0, dX, xlo16, dW, wlo16, (uint32_t)U.N, idesc, acc); break;
+#define SOBEK_MMA(d) case 2 * d + 1: ms_issue<d, 1>(d0, dX, xlo16, dW, uN * 2u, uN, idesc, acc); break; \
+                     case 2 * d + 2: ms_issue<d, 2>(d0, dX, xlo16, dW, uN * 4u, uN, idesc, acc); break;
                             SOBEK_MMA(1) SOBEK_MMA(3) SOBEK_MMA(5) SOBEK_MMA(7) SOBEK_MMA(9)
 #undef SOBEK_MMA
                             default: break;
