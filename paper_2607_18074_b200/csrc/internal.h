@@ -165,7 +165,17 @@ struct TcSets {
 
 // --- moment-form edge stream (moment_stream.cu) --------------------------------------------
 struct MSet {          // a run of source blocks whose gathered rows share the slots of the shared-memory ring
-    int32_t unit_begin, nunit, blk_begin, nblk;
+    int32_t blk_begin, nblk;
+    int32_t grp_begin, ngrp;  // groups of radial indices, one after another
+    int32_t nunit;            // units of all groups
+    int32_t nq;               // radial indices side by side in the columns (1, 2 or 4)
+    int32_t pad[2];
+};
+struct MGrp {          // radial indices whose W is built at once, and the units that use it
+    int32_t q0, rows;         // first radial index; rows of W per lane half
+    int32_t row_begin;        // first entry of the row table (the upper half's rows follow the lower half's)
+    int32_t unit_begin, nunit;
+    int32_t pad[3];
 };
 struct MBlk {          // (part of) a source block: at most 128 multiplicities
     int32_t src_off, c;       // first element inside a source feature row, multiplicities
@@ -173,33 +183,37 @@ struct MBlk {          // (part of) a source block: at most 128 multiplicities
     int32_t slab0, nch;       // first slab of the block in a slot, slabs (64 multiplicities each) per component
     int32_t pad[2];
 };
-struct MUnit {         // one accumulator: a block x radial indices q0.. x a run of harmonic orders
-    int32_t slab0, d_src;     // first slab of the block, components
-    int32_t halves;           // 2: M = 64 products, even / odd radial indices in the lane halves; 1: M = 128
-    int32_t N, nq, q0;        // columns of one product; radial indices per lane half; first of them
-    int32_t c, c_row;         // multiplicities, those of the whole source block
-    int32_t row_begin;        // first entry of the column table
+struct MUnit {         // one accumulator: components of neighbouring blocks x rows of W
+    int32_t slab0, d;         // first slab, components
+    int32_t halves;           // 2: M = 64 products, even / odd radial indices in the lane halves; 1: M = 128, one of the two
+    int32_t row0, N;          // first row of W (of the lower half if halves == 2), rows = columns of one product
+    int32_t nqs, rows_q;      // runs of radial indices side by side, columns from one to the next
+    int32_t q0;               // first radial index
+    int32_t c;                // multiplicities
+    int32_t blk0, nblk;       // blocks, relative to the set's
     int32_t out_begin, n_out; // state components
-    int32_t pad;
+    int32_t pad[3];
 };
 struct MOut {          // a state component (path, o) and its coupling terms
     int64_t a;                // state offset of radial index 0, multiplicity 0 for node 0, without the group's share:
     int64_t zoff;             // state offset per node of the destination group
     int32_t b;                // state elements from one node to the next
-    int32_t term, n, pad;     // first term, terms (even)
+    int32_t c_row;            // state elements from one radial index to the next
+    int32_t term, n;          // first term, terms (even)
 };
 struct MTerm { uint32_t col; float coef; };      // column of the term's moment (radial index 0 of the unit), coefficient
 struct MomentSets {
     bool ok = false;
     std::vector<MSet> sets;
+    std::vector<MGrp> grps;
     std::vector<MBlk> blks;
     std::vector<MUnit> units;
     std::vector<MOut> outs;
     std::vector<MTerm> terms;
-    std::vector<uint16_t> rows;      // per column of a unit: radial index inside the unit | harmonic << 8; 0xffff: padding
-    MSet* d_sets = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
+    std::vector<uint16_t> rows;      // per row of W: radial index inside the group | harmonic << 8; padding rows repeat another
+    MSet* d_sets = nullptr; MGrp* d_grps = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
     uint16_t* d_rows = nullptr;
-    int32_t x_cap = 0, slot_bytes = 0, ns = 0, w_bytes = 0, smem_bytes = 0;
+    int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;
 };
 
 struct FStage {        // one 256-column stage of the fused kernel's contraction axis

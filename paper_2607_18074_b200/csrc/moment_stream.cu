@@ -8,6 +8,8 @@ namespace sobek {
 // Sets, units and read-out tables of one direction for the plain ([0]) and the dual ([1]) stream.
 void build_moment_sets(const sobek_plan* p, Direction& dir) {
     constexpr int kSmem = 227 * 1024;
+    constexpr int kSlotBytes = 37 * 1024;      // gathered rows of a slot, hi and lo, beyond which a block starts a set of its own
+    constexpr int kWRows = 224;                // rows of W at a time at most (both lane halves)
     for (int dual = 0; dual < 2; ++dual) {
         MomentSets& T = dir.ms[dual];
         T = MomentSets{};
@@ -34,118 +36,152 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
             const int n = (blocks[b].c + 127) / 128, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
             for (int u = 0; u < blocks[b].c; u += per) parts.push_back(Part{(int)b, u, std::min(per, blocks[b].c - u)});
         }
-        int max_rows = 16;
-        std::vector<std::vector<MUnit>> units(parts.size());
-        for (size_t pi = 0; pi < parts.size() && ok; ++pi) {
-            const Blk& B = blocks[parts[pi].blk];
-            const int halves = parts[pi].c > 64 ? 1 : 2, gran = halves == 2 ? 8 : 16;
-            std::vector<int> lbs, lboff(1, 0);
-            for (int lb = 0; lb <= p->l_max; ++lb)
-                if (std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb == lb; })) { lbs.push_back(lb); lboff.push_back(lboff.back() + 2 * lb + 1); }
-            // Harmonic orders that share a unit, and how many radial indices it takes: the partition with the fewest MMA cycles.
-            // (see the rates at ms_issue: M = 64 takes about max(N/2, 16 + 0.24 N) cycles, M = 128 max(N/2, 27 + 0.23 N))
-            const int nl = (int)lbs.size(), KH = (p->K + halves - 1) / halves;     // radial indices per lane half
-            const int cap = std::min(MS_NMAX, MS_HALF / B.d & ~(gran - 1));
-            auto cycles = [&](int n) { return halves == 2 ? 2.0 * std::max(0.5 * n, 16.0 + 0.24 * n) : std::max(0.5 * n, 27.0 + 0.23 * n); };
-            // columns of nb harmonics x nq radial indices: the read-out takes four or eight indices at a time from three or five
-            // on, and its last read may reach past them
-            auto width = [&](int nb, int nq) { return (nb * nq + (nq > 4 ? (8 - nq % 8) % 8 : nq == 3 ? 1 : 0) + gran - 1) & ~(gran - 1); };
-            double best = 1e30; int best_mask = 0; std::vector<int> best_nq;
-            for (int mask = 0; mask < (1 << (nl - 1)); ++mask) {      // bit i: cut after order i
-                double cost = 0; std::vector<int> nqs; bool good = true;
-                for (int i = 0; i < nl && good;) {
-                    int j = i;
-                    while (j + 1 < nl && !((mask >> j) & 1)) ++j;
-                    const int nb = lboff[j + 1] - lboff[i];
-                    int nout = 0;
-                    for (const Pth& t : B.paths) if (t.lb >= lbs[i] && t.lb <= lbs[j]) nout += t.P->d_dst;
-                    // as many radial indices as fit, in equal units; then the cheapest count by products and read-out steps (some
-                    // 8 + 4 R cycles per component)
-                    double c_best = 1e30; int nq = 0;
-                    for (int t = 1; t <= KH; ++t) {
-                        if (width(nb, t) > cap) break;
-                        const int nu = (KH + t - 1) / t;
-                        const double c = nu * (B.d * 3.0 * cycles(width(nb, t)) + nout * (8.0 + 4.0 * (t > 4 ? 8 : (t > 2 ? 4 : t))));
-                        if (c <= c_best) { c_best = c; nq = t; }
-                    }
-                    if (!nq) { good = false; break; }
-                    cost += c_best;
-                    nqs.push_back(nq);
-                    i = j + 1;
-                }
-                if (good && cost < best) { best = cost; best_mask = mask; best_nq = nqs; }
-            }
-            if (best > 1e29) { ok = false; break; }
-            for (int i = 0, gi = 0; i < nl; ++gi) {
-                int j = i;
-                while (j + 1 < nl && !((best_mask >> j) & 1)) ++j;
-                const int nb = lboff[j + 1] - lboff[i], nq = best_nq[gi];
-                MUnit U{};
-                U.d_src = B.d; U.halves = halves; U.N = width(nb, nq); U.nq = nq; U.c = parts[pi].c; U.c_row = B.c;
-                // columns: radial index fastest, so that one read-out instruction takes several of them
-                U.row_begin = (int)T.rows.size();
-                for (int h = 0; h < halves; ++h)
-                    for (int n = 0; n < U.N; ++n) {
-                        if (n >= nb * nq) { T.rows.push_back(0xffff); continue; }
-                        int r = n / nq, b = 0;
-                        for (int k = i; k <= j; ++k) { const int db = 2 * lbs[k] + 1; if (r < db) { b = lbs[k] * lbs[k] + r; break; } r -= db; }
-                        T.rows.push_back((uint16_t)(((n % nq) * halves + h) | (b << 8)));
-                    }
-                U.out_begin = (int)T.outs.size();
-                for (int k = i; k <= j; ++k)
-                    for (const Pth& t : B.paths) {
-                        if (t.lb != lbs[k]) continue;
-                        for (int o = 0; o < t.P->d_dst; ++o) {
-                            const int ld = dir.nk_ld[t.group];
-                            MOut e{(int64_t)o * ld + t.P->koff + parts[pi].u0, dir.zb_off[t.group], t.P->d_dst * ld, (int)T.terms.size(), 0, 0};
-                            for (int sc = 0; sc < B.d; ++sc)
-                                for (int z = p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o]; z < p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o + 1]; ++z)
-                                    T.terms.push_back(MTerm{(uint32_t)(sc * U.N + (lboff[k] - lboff[i] + p->tab_idx[z]) * nq), p->tab_coef[z]});
-                            if ((int)T.terms.size() == e.term) T.terms.push_back(MTerm{0, 0.f});
-                            if ((T.terms.size() - e.term) & 1) T.terms.push_back(MTerm{T.terms.back().col, 0.f});
-                            e.n = (int)T.terms.size() - e.term;
-                            T.outs.push_back(e);
-                        }
-                    }
-                U.n_out = (int)T.outs.size() - U.out_begin;
-                max_rows = std::max(max_rows, U.N * halves);
-                for (int q0 = 0; q0 < p->K; q0 += nq * halves) { U.q0 = q0; units[pi].push_back(U); }
-                i = j + 1;
-            }
-        }
-        if (!ok) { T = MomentSets{}; continue; }
-        size_t n_units = 0;
-        for (const auto& u : units) n_units += u.size();
-        T.w_bytes = max_rows * 64;
-        const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + parts.size() * (sizeof(MSet) + sizeof(MBlk)) + n_units * sizeof(MUnit) +
-                                 T.rows.size() * 2 + 64);
-        const int fixed = 1024 + MS_NW * T.w_bytes + MS_NBAR * 8 + 16 + tables;
-        // Sets: consecutive parts whose rows of 16 edges leave room for four slots (a node of 32 edges and the next one's
-        // first rows); a wider part is a set of its own with the slots it leaves, at least two.
-        const int slot4 = ((kSmem - fixed) / 4) & ~1023;
+        // Sets: consecutive parts whose rows of 16 edges leave room for four slots with their W (a node of 32 edges and the next
+        // one's first rows); a wider part is a set of its own with the slots it leaves, at least two.
+        auto slabs_of = [&](const Part& q) { return blocks[q.blk].d * ((q.c + 63) / 64); };
         int x_cap = 0;
-        for (size_t i = 0; i < parts.size();) {
+        for (size_t i = 0; i < parts.size() && ok;) {
             MSet S{};
-            S.blk_begin = (int)T.blks.size(); S.unit_begin = (int)T.units.size();
-            int slabs = 0;
+            S.blk_begin = (int)T.blks.size(); S.grp_begin = (int)T.grps.size();
+            int slabs = 0, dmax = 0;
+            bool wide = false;
             size_t j = i;
             for (; j < parts.size(); ++j) {
                 const Blk& B = blocks[parts[j].blk];
-                const int nch = (parts[j].c + 63) / 64;
-                if (j > i && 2 * (slabs + B.d * nch) * MS_SLAB + raw > slot4) break;
-                T.blks.push_back(MBlk{B.so + parts[j].u0, parts[j].c, B.c, B.d, slabs, nch, {0, 0}});
-                for (MUnit U : units[j]) { U.slab0 = slabs; T.units.push_back(U); }
-                slabs += B.d * nch;
+                if (j > i && 2 * (slabs + slabs_of(parts[j])) * MS_SLAB > kSlotBytes) break;
+                T.blks.push_back(MBlk{B.so + parts[j].u0, parts[j].c, B.c, B.d, slabs, (parts[j].c + 63) / 64, {0, 0}});
+                slabs += slabs_of(parts[j]);
+                dmax = std::max(dmax, B.d);
+                wide |= parts[j].c > 64;
             }
-            S.nblk = (int)T.blks.size() - S.blk_begin; S.nunit = (int)T.units.size() - S.unit_begin;
-            T.sets.push_back(S);
+            S.nblk = (int)T.blks.size() - S.blk_begin;
             x_cap = std::max(x_cap, slabs * MS_SLAB);
+            // Rows of W: runs of nq radial indices (those of one lane half), per run the harmonics order by order, the radial
+            // index fastest, so that one read-out instruction takes nq of them.  The orders are cut into segments of whole
+            // 8-row (M = 128: 16-row) groups such that every block's components x a segment fit the columns of one TMEM half.
+            const int gran = wide ? 16 : 8, KH = (p->K + 1) / 2;
+            struct Seg { int l0, l1, row, rows; };
+            std::vector<Seg> segs;
+            int nq = KH >= 3 ? 4 : KH, rows_q = 0;
+            for (; nq >= 1; nq >>= 1) {
+                segs.clear(); rows_q = 0;
+                bool fits = true;
+                for (int l = 0; l <= p->l_max && fits;) {
+                    int e = l, rows = 0;
+                    for (; e <= p->l_max; ++e) {
+                        const int r = (((e + 1) * (e + 1) - l * l) * nq + gran - 1) & ~(gran - 1);
+                        if (dmax * r > MS_HALF) break;
+                        rows = r;
+                    }
+                    if (e == l) { fits = false; break; }
+                    segs.push_back(Seg{l, e - 1, rows_q, rows});
+                    rows_q += rows;
+                    l = e;
+                }
+                if (fits) break;
+            }
+            if (!nq) { ok = false; break; }
+            S.nq = nq;
+            const int runs = (KH + nq - 1) / nq;                                  // runs of radial indices per lane half
+            const int nqs = std::max(1, std::min(runs, kWRows / 2 / rows_q)), ngrp = (runs + nqs - 1) / nqs;
+            const int nqs_g = (runs + ngrp - 1) / ngrp, rows_h = nqs_g * rows_q;
+            S.ngrp = ngrp;
+            T.w_bytes = std::max(T.w_bytes, 2 * rows_h * 64);
+            const int row_begin = (int)T.rows.size();
+            for (int h = 0; h < 2; ++h)
+                for (int r = 0; r < nqs_g; ++r)
+                    for (const Seg& g : segs)
+                        for (int n = 0; n < g.rows; ++n) {
+                            const int nb = (g.l1 + 1) * (g.l1 + 1) - g.l0 * g.l0, m = std::min(n, nb * nq - 1);
+                            T.rows.push_back((uint16_t)((2 * (r * nq + m % nq) + h) | ((g.l0 * g.l0 + m / nq) << 8)));
+                        }
+            // units of one group; `used` tells which segments a block has paths in
+            std::vector<MUnit> us;
+            for (size_t k = i; k < j; ++k) {
+                const Blk& B = blocks[parts[k].blk];
+                const MBlk& M = T.blks[S.blk_begin + (int)(k - i)];
+                const int halves = parts[k].c > 64 ? 1 : 2;
+                auto used = [&](size_t g) { return std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb >= segs[g].l0 && t.lb <= segs[g].l1; }); };
+                auto emit = [&](int h, int run, int n_runs, size_t ga, size_t gb) {          // segments [ga, gb)
+                    MUnit U{};
+                    U.slab0 = M.slab0; U.d = B.d; U.halves = halves; U.c = M.c; U.blk0 = (int)(k - i); U.nblk = 1;
+                    U.row0 = (halves == 1 ? h * rows_h : 0) + run * rows_q + segs[ga].row;
+                    U.N = n_runs > 1 ? n_runs * rows_q : segs[gb - 1].row + segs[gb - 1].rows - segs[ga].row;
+                    U.nqs = n_runs; U.rows_q = rows_q; U.q0 = 2 * run * nq + (halves == 1 ? h : 0);
+                    U.pad[0] = (int)ga; U.pad[1] = (int)gb;
+                    if (!us.empty()) {       // together with the block before it, where the columns hold both
+                        MUnit& V = us.back();
+                        if (V.row0 == U.row0 && V.N == U.N && V.halves == halves && V.c == U.c && V.blk0 + V.nblk == U.blk0 &&
+                            V.slab0 + V.d * ((V.c + 63) / 64) == U.slab0 && (V.d + U.d) * U.N <= MS_HALF) {
+                            V.d += U.d; ++V.nblk;
+                            return;
+                        }
+                    }
+                    us.push_back(U);
+                };
+                const size_t ns = segs.size();
+                for (int h = 0; h < (halves == 1 ? 2 : 1); ++h) {
+                    size_t ga = 0, gb = ns;
+                    while (ga < ns && !used(ga)) ++ga;
+                    while (gb > ga && !used(gb - 1)) --gb;
+                    if (ga == 0 && gb == ns && B.d * nqs_g * rows_q <= MS_HALF) { emit(h, 0, nqs_g, 0, ns); continue; }
+                    for (int run = 0; run < nqs_g; ++run)
+                        for (size_t x = ga; x < gb;) {
+                            if (!used(x)) { ++x; continue; }
+                            size_t y = x + 1;
+                            while (y < gb && B.d * (segs[y].row + segs[y].rows - segs[x].row) <= MS_HALF) ++y;
+                            emit(h, run, 1, x, y);
+                            x = y;
+                        }
+                }
+            }
+            // read-out tables (the same for every group)
+            for (MUnit& U : us) {
+                U.out_begin = (int)T.outs.size();
+                int s0 = 0;
+                for (int k = 0; k < U.nblk; ++k) {
+                    const Part& Pt = parts[i + U.blk0 + k];
+                    const Blk& B = blocks[Pt.blk];
+                    for (int g = U.pad[0]; g < U.pad[1]; ++g)
+                        for (const Pth& t : B.paths) {
+                            if (t.lb < segs[g].l0 || t.lb > segs[g].l1) continue;
+                            for (int o = 0; o < t.P->d_dst; ++o) {
+                                const int ld = dir.nk_ld[t.group];
+                                MOut e{(int64_t)o * ld + t.P->koff + Pt.u0, dir.zb_off[t.group], t.P->d_dst * ld, B.c, (int)T.terms.size(), 0};
+                                const int col0 = segs[g].row - segs[U.pad[0]].row + (t.lb * t.lb - segs[g].l0 * segs[g].l0) * nq;
+                                for (int sc = 0; sc < B.d; ++sc)
+                                    for (int z = p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o]; z < p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o + 1]; ++z)
+                                        T.terms.push_back(MTerm{(uint32_t)((s0 + sc) * U.N + col0 + p->tab_idx[z] * nq), p->tab_coef[z]});
+                                if ((int)T.terms.size() == e.term) T.terms.push_back(MTerm{(uint32_t)col0, 0.f});
+                                if ((T.terms.size() - e.term) & 1) T.terms.push_back(MTerm{T.terms.back().col, 0.f});
+                                e.n = (int)T.terms.size() - e.term;
+                                T.outs.push_back(e);
+                            }
+                        }
+                    s0 += B.d;
+                }
+                U.n_out = (int)T.outs.size() - U.out_begin;
+            }
+            for (int g = 0; g < ngrp; ++g) {
+                MGrp G{};
+                G.q0 = 2 * g * nqs_g * nq; G.rows = rows_h; G.row_begin = row_begin; G.unit_begin = (int)T.units.size(); G.nunit = (int)us.size();
+                for (MUnit U : us) { U.q0 += G.q0; T.units.push_back(U); }
+                T.grps.push_back(G);
+            }
+            S.nunit = ngrp * (int)us.size();
+            T.sets.push_back(S);
             i = j;
         }
+        if (!ok) { T = MomentSets{}; continue; }
+        const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + T.sets.size() * sizeof(MSet) + T.grps.size() * sizeof(MGrp) +
+                                 T.blks.size() * sizeof(MBlk) + T.units.size() * sizeof(MUnit) + T.rows.size() * 2 + 64);
+        const int fixed = 1024 + MS_NBAR * 8 + 16 + tables;
         T.x_cap = x_cap;
         T.slot_bytes = 2 * x_cap + raw;
-        T.ns = std::min(MS_MAXNS, (kSmem - fixed) / T.slot_bytes);
-        T.smem_bytes = fixed + T.ns * T.slot_bytes;
+        // as many slots as fit with an entry of W each
+        T.ns = T.nw = std::min(std::min(MS_MAXNS, MS_MAXNW), (kSmem - fixed) / (T.slot_bytes + T.w_bytes));
+        if (fixed + T.ns * (T.slot_bytes + T.w_bytes) + T.w_bytes <= kSmem && T.nw < MS_MAXNW) ++T.nw;
+        T.smem_bytes = fixed + T.ns * T.slot_bytes + T.nw * T.w_bytes;
         T.ok = T.ns >= 2;
     }
 }
@@ -157,8 +193,8 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
     if (!T.ok || !ss.h || !ss.l) return cudaErrorInvalidValue;
     if (n_nodes <= 0) return cudaSuccess;
     MsArgs a{};
-    a.sets = T.d_sets; a.blks = T.d_blks; a.units = T.d_units; a.outs = T.d_outs; a.terms = T.d_terms; a.rows = T.d_rows;
-    a.nsets = (int)T.sets.size(); a.n_blks = (int)T.blks.size(); a.n_units = (int)T.units.size(); a.n_terms = (int)T.terms.size();
+    a.sets = T.d_sets; a.grps = T.d_grps; a.blks = T.d_blks; a.units = T.d_units; a.outs = T.d_outs; a.terms = T.d_terms; a.rows = T.d_rows;
+    a.nsets = (int)T.sets.size(); a.n_grps = (int)T.grps.size(); a.n_blks = (int)T.blks.size(); a.n_units = (int)T.units.size(); a.n_terms = (int)T.terms.size();
     a.n_outs = (int)T.outs.size(); a.n_rows = (int)T.rows.size();
     a.ev = ev; a.node0 = node0; a.n_nodes = n_nodes;
     a.oseg = ss.oseg ? ss.oseg + node0 : nullptr;
@@ -169,7 +205,7 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
     a.vrvec = dual ? ss.vrvec : nullptr;
     a.zh = (__nv_bfloat16*)zh; a.zl = (__nv_bfloat16*)zl;
     a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src;
-    a.x_cap = T.x_cap; a.slot_bytes = T.slot_bytes; a.ns = T.ns; a.w_bytes = T.w_bytes;
+    a.x_cap = T.x_cap; a.slot_bytes = T.slot_bytes; a.ns = T.ns; a.w_bytes = T.w_bytes; a.nw = T.nw;
     a.status = status;
     const int grid = (int)std::min<int64_t>(n_nodes * a.nsets, (int64_t)148);
     KernelTimer kt(K_STATE, s);

@@ -13,21 +13,21 @@ constexpr int MS_NLW = 2;               // loader warps
 constexpr int MS_NBW = 4;               // builder warps
 constexpr int MS_TT = (MS_NDW + MS_NLW + MS_NBW + 2) * 32;      // plus the MMA warp and the geometry warp
 constexpr int MS_MAXNS = 8;             // ring slots at most
-constexpr int MS_NW = 3;                // slots of the W ring
+constexpr int MS_MAXNW = 8;             // entries of the W ring at most
 constexpr int MS_HALF = 256;            // columns of one TMEM half
-constexpr int MS_NMAX = 80;             // columns of one product at most
 constexpr int MS_PS = 20;               // pitch (floats) of the transposed phi / Y rows: 16 values + 4 (bank spread)
 constexpr int MS_SLAB = MS_TB * 128;    // bytes of 64 multiplicities of one component: 16 edges x 64 bf16
-constexpr int MS_NBAR = 2 * MS_MAXNS + 2 * MS_NW + 4;
+constexpr int MS_NBAR = 2 * MS_MAXNS + 2 * MS_MAXNW + 4;
 
 struct MsArgs {
     const MSet* sets;
+    const MGrp* grps;
     const MBlk* blks;
     const MUnit* units;
     const MOut* outs;
     const MTerm* terms;
     const uint16_t* rows;
-    int32_t nsets, n_blks, n_units, n_outs, n_terms, n_rows;
+    int32_t nsets, n_grps, n_blks, n_units, n_outs, n_terms, n_rows;
     EdgeView ev;
     int64_t node0, n_nodes;
     const int4* oseg;           // the chunk's nodes in processing order {local node, segment begin, end} or NULL
@@ -46,7 +46,7 @@ struct MsArgs {
     __nv_bfloat16* zh;
     __nv_bfloat16* zl;
     int32_t K, dsh, C_src;
-    int32_t x_cap, slot_bytes, ns, w_bytes;
+    int32_t x_cap, slot_bytes, ns, w_bytes, nw;
     int* status;
 };
 

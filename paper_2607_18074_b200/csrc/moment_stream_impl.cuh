@@ -80,14 +80,9 @@ __device__ __forceinline__ void tm_ld4(uint32_t t, float* v) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
 }
-__device__ __forceinline__ void tm_ld8(uint32_t t, float* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(t) : "memory");
-}
 template <int R>
 __device__ __forceinline__ void tm_ld(uint32_t t, float* v) {
-    if constexpr (R == 8) tm_ld8(t, v);
-    else if constexpr (R == 4) tm_ld4(t, v);
+    if constexpr (R == 4) tm_ld4(t, v);
     else if constexpr (R == 2) tm_ld2(t, v);
     else tm_ld1(t, v);
 }
@@ -108,9 +103,9 @@ __device__ __forceinline__ void st_b32_if(uint32_t ok, void* p, uint32_t v) {
 template <int R>
 __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
                                          int team, int u, int qh) {
-    constexpr int G = R == 8 ? 1 : 2;      // pairs of terms per wait
-    const int nq = U.nq, q0 = U.q0 + qh, qs = U.halves, n_out = U.n_out, c_row = U.c_row, Kq = u < U.c ? min(a.K, U.q0 + nq * qs) : 0;
-    const uint32_t q_step = (uint32_t)(qs * c_row), sel = u & 1 ? 0x1054u : 0x7632u;
+    constexpr int G = 2;                   // pairs of terms per wait
+    const int q0 = U.q0 + qh, n_out = U.n_out, nqs = U.nqs, rows_q = U.rows_q, Kq = u < U.c ? a.K : 0;
+    const uint32_t sel = u & 1 ? 0x1054u : 0x7632u;
     __nv_bfloat16* const z0 = u & 1 ? a.zl + u - 1 : a.zh + u;
     outs += U.out_begin;
     MOut e = outs[team < n_out ? team : 0];
@@ -119,13 +114,15 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
         __nv_bfloat16* const z = z0 + (e.a + nl * e.b);
         const uint4* tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
         const int n = full ? e.n : 0;
+        const uint32_t q_step = 2u * (uint32_t)e.c_row;
+        uint32_t off = (uint32_t)(q0 * e.c_row);
         e = outs[min(o + MS_NDT, n_out - 1)];
 #pragma unroll 1
-        for (int qc = 0; qc < nq; qc += R) {
+        for (int qc = 0; qc < nqs; ++qc) {
             float acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = 0.f;
-            const uint32_t t = t0 + (uint32_t)qc;
+            const uint32_t t = t0 + (uint32_t)(qc * rows_q);
 #pragma unroll 1
             for (int k = 0; k < n; k += 2 * G) {
                 float p[2 * G][R];
@@ -153,14 +150,13 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
                 }
             }
             // Two neighbouring lanes swap halves: the even one writes the hi, the odd one the lo parts of both multiplicities.
-            const int q = q0 + qc * qs;
-            uint32_t off = (uint32_t)(q * c_row);
+            const int q = q0 + 2 * R * qc;
 #pragma unroll
             for (int r = 0; r < R; ++r, off += q_step) {
                 uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
-                st_b32_if(q + r * qs < Kq, z + off, __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel));
+                st_b32_if(q + 2 * r < Kq, z + off, __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel));
             }
         }
     }
@@ -178,9 +174,9 @@ struct MsItem { int set; int64_t nl, seg0; int len, nslot; bool resident; };
 struct MsWalk {
     const MsArgs& a;
     int64_t v, nl, s0, s1;
-    int set, nsub, ns;
+    int set, nsub;
     int* st;
-    __device__ MsWalk(const MsArgs& a_, int nsub_, int ns_, int* st_) : a(a_), nl(0), s0(0), s1(0), nsub(nsub_), ns(ns_), st(st_) {
+    __device__ MsWalk(const MsArgs& a_, int nsub_, int* st_) : a(a_), nl(0), s0(0), s1(0), nsub(nsub_), st(st_) {
         v = blockIdx.x % a.n_nodes; set = (int)(blockIdx.x / a.n_nodes);
         fetch();
     }
@@ -194,7 +190,7 @@ struct MsWalk {
         if (set >= a.nsets) return false;
         it.set = set; it.nl = nl; it.seg0 = s0; it.len = nsub ? (int)(s1 - s0) : 0;
         it.nslot = ((it.len + MS_TB - 1) / MS_TB) * nsub;
-        it.resident = it.nslot <= ns;
+        it.resident = it.nslot <= min(a.ns, a.nw);
         v += gridDim.x;
         while (v >= a.n_nodes && set < a.nsets) { v -= a.n_nodes; ++set; }
         fetch();
@@ -202,17 +198,17 @@ struct MsWalk {
     }
 };
 
-// The products of one slot: x_hi W_hi, x_hi W_lo, x_lo W_hi per component and lane half.  Unrolled: a loop over runtime counts
-// issues M = 64, N = 40 products every 38 cycles, this every 26 (N = 24 / 48 / 72: 22 / 28 / 36; M = 128, N = 48 / 80: 37 / 46).
-// (x_hi stays in the collector for two products of one lane half; a product into the other half does not find it there.)
-template <int D, int HALVES>
-__device__ __forceinline__ void ms_issue(uint32_t d0, uint64_t dX, uint32_t xlo16, uint64_t dW, uint32_t wlo16, uint32_t N, uint32_t idesc, uint32_t acc) {
-#pragma unroll
-    for (int s = 0; s < D; ++s)
+// The products of one slot: x_hi W_hi, x_hi W_lo, x_lo W_hi per component and lane half.  (x_hi stays in the collector for two
+// products of one lane half; a product into the other half does not find it there.)
+template <int HALVES>
+__device__ __forceinline__ void ms_issue(uint32_t d, uint32_t d0, uint64_t dX, uint32_t xlo16, uint64_t dW, uint32_t wlo16, uint32_t whalf16, uint32_t N,
+                                         uint32_t idesc, uint32_t acc) {
+#pragma unroll 2
+    for (uint32_t s = 0; s < d; ++s, d0 += N, dX += (HALVES == 2 ? 1 : 2) * (MS_SLAB >> 4))
 #pragma unroll
         for (int h = 0; h < HALVES; ++h) {
-            const uint64_t x = dX + (uint32_t)(s * (HALVES == 2 ? 1 : 2) * (MS_SLAB >> 4)), w = dW + (uint32_t)h * 2u * N;
-            tc_mma_bf16_x3(d0 + (uint32_t)s * N + (uint32_t)(h * 16 << 16), x, x + xlo16, w, w + wlo16, idesc, acc);
+            const uint64_t w = dW + (h ? whalf16 : 0u);
+            tc_mma_bf16_x3(d0 + (uint32_t)(h * 16 << 16), dX, dX + xlo16, w, w + wlo16, idesc, acc);
         }
 }
 
@@ -220,9 +216,9 @@ template <bool DUAL>
 __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);       // (keeps the pointer in the shared address space)
-    constexpr int TB = MS_TB, PS = MS_PS, NW = MS_NW, SLAB = MS_SLAB, HALF = MS_HALF;
+    constexpr int TB = MS_TB, PS = MS_PS, SLAB = MS_SLAB, HALF = MS_HALF;
     constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_GEO = W_MMA + 1;
-    const int NS = a.ns;
+    const int NS = a.ns, NW = a.nw;
     uint8_t* sRing = smem;                                            // slots: x hi, x lo, raw phi / Y (+ directions)
     uint8_t* sW = sRing + (size_t)NS * a.slot_bytes;                  // W ring: hi rows, lo rows
     uint64_t* bars = reinterpret_cast<uint64_t*>(sW + (size_t)NW * a.w_bytes);
@@ -230,12 +226,13 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     MTerm* sTerm = reinterpret_cast<MTerm*>(tmem_holder + 4);
     MOut* sOut = reinterpret_cast<MOut*>(sTerm + a.n_terms);
     MSet* sSet = reinterpret_cast<MSet*>(sOut + a.n_outs);
-    MBlk* sBlk = reinterpret_cast<MBlk*>(sSet + a.nsets);
+    MGrp* sGrp = reinterpret_cast<MGrp*>(sSet + a.nsets);
+    MBlk* sBlk = reinterpret_cast<MBlk*>(sGrp + a.n_grps);
     MUnit* sUnit = reinterpret_cast<MUnit*>(sBlk + a.n_blks);
     uint16_t* sRow = reinterpret_cast<uint16_t*>(sUnit + a.n_units);
     const uint32_t bar0 = smem_u32(bars);
-    const uint32_t bar_full = bar0, bar_sfree = bar0 + 8 * MS_MAXNS, bar_wfull = bar0 + 16 * MS_MAXNS, bar_wfree = bar_wfull + 8 * NW,
-                   bar_accfull = bar_wfree + 8 * NW, bar_accfree = bar_accfull + 16;
+    const uint32_t bar_full = bar0, bar_sfree = bar0 + 8 * MS_MAXNS, bar_wfull = bar0 + 16 * MS_MAXNS, bar_wfree = bar_wfull + 8 * MS_MAXNW,
+                   bar_accfull = bar_wfree + 8 * MS_MAXNW, bar_accfree = bar_accfull + 16;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool has_vx = DUAL && a.vsh != nullptr, has_vY = DUAL && (a.rvec ? a.vrvec != nullptr : a.vY != nullptr),
@@ -246,7 +243,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
 
     if (tid == 0) {
         for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, NLW * 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 1); }
-        for (int s = 0; s < NW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 1); }
+        for (int s = 0; s < MS_MAXNW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 1); }
         for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, 4 * MS_NDT); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -259,6 +256,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         for (int i = tid; i < bytes / 2; i += MS_TT) reinterpret_cast<uint16_t*>(dst)[i] = reinterpret_cast<const uint16_t*>(src)[i];
     };
     table(sTerm, a.terms, a.n_terms * (int)sizeof(MTerm)); table(sSet, a.sets, a.nsets * (int)sizeof(MSet));
+    table(sGrp, a.grps, a.n_grps * (int)sizeof(MGrp));
     table(sBlk, a.blks, a.n_blks * (int)sizeof(MBlk)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit)); table(sRow, a.rows, a.n_rows * 2);
     for (int i = tid; i < a.n_outs; i += MS_TT) {
         MOut e = a.outs[i];
@@ -278,7 +276,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // =========================== loader warps ===========================
         const int lt = (warp - W_LOAD) * 32 + lane;
         const int le = lane & (TB - 1);
-        MsWalk walk(a, nsub, NS, a.status);
+        MsWalk walk(a, nsub, a.status);
         MsItem it{};
         int rep = 0, nrep = 0, b0 = 0, sub = 0;
         // position of the next slot's batch; false at the end
@@ -326,7 +324,11 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         if (have) ids = request();
         int st = 0; uint32_t round = 0;
         while (have) {
-            const MSet S = sSet[it.set];
+            int blk0 = sSet[it.set].blk_begin, nblk = sSet[it.set].nblk;
+            if (!it.resident) {          // a unit's turn: its blocks only
+                const MUnit& U = sUnit[sGrp[sSet[it.set].grp_begin].unit_begin + rep];
+                blk0 += U.blk0; nblk = U.nblk;
+            }
             const int op = has_a1 ? sub : 1;
             int64_t eid; int32_t sn;
             const uint32_t msk = settle(ids, eid, sn);
@@ -351,8 +353,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: up to sixteen consecutive threads per row
             const __nv_bfloat16* baseh = op == 0 ? a.sh : a.vsh;
             const __nv_bfloat16* basel = op == 0 ? a.sl : a.vsl;
-            for (int bi = 0; bi < S.nblk; ++bi) {
-                const MBlk B = sBlk[S.blk_begin + bi];
+            for (int bi = blk0; bi < blk0 + nblk; ++bi) {
+                const MBlk B = sBlk[bi];
                 const int cpr = (B.c + 7) >> 3;
                 const int lgp = cpr > 8 ? 4 : (cpr > 4 ? 3 : (cpr > 2 ? 2 : 1));
                 const int j = lt & ((1 << lgp) - 1), rows = (NLW * 32) >> lgp, nsg = rows > TB ? rows / TB : 1, sg = (lt >> lgp) / TB;
@@ -384,7 +386,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // Walks the same slots as the loaders and fills their phi and Y rows from the edge vectors (lane <-> edge lane & 15, half
         // of the radial indices / components each).
         if (a.rvec != nullptr) {
-            MsWalk walk(a, nsub, NS, nullptr);
+            MsWalk walk(a, nsub, nullptr);
             MsItem it{};
             const int le = lane & (TB - 1), hf = lane >> 4;
             int st = 0; uint32_t round = 0;
@@ -435,19 +437,26 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     } else if (warp >= W_BUILD && warp < W_BUILD + NBW) {
         // =========================== builder warps ===========================
         const int bt = (warp - W_BUILD) * 32 + lane;
-        MsWalk walk(a, nsub, NS, nullptr);
+        MsWalk walk(a, nsub, nullptr);
         MsItem it{};
         int st0 = 0; uint32_t r0 = 0;          // slot and round of the item's first slot
         int ws = 0; uint32_t wr = 0;
         while (walk.next(it)) {
             if (it.len == 0) continue;
-            const MSet S = sSet[it.set];
+            const int g0 = sSet[it.set].grp_begin, g1 = g0 + sSet[it.set].ngrp;
             int st = st0; uint32_t rd = r0;
-            for (int ui = 0; ui < S.nunit; ++ui) {
+            for (int gi = g0; gi < g1; ++gi)
+            for (int ui = 0; ui < (it.resident ? 1 : sGrp[gi].nunit); ++ui) {          // resident: one W for the units of the group
                 if (it.resident) { st = st0; rd = r0; }
-                const MUnit U = sUnit[S.unit_begin + ui];
-                const uint16_t* rt = sRow + U.row_begin;
-                const int rows = U.N * U.halves;
+                const MGrp& G = sGrp[gi];
+                const uint16_t* rt = sRow + G.row_begin;
+                const int rows = 2 * G.rows, q_first = G.q0;
+                int lo = 0, n_lo = rows, hi = 0, n_hi = 0;                             // rows [lo, lo + n_lo) and [hi, hi + n_hi)
+                if (!it.resident) {
+                    const MUnit& U = sUnit[G.unit_begin + ui];
+                    lo = U.row0; n_lo = U.N;
+                    if (U.halves == 2) { hi = U.row0 + G.rows; n_hi = U.N; }
+                }
                 for (int j = 0; j < it.nslot; ++j) {
                     const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
                     if (warp == W_BUILD) {
@@ -460,9 +469,9 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     const int dv = (a.K + a.dsh) * PS;
                     uint8_t* w = sW + (size_t)ws * a.w_bytes;
                     auto build = [&](int i) {                  // (row, eight edges)
-                        const int n = ((i >> 4) << 3) | (i & 7), h = (i >> 3) & 1;
+                        const int m = ((i >> 4) << 3) | (i & 7), h = (i >> 3) & 1, n = m < n_lo ? lo + m : hi + m - n_lo;
                         const uint32_t qb = rt[n];
-                        const int q = min(U.q0 + (int)(qb & 255u), a.K - 1), b = min((int)(qb >> 8), a.dsh - 1);   // (padding: any value)
+                        const int q = min(q_first + (int)(qb & 255u), a.K - 1), b = (int)(qb >> 8);   // (indices past K: any value)
                         float f[8], y[8], v[8];
                         *reinterpret_cast<float4*>(f) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h);
                         *reinterpret_cast<float4*>(f + 4) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h + 4);
@@ -489,8 +498,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     };
                     int i = bt;
 #pragma unroll 1
-                    for (; i + NBW * 32 < 2 * rows; i += 2 * NBW * 32) { build(i); build(i + NBW * 32); }
-                    if (i < 2 * rows) build(i);
+                    for (; i + NBW * 32 < 2 * (n_lo + n_hi); i += 2 * NBW * 32) { build(i); build(i + NBW * 32); }
+                    if (i < 2 * (n_lo + n_hi)) build(i);
                     fence_async_smem();
                     mbar_arrive(bar_wfull + 8 * ws);
                     if (++ws == NW) { ws = 0; ++wr; }
@@ -501,7 +510,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         }
     } else if (warp == W_MMA) {
         // =========================== MMA warp ===========================
-        MsWalk walk(a, nsub, NS, nullptr);
+        MsWalk walk(a, nsub, nullptr);
         MsItem it{};
         int st0 = 0; uint32_t r0 = 0;
         int ws = 0; uint32_t wr = 0, ai = 0;
@@ -511,43 +520,45 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         const uint32_t slot16 = (uint32_t)a.slot_bytes >> 4, w16 = (uint32_t)a.w_bytes >> 4, xlo16 = (uint32_t)a.x_cap >> 4;
         while (walk.next(it)) {
             if (it.len == 0) continue;
-            const MSet S = sSet[it.set];
+            const int g0 = sSet[it.set].grp_begin, g1 = g0 + sSet[it.set].ngrp;
             int st = st0; uint32_t rd = r0;
-            for (int ui = 0; ui < S.nunit; ++ui, ++ai) {
-                if (it.resident) { st = st0; rd = r0; }
-                const MUnit U = sUnit[S.unit_begin + ui];
-                const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0);
-                // D = F32, A = B = BF16, A MN-major, B K-major, M = 128 / halves
-                const uint32_t uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0);
-                const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | (__shfl_sync(0xffffffffu, 8u / (uint32_t)U.halves, 0) << 24);
-                if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
-                tc_fence_after();
-                const uint32_t d0 = tm_u + buf * HALF;
-                const bool release = ui + 1 == S.nunit || !it.resident;
-                for (int j = 0; j < it.nslot; ++j) {
-                    mbar_spin(bar_full + 8 * st, rd & 1, a.status);
-                    mbar_spin(bar_wfull + 8 * ws, wr & 1, a.status);
-                    if (ui == 0 || !it.resident) fence_async_smem();      // the gathered rows were written through the generic proxy
-                    tc_fence_after();
-                    // (broadcasts: operands that the compiler knows to be uniform take no transfer per instruction)
-                    const uint64_t dX = dX0 + __shfl_sync(0xffffffffu, (uint32_t)st * slot16 + (uint32_t)U.slab0 * (SLAB >> 4), 0),
-                                   dW = dW0 + __shfl_sync(0xffffffffu, (uint32_t)ws * w16, 0);
-                    if (elect_one()) {
-                        const uint32_t acc = j > 0 ? 1u : 0u;
-                        switch (U.d_src * 2 + U.halves) {
-#define SOBEK_MMA(d) case 2 * d + 1: ms_issue<d, 1>(d0, dX, xlo16, dW, uN * 2u, uN, idesc, acc); break; \
-                     case 2 * d + 2: ms_issue<d, 2>(d0, dX, xlo16, dW, uN * 4u, uN, idesc, acc); break;
-                            SOBEK_MMA(1) SOBEK_MMA(3) SOBEK_MMA(5) SOBEK_MMA(7) SOBEK_MMA(9)
-#undef SOBEK_MMA
-                            default: break;
+            for (int gi = g0; gi < g1; ++gi) {
+                const int ws0 = ws; const uint32_t wr0 = wr;
+                const int nu = sGrp[gi].nunit, u_begin = sGrp[gi].unit_begin;
+                const uint32_t grows = __shfl_sync(0xffffffffu, (uint32_t)sGrp[gi].rows, 0);
+                for (int ui = 0; ui < nu; ++ui, ++ai) {
+                    if (it.resident) { st = st0; rd = r0; ws = ws0; wr = wr0; }
+                    const MUnit& U = sUnit[u_begin + ui];
+                    const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0), uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0),
+                                   ud = __shfl_sync(0xffffffffu, (uint32_t)U.d, 0), uh = __shfl_sync(0xffffffffu, (uint32_t)U.halves, 0),
+                                   x0 = __shfl_sync(0xffffffffu, (uint32_t)U.slab0 * (SLAB >> 4), 0), w0 = __shfl_sync(0xffffffffu, (uint32_t)U.row0 * 2u, 0);
+                    // D = F32, A = B = BF16, A MN-major, B K-major, M = 128 / halves
+                    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | ((8u / uh) << 24);
+                    if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
+                    const uint32_t d0 = tm_u + buf * HALF;
+                    const bool wlast = ui + 1 == nu || !it.resident, xlast = (wlast && gi + 1 == g1) || !it.resident;
+                    for (int j = 0; j < it.nslot; ++j) {
+                        if (ui == 0 || !it.resident) {       // (later units of a group find the slot's rows and W in place)
+                            mbar_spin(bar_full + 8 * st, rd & 1, a.status);
+                            mbar_spin(bar_wfull + 8 * ws, wr & 1, a.status);
+                            fence_async_smem();      // the gathered rows were written through the generic proxy
                         }
-                        tc_commit(bar_wfree + 8 * ws);
-                        if (release) tc_commit(bar_sfree + 8 * st);
-                        if (j + 1 == it.nslot) tc_commit(bar_accfull + 8 * buf);
+                        tc_fence_after();
+                        // (broadcasts: operands that the compiler knows to be uniform take no transfer per instruction)
+                        const uint64_t dX = dX0 + (x0 + __shfl_sync(0xffffffffu, (uint32_t)st * slot16, 0)),
+                                       dW = dW0 + (w0 + __shfl_sync(0xffffffffu, (uint32_t)ws * w16, 0));
+                        if (elect_one()) {
+                            const uint32_t acc = j > 0 ? 1u : 0u;
+                            if (uh == 2) ms_issue<2>(ud, d0, dX, xlo16, dW, grows * 4u, grows * 2u, uN, idesc, acc);
+                            else ms_issue<1>(ud, d0, dX, xlo16, dW, grows * 4u, 0u, uN, idesc, acc);
+                            if (wlast) tc_commit(bar_wfree + 8 * ws);
+                            if (xlast) tc_commit(bar_sfree + 8 * st);
+                            if (j + 1 == it.nslot) tc_commit(bar_accfull + 8 * buf);
+                        }
+                        __syncwarp();
+                        if (++ws == NW) { ws = 0; ++wr; }
+                        if (++st == NS) { st = 0; ++rd; }
                     }
-                    __syncwarp();
-                    if (++ws == NW) { ws = 0; ++wr; }
-                    if (++st == NS) { st = 0; ++rd; }
                 }
             }
             st0 = st; r0 = rd;
@@ -555,12 +566,12 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     } else if (warp < NDW) {
         // =========================== drain warps ===========================
         const int grp = warp / (4 * MS_NDT), quarter = warp & 3;
-        MsWalk walk(a, nsub, NS, nullptr);
+        MsWalk walk(a, nsub, nullptr);
         MsItem it{};
         uint32_t ai = 0;
         const int team = (warp >> 2) % MS_NDT;
         while (walk.next(it)) {
-            const int u_begin = sSet[it.set].unit_begin, nunit = sSet[it.set].nunit;
+            const int u_begin = sGrp[sSet[it.set].grp_begin].unit_begin, nunit = sSet[it.set].nunit, R = sSet[it.set].nq;
             const bool full = it.len > 0;
             for (int ui = 0; ui < nunit; ++ui) {
                 const uint32_t buf = full ? (ai & 1) : (uint32_t)(ui & 1);
@@ -576,9 +587,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (quarter * uw < U.c) {
                     const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
                     const int u = quarter * uw + (lane & (uw - 1)), qh = lane >= uw ? 1 : 0;
-                    if (U.nq > 4) read_out<8>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
-                    else if (U.nq > 2) read_out<4>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
-                    else if (U.nq == 2) read_out<2>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    if (R == 4) read_out<4>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    else if (R == 2) read_out<2>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
                     else read_out<1>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
                 }
                 if (full) {

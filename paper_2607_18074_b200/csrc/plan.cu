@@ -515,6 +515,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
         for (MomentSets& t : d->ms) {
             if (!t.ok) continue;
             if (e == cudaSuccess) e = upload(t.sets, &t.d_sets);
+            if (e == cudaSuccess) e = upload(t.grps, &t.d_grps);
             if (e == cudaSuccess) e = upload(t.blks, &t.d_blks);
             if (e == cudaSuccess) e = upload(t.units, &t.d_units);
             if (e == cudaSuccess) e = upload(t.terms, &t.d_terms);
@@ -572,7 +573,7 @@ extern "C" void sobek_plan_destroy(sobek_plan* p) {
         cudaFree(d->d_stasks); cudaFree(d->d_scomps); cudaFree(d->d_etasks); cudaFree(d->d_ecomps); cudaFree(d->d_zb_off);
         cudaFree(d->d_fstages); cudaFree(d->d_fs_begin); cudaFree(d->d_fs_count); cudaFree(d->d_fk_off);
         for (MomentSets& t : d->ms) {
-            cudaFree(t.d_sets); cudaFree(t.d_blks); cudaFree(t.d_units); cudaFree(t.d_terms); cudaFree(t.d_outs); cudaFree(t.d_rows);
+            cudaFree(t.d_sets); cudaFree(t.d_grps); cudaFree(t.d_blks); cudaFree(t.d_units); cudaFree(t.d_terms); cudaFree(t.d_outs); cudaFree(t.d_rows);
         }
         for (TcSets* tp : {&d->etc[0], &d->etc[1]}) {
             TcSets& t = *tp;
