@@ -24,8 +24,10 @@
 //   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
 //   builder warps  W of one (unit, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
 //   MMA warp       one elected lane issues the three products per component (and lane half);
-//   drain warps    two groups, one per TMEM half, of two teams of four warps that share the unit's state components: a lane holds one
-//                  multiplicity, sums the coupling terms and writes bf16 hi / lo.
+//   drain warps    four teams of four warps (one per TMEM lane quarter) that share the state components of a unit: a lane holds one
+//                  multiplicity, sums the coupling terms and writes bf16 hi / lo.  All of them work on one accumulator while the
+//                  other is filled: with a group of its own for each, the read-out took twice as long as the products and both
+//                  waited a third of the time.
 // With DUAL the kernel produces the directional state of the double backward (Eq. receiver_double_adjoint)
 //     dP = sum_e (vphi Y + phi vY)[q,b] x[s,u] + (phi Y)[q,b] vx[s,u]
 // as two slots per batch of edges.  The same kernel runs the sender-owned transposed traversal.  Every wait is bounded.
@@ -565,22 +567,19 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         }
     } else if (warp < NDW) {
         // =========================== drain warps ===========================
-        const int grp = warp / (4 * MS_NDT), quarter = warp & 3;
+        const int quarter = warp & 3, team = warp >> 2;
         MsWalk walk(a, nsub, nullptr);
         MsItem it{};
         uint32_t ai = 0;
-        const int team = (warp >> 2) % MS_NDT;
         while (walk.next(it)) {
             const int u_begin = sGrp[sSet[it.set].grp_begin].unit_begin, nunit = sSet[it.set].nunit, R = sSet[it.set].nq;
             const bool full = it.len > 0;
             for (int ui = 0; ui < nunit; ++ui) {
-                const uint32_t buf = full ? (ai & 1) : (uint32_t)(ui & 1);
-                const uint32_t par = (ai >> 1) & 1;
+                const uint32_t buf = ai & 1, par = (ai >> 1) & 1;
                 if (full) ++ai;
-                if (buf != (uint32_t)grp) continue;
                 const MUnit& U = sUnit[u_begin + ui];
                 if (full) {
-                    role_wait(warp % (4 * MS_NDT) == 0, 1 + grp, 4 * MS_NDT * 32, bar_accfull + 8 * buf, par, a.status);
+                    role_wait(warp == 0, 1, NDW * 32, bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
                 const int uw = 32 / U.halves;          // multiplicities of a quarter
