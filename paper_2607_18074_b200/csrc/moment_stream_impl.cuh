@@ -102,63 +102,51 @@ __device__ __forceinline__ void st_b32_if(uint32_t ok, void* p, uint32_t v) {
 // cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients the same sums ran at
 // 8 - 10 cycles an instruction, however many warps and independent chains there were: every warp streamed kilobytes of code
 // through the instruction cache for each radial index.)
-template <int R>
+// FULL: every lane and radial index of the unit is wanted.
+template <int R, bool FULL>
 __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
                                          int team, int u, int qh) {
-    constexpr int G = 2;                   // pairs of terms per wait
-    const int q0 = U.q0 + qh, n_out = U.n_out, nqs = U.nqs, rows_q = U.rows_q, Kq = u < U.c ? a.K : 0;
+    const int q0 = U.q0 + qh, n_out = U.n_out, nqs = U.nqs, rows_q = U.rows_q, Kq = FULL ? 0 : (u < U.c ? a.K : 0);
     const uint32_t sel = u & 1 ? 0x1054u : 0x7632u;
     __nv_bfloat16* const z0 = u & 1 ? a.zl + u - 1 : a.zh + u;
     outs += U.out_begin;
-    MOut e = outs[team < n_out ? team : 0];
 #pragma unroll 1
     for (int o = team; o < n_out; o += MS_NDT) {
-        __nv_bfloat16* const z = z0 + (e.a + nl * e.b);
-        const uint4* tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
-        const int n = full ? e.n : 0;
-        const uint32_t q_step = 2u * (uint32_t)e.c_row;
-        uint32_t off = (uint32_t)(q0 * e.c_row);
-        e = outs[min(o + MS_NDT, n_out - 1)];
+        const MOut e = outs[o];
+        const uint4* const tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
+        const uint32_t step = 4u * (uint32_t)e.c_row;                                  // bytes from one radial index of this lane to the next
+        char* z = reinterpret_cast<char*>(z0 + (e.a + nl * e.b + (uint32_t)(q0 * e.c_row)));
+        const int n = full ? e.n >> 1 : 0;
+        uint32_t t = t0;
+        int q = q0;
 #pragma unroll 1
-        for (int qc = 0; qc < nqs; ++qc) {
+        for (int qc = 0; qc < nqs; ++qc, t += (uint32_t)rows_q, q += 2 * R, z += (size_t)(R * step)) {
             float acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = 0.f;
-            const uint32_t t = t0 + (uint32_t)(qc * rows_q);
 #pragma unroll 1
-            for (int k = 0; k < n; k += 2 * G) {
-                float p[2 * G][R];
-                uint4 c[G];
-                c[0] = tp[k >> 1];
-                tm_ld<R>(t + c[0].x, p[0]);
-                tm_ld<R>(t + c[0].z, p[1]);
-                const bool more = G > 1 && k + 2 < n;
-                if (more) {
-                    c[G - 1] = tp[(k >> 1) + G - 1];
-                    tm_ld<R>(t + c[G - 1].x, p[2 * G - 2]);
-                    tm_ld<R>(t + c[G - 1].z, p[2 * G - 1]);
-                }
+            for (int k = 0; k < n; ++k) {
+                float p0[R], p1[R];
+                const uint4 c = tp[k];
+                tm_ld<R>(t + c.x, p0);
+                tm_ld<R>(t + c.z, p1);
                 tc_wait_ld();
-                tm_pin<R>(p[0]);
-                tm_pin<R>(p[1]);
+                tm_pin<R>(p0);
+                tm_pin<R>(p1);
 #pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c[0].w), p[1][r], fmaf(__uint_as_float(c[0].y), p[0][r], acc[r]));
-                if (more) {
-                    tm_pin<R>(p[2 * G - 2]);
-                    tm_pin<R>(p[2 * G - 1]);
+                for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c.y), p0[r], acc[r]);
 #pragma unroll
-                    for (int r = 0; r < R; ++r)
-                        acc[r] = fmaf(__uint_as_float(c[G - 1].w), p[2 * G - 1][r], fmaf(__uint_as_float(c[G - 1].y), p[2 * G - 2][r], acc[r]));
-                }
+                for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c.w), p1[r], acc[r]);
             }
             // Two neighbouring lanes swap halves: the even one writes the hi, the odd one the lo parts of both multiplicities.
-            const int q = q0 + 2 * R * qc;
 #pragma unroll
-            for (int r = 0; r < R; ++r, off += q_step) {
+            for (int r = 0; r < R; ++r) {
                 uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
-                st_b32_if(q + 2 * r < Kq, z + off, __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel));
+                const uint32_t y = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel);
+                if (FULL) *reinterpret_cast<uint32_t*>(z + (size_t)(r * step)) = y;
+                else st_b32_if(q + 2 * r < Kq, z + (size_t)(r * step), y);
             }
         }
     }
@@ -586,9 +574,12 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (quarter * uw < U.c) {
                     const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
                     const int u = quarter * uw + (lane & (uw - 1)), qh = lane >= uw ? 1 : 0;
-                    if (R == 4) read_out<4>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
-                    else if (R == 2) read_out<2>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
-                    else read_out<1>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh);
+                    const bool all = (quarter + 1) * uw <= U.c && U.q0 + U.halves + 2 * (R * U.nqs - 1) <= a.K;
+#define SOBEK_READ(r) (all ? read_out<r, true>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh) : read_out<r, false>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh))
+                    if (R == 4) SOBEK_READ(4);
+                    else if (R == 2) SOBEK_READ(2);
+                    else SOBEK_READ(1);
+#undef SOBEK_READ
                 }
                 if (full) {
                     tc_fence_before();
