@@ -72,26 +72,18 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
 }
 
 // ---- read-out: n consecutive columns of this thread's TMEM lane ----------------
-__device__ __forceinline__ void tm_ld1(uint32_t t, float* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(v[0]) : "r"(t) : "memory");
-}
-__device__ __forceinline__ void tm_ld2(uint32_t t, float* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(t) : "memory");
-}
-__device__ __forceinline__ void tm_ld4(uint32_t t, float* v) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
-                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
-}
+// R columns from each of two places, waited for
 template <int R>
-__device__ __forceinline__ void tm_ld(uint32_t t, float* v) {
-    if constexpr (R == 4) tm_ld4(t, v);
-    else if constexpr (R == 2) tm_ld2(t, v);
-    else tm_ld1(t, v);
-}
-template <int R>
-__device__ __forceinline__ void tm_pin(float* v) {      // after the wait: nothing that reads the registers is scheduled ahead of it
-#pragma unroll
-    for (int r = 0; r < R; ++r) asm volatile("" : "+f"(v[r]));
+__device__ __forceinline__ void tm_ld_pair(uint32_t ta, uint32_t tb, float* p, float* q) {
+    if constexpr (R == 4)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n\ttcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n\ttcgen05.wait::ld.sync.aligned;"
+                     : "=f"(p[0]), "=f"(p[1]), "=f"(p[2]), "=f"(p[3]), "=f"(q[0]), "=f"(q[1]), "=f"(q[2]), "=f"(q[3]) : "r"(ta), "r"(tb) : "memory");
+    else if constexpr (R == 2)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%4];\n\ttcgen05.ld.sync.aligned.32x32b.x2.b32 {%2,%3}, [%5];\n\ttcgen05.wait::ld.sync.aligned;"
+                     : "=f"(p[0]), "=f"(p[1]), "=f"(q[0]), "=f"(q[1]) : "r"(ta), "r"(tb) : "memory");
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%2];\n\ttcgen05.ld.sync.aligned.32x32b.x1.b32 {%1}, [%3];\n\ttcgen05.wait::ld.sync.aligned;"
+                     : "=f"(p[0]), "=f"(q[0]) : "r"(ta), "r"(tb) : "memory");
 }
 __device__ __forceinline__ void st_b32_if(uint32_t ok, void* p, uint32_t v) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(p), "r"(v), "r"(ok) : "memory");
@@ -128,11 +120,7 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
             for (int k = 0; k < n; ++k) {
                 float p0[R], p1[R];
                 const uint4 c = tp[k];
-                tm_ld<R>(t + c.x, p0);
-                tm_ld<R>(t + c.z, p1);
-                tc_wait_ld();
-                tm_pin<R>(p0);
-                tm_pin<R>(p1);
+                tm_ld_pair<R>(t + c.x, t + c.z, p0, p1);
 #pragma unroll
                 for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c.y), p0[r], acc[r]);
 #pragma unroll
