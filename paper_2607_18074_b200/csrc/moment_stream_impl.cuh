@@ -106,13 +106,13 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
     for (int o = team; o < n_out; o += MS_NDT) {
         const MOut e = outs[o];
         const uint4* const tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
-        const uint32_t step = 4u * (uint32_t)e.c_row;                                  // bytes from one radial index of this lane to the next
-        char* z = reinterpret_cast<char*>(z0 + (e.a + nl * e.b + (uint32_t)(q0 * e.c_row)));
+        const uint32_t step = (uint32_t)e.c_row;         // words from one radial index of this lane to the next
+        uint32_t* z = reinterpret_cast<uint32_t*>(z0 + (e.a + nl * e.b + (uint32_t)(q0 * e.c_row)));
         const int n = full ? e.n >> 1 : 0;
         uint32_t t = t0;
         int q = q0;
 #pragma unroll 1
-        for (int qc = 0; qc < nqs; ++qc, t += (uint32_t)rows_q, q += 2 * R, z += (size_t)(R * step)) {
+        for (int qc = 0; qc < nqs; ++qc, t += (uint32_t)rows_q) {
             float acc[R];
 #pragma unroll
             for (int r = 0; r < R; ++r) acc[r] = 0.f;
@@ -133,8 +133,9 @@ __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const 
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
                 asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
                 const uint32_t y = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel);
-                if (FULL) *reinterpret_cast<uint32_t*>(z + (size_t)(r * step)) = y;
-                else st_b32_if(q + 2 * r < Kq, z + (size_t)(r * step), y);
+                if (FULL) *z = y;
+                else { st_b32_if(q < Kq, z, y); q += 2; }
+                z += step;
             }
         }
     }
