@@ -9,7 +9,7 @@ namespace sobek {
 constexpr int MS_TB = 16;               // edges per slot = k extent of one MMA
 constexpr int MS_NDT = 4;               // drain teams (four warps each, one per TMEM lane quarter)
 constexpr int MS_NDW = 4 * MS_NDT;
-constexpr int MS_NLW = 2;               // loader warps
+constexpr int MS_NLW = 4;               // loader warps
 constexpr int MS_NBW = 4;               // builder warps
 constexpr int MS_TT = (MS_NDW + MS_NLW + MS_NBW + 2) * 32;      // plus the MMA warp and the geometry warp
 constexpr int MS_MAXNS = 8;             // ring slots at most

@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     const int nsub = (has_a1 ? 1 : 0) + (has_a2 ? 1 : 0);
 
     if (tid == 0) {
-        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, NLW * 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 1); }
+        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 1); }
         for (int s = 0; s < MS_MAXNW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 1); }
         for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, 4 * MS_NDT); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -253,7 +253,9 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
 
     if (warp >= W_LOAD && warp < W_LOAD + NLW) {
         // =========================== loader warps ===========================
-        const int lt = (warp - W_LOAD) * 32 + lane;
+        // A slot is filled by one warp alone, the warps take turns: a warp spends most of its time on index arithmetic, a few cycles an instruction
+        // whatever the others do, so slots side by side go faster than warps side by side on one slot (2.3 against 0.8 us).
+        const int me = warp - W_LOAD;
         const int le = lane & (TB - 1);
         MsWalk walk(a, nsub, a.status);
         MsItem it{};
@@ -298,11 +300,26 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             }
             return __ballot_sync(0xffffffffu, ok);
         };
-        bool have = advance(true);
+        int st = 0; uint32_t round = 0;      // of the slot at hand
+        // its index mod the number of warps that take part: no more than slots, so that the free barrier of a slot is never waited
+        // for two phases ahead
+        const int nlw = min(NLW, NS);
+        int turn = 0;
+        auto to_mine = [&](bool first) -> bool {
+            bool more = advance(first);
+            if (!first) { if (++st == NS) { st = 0; ++round; } if (++turn == nlw) turn = 0; }
+            while (more && turn != me) {
+                more = advance(false);
+                if (++st == NS) { st = 0; ++round; }
+                if (++turn == nlw) turn = 0;
+            }
+            return more;
+        };
+        bool have = me < nlw && to_mine(true);
         Ids ids{0, 0, false};
         if (have) ids = request();
-        int st = 0; uint32_t round = 0;
         while (have) {
+            const int st_now = st; const uint32_t round_now = round;
             int blk0 = sSet[it.set].blk_begin, nblk = sSet[it.set].nblk;
             if (!it.resident) {          // a unit's turn: its blocks only
                 const MUnit& U = sUnit[sGrp[sSet[it.set].grp_begin].unit_begin + rep];
@@ -311,54 +328,56 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             const int op = has_a1 ? sub : 1;
             int64_t eid; int32_t sn;
             const uint32_t msk = settle(ids, eid, sn);
-            have = advance(false);
+            have = to_mine(false);
             if (have) ids = request();
-            if (round > 0) role_wait(warp == W_LOAD, 4, NLW * 32, bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
-            const uint32_t slot_u = smem_u32(sRing + (size_t)st * a.slot_bytes);
+            if (round_now > 0) mbar_spin(bar_sfree + 8 * st_now, (round_now & 1) ^ 1, a.status);
+            const uint32_t slot_u = smem_u32(sRing + (size_t)st_now * a.slot_bytes);
             const uint32_t raw_u = slot_u + (uint32_t)(2 * a.x_cap);
             if (!a.rvec) {
-                // phi and Y, transposed: thread <-> (edge le, every eighth radial index / harmonic)
+                // phi and Y, transposed: thread <-> (edge le, every second radial index / harmonic)
                 const int64_t ee = __shfl_sync(0xffffffffu, eid, le);
                 const uint32_t ok = ((msk >> le) & 1u) * 4u;
-                for (int q = lt >> 4; q < a.K; q += NLW * 32 / TB) {
+                for (int q = lane >> 4; q < a.K; q += 32 / TB) {
                     cp_async4_zfill(raw_u + (uint32_t)(q * PS + le) * 4, a.phi + ee * a.K + q, ok);
                     if (has_vphi) cp_async4_zfill(raw_u + (uint32_t)((a.K + a.dsh + q) * PS + le) * 4, a.vphi + ee * a.K + q, ok);
                 }
-                for (int b = lt >> 4; b < a.dsh; b += NLW * 32 / TB) {
+                for (int b = lane >> 4; b < a.dsh; b += 32 / TB) {
                     cp_async4_zfill(raw_u + (uint32_t)((a.K + b) * PS + le) * 4, a.Y + ee * a.dsh + b, ok);
                     if (has_vY) cp_async4_zfill(raw_u + (uint32_t)((2 * a.K + a.dsh + b) * PS + le) * 4, a.vY + ee * a.dsh + b, ok);
                 }
             }
-            // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: up to sixteen consecutive threads per row
+            // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: two to sixteen consecutive threads per row
             const __nv_bfloat16* baseh = op == 0 ? a.sh : a.vsh;
             const __nv_bfloat16* basel = op == 0 ? a.sl : a.vsl;
             for (int bi = blk0; bi < blk0 + nblk; ++bi) {
                 const MBlk B = sBlk[bi];
                 const int cpr = (B.c + 7) >> 3;
                 const int lgp = cpr > 8 ? 4 : (cpr > 4 ? 3 : (cpr > 2 ? 2 : 1));
-                const int j = lt & ((1 << lgp) - 1), rows = (NLW * 32) >> lgp, nsg = rows > TB ? rows / TB : 1, sg = (lt >> lgp) / TB;
+                const int j = lane & ((1 << lgp) - 1), rows = 32 >> lgp;
+                const int step = B.nch * SLAB;
+                const int64_t g0 = B.src_off + 8 * j;
+                const uint32_t d0 = slot_u + (uint32_t)((B.slab0 + (j >> 3)) * SLAB);
 #pragma unroll 1
                 for (int re0 = 0; re0 < TB; re0 += rows) {
-                    const int re = re0 + ((lt >> lgp) & (TB - 1));
+                    const int re = re0 + (lane >> lgp);
                     const int32_t sne = __shfl_sync(0xffffffffu, sn, re);
                     if (j < cpr) {
                         const uint32_t ok = ((msk >> re) & 1u) * 16u;
-                        const int64_t g = (int64_t)sne * a.C_src + B.src_off + 8 * j;
-                        const int step = nsg * B.nch * SLAB;
-                        uint32_t dst = slot_u + (uint32_t)((B.slab0 + sg * B.nch + (j >> 3)) * SLAB + re * 128 + (((j & 7) ^ (re & 7)) << 4));
-                        const __nv_bfloat16* ph = baseh + g + sg * B.c_row;
-                        const __nv_bfloat16* pl = basel + g + sg * B.c_row;
-                        for (int s = sg; s < B.d_src; s += nsg) {
+                        const int64_t g = (int64_t)sne * a.C_src + g0;
+                        uint32_t dst = d0 + (uint32_t)(re * 128 + (((j & 7) ^ (re & 7)) << 4));
+                        const __nv_bfloat16* ph = baseh + g;
+                        const __nv_bfloat16* pl = basel + g;
+#pragma unroll 3
+                        for (int s = 0; s < B.d_src; ++s) {
                             cp_async16_zfill(dst, ph, ok);
                             cp_async16_zfill(dst + (uint32_t)a.x_cap, pl, ok);
-                            dst += (uint32_t)step; ph += nsg * B.c_row; pl += nsg * B.c_row;
+                            dst += (uint32_t)step; ph += B.c_row; pl += B.c_row;
                         }
                     }
                 }
             }
             // this thread's arrival on the slot's barrier fires when all its copies above have landed
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st) : "memory");
-            if (++st == NS) { st = 0; ++round; }
+            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st_now) : "memory");
         }
     } else if (warp == W_GEO) {
         // =========================== geometry warp ===========================
