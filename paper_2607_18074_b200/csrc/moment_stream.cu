@@ -29,11 +29,13 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
         if (!ok) continue;
         std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
         const int raw = ((dual ? 2 : 1) * (p->K + p->dim_sh) * MS_PS * 4 + 1023) & ~1023;
-        // blocks of more than 128 multiplicities are cut into equal parts
+        // blocks of more than 128 multiplicities are cut into equal parts, and wider ones than a slot should hold into parts of 64
+        // at most (a node whose slots do not all fit the ring is gathered again for every unit)
         struct Part { int blk, u0, c; };
         std::vector<Part> parts;
         for (size_t b = 0; b < blocks.size(); ++b) {
-            const int n = (blocks[b].c + 127) / 128, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
+            const int most = 2 * blocks[b].d * ((std::min(blocks[b].c, 128) + 63) / 64) * MS_SLAB > kSlotBytes ? 64 : 128;
+            const int n = (blocks[b].c + most - 1) / most, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
             for (int u = 0; u < blocks[b].c; u += per) parts.push_back(Part{(int)b, u, std::min(per, blocks[b].c - u)});
         }
         // Sets: consecutive parts whose rows of 16 edges leave room for four slots with their W (a node of 32 edges and the next
