@@ -11,6 +11,9 @@ namespace {
 
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
+// the stream of a direction runs on the tensor cores, in one of its two forms
+bool tc_stream_ok(const Direction& d, int dual) { return d.ms[dual].ok || d.tc[dual].ok; }
+
 struct Workspace {
     int* status;
     // bf16 (hi, lo) copies of R as tensor-core operands
@@ -98,9 +101,9 @@ Workspace carve(const sobek_plan* p, int64_t N, int order, void* ws) {
     }
     if (p->use_tc_stream || (p->use_tc_edge && p->fwd.etc[0].ok)) {
         const size_t nx = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_x * 2, ny = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_y * 2;
-        if (p->fwd.ms[0].ok || (order >= 2 && p->fwd.ms[1].ok) || (order >= 1 && w.zqh)) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
-        if (order >= 1 && (p->tr.ms[0].ok || (order >= 2 && p->tr.ms[1].ok))) { w.gsh = (uint16_t*)take(ny); w.gsl = (uint16_t*)take(ny); }
-        if (order >= 2 && (p->fwd.ms[1].ok || (w.zqh && p->fwd.etc[1].ok))) { w.vsh = (uint16_t*)take(nx); w.vsl = (uint16_t*)take(nx); }
+        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || (order >= 1 && w.zqh)) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
+        if (order >= 1 && (tc_stream_ok(p->tr, 0) || (order >= 2 && tc_stream_ok(p->tr, 1)))) { w.gsh = (uint16_t*)take(ny); w.gsl = (uint16_t*)take(ny); }
+        if (order >= 2 && (tc_stream_ok(p->fwd, 1) || (w.zqh && p->fwd.etc[1].ok))) { w.vsh = (uint16_t*)take(nx); w.vsl = (uint16_t*)take(nx); }
         // load balance of the persistent edge kernels: only where a CTA takes several nodes of a chunk
         if (w.chunk >= kOrderMinChunk && N >= kOrderMinChunk) {
             w.oseg_r = (int4*)take((size_t)N * sizeof(int4));
@@ -335,8 +338,8 @@ namespace {
 // Geometry mode (Y and phi recomputed from edge vectors inside the edge kernels) exists in the tensor-core edge
 // kernels only: the plan must run them in both directions, unfused, in the ir_mul layout, with l_max <= 4.
 bool geo_supported(const sobek_plan* p, const Workspace& w, int order) {
-    if (!p->use_tc_stream || !p->fwd.ms[0].ok || !w.xsh || w.fused_f || p->mul_ir || p->dim_sh > 25) return false;
-    return order == 0 || (p->tr.ms[0].ok && p->fwd.etc[0].ok && w.gsh && w.zqh && !w.fused_t);
+    if (!p->use_tc_stream || !tc_stream_ok(p->fwd, 0) || !w.xsh || w.fused_f || p->mul_ir || p->dim_sh > 25) return false;
+    return order == 0 || (tc_stream_ok(p->tr, 0) && p->fwd.etc[0].ok && w.gsh && w.zqh && !w.fused_t);
 }
 // `order` is the workspace layout to use (0, or 1 when the state is to be found by a following backward call);
 // *retained is set to 1 when the state of every receiver is left in the workspace (one chunk, state schedule)
@@ -490,7 +493,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
     if (hx && g->E > 0 && (!g->src_ptr || !g->src_perm)) return SOBEK_ERR_NEED_TRANSPOSE;
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(p, g->N, 2, ws);
-    if (geo && !(geo_supported(p, w, 1) && p->fwd.ms[1].ok && p->tr.ms[1].ok && w.vsh)) return SOBEK_ERR_UNSUPPORTED;
+    if (geo && !(geo_supported(p, w, 1) && tc_stream_ok(p->fwd, 1) && tc_stream_ok(p->tr, 1) && w.vsh)) return SOBEK_ERR_UNSUPPORTED;
     CK(cudaMemsetAsync(w.status, 0, kHeaderBytes, s));
     const int64_t KN = (int64_t)p->K * p->N_w;
     const bool any_edge_dir = vx || vY || vphi;

@@ -62,8 +62,10 @@ cudaError_t launch_stream(const sobek_plan* p, const Direction& dir, const EdgeV
                           int* status, cudaStream_t s) {
     if (n_nodes <= 0 || dir.stasks.empty()) return cudaSuccess;
     // tensor-core stream when the profile allows it and the caller made the bf16 copies of the sources
-    if (p->use_tc_stream && dir.ms[dual ? 1 : 0].ok && status && ss.h && ss.l && (!vsrc || (ss.vh && ss.vl)))
-        return launch_moment_stream(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
+    if (p->use_tc_stream && status && ss.h && ss.l && (!vsrc || (ss.vh && ss.vl))) {
+        if (dir.ms[dual ? 1 : 0].ok) return launch_moment_stream(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
+        if (dir.tc[dual ? 1 : 0].ok) return launch_stream_tc(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
+    }
     if (ss.rvec) return cudaErrorNotSupported;      // the geometry mode exists in the tensor-core kernels only
     const int KC = p->K <= 8 ? 8 : 16;
     StreamArgsHost a{};

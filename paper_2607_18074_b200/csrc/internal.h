@@ -177,22 +177,21 @@ struct MGrp {          // radial indices whose W is built at once, and the units
     int32_t unit_begin, nunit;
     int32_t pad[3];
 };
-struct MBlk {          // (part of) a source block: at most 128 multiplicities
+struct MBlk {          // (part of) a source block: at most 64 multiplicities
     int32_t src_off, c;       // first element inside a source feature row, multiplicities
     int32_t c_row, d_src;     // elements between consecutive components, components
-    int32_t slab0, nch;       // first slab of the block in a slot, slabs (64 multiplicities each) per component
-    int32_t pad[2];
+    int32_t slab0;            // first slab of the block in a slot (one per component)
+    int32_t pad[3];
 };
 struct MUnit {         // one accumulator: components of neighbouring blocks x rows of W
     int32_t slab0, d;         // first slab, components
-    int32_t halves;           // 2: M = 64 products, even / odd radial indices in the lane halves; 1: M = 128, one of the two
-    int32_t row0, N;          // first row of W (of the lower half if halves == 2), rows = columns of one product
+    int32_t row0, N;          // first row of W (in either lane half), rows = columns of one product
     int32_t nqs, rows_q;      // runs of radial indices side by side, columns from one to the next
     int32_t q0;               // first radial index
     int32_t c;                // multiplicities
     int32_t blk0, nblk;       // blocks, relative to the set's
     int32_t out_begin, n_out; // state components
-    int32_t pad[3];
+    int32_t pad[4];
 };
 struct MOut {          // a state component (path, o) and its coupling terms
     int64_t a;                // state offset of radial index 0, multiplicity 0 for node 0, without the group's share:
@@ -245,6 +244,7 @@ struct Direction {
     std::vector<SClass> sclasses;
     STask* d_stasks = nullptr;
     SComp* d_scomps = nullptr;
+    TcSets tc[2];                     // coupling-in-operand stream on the tensor cores: [0] plain, [1] dual
     MomentSets ms[2];                 // moment-form stream: [0] plain, [1] dual
     TcSets etc[2];                    // tensor-core edge pass: [0] plain, [1] dual
     // receiver-owned edge pass: source-major tasks over all multiplicities
@@ -422,6 +422,11 @@ cudaError_t launch_edge_pass_tc(const sobek_plan* p, const Direction& dir, const
                                 int64_t n_nodes, const SplitSrc& ss, const float* Y, const float* vY, const float* phi,
                                 const float* vphi, int dual, const void* zqh, const void* zql, float* gphi, float* gY,
                                 int phi_mode, int Y_mode, int* status, cudaStream_t s);
+// --- stream_tc.cu ---------------------------------------------------------------------
+void build_tc_sets(const sobek_plan* p, Direction& dir);
+cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
+                             int64_t n_nodes, const SplitSrc& ss, const float* Y, const float* vY, const float* phi,
+                             const float* vphi, int dual, void* zh, void* zl, int* status, cudaStream_t s);
 // --- moment_stream.cu -------------------------------------------------------------------
 void build_moment_sets(const sobek_plan* p, Direction& dir);
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,

@@ -5,6 +5,24 @@
 
 namespace sobek {
 
+// Where both forms of the stream apply, which one: measured on 2,000 nodes of degree 30 in whole calls, time of the other form over
+// that of this one, m x (0..L).
+//   forward   K = 8:  L = 1 1.26 - 1.37, L = 2 1.06 - 1.15, L = 3 1.04 - 1.17, L = 4 1.03 - 1.14   (m = 8 .. 64)
+//             K = 16: L = 1 1.04 - 1.12, L = 2 1.01 - 1.21, L = 3 0.91 - 1.06, L = 4 0.80 - 0.95
+//   second order (the dual stream and the plain one of the transposed direction)  1.01 - 1.25 throughout
+//   m = 96, cut into 48 + 48 of 64 rows: 0.76 - 1.13, mostly below one; m = 128: 0.94 - 1.26
+// The plain form loses where a run of radial indices has to be split over many narrow products: orders from three on with more
+// than eight radial indices; both lose where cutting a wide block leaves the products a quarter empty.
+static bool moment_form_pays(const sobek_plan* p, const Direction& dir, int dual) {
+    int d = 0, rows = 0, used = 0;
+    for (const DPath& P : dir.paths) {
+        d = std::max(d, P.d_src);
+        if (P.c_src > 64) { rows += P.d_src * 64 * ((P.c_src + 63) / 64); used += P.d_src * P.c_src; }
+    }
+    if (rows && used * 5 < rows * 4) return false;
+    return dual || p->K <= 8 || d <= 5;
+}
+
 // Sets, units and read-out tables of one direction for the plain ([0]) and the dual ([1]) stream.
 void build_moment_sets(const sobek_plan* p, Direction& dir) {
     constexpr int kSmem = 227 * 1024;
@@ -14,6 +32,7 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
         MomentSets& T = dir.ms[dual];
         T = MomentSets{};
         if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) continue;
+        if (dir.tc[dual].ok && !moment_form_pays(p, dir, dual)) continue;
         bool ok = true;
         struct Pth { const DPath* P; int lb, group; };
         struct Blk { int so, c, d; std::vector<Pth> paths; };
@@ -29,39 +48,34 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
         if (!ok) continue;
         std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
         const int raw = ((dual ? 2 : 1) * (p->K + p->dim_sh) * MS_PS * 4 + 1023) & ~1023;
-        // blocks of more than 128 multiplicities are cut into equal parts, and wider ones than a slot should hold into parts of 64
-        // at most (a node whose slots do not all fit the ring is gathered again for every unit)
+        // blocks of more than 64 multiplicities are cut into equal parts
         struct Part { int blk, u0, c; };
         std::vector<Part> parts;
         for (size_t b = 0; b < blocks.size(); ++b) {
-            const int most = 2 * blocks[b].d * ((std::min(blocks[b].c, 128) + 63) / 64) * MS_SLAB > kSlotBytes ? 64 : 128;
-            const int n = (blocks[b].c + most - 1) / most, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
+            const int n = (blocks[b].c + 63) / 64, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
             for (int u = 0; u < blocks[b].c; u += per) parts.push_back(Part{(int)b, u, std::min(per, blocks[b].c - u)});
         }
         // Sets: consecutive parts whose rows of 16 edges leave room for four slots with their W (a node of 32 edges and the next
         // one's first rows); a wider part is a set of its own with the slots it leaves, at least two.
-        auto slabs_of = [&](const Part& q) { return blocks[q.blk].d * ((q.c + 63) / 64); };
         int x_cap = 0;
         for (size_t i = 0; i < parts.size() && ok;) {
             MSet S{};
             S.blk_begin = (int)T.blks.size(); S.grp_begin = (int)T.grps.size();
             int slabs = 0, dmax = 0;
-            bool wide = false;
             size_t j = i;
             for (; j < parts.size(); ++j) {
                 const Blk& B = blocks[parts[j].blk];
-                if (j > i && 2 * (slabs + slabs_of(parts[j])) * MS_SLAB > kSlotBytes) break;
-                T.blks.push_back(MBlk{B.so + parts[j].u0, parts[j].c, B.c, B.d, slabs, (parts[j].c + 63) / 64, {0, 0}});
-                slabs += slabs_of(parts[j]);
+                if (j > i && 2 * (slabs + B.d) * MS_SLAB > kSlotBytes) break;
+                T.blks.push_back(MBlk{B.so + parts[j].u0, parts[j].c, B.c, B.d, slabs, {0, 0, 0}});
+                slabs += B.d;
                 dmax = std::max(dmax, B.d);
-                wide |= parts[j].c > 64;
             }
             S.nblk = (int)T.blks.size() - S.blk_begin;
             x_cap = std::max(x_cap, slabs * MS_SLAB);
             // Rows of W: runs of nq radial indices (those of one lane half), per run the harmonics order by order, the radial
             // index fastest, so that one read-out instruction takes nq of them.  The orders are cut into segments of whole
-            // 8-row (M = 128: 16-row) groups such that every block's components x a segment fit the columns of one TMEM half.
-            const int gran = wide ? 16 : 8, KH = (p->K + 1) / 2;
+            // groups of eight rows such that every block's components x a segment fit the columns of one TMEM half.
+            const int KH = (p->K + 1) / 2;
             struct Seg { int l0, l1, row, rows; };
             std::vector<Seg> segs;
             int nq = KH >= 3 ? 4 : KH, rows_q = 0;
@@ -71,7 +85,7 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
                 for (int l = 0; l <= p->l_max && fits;) {
                     int e = l, rows = 0;
                     for (; e <= p->l_max; ++e) {
-                        const int r = (((e + 1) * (e + 1) - l * l) * nq + gran - 1) & ~(gran - 1);
+                        const int r = (((e + 1) * (e + 1) - l * l) * nq + 7) & ~7;
                         if (dmax * r > MS_HALF) break;
                         rows = r;
                     }
@@ -102,19 +116,18 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
             for (size_t k = i; k < j; ++k) {
                 const Blk& B = blocks[parts[k].blk];
                 const MBlk& M = T.blks[S.blk_begin + (int)(k - i)];
-                const int halves = parts[k].c > 64 ? 1 : 2;
                 auto used = [&](size_t g) { return std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb >= segs[g].l0 && t.lb <= segs[g].l1; }); };
-                auto emit = [&](int h, int run, int n_runs, size_t ga, size_t gb) {          // segments [ga, gb)
+                auto emit = [&](int run, int n_runs, size_t ga, size_t gb) {          // segments [ga, gb)
                     MUnit U{};
-                    U.slab0 = M.slab0; U.d = B.d; U.halves = halves; U.c = M.c; U.blk0 = (int)(k - i); U.nblk = 1;
-                    U.row0 = (halves == 1 ? h * rows_h : 0) + run * rows_q + segs[ga].row;
+                    U.slab0 = M.slab0; U.d = B.d; U.c = M.c; U.blk0 = (int)(k - i); U.nblk = 1;
+                    U.row0 = run * rows_q + segs[ga].row;
                     U.N = n_runs > 1 ? n_runs * rows_q : segs[gb - 1].row + segs[gb - 1].rows - segs[ga].row;
-                    U.nqs = n_runs; U.rows_q = rows_q; U.q0 = 2 * run * nq + (halves == 1 ? h : 0);
+                    U.nqs = n_runs; U.rows_q = rows_q; U.q0 = 2 * run * nq;
                     U.pad[0] = (int)ga; U.pad[1] = (int)gb;
                     if (!us.empty()) {       // together with the block before it, where the columns hold both
                         MUnit& V = us.back();
-                        if (V.row0 == U.row0 && V.N == U.N && V.halves == halves && V.c == U.c && V.blk0 + V.nblk == U.blk0 &&
-                            V.slab0 + V.d * ((V.c + 63) / 64) == U.slab0 && (V.d + U.d) * U.N <= MS_HALF) {
+                        if (V.row0 == U.row0 && V.N == U.N && V.c == U.c && V.blk0 + V.nblk == U.blk0 &&
+                            V.slab0 + V.d == U.slab0 && (V.d + U.d) * U.N <= MS_HALF) {
                             V.d += U.d; ++V.nblk;
                             return;
                         }
@@ -122,20 +135,18 @@ void build_moment_sets(const sobek_plan* p, Direction& dir) {
                     us.push_back(U);
                 };
                 const size_t ns = segs.size();
-                for (int h = 0; h < (halves == 1 ? 2 : 1); ++h) {
-                    size_t ga = 0, gb = ns;
-                    while (ga < ns && !used(ga)) ++ga;
-                    while (gb > ga && !used(gb - 1)) --gb;
-                    if (ga == 0 && gb == ns && B.d * nqs_g * rows_q <= MS_HALF) { emit(h, 0, nqs_g, 0, ns); continue; }
-                    for (int run = 0; run < nqs_g; ++run)
-                        for (size_t x = ga; x < gb;) {
-                            if (!used(x)) { ++x; continue; }
-                            size_t y = x + 1;
-                            while (y < gb && B.d * (segs[y].row + segs[y].rows - segs[x].row) <= MS_HALF) ++y;
-                            emit(h, run, 1, x, y);
-                            x = y;
-                        }
-                }
+                size_t ga = 0, gb = ns;
+                while (ga < ns && !used(ga)) ++ga;
+                while (gb > ga && !used(gb - 1)) --gb;
+                if (ga == 0 && gb == ns && B.d * nqs_g * rows_q <= MS_HALF) { emit(0, nqs_g, 0, ns); continue; }
+                for (int run = 0; run < nqs_g; ++run)
+                    for (size_t x = ga; x < gb;) {
+                        if (!used(x)) { ++x; continue; }
+                        size_t y = x + 1;
+                        while (y < gb && B.d * (segs[y].row + segs[y].rows - segs[x].row) <= MS_HALF) ++y;
+                        emit(run, 1, x, y);
+                        x = y;
+                    }
             }
             // read-out tables (the same for every group)
             for (MUnit& U : us) {

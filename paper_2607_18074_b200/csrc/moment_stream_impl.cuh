@@ -14,16 +14,17 @@
 // 400 at 64 x (0..4), and that build bound the kernel.  fp32 parity comes from the split-bf16 product
 // a*b ~= a_hi*b_hi + a_hi*b_lo + a_lo*b_hi with fp32 accumulation in TMEM; the coupling sums run in fp32.
 //
-// Work items are (set, node): a set is a run of source blocks (128 multiplicities at most each, wider ones are cut) whose gathered
-// rows of 16 edges fit one slot of the shared-memory ring.  An item's accumulators are produced unit after unit: a unit is one
-// block x a range of radial indices x some harmonic orders, at most 256 TMEM columns, so that the two TMEM halves alternate
-// between products and read-out.  Blocks of at most 64 multiplicities use M = 64 products, whose 64 rows take 16 lanes of each
-// 32-lane quarter: the even radial indices go to the lower 16, the odd ones to the upper 16, and every lane has work in the
-// read-out.  When the slots of a node's edges all fit the ring they stay there for all units; longer segments are gathered again
-// for every unit.
+// Work items are (set, node): a set is a run of source blocks (64 multiplicities at most each, wider ones are cut) whose gathered
+// rows of 16 edges fit one slot of the shared-memory ring.  W of a group of radial indices is built once per slot; an item's
+// accumulators are then produced unit after unit: a unit is a run of components x a run of W's rows, at most 256 TMEM columns, so
+// that the two TMEM halves alternate between products and read-out.  The products have M = 64, whose 64 rows take 16 lanes of
+// each 32-lane quarter: the even radial indices go to the lower 16, the odd ones to the upper 16, and every lane has work in the
+// read-out.  (M = 128 for wider blocks has half the products but needs slots twice as large: 128 x (0..2) ran 3 to 17 % slower.)
+// When the slots of a node's edges all fit the rings they stay there for all units; longer segments are gathered again for every
+// unit.
 //   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
-//   builder warps  W of one (unit, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
-//   MMA warp       one elected lane issues the three products per component (and lane half);
+//   builder warps  W of one (group, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
+//   MMA warp       one elected lane issues the three products per component and lane half;
 //   drain warps    four teams of four warps (one per TMEM lane quarter) that share the state components of a unit: a lane holds one
 //                  multiplicity, sums the coupling terms and writes bf16 hi / lo.  All of them work on one accumulator while the
 //                  other is filled: with a group of its own for each, the read-out took twice as long as the products and both
@@ -179,13 +180,12 @@ struct MsWalk {
 
 // The products of one slot: x_hi W_hi, x_hi W_lo, x_lo W_hi per component and lane half.  (x_hi stays in the collector for two
 // products of one lane half; a product into the other half does not find it there.)
-template <int HALVES>
 __device__ __forceinline__ void ms_issue(uint32_t d, uint32_t d0, uint64_t dX, uint32_t xlo16, uint64_t dW, uint32_t wlo16, uint32_t whalf16, uint32_t N,
                                          uint32_t idesc, uint32_t acc) {
 #pragma unroll 2
-    for (uint32_t s = 0; s < d; ++s, d0 += N, dX += (HALVES == 2 ? 1 : 2) * (MS_SLAB >> 4))
+    for (uint32_t s = 0; s < d; ++s, d0 += N, dX += MS_SLAB >> 4)
 #pragma unroll
-        for (int h = 0; h < HALVES; ++h) {
+        for (int h = 0; h < 2; ++h) {
             const uint64_t w = dW + (h ? whalf16 : 0u);
             tc_mma_bf16_x3(d0 + (uint32_t)(h * 16 << 16), dX, dX + xlo16, w, w + wlo16, idesc, acc);
         }
@@ -346,17 +346,16 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     if (has_vY) cp_async4_zfill(raw_u + (uint32_t)((2 * a.K + a.dsh + b) * PS + le) * 4, a.vY + ee * a.dsh + b, ok);
                 }
             }
-            // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: two to sixteen consecutive threads per row
+            // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: two to eight consecutive threads per row
             const __nv_bfloat16* baseh = op == 0 ? a.sh : a.vsh;
             const __nv_bfloat16* basel = op == 0 ? a.sl : a.vsl;
             for (int bi = blk0; bi < blk0 + nblk; ++bi) {
                 const MBlk B = sBlk[bi];
                 const int cpr = (B.c + 7) >> 3;
-                const int lgp = cpr > 8 ? 4 : (cpr > 4 ? 3 : (cpr > 2 ? 2 : 1));
+                const int lgp = cpr > 4 ? 3 : (cpr > 2 ? 2 : 1);
                 const int j = lane & ((1 << lgp) - 1), rows = 32 >> lgp;
-                const int step = B.nch * SLAB;
                 const int64_t g0 = B.src_off + 8 * j;
-                const uint32_t d0 = slot_u + (uint32_t)((B.slab0 + (j >> 3)) * SLAB);
+                const uint32_t d0 = slot_u + (uint32_t)(B.slab0 * SLAB);
 #pragma unroll 1
                 for (int re0 = 0; re0 < TB; re0 += rows) {
                     const int re = re0 + (lane >> lgp);
@@ -364,14 +363,14 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     if (j < cpr) {
                         const uint32_t ok = ((msk >> re) & 1u) * 16u;
                         const int64_t g = (int64_t)sne * a.C_src + g0;
-                        uint32_t dst = d0 + (uint32_t)(re * 128 + (((j & 7) ^ (re & 7)) << 4));
+                        uint32_t dst = d0 + (uint32_t)(re * 128 + ((j ^ (re & 7)) << 4));
                         const __nv_bfloat16* ph = baseh + g;
                         const __nv_bfloat16* pl = basel + g;
 #pragma unroll 3
                         for (int s = 0; s < B.d_src; ++s) {
                             cp_async16_zfill(dst, ph, ok);
                             cp_async16_zfill(dst + (uint32_t)a.x_cap, pl, ok);
-                            dst += (uint32_t)step; ph += B.c_row; pl += B.c_row;
+                            dst += (uint32_t)SLAB; ph += B.c_row; pl += B.c_row;
                         }
                     }
                 }
@@ -452,8 +451,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 int lo = 0, n_lo = rows, hi = 0, n_hi = 0;                             // rows [lo, lo + n_lo) and [hi, hi + n_hi)
                 if (!it.resident) {
                     const MUnit& U = sUnit[G.unit_begin + ui];
-                    lo = U.row0; n_lo = U.N;
-                    if (U.halves == 2) { hi = U.row0 + G.rows; n_hi = U.N; }
+                    lo = U.row0; hi = U.row0 + G.rows; n_lo = n_hi = U.N;
                 }
                 for (int j = 0; j < it.nslot; ++j) {
                     const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
@@ -513,7 +511,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         int st0 = 0; uint32_t r0 = 0;
         int ws = 0; uint32_t wr = 0, ai = 0;
         const uint32_t tm_u = __shfl_sync(0xffffffffu, tmem_base, 0);
-        const uint64_t dX0 = make_desc(smem_u32(sRing), SLAB, 1024);          // 64 multiplicities per row, the next 64 a slab on
+        const uint64_t dX0 = make_desc(smem_u32(sRing), SLAB, 1024);          // 64 multiplicities per row
         const uint64_t dW0 = make_desc_plain(smem_u32(sW), 128, 256);
         const uint32_t slot16 = (uint32_t)a.slot_bytes >> 4, w16 = (uint32_t)a.w_bytes >> 4, xlo16 = (uint32_t)a.x_cap >> 4;
         while (walk.next(it)) {
@@ -528,10 +526,10 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     if (it.resident) { st = st0; rd = r0; ws = ws0; wr = wr0; }
                     const MUnit& U = sUnit[u_begin + ui];
                     const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0), uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0),
-                                   ud = __shfl_sync(0xffffffffu, (uint32_t)U.d, 0), uh = __shfl_sync(0xffffffffu, (uint32_t)U.halves, 0),
+                                   ud = __shfl_sync(0xffffffffu, (uint32_t)U.d, 0),
                                    x0 = __shfl_sync(0xffffffffu, (uint32_t)U.slab0 * (SLAB >> 4), 0), w0 = __shfl_sync(0xffffffffu, (uint32_t)U.row0 * 2u, 0);
-                    // D = F32, A = B = BF16, A MN-major, B K-major, M = 128 / halves
-                    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | ((8u / uh) << 24);
+                    // D = F32, A = B = BF16, A MN-major, B K-major, M = 64
+                    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | (4u << 24);
                     if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
                     const uint32_t d0 = tm_u + buf * HALF;
                     const bool wlast = ui + 1 == nu || !it.resident, xlast = (wlast && gi + 1 == g1) || !it.resident;
@@ -547,8 +545,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                                        dW = dW0 + (w0 + __shfl_sync(0xffffffffu, (uint32_t)ws * w16, 0));
                         if (elect_one()) {
                             const uint32_t acc = j > 0 ? 1u : 0u;
-                            if (uh == 2) ms_issue<2>(ud, d0, dX, xlo16, dW, grows * 4u, grows * 2u, uN, idesc, acc);
-                            else ms_issue<1>(ud, d0, dX, xlo16, dW, grows * 4u, 0u, uN, idesc, acc);
+                            ms_issue(ud, d0, dX, xlo16, dW, grows * 4u, grows * 2u, uN, idesc, acc);
                             if (wlast) tc_commit(bar_wfree + 8 * ws);
                             if (xlast) tc_commit(bar_sfree + 8 * st);
                             if (j + 1 == it.nslot) tc_commit(bar_accfull + 8 * buf);
@@ -578,11 +575,10 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     role_wait(warp == 0, 1, NDW * 32, bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
-                const int uw = 32 / U.halves;          // multiplicities of a quarter
-                if (quarter * uw < U.c) {
+                if (quarter * 16 < U.c) {
                     const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
-                    const int u = quarter * uw + (lane & (uw - 1)), qh = lane >= uw ? 1 : 0;
-                    const bool all = (quarter + 1) * uw <= U.c && U.q0 + U.halves + 2 * (R * U.nqs - 1) <= a.K;
+                    const int u = quarter * 16 + (lane & 15), qh = lane >> 4;
+                    const bool all = quarter * 16 + 16 <= U.c && U.q0 + 2 * R * U.nqs <= a.K;
 #define SOBEK_READ(r) (all ? read_out<r, true>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh) : read_out<r, false>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh))
                     if (R == 4) SOBEK_READ(4);
                     else if (R == 2) SOBEK_READ(2);

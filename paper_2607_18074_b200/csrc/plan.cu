@@ -460,6 +460,8 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
     build_direction(p, 1, p->tr);
     build_stream_tasks(p, p->fwd);
     build_stream_tasks(p, p->tr);
+    build_tc_sets(p, p->fwd);
+    build_tc_sets(p, p->tr);
     build_moment_sets(p, p->fwd);
     build_moment_sets(p, p->tr);
     build_tc_edge_sets(p, p->fwd);
@@ -522,7 +524,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
             if (e == cudaSuccess) e = upload(t.outs, &t.d_outs);
             if (e == cudaSuccess) e = upload(t.rows, &t.d_rows);
         }
-        for (TcSets* tp : {&d->etc[0], &d->etc[1]}) {
+        for (TcSets* tp : {&d->tc[0], &d->tc[1], &d->etc[0], &d->etc[1]}) {
             TcSets& t = *tp;
             if (!t.ok) continue;
             if (e == cudaSuccess) e = upload(t.ents_s, &t.d_ents_s);
@@ -575,7 +577,7 @@ extern "C" void sobek_plan_destroy(sobek_plan* p) {
         for (MomentSets& t : d->ms) {
             cudaFree(t.d_sets); cudaFree(t.d_grps); cudaFree(t.d_blks); cudaFree(t.d_units); cudaFree(t.d_terms); cudaFree(t.d_outs); cudaFree(t.d_rows);
         }
-        for (TcSets* tp : {&d->etc[0], &d->etc[1]}) {
+        for (TcSets* tp : {&d->tc[0], &d->tc[1], &d->etc[0], &d->etc[1]}) {
             TcSets& t = *tp;
             cudaFree(t.d_inv_ptr); cudaFree(t.d_inv);
             cudaFree(t.d_ents_s); cudaFree(t.d_nz); cudaFree(t.d_comps_s); cudaFree(t.d_slabs);
