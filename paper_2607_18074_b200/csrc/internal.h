@@ -423,12 +423,12 @@ cudaError_t launch_edge_pass_tc(const sobek_plan* p, const Direction& dir, const
                                 const float* vphi, int dual, const void* zqh, const void* zql, float* gphi, float* gY,
                                 int phi_mode, int Y_mode, int* status, cudaStream_t s);
 // --- stream_tc.cu ---------------------------------------------------------------------
-void build_tc_sets(const sobek_plan* p, Direction& dir);
+void build_tc_sets(const sobek_plan* p, Direction& dir, int dual);
 cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
                              int64_t n_nodes, const SplitSrc& ss, const float* Y, const float* vY, const float* phi,
                              const float* vphi, int dual, void* zh, void* zl, int* status, cudaStream_t s);
 // --- moment_stream.cu -------------------------------------------------------------------
-void build_moment_sets(const sobek_plan* p, Direction& dir);
+void build_stream_sets(const sobek_plan* p, Direction& dir);
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
                                  const SplitSrc& ss, const float* Y, const float* vY, const float* phi, const float* vphi, int dual,
                                  void* zh, void* zl, int* status, cudaStream_t s);

@@ -23,180 +23,189 @@ static bool moment_form_pays(const sobek_plan* p, const Direction& dir, int dual
     return dual || p->K <= 8 || d <= 5;
 }
 
-// Sets, units and read-out tables of one direction for the plain ([0]) and the dual ([1]) stream.
-void build_moment_sets(const sobek_plan* p, Direction& dir) {
+// Sets, units and read-out tables of one direction, plain or dual stream.
+static void build_moment_set(const sobek_plan* p, Direction& dir, int dual);
+
+// Which form each stream of a direction takes, and its tables (of that form only: a plan is made for every layer of a model).
+void build_stream_sets(const sobek_plan* p, Direction& dir) {
+    for (int dual = 0; dual < 2; ++dual) {
+        const bool pays = moment_form_pays(p, dir, dual);
+        if (pays) build_moment_set(p, dir, dual);
+        if (!dir.ms[dual].ok) build_tc_sets(p, dir, dual);
+        if (!pays && !dir.tc[dual].ok) build_moment_set(p, dir, dual);
+    }
+}
+
+static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
     constexpr int kSmem = 227 * 1024;
     constexpr int kSlotBytes = 37 * 1024;      // gathered rows of a slot, hi and lo, beyond which a block starts a set of its own
     constexpr int kWRows = 224;                // rows of W at a time at most (both lane halves)
-    for (int dual = 0; dual < 2; ++dual) {
-        MomentSets& T = dir.ms[dual];
-        T = MomentSets{};
-        if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) continue;
-        if (dir.tc[dual].ok && !moment_form_pays(p, dir, dual)) continue;
-        bool ok = true;
-        struct Pth { const DPath* P; int lb, group; };
-        struct Blk { int so, c, d; std::vector<Pth> paths; };
-        std::vector<Blk> blocks;
-        for (size_t gi = 0; gi < dir.groups.size(); ++gi)
-            for (int k = dir.groups[gi].path_begin; k < dir.groups[gi].path_end; ++k) {
-                const DPath& P = dir.paths[k];
-                if ((P.c_src & 7) || (P.src_off & 7)) ok = false;
-                auto it = std::find_if(blocks.begin(), blocks.end(), [&](const Blk& b) { return b.so == P.src_off; });
-                if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
-                it->paths.push_back(Pth{&P, (P.d_sh - 1) / 2, (int)gi});
-            }
-        if (!ok) continue;
-        std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
-        const int raw = ((dual ? 2 : 1) * (p->K + p->dim_sh) * MS_PS * 4 + 1023) & ~1023;
-        // blocks of more than 64 multiplicities are cut into equal parts
-        struct Part { int blk, u0, c; };
-        std::vector<Part> parts;
-        for (size_t b = 0; b < blocks.size(); ++b) {
-            const int n = (blocks[b].c + 63) / 64, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
-            for (int u = 0; u < blocks[b].c; u += per) parts.push_back(Part{(int)b, u, std::min(per, blocks[b].c - u)});
+    MomentSets& T = dir.ms[dual];
+    T = MomentSets{};
+    if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) return;
+    bool ok = true;
+    struct Pth { const DPath* P; int lb, group; };
+    struct Blk { int so, c, d; std::vector<Pth> paths; };
+    std::vector<Blk> blocks;
+    for (size_t gi = 0; gi < dir.groups.size(); ++gi)
+        for (int k = dir.groups[gi].path_begin; k < dir.groups[gi].path_end; ++k) {
+            const DPath& P = dir.paths[k];
+            if ((P.c_src & 7) || (P.src_off & 7)) ok = false;
+            auto it = std::find_if(blocks.begin(), blocks.end(), [&](const Blk& b) { return b.so == P.src_off; });
+            if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
+            it->paths.push_back(Pth{&P, (P.d_sh - 1) / 2, (int)gi});
         }
-        // Sets: consecutive parts whose rows of 16 edges leave room for four slots with their W (a node of 32 edges and the next
-        // one's first rows); a wider part is a set of its own with the slots it leaves, at least two.
-        int x_cap = 0;
-        for (size_t i = 0; i < parts.size() && ok;) {
-            MSet S{};
-            S.blk_begin = (int)T.blks.size(); S.grp_begin = (int)T.grps.size();
-            int slabs = 0, dmax = 0;
-            size_t j = i;
-            for (; j < parts.size(); ++j) {
-                const Blk& B = blocks[parts[j].blk];
-                if (j > i && 2 * (slabs + B.d) * MS_SLAB > kSlotBytes) break;
-                T.blks.push_back(MBlk{B.so + parts[j].u0, parts[j].c, B.c, B.d, slabs, {0, 0, 0}});
-                slabs += B.d;
-                dmax = std::max(dmax, B.d);
-            }
-            S.nblk = (int)T.blks.size() - S.blk_begin;
-            x_cap = std::max(x_cap, slabs * MS_SLAB);
-            // Rows of W: runs of nq radial indices (those of one lane half), per run the harmonics order by order, the radial
-            // index fastest, so that one read-out instruction takes nq of them.  The orders are cut into segments of whole
-            // groups of eight rows such that every block's components x a segment fit the columns of one TMEM half.
-            const int KH = (p->K + 1) / 2;
-            struct Seg { int l0, l1, row, rows; };
-            std::vector<Seg> segs;
-            int nq = KH >= 3 ? 4 : KH, rows_q = 0;
-            for (; nq >= 1; nq >>= 1) {
-                segs.clear(); rows_q = 0;
-                bool fits = true;
-                for (int l = 0; l <= p->l_max && fits;) {
-                    int e = l, rows = 0;
-                    for (; e <= p->l_max; ++e) {
-                        const int r = (((e + 1) * (e + 1) - l * l) * nq + 7) & ~7;
-                        if (dmax * r > MS_HALF) break;
-                        rows = r;
-                    }
-                    if (e == l) { fits = false; break; }
-                    segs.push_back(Seg{l, e - 1, rows_q, rows});
-                    rows_q += rows;
-                    l = e;
-                }
-                if (fits) break;
-            }
-            if (!nq) { ok = false; break; }
-            S.nq = nq;
-            const int runs = (KH + nq - 1) / nq;                                  // runs of radial indices per lane half
-            const int nqs = std::max(1, std::min(runs, kWRows / 2 / rows_q)), ngrp = (runs + nqs - 1) / nqs;
-            const int nqs_g = (runs + ngrp - 1) / ngrp, rows_h = nqs_g * rows_q;
-            S.ngrp = ngrp;
-            T.w_bytes = std::max(T.w_bytes, 2 * rows_h * 64);
-            const int row_begin = (int)T.rows.size();
-            for (int h = 0; h < 2; ++h)
-                for (int r = 0; r < nqs_g; ++r)
-                    for (const Seg& g : segs)
-                        for (int n = 0; n < g.rows; ++n) {
-                            const int nb = (g.l1 + 1) * (g.l1 + 1) - g.l0 * g.l0, m = std::min(n, nb * nq - 1);
-                            T.rows.push_back((uint16_t)((2 * (r * nq + m % nq) + h) | ((g.l0 * g.l0 + m / nq) << 8)));
-                        }
-            // units of one group; `used` tells which segments a block has paths in
-            std::vector<MUnit> us;
-            for (size_t k = i; k < j; ++k) {
-                const Blk& B = blocks[parts[k].blk];
-                const MBlk& M = T.blks[S.blk_begin + (int)(k - i)];
-                auto used = [&](size_t g) { return std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb >= segs[g].l0 && t.lb <= segs[g].l1; }); };
-                auto emit = [&](int run, int n_runs, size_t ga, size_t gb) {          // segments [ga, gb)
-                    MUnit U{};
-                    U.slab0 = M.slab0; U.d = B.d; U.c = M.c; U.blk0 = (int)(k - i); U.nblk = 1;
-                    U.row0 = run * rows_q + segs[ga].row;
-                    U.N = n_runs > 1 ? n_runs * rows_q : segs[gb - 1].row + segs[gb - 1].rows - segs[ga].row;
-                    U.nqs = n_runs; U.rows_q = rows_q; U.q0 = 2 * run * nq;
-                    U.pad[0] = (int)ga; U.pad[1] = (int)gb;
-                    if (!us.empty()) {       // together with the block before it, where the columns hold both
-                        MUnit& V = us.back();
-                        if (V.row0 == U.row0 && V.N == U.N && V.c == U.c && V.blk0 + V.nblk == U.blk0 &&
-                            V.slab0 + V.d == U.slab0 && (V.d + U.d) * U.N <= MS_HALF) {
-                            V.d += U.d; ++V.nblk;
-                            return;
-                        }
-                    }
-                    us.push_back(U);
-                };
-                const size_t ns = segs.size();
-                size_t ga = 0, gb = ns;
-                while (ga < ns && !used(ga)) ++ga;
-                while (gb > ga && !used(gb - 1)) --gb;
-                if (ga == 0 && gb == ns && B.d * nqs_g * rows_q <= MS_HALF) { emit(0, nqs_g, 0, ns); continue; }
-                for (int run = 0; run < nqs_g; ++run)
-                    for (size_t x = ga; x < gb;) {
-                        if (!used(x)) { ++x; continue; }
-                        size_t y = x + 1;
-                        while (y < gb && B.d * (segs[y].row + segs[y].rows - segs[x].row) <= MS_HALF) ++y;
-                        emit(run, 1, x, y);
-                        x = y;
-                    }
-            }
-            // read-out tables (the same for every group)
-            for (MUnit& U : us) {
-                U.out_begin = (int)T.outs.size();
-                int s0 = 0;
-                for (int k = 0; k < U.nblk; ++k) {
-                    const Part& Pt = parts[i + U.blk0 + k];
-                    const Blk& B = blocks[Pt.blk];
-                    for (int g = U.pad[0]; g < U.pad[1]; ++g)
-                        for (const Pth& t : B.paths) {
-                            if (t.lb < segs[g].l0 || t.lb > segs[g].l1) continue;
-                            for (int o = 0; o < t.P->d_dst; ++o) {
-                                const int ld = dir.nk_ld[t.group];
-                                MOut e{(int64_t)o * ld + t.P->koff + Pt.u0, dir.zb_off[t.group], t.P->d_dst * ld, B.c, (int)T.terms.size(), 0};
-                                const int col0 = segs[g].row - segs[U.pad[0]].row + (t.lb * t.lb - segs[g].l0 * segs[g].l0) * nq;
-                                for (int sc = 0; sc < B.d; ++sc)
-                                    for (int z = p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o]; z < p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o + 1]; ++z)
-                                        T.terms.push_back(MTerm{(uint32_t)((s0 + sc) * U.N + col0 + p->tab_idx[z] * nq), p->tab_coef[z]});
-                                if ((int)T.terms.size() == e.term) T.terms.push_back(MTerm{(uint32_t)col0, 0.f});
-                                if ((T.terms.size() - e.term) & 1) T.terms.push_back(MTerm{T.terms.back().col, 0.f});
-                                e.n = (int)T.terms.size() - e.term;
-                                T.outs.push_back(e);
-                            }
-                        }
-                    s0 += B.d;
-                }
-                U.n_out = (int)T.outs.size() - U.out_begin;
-            }
-            for (int g = 0; g < ngrp; ++g) {
-                MGrp G{};
-                G.q0 = 2 * g * nqs_g * nq; G.rows = rows_h; G.row_begin = row_begin; G.unit_begin = (int)T.units.size(); G.nunit = (int)us.size();
-                for (MUnit U : us) { U.q0 += G.q0; T.units.push_back(U); }
-                T.grps.push_back(G);
-            }
-            S.nunit = ngrp * (int)us.size();
-            T.sets.push_back(S);
-            i = j;
-        }
-        if (!ok) { T = MomentSets{}; continue; }
-        const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + T.sets.size() * sizeof(MSet) + T.grps.size() * sizeof(MGrp) +
-                                 T.blks.size() * sizeof(MBlk) + T.units.size() * sizeof(MUnit) + T.rows.size() * 2 + 64);
-        const int fixed = 1024 + MS_NBAR * 8 + 16 + tables;
-        T.x_cap = x_cap;
-        T.slot_bytes = 2 * x_cap + raw;
-        // as many slots as fit with an entry of W each
-        T.ns = T.nw = std::min(std::min(MS_MAXNS, MS_MAXNW), (kSmem - fixed) / (T.slot_bytes + T.w_bytes));
-        if (fixed + T.ns * (T.slot_bytes + T.w_bytes) + T.w_bytes <= kSmem && T.nw < MS_MAXNW) ++T.nw;
-        T.smem_bytes = fixed + T.ns * T.slot_bytes + T.nw * T.w_bytes;
-        T.ok = T.ns >= 2;
+    if (!ok) return;
+    std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
+    const int raw = ((dual ? 2 : 1) * (p->K + p->dim_sh) * MS_PS * 4 + 1023) & ~1023;
+    // blocks of more than 64 multiplicities are cut into equal parts
+    struct Part { int blk, u0, c; };
+    std::vector<Part> parts;
+    for (size_t b = 0; b < blocks.size(); ++b) {
+        const int n = (blocks[b].c + 63) / 64, per = ((blocks[b].c / 8 + n - 1) / n) * 8;
+        for (int u = 0; u < blocks[b].c; u += per) parts.push_back(Part{(int)b, u, std::min(per, blocks[b].c - u)});
     }
+    // Sets: consecutive parts whose rows of 16 edges leave room for four slots with their W (a node of 32 edges and the next
+    // one's first rows); a wider part is a set of its own with the slots it leaves, at least two.
+    int x_cap = 0;
+    for (size_t i = 0; i < parts.size() && ok;) {
+        MSet S{};
+        S.blk_begin = (int)T.blks.size(); S.grp_begin = (int)T.grps.size();
+        int slabs = 0, dmax = 0;
+        size_t j = i;
+        for (; j < parts.size(); ++j) {
+            const Blk& B = blocks[parts[j].blk];
+            if (j > i && 2 * (slabs + B.d) * MS_SLAB > kSlotBytes) break;
+            T.blks.push_back(MBlk{B.so + parts[j].u0, parts[j].c, B.c, B.d, slabs, {0, 0, 0}});
+            slabs += B.d;
+            dmax = std::max(dmax, B.d);
+        }
+        S.nblk = (int)T.blks.size() - S.blk_begin;
+        x_cap = std::max(x_cap, slabs * MS_SLAB);
+        // Rows of W: runs of nq radial indices (those of one lane half), per run the harmonics order by order, the radial
+        // index fastest, so that one read-out instruction takes nq of them.  The orders are cut into segments of whole
+        // groups of eight rows such that every block's components x a segment fit the columns of one TMEM half.
+        const int KH = (p->K + 1) / 2;
+        struct Seg { int l0, l1, row, rows; };
+        std::vector<Seg> segs;
+        int nq = KH >= 3 ? 4 : KH, rows_q = 0;
+        for (; nq >= 1; nq >>= 1) {
+            segs.clear(); rows_q = 0;
+            bool fits = true;
+            for (int l = 0; l <= p->l_max && fits;) {
+                int e = l, rows = 0;
+                for (; e <= p->l_max; ++e) {
+                    const int r = (((e + 1) * (e + 1) - l * l) * nq + 7) & ~7;
+                    if (dmax * r > MS_HALF) break;
+                    rows = r;
+                }
+                if (e == l) { fits = false; break; }
+                segs.push_back(Seg{l, e - 1, rows_q, rows});
+                rows_q += rows;
+                l = e;
+            }
+            if (fits) break;
+        }
+        if (!nq) { ok = false; break; }
+        S.nq = nq;
+        const int runs = (KH + nq - 1) / nq;                                  // runs of radial indices per lane half
+        const int nqs = std::max(1, std::min(runs, kWRows / 2 / rows_q)), ngrp = (runs + nqs - 1) / nqs;
+        const int nqs_g = (runs + ngrp - 1) / ngrp, rows_h = nqs_g * rows_q;
+        S.ngrp = ngrp;
+        T.w_bytes = std::max(T.w_bytes, 2 * rows_h * 64);
+        const int row_begin = (int)T.rows.size();
+        for (int h = 0; h < 2; ++h)
+            for (int r = 0; r < nqs_g; ++r)
+                for (const Seg& g : segs)
+                    for (int n = 0; n < g.rows; ++n) {
+                        const int nb = (g.l1 + 1) * (g.l1 + 1) - g.l0 * g.l0, m = std::min(n, nb * nq - 1);
+                        T.rows.push_back((uint16_t)((2 * (r * nq + m % nq) + h) | ((g.l0 * g.l0 + m / nq) << 8)));
+                    }
+        // units of one group; `used` tells which segments a block has paths in
+        std::vector<MUnit> us;
+        for (size_t k = i; k < j; ++k) {
+            const Blk& B = blocks[parts[k].blk];
+            const MBlk& M = T.blks[S.blk_begin + (int)(k - i)];
+            auto used = [&](size_t g) { return std::any_of(B.paths.begin(), B.paths.end(), [&](const Pth& t) { return t.lb >= segs[g].l0 && t.lb <= segs[g].l1; }); };
+            auto emit = [&](int run, int n_runs, size_t ga, size_t gb) {          // segments [ga, gb)
+                MUnit U{};
+                U.slab0 = M.slab0; U.d = B.d; U.c = M.c; U.blk0 = (int)(k - i); U.nblk = 1;
+                U.row0 = run * rows_q + segs[ga].row;
+                U.N = n_runs > 1 ? n_runs * rows_q : segs[gb - 1].row + segs[gb - 1].rows - segs[ga].row;
+                U.nqs = n_runs; U.rows_q = rows_q; U.q0 = 2 * run * nq;
+                U.pad[0] = (int)ga; U.pad[1] = (int)gb;
+                if (!us.empty()) {       // together with the block before it, where the columns hold both
+                    MUnit& V = us.back();
+                    if (V.row0 == U.row0 && V.N == U.N && V.c == U.c && V.blk0 + V.nblk == U.blk0 &&
+                        V.slab0 + V.d == U.slab0 && (V.d + U.d) * U.N <= MS_HALF) {
+                        V.d += U.d; ++V.nblk;
+                        return;
+                    }
+                }
+                us.push_back(U);
+            };
+            const size_t ns = segs.size();
+            size_t ga = 0, gb = ns;
+            while (ga < ns && !used(ga)) ++ga;
+            while (gb > ga && !used(gb - 1)) --gb;
+            if (ga == 0 && gb == ns && B.d * nqs_g * rows_q <= MS_HALF) { emit(0, nqs_g, 0, ns); continue; }
+            for (int run = 0; run < nqs_g; ++run)
+                for (size_t x = ga; x < gb;) {
+                    if (!used(x)) { ++x; continue; }
+                    size_t y = x + 1;
+                    while (y < gb && B.d * (segs[y].row + segs[y].rows - segs[x].row) <= MS_HALF) ++y;
+                    emit(run, 1, x, y);
+                    x = y;
+                }
+        }
+        // read-out tables (the same for every group)
+        for (MUnit& U : us) {
+            U.out_begin = (int)T.outs.size();
+            int s0 = 0;
+            for (int k = 0; k < U.nblk; ++k) {
+                const Part& Pt = parts[i + U.blk0 + k];
+                const Blk& B = blocks[Pt.blk];
+                for (int g = U.pad[0]; g < U.pad[1]; ++g)
+                    for (const Pth& t : B.paths) {
+                        if (t.lb < segs[g].l0 || t.lb > segs[g].l1) continue;
+                        for (int o = 0; o < t.P->d_dst; ++o) {
+                            const int ld = dir.nk_ld[t.group];
+                            MOut e{(int64_t)o * ld + t.P->koff + Pt.u0, dir.zb_off[t.group], t.P->d_dst * ld, B.c, (int)T.terms.size(), 0};
+                            const int col0 = segs[g].row - segs[U.pad[0]].row + (t.lb * t.lb - segs[g].l0 * segs[g].l0) * nq;
+                            for (int sc = 0; sc < B.d; ++sc)
+                                for (int z = p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o]; z < p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o + 1]; ++z)
+                                    T.terms.push_back(MTerm{(uint32_t)((s0 + sc) * U.N + col0 + p->tab_idx[z] * nq), p->tab_coef[z]});
+                            if ((int)T.terms.size() == e.term) T.terms.push_back(MTerm{(uint32_t)col0, 0.f});
+                            if ((T.terms.size() - e.term) & 1) T.terms.push_back(MTerm{T.terms.back().col, 0.f});
+                            e.n = (int)T.terms.size() - e.term;
+                            T.outs.push_back(e);
+                        }
+                    }
+                s0 += B.d;
+            }
+            U.n_out = (int)T.outs.size() - U.out_begin;
+        }
+        for (int g = 0; g < ngrp; ++g) {
+            MGrp G{};
+            G.q0 = 2 * g * nqs_g * nq; G.rows = rows_h; G.row_begin = row_begin; G.unit_begin = (int)T.units.size(); G.nunit = (int)us.size();
+            for (MUnit U : us) { U.q0 += G.q0; T.units.push_back(U); }
+            T.grps.push_back(G);
+        }
+        S.nunit = ngrp * (int)us.size();
+        T.sets.push_back(S);
+        i = j;
+    }
+    if (!ok) { T = MomentSets{}; return; }
+    const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + T.sets.size() * sizeof(MSet) + T.grps.size() * sizeof(MGrp) +
+                             T.blks.size() * sizeof(MBlk) + T.units.size() * sizeof(MUnit) + T.rows.size() * 2 + 64);
+    const int fixed = 1024 + MS_NBAR * 8 + 16 + tables;
+    T.x_cap = x_cap;
+    T.slot_bytes = 2 * x_cap + raw;
+    // as many slots as fit with an entry of W each
+    T.ns = T.nw = std::min(std::min(MS_MAXNS, MS_MAXNW), (kSmem - fixed) / (T.slot_bytes + T.w_bytes));
+    if (fixed + T.ns * (T.slot_bytes + T.w_bytes) + T.w_bytes <= kSmem && T.nw < MS_MAXNW) ++T.nw;
+    T.smem_bytes = fixed + T.ns * T.slot_bytes + T.nw * T.w_bytes;
+    T.ok = T.ns >= 2;
 }
 
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,

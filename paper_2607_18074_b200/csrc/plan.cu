@@ -460,10 +460,8 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
     build_direction(p, 1, p->tr);
     build_stream_tasks(p, p->fwd);
     build_stream_tasks(p, p->tr);
-    build_tc_sets(p, p->fwd);
-    build_tc_sets(p, p->tr);
-    build_moment_sets(p, p->fwd);
-    build_moment_sets(p, p->tr);
+    build_stream_sets(p, p->fwd);
+    build_stream_sets(p, p->tr);
     build_tc_edge_sets(p, p->fwd);
     p->uvu_state = (flags & SOBEK_FLAG_UVU_STATE) != 0;
     build_uvu_direct(p, in, n_in, out, n_out);

@@ -823,10 +823,10 @@ int smem_need(int KP, bool dual, int dsh, int ns, int b_cap, int max_ent, int n_
 
 }  // namespace
 
-// Units, passes ("sets") and entries of one direction for the plain ([0]) and the dual ([1]) stream.
-void build_tc_sets(const sobek_plan* p, Direction& dir) {
+// Units, passes ("sets") and entries of one direction, plain (0) or dual (1) stream.
+void build_tc_sets(const sobek_plan* p, Direction& dir, int only) {
     const int KP = p->K <= 8 ? 8 : 16;
-    for (int dual = 0; dual < 2; ++dual) {
+    for (int dual = only; dual <= only; ++dual) {
         TcSets& T = dir.tc[dual];
         T = TcSets{};
         if (p->K > 16) continue;

@@ -71,6 +71,25 @@ def test_double_backward(cases, name):
         assert rel_err(got, ref) <= BWD_TOL, nm
 
 
+# The moment form of the stream where its tables change shape: radial indices of one, of two and of more than one run per lane
+# half with and without padding, blocks cut into parts, orders split over units and groups, nodes whose edges fill one slot, all
+# slots and more than the ring holds.  (All sums are fp32 over split-bf16 products, 2^-17 per factor: the common tolerances.)
+MOMENT = [("8x0e+8x1o", "8x0e+8x1o", 2, 1, 40, 15), ("16x0e+8x1o", "24x0e+16x1o", 2, 2, 40, 16), ("8x0e+64x1o", "8x0e+16x1o", 2, 5, 40, 17),
+          ("72x0e+16x1o", "16x0e+136x1o", 1, 9, 30, 12), ("64x1o+64x2e", "32x0e+8x3o", 3, 8, 40, 33), ("16x3o+8x4e", "16x0e+8x1o+8x4e", 4, 7, 30, 20),
+          ("8x0e+8x1o+8x2e+8x3o", "8x0e+8x2e", 3, 16, 25, 9), ("8x0e+8x1o", "8x0e+8x1o", 1, 8, 260, 140), ("64x0e+64x2e", "64x2e", 2, 16, 160, 75)]
+
+
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg", MOMENT)
+def test_moment_stream_shapes(ir_in, ir_out, l_max, K, N, deg):
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    c = Case(synth.Workload("moment", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=17))
+    assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
+    for got, ref, nm in zip(c.bwd(), c.o_bwd(), ("gx", "gY", "gphi", "gR")):
+        assert rel_err(got, ref) <= BWD_TOL, nm
+    for got, ref, nm in zip(c.dbwd(), c.o_dbwd(), ("ggy", "hx", "hY", "hphi", "hR")):
+        assert rel_err(got, ref) <= BWD_TOL, nm
+
+
 @pytest.mark.parametrize("dirs", [(1, 0, 0, 0), (0, 1, 0, 0), (0, 0, 1, 0), (0, 0, 0, 1), (0, 0, 0, 0), (1, 0, 1, 0)])
 def test_double_backward_null_directions(cases, dirs):
     c = get(cases, "cfg1")
