@@ -31,6 +31,7 @@ struct Workspace {
     uint16_t *gbh, *gbl;      // bf16 (hi, lo) rows of the chunk's output adjoint
     // bf16 (hi, lo) copies of x, gy and vx, [N][C] each: the gathered operand of the tensor-core stream
     uint16_t *xsh, *xsl, *gsh, *gsl, *vsh, *vsl;
+    float* zf;                // fp32 adjoint state of one chunk (input of the edge pass in moment form); NULL: not used
     uint16_t *zqh, *zql;      // bf16 (hi, lo) adjoint state of one chunk (input of the tensor-core edge pass)
     int4 *oseg_r, *oseg_s;    // processing order of the nodes of every chunk, receiver / sender view (launch_chunk_order)
     // mul_ir plans: ir_mul copies of the node feature arrays of a call (inputs x, gy, vx; outputs on C_y, on C_x)
@@ -95,6 +96,8 @@ Workspace carve(const sobek_plan* p, int64_t N, int order, void* ws) {
             // weight-adjoint contractions): the two share one buffer
             w.zqh = w.zbh;
             w.zql = w.zbl;
+            // (the edge pass in moment form takes it in fp32, in the place of both halves)
+            if (p->fwd.me.ok) w.zf = (float*)w.zbh;
         } else {
             w.zbar = (float*)take((size_t)w.chunk * (size_t)p->fwd.state_floats * 4);
         }
@@ -442,7 +445,10 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
                 CK(weight_grad(p, p->fwd, n0, nn, w.zbh, w.zbl, w.gbh, w.gbl, gy, w.gRp, w.part, w.splits, w.status, s));
             }
             if (gphi || gY) {
-                if (tc_edge) {
+                if (w.zf && !geo) {
+                    CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s));
+                    CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xs, Y, nullptr, phi, nullptr, 0, w.zf, gphi, gY, gphi ? 1 : 0, gY ? 1 : 0, w.status, s));
+                } else if (tc_edge) {
                     CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, nullptr, w.status, s, w.zqh, w.zql));
                     CK(launch_edge_pass_tc(p, p->fwd, rv, n0, nn, xs, Y, nullptr, phi, nullptr, 0, w.zqh, w.zql,
                                            g_edge ? nullptr : gphi, g_edge ? nullptr : gY, gphi ? 1 : 0, gY ? 1 : 0, w.status, s));
@@ -583,7 +589,10 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                 int pm = 1, ym = 1;   // first writer overwrites, later ones accumulate
                 if (any_edge_dir) {
                     // the three direction terms that share Zbar = gy R^T, in one pass
-                    if (tc_edge_dual) {
+                    if (w.zf && !geo && (!vx || w.vsh)) {
+                        CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s));
+                        CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xs, Y, vY, phi, vphi, 1, w.zf, hphi, hY, hphi ? pm : 0, hY ? ym : 0, w.status, s));
+                    } else if (tc_edge_dual) {
                         CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, nullptr, w.status, s, w.zqh, w.zql));
                         CK(launch_edge_pass_tc(p, p->fwd, rv, n0, nn, xs, Y, vY, phi, vphi, 1, w.zqh, w.zql, hphi, hY,
                                                hphi ? pm : 0, hY ? ym : 0, w.status, s));
@@ -595,9 +604,12 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                     pm = ym = 2;
                 }
                 if (vR) {   // the term through dZbar = gy vR^T
-                    if (tc_edge_plain) {
+                    SplitSrc xp{}; xp.h = xs.h; xp.l = xs.l; xp.oseg = xs.oseg;
+                    if (w.zf && !geo) {
+                        CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.vfKNh, w.vfKNl, gy, vR, w.zf, w.status, s));
+                        CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xp, Y, nullptr, phi, nullptr, 0, w.zf, hphi, hY, hphi ? pm : 0, hY ? ym : 0, w.status, s));
+                    } else if (tc_edge_plain) {
                         CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.vfKNh, w.vfKNl, gy, vR, nullptr, w.status, s, w.zqh, w.zql));
-                        SplitSrc xp{}; xp.h = xs.h; xp.l = xs.l;
                         CK(launch_edge_pass_tc(p, p->fwd, rv, n0, nn, xp, Y, nullptr, phi, nullptr, 0, w.zqh, w.zql, hphi, hY,
                                                hphi ? pm : 0, hY ? ym : 0, w.status, s));
                     } else {

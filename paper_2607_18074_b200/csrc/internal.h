@@ -215,6 +215,28 @@ struct MomentSets {
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;
 };
 
+// --- moment-form edge pass (moment_edge.cu) ------------------------------------------------
+struct MEComp {        // a state component (path, o): where its adjoint lies in the fp32 adjoint state
+    int64_t zoff;             // floats per node of the groups before its own
+    int64_t a;                // offset of radial index 0, multiplicity 0 of the block for the group's node 0
+    int32_t b, c_row;         // floats from one node / one radial index to the next
+};
+struct MEBlk {         // (part of) a source block: at most 64 multiplicities
+    int32_t src_off, c, c_row, d;     // as MBlk
+    int32_t ksteps;                   // contraction steps of 16 multiplicities
+    int32_t comp_begin, ncomp;        // its state components
+    int32_t t_begin;                  // first entry of its term pointers: (component s, harmonic b) -> terms
+};
+struct MomentEdge {
+    bool ok = false;
+    std::vector<MEBlk> blks;
+    std::vector<MEComp> comps;
+    std::vector<int32_t> tptr;
+    std::vector<MTerm> terms;         // {offset of the component in the staged Zbar, coefficient}
+    MEBlk* d_blks = nullptr; MEComp* d_comps = nullptr; int32_t* d_tptr = nullptr; MTerm* d_terms = nullptr;
+    int32_t nq = 0, n_cols = 0, nx = 0, np = 0, nz = 0, p_bytes = 0, z_bytes = 0, smem_bytes = 0;
+};
+
 struct FStage {        // one 256-column stage of the fused kernel's contraction axis
     int32_t path;
     int32_t u0;        // first multiplicity of the block (256/KP wide)
@@ -246,6 +268,7 @@ struct Direction {
     SComp* d_scomps = nullptr;
     TcSets tc[2];                     // coupling-in-operand stream on the tensor cores: [0] plain, [1] dual
     MomentSets ms[2];                 // moment-form stream: [0] plain, [1] dual
+    MomentEdge me;                    // edge pass in moment form (receiver direction)
     TcSets etc[2];                    // tensor-core edge pass: [0] plain, [1] dual
     // receiver-owned edge pass: source-major tasks over all multiplicities
     std::vector<STask> etasks;
@@ -432,6 +455,12 @@ void build_stream_sets(const sobek_plan* p, Direction& dir);
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
                                  const SplitSrc& ss, const float* Y, const float* vY, const float* phi, const float* vphi, int dual,
                                  void* zh, void* zl, int* status, cudaStream_t s);
+
+// --- moment_edge.cu ---------------------------------------------------------------------
+void build_moment_edge(const sobek_plan* p, Direction& dir);
+cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes, const SplitSrc& ss,
+                               const float* Y, const float* vY, const float* phi, const float* vphi, int dual, const float* zbar, float* gphi,
+                               float* gY, int phi_mode, int Y_mode, int* status, cudaStream_t s);
 
 cudaError_t stream_launch_k8(const void* args, int cls, int t_begin, int t_count, cudaStream_t s);
 cudaError_t stream_launch_k16(const void* args, int cls, int t_begin, int t_count, cudaStream_t s);

@@ -1,0 +1,550 @@
+// Receiver-owned edge pass in moment form (sm_100a, tcgen05 / TMEM), warp-specialised.
+//
+// The edge outputs of the backward program (Eqs. streamed_radial_adjoints, streamed_operand_adjoints) are adjoints of the moments
+//     P_i[q,b,s,u] = sum_e phi_e[q] Y_e[b] x_{src(e)}[s,u],     Z_i[path,o,q,u] = sum_{s,b} c[s,b,o] P_i[q,b,s,u]
+// so with the moments' adjoint, made once per node from the state's adjoint Zbar = gy R^T,
+//     Pbar_i[(q,b),(s,u)] = sum_{path,o} c[s,b,o] Zbar_i[path,o,q,u]
+// they are one dense contraction per node and two short sums per edge:
+//     G_e[(q,b)] = sum_{s,u} x_{src(e)}[s,u] Pbar_i[(q,b),(s,u)]
+//     gphi_e[q] = sum_b G_e[(q,b)] Y_e[b],     gY_e[b] = sum_q G_e[(q,b)] phi_e[q]
+// G has K x (harmonics) values per edge; the contraction with the coupling left in (k_edge_tc) has K sum d_src d_dst of them, each
+// of which its epilogue reads twice: 1,840 against 144 at 64 x (0..2), K = 16.  What binds here is building Pbar (per node, not
+// per edge).  fp32 parity: coupling sums in fp32, split-bf16 product with fp32 accumulation in TMEM.
+//
+// With DUAL the pass gives the second-order terms that share Zbar (Eq. streamed_operand_second_adjoints) from G (rows of x) and Gv
+// (rows of vx):   hphi[q] = sum_b Gv Y + G vY,     hY[b] = sum_q Gv phi + G vphi.
+//
+// A CTA takes nodes round-robin.  A node's edges are taken in passes of as many tiles of 64 as the accumulators hold, the radial
+// indices in runs of NQ; for every run the blocks' slabs (64 multiplicities of one component) go by:
+//   state warps    cp.async of the Zbar rows of one (block, run), fp32, into shared memory;
+//   builder warps  Pbar of one slab: a warp takes (harmonic b) x NQ rows, a lane two multiplicities; K-major, 128-byte swizzle;
+//   row warps      cp.async of the sender rows of one (slab, tile), taking turns;
+//   MMA warp       M = 64 edges, N = NQ x harmonics; even tiles in the lower 16 lanes of each TMEM lane quarter, odd ones in the
+//                  upper 16;
+//   output warps   the two sums, one thread per edge; the two TMEM halves alternate between products and read-out.
+// Every wait is bounded.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "guard.cuh"
+#include "internal.h"
+#include "ptx.cuh"
+
+namespace sobek {
+namespace {
+
+using namespace ptx;
+
+constexpr int NOW = 4;                  // output warps (one per TMEM lane quarter)
+constexpr int NBW = 12;                 // builder warps
+constexpr int NXW = 4;                  // row warps
+constexpr int NZW = 2;                  // state warps
+constexpr int W_B = NOW, W_X = W_B + NBW, W_Z = W_X + NXW, W_M = W_Z + NZW;
+constexpr int TT = (W_M + 1) * 32;
+constexpr int TILE = 64;                // edges of a tile
+constexpr int SLAB = TILE * 128;        // bytes of one copy of a (slab, tile): 64 edges x 64 bf16
+constexpr int MAXNX = 8, MAXNP = 4, MAXNZ = 2;
+constexpr int HALF = 256;
+constexpr int NBAR = 2 * MAXNX + 2 * MAXNP + 2 * MAXNZ + 4;
+
+struct MeArgs {
+    const MEBlk* blks;
+    const MEComp* comps;
+    const int32_t* tptr;        // per (component of a block, harmonic): first term (MEBlk::t_begin)
+    const MTerm* terms;         // {component of the block, coefficient}
+    int32_t n_blks, n_comps, n_tptr, n_terms;
+    const int64_t* row_ptr;
+    const int32_t* col;
+    int64_t node0, n_nodes, N, E;
+    const int4* oseg;           // the chunk's nodes in processing order {local node, segment begin, end} or NULL
+    const __nv_bfloat16 *sh, *sl, *vsh, *vsl;
+    const float *Y, *vY, *phi, *vphi;
+    const float* zbar;
+    float *gphi, *gY;
+    int32_t phi_mode, Y_mode;   // 0 skip, 1 overwrite, 2 accumulate
+    int32_t K, dsh, C_src, nq, N_cols, nx, np, nz, p_bytes, z_bytes;
+    int* status;
+};
+
+__device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+__device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, uint32_t bytes) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const float ra = a - __uint_as_float(hi << 16);
+    const float rb = b - __uint_as_float(hi & 0xffff0000u);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(ra, rb);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+// NQ columns of this thread's TMEM lane, waited for
+template <int NQ>
+__device__ __forceinline__ void tm_read(uint32_t t, float* v) {
+    if constexpr (NQ == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\ttcgen05.wait::ld.sync.aligned;"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7]) : "r"(t) : "memory");
+    else if constexpr (NQ == 4)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];\n\ttcgen05.wait::ld.sync.aligned;"
+                     : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(t) : "memory");
+    else
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];\n\ttcgen05.wait::ld.sync.aligned;" : "=f"(v[0]), "=f"(v[1]) : "r"(t) : "memory");
+}
+
+// Nodes of a CTA; the next one's bounds are requested one node ahead.
+struct Walk {
+    const MeArgs& a;
+    int64_t v, nl, s0, s1;
+    int* st;
+    __device__ Walk(const MeArgs& a_, int* st_) : a(a_), v(blockIdx.x), nl(0), s0(0), s1(0), st(st_) { fetch(); }
+    __device__ void fetch() {
+        if (v >= a.n_nodes) return;
+        if (a.oseg) { const int4 q = __ldg(a.oseg + v); nl = q.x; s0 = q.y; s1 = q.z; return; }
+        seg_bounds(a.row_ptr, a.node0 + v, a.E, st, s0, s1);
+        nl = v;
+    }
+    __device__ bool next(int64_t& node, int64_t& seg0, int& len) {
+        while (v < a.n_nodes) {
+            node = nl; seg0 = s0; len = (int)(s1 - s0);
+            v += gridDim.x;
+            fetch();
+            if (len > 0) return true;
+        }
+        return false;
+    }
+};
+
+// The two sums of one run of radial indices for the edge of this thread.
+template <int NQ, bool DUAL>
+__device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t tv, int64_t e, bool ok, int q0, bool first_run, bool has_vx) {
+    float f[NQ], vf[NQ], gp[NQ];
+    const bool has_vY = DUAL && a.vY, has_vphi = DUAL && a.vphi;
+#pragma unroll
+    for (int r = 0; r < NQ; ++r) {
+        const bool in = ok && q0 + r < a.K;
+        f[r] = in ? __ldg(a.phi + e * a.K + q0 + r) : 0.f;
+        vf[r] = in && has_vphi ? __ldg(a.vphi + e * a.K + q0 + r) : 0.f;
+        gp[r] = 0.f;
+    }
+#pragma unroll 2
+    for (int b = 0; b < a.dsh; ++b) {
+        const float y = ok ? __ldg(a.Y + e * a.dsh + b) : 0.f, vy = ok && has_vY ? __ldg(a.vY + e * a.dsh + b) : 0.f;
+        float g[NQ], gv[NQ];
+        tm_read<NQ>(t + (uint32_t)(b * NQ), g);
+        float gy = 0.f;
+        if (DUAL) {
+            if (has_vx) {
+                tm_read<NQ>(tv + (uint32_t)(b * NQ), gv);
+            } else {
+#pragma unroll
+                for (int r = 0; r < NQ; ++r) gv[r] = 0.f;
+            }
+#pragma unroll
+            for (int r = 0; r < NQ; ++r) {
+                gp[r] = fmaf(gv[r], y, fmaf(g[r], vy, gp[r]));
+                if (q0 + r < a.K) gy = fmaf(gv[r], f[r], fmaf(g[r], vf[r], gy));       // (columns past K hold no sums)
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < NQ; ++r) {
+                gp[r] = fmaf(g[r], y, gp[r]);
+                if (q0 + r < a.K) gy = fmaf(g[r], f[r], gy);
+            }
+        }
+        if (ok && a.Y_mode) {
+            float* d = a.gY + e * a.dsh + b;
+            *d = (first_run && a.Y_mode == 1) ? gy : *d + gy;
+        }
+    }
+    if (ok && a.phi_mode) {
+#pragma unroll
+        for (int r = 0; r < NQ; ++r)
+            if (q0 + r < a.K) {
+                float* d = a.gphi + e * a.K + q0 + r;
+                *d = a.phi_mode == 1 ? gp[r] : *d + gp[r];
+            }
+    }
+}
+
+template <int NQ, bool DUAL>
+__global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
+    uint8_t* sX = smem;                                                // rows of (slab, tile): hi, lo
+    uint8_t* sP = sX + (size_t)a.nx * 2 * SLAB;                        // Pbar of a slab: hi rows, lo rows
+    uint8_t* sZ = sP + (size_t)a.np * a.p_bytes;                       // Zbar of (block, run): [component][NQ][64]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(sZ + (size_t)a.nz * a.z_bytes);
+    uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + NBAR);
+    MEComp* sComp = reinterpret_cast<MEComp*>(tmem_holder + 4);
+    MEBlk* sBlk = reinterpret_cast<MEBlk*>(sComp + a.n_comps);
+    MTerm* sTerm = reinterpret_cast<MTerm*>(sBlk + a.n_blks);
+    int32_t* sTp = reinterpret_cast<int32_t*>(sTerm + a.n_terms);
+    const uint32_t bar0 = smem_u32(bars);
+    const uint32_t bar_xfull = bar0, bar_xfree = bar0 + 8 * MAXNX, bar_pfull = bar_xfree + 8 * MAXNX, bar_pfree = bar_pfull + 8 * MAXNP,
+                   bar_zfull = bar_pfree + 8 * MAXNP, bar_zfree = bar_zfull + 8 * MAXNZ, bar_accfull = bar_zfree + 8 * MAXNZ, bar_accfree = bar_accfull + 16;
+
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool has_vx = DUAL && a.vsh != nullptr;
+    const int nop = has_vx ? 2 : 1;                                    // operands: rows of x, of vx
+    const int n_cols = a.N_cols, runs = (a.K + NQ - 1) / NQ;
+    const int pass_tiles = 2 * (HALF / (n_cols * nop));                // tiles that one accumulator holds
+    if (tid == 0) {
+        for (int s = 0; s < MAXNX; ++s) { mbar_init(bar_xfull + 8 * s, 32); mbar_init(bar_xfree + 8 * s, 1); }
+        for (int s = 0; s < MAXNP; ++s) { mbar_init(bar_pfull + 8 * s, NBW * 32); mbar_init(bar_pfree + 8 * s, 1); }
+        for (int s = 0; s < MAXNZ; ++s) { mbar_init(bar_zfull + 8 * s, NZW * 32); mbar_init(bar_zfree + 8 * s, NBW); }
+        for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, NOW); }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    auto table = [&](void* dst, const void* src, int bytes) {
+        for (int i = tid; i < bytes / 4; i += TT) reinterpret_cast<uint32_t*>(dst)[i] = reinterpret_cast<const uint32_t*>(src)[i];
+    };
+    table(sComp, a.comps, a.n_comps * (int)sizeof(MEComp)); table(sBlk, a.blks, a.n_blks * (int)sizeof(MEBlk));
+    table(sTerm, a.terms, a.n_terms * (int)sizeof(MTerm)); table(sTp, a.tptr, a.n_tptr * 4);
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_holder)), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_holder;
+    int64_t node, seg0;
+    int len;
+
+    if (warp >= W_X && warp < W_X + NXW) {
+        // =========================== row warps ===========================
+        // An entry is one (run, block, slab, tile, operand), filled by one warp; the warps that take part (no more than entries,
+        // so that a free barrier is never waited for two phases ahead) take turns.
+        const int nw = min(NXW, a.nx), me = warp - W_X;
+        Walk walk(a, a.status);
+        int xs = 0; uint32_t xr = 0;
+        int turn = 0;
+        while (me < nw && walk.next(node, seg0, len)) {
+            for (int p0 = 0; p0 < len; p0 += pass_tiles * TILE) {
+                const int plen = min(len - p0, pass_tiles * TILE), tiles = (plen + TILE - 1) / TILE;
+                int32_t id0 = 0, id1 = 0;
+                uint32_t m0 = 0, m1 = 0;
+                int have = -1;                                         // tile whose sender ids the lanes hold
+                for (int run = 0; run < runs; ++run)
+                for (int bi = 0; bi < a.n_blks; ++bi) {
+                    const MEBlk B = sBlk[bi];
+                    const int cpr = B.c >> 3, pieces = 2 * B.ksteps;   // 16-byte pieces with multiplicities / that the products read
+                    for (int s = 0; s < B.d; ++s)
+                    for (int t = 0; t < tiles; ++t)
+                    for (int op = 0; op < nop; ++op) {
+                        if (turn == me) {
+                            if (have != t) {
+                                const int64_t pos = seg0 + p0 + t * TILE + lane;
+                                const int left = plen - t * TILE;
+                                bool ok0 = lane < left, ok1 = lane + 32 < left;
+                                const int64_t v0 = ok0 ? (int64_t)a.col[pos] : 0, v1 = ok1 ? (int64_t)a.col[pos + 32] : 0;
+                                ok0 = ok0 && id_ok(v0, a.N, a.status); ok1 = ok1 && id_ok(v1, a.N, a.status);
+                                id0 = ok0 ? (int32_t)v0 : 0; id1 = ok1 ? (int32_t)v1 : 0;
+                                m0 = __ballot_sync(0xffffffffu, ok0); m1 = __ballot_sync(0xffffffffu, ok1);
+                                have = t;
+                            }
+                            if (xr > 0) mbar_spin(bar_xfree + 8 * xs, (xr & 1) ^ 1, a.status);
+                            const uint32_t dst0 = smem_u32(sX + (size_t)xs * 2 * SLAB);
+                            const __nv_bfloat16* bh = (op == 0 ? a.sh : a.vsh) + B.src_off + s * B.c_row;
+                            const __nv_bfloat16* bl = (op == 0 ? a.sl : a.vsl) + B.src_off + s * B.c_row;
+                            const int j = lane & 7, rmax = min(TILE, plen - t * TILE);
+#pragma unroll 2
+                            for (int r0 = 0; r0 < rmax; r0 += 4) {     // eight threads per row; rows past the edges are not read by anyone
+                                const int r = r0 + (lane >> 3);
+                                const int32_t ia = __shfl_sync(0xffffffffu, id0, r & 31), ib = __shfl_sync(0xffffffffu, id1, r & 31);
+                                const int64_t g = (int64_t)(r < 32 ? ia : ib) * a.C_src + 8 * j;
+                                const uint32_t ok = ((r < 32 ? m0 >> r : m1 >> (r - 32)) & 1u) && j < cpr ? 16u : 0u;
+                                const uint32_t d = dst0 + (uint32_t)(r * 128 + ((j ^ (r & 7)) << 4));
+                                if (j < pieces) {
+                                    cp_async16_zfill(d, bh + (ok ? g : 0), ok);
+                                    cp_async16_zfill(d + SLAB, bl + (ok ? g : 0), ok);
+                                }
+                            }
+                            cp_async_arrive(bar_xfull + 8 * xs);
+                        }
+                        if (++turn == nw) turn = 0;
+                        if (++xs == a.nx) { xs = 0; ++xr; }
+                    }
+                }
+            }
+        }
+    } else if (warp >= W_Z && warp < W_Z + NZW) {
+        // =========================== state warps ===========================
+        const int lt = (warp - W_Z) * 32 + lane;
+        Walk walk(a, nullptr);
+        int zs = 0; uint32_t zr = 0;
+        while (walk.next(node, seg0, len)) {
+            for (int p0 = 0; p0 < len; p0 += pass_tiles * TILE)
+            for (int run = 0; run < runs; ++run)
+            for (int bi = 0; bi < a.n_blks; ++bi) {
+                const MEBlk B = sBlk[bi];
+                if (zr > 0) mbar_spin(bar_zfree + 8 * zs, (zr & 1) ^ 1, a.status);
+                const uint32_t dst0 = smem_u32(sZ + (size_t)zs * a.z_bytes);
+                const int c4 = B.c >> 2, rows = B.ncomp * NQ, j = lt & 15, q0 = run * NQ;
+                for (int i = lt >> 4; i < rows; i += NZW * 2) {        // sixteen threads per row of 64 multiplicities
+                    const MEComp cp = sComp[B.comp_begin + i / NQ];
+                    const int q = q0 + i % NQ;
+                    const uint32_t ok = q < a.K && j < c4 ? 16u : 0u;
+                    const float* src = a.zbar + (ok ? a.n_nodes * cp.zoff + node * cp.b + cp.a + (int64_t)q * cp.c_row + 4 * j : 0);
+                    cp_async16_zfill(dst0 + (uint32_t)((i * 64 + 4 * j) * 4), src, ok);
+                }
+                cp_async_arrive(bar_zfull + 8 * zs);
+                if (++zs == a.nz) { zs = 0; ++zr; }
+            }
+        }
+    } else if (warp >= W_B && warp < W_B + NBW) {
+        // =========================== builder warps ===========================
+        const int me = warp - W_B;
+        Walk walk(a, nullptr);
+        int zs = 0, ps = 0; uint32_t zr = 0, pr = 0;
+        int turn = 0;                                                  // harmonics go round the warps
+        while (walk.next(node, seg0, len)) {
+            for (int p0 = 0; p0 < len; p0 += pass_tiles * TILE)
+            for (int run = 0; run < runs; ++run)
+            for (int bi = 0; bi < a.n_blks; ++bi) {
+                const MEBlk B = sBlk[bi];
+                mbar_spin(bar_zfull + 8 * zs, zr & 1, a.status);
+                const float* z = reinterpret_cast<const float*>(sZ + (size_t)zs * a.z_bytes) + 2 * lane;
+                const int32_t* tp = sTp + B.t_begin;
+                for (int s = 0; s < B.d; ++s, tp += a.dsh) {
+                    if (pr > 0) mbar_spin(bar_pfree + 8 * ps, (pr & 1) ^ 1, a.status);
+                    uint8_t* P = sP + (size_t)ps * a.p_bytes;
+                    int b = me - turn;
+                    if (b < 0) b += NBW;
+                    for (; b < a.dsh; b += NBW) {
+                        float v[NQ][2];
+#pragma unroll
+                        for (int r = 0; r < NQ; ++r) { v[r][0] = 0.f; v[r][1] = 0.f; }
+                        const int k1 = tp[b + 1];
+#pragma unroll 1
+                        for (int k = tp[b]; k < k1; ++k) {
+                            const MTerm m = sTerm[k];
+                            const float* zc = z + m.col;
+#pragma unroll
+                            for (int r = 0; r < NQ; ++r) {
+                                const float2 w = *reinterpret_cast<const float2*>(zc + r * 64);
+                                v[r][0] = fmaf(m.coef, w.x, v[r][0]);
+                                v[r][1] = fmaf(m.coef, w.y, v[r][1]);
+                            }
+                        }
+                        uint8_t* d = P + (size_t)(b * NQ) * 128 + (lane & 3) * 4;
+                        const int ch = lane >> 2;
+#pragma unroll
+                        for (int r = 0; r < NQ; ++r) {
+                            uint32_t hi, lo;
+                            split2(v[r][0], v[r][1], hi, lo);
+                            const uint32_t o = (uint32_t)(r * 128 + ((ch ^ ((b * NQ + r) & 7)) << 4));
+                            *reinterpret_cast<uint32_t*>(d + o) = hi;
+                            *reinterpret_cast<uint32_t*>(d + o + n_cols * 128) = lo;
+                        }
+                    }
+                    turn = (turn + a.dsh) % NBW;
+                    fence_async_smem();
+                    mbar_arrive(bar_pfull + 8 * ps);
+                    if (++ps == a.np) { ps = 0; ++pr; }
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar_zfree + 8 * zs);
+                if (++zs == a.nz) { zs = 0; ++zr; }
+            }
+        }
+    } else if (warp == W_M) {
+        // =========================== MMA warp ===========================
+        Walk walk(a, nullptr);
+        int xs = 0, ps = 0; uint32_t xr = 0, pr = 0, ai = 0;
+        // D = F32, A = B = BF16, both K-major, M = 64
+        const uint32_t uN = __shfl_sync(0xffffffffu, (uint32_t)n_cols, 0), tm_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+        const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uN >> 3) << 17) | (4u << 24);
+        const uint64_t dX0 = make_desc(smem_u32(sX), 16, 1024), dP0 = make_desc(smem_u32(sP), 16, 1024);
+        while (walk.next(node, seg0, len)) {
+            for (int p0 = 0; p0 < len; p0 += pass_tiles * TILE) {
+                const int tiles = (min(len - p0, pass_tiles * TILE) + TILE - 1) / TILE;
+                for (int run = 0; run < runs; ++run, ++ai) {
+                    const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0);
+                    if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
+                    tc_fence_after();
+                    for (int bi = 0; bi < a.n_blks; ++bi) {
+                        const int d = sBlk[bi].d;
+                        const uint32_t ks = __shfl_sync(0xffffffffu, (uint32_t)sBlk[bi].ksteps, 0);
+                        for (int s = 0; s < d; ++s) {
+                            mbar_spin(bar_pfull + 8 * ps, pr & 1, a.status);
+                            const uint64_t dP = dP0 + __shfl_sync(0xffffffffu, (uint32_t)ps * ((uint32_t)a.p_bytes >> 4), 0);
+                            const uint32_t acc = __shfl_sync(0xffffffffu, bi + s > 0 ? 1u : 0u, 0);
+                            for (int t = 0; t < tiles; ++t)
+                            for (int op = 0; op < nop; ++op) {
+                                mbar_spin(bar_xfull + 8 * xs, xr & 1, a.status);
+                                fence_async_smem();      // the gathered rows were written through the generic proxy
+                                tc_fence_after();
+                                const uint64_t dX = dX0 + __shfl_sync(0xffffffffu, (uint32_t)xs * (2u * SLAB >> 4), 0);
+                                const uint32_t dt = tm_u + buf * HALF + __shfl_sync(0xffffffffu, (uint32_t)((t >> 1) * nop + op) * uN + (uint32_t)((t & 1) * 16 << 16), 0);
+                                if (elect_one()) {
+#pragma unroll 1
+                                    for (uint32_t k = 0; k < ks; ++k)
+                                        tc_mma_bf16_x3(dt, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                    tc_commit(bar_xfree + 8 * xs);
+                                    if (t + 1 == tiles && op + 1 == nop) {
+                                        tc_commit(bar_pfree + 8 * ps);
+                                        if (bi + 1 == a.n_blks && s + 1 == d) tc_commit(bar_accfull + 8 * buf);
+                                    }
+                                }
+                                __syncwarp();
+                                if (++xs == a.nx) { xs = 0; ++xr; }
+                            }
+                            if (++ps == a.np) { ps = 0; ++pr; }
+                        }
+                    }
+                }
+            }
+        }
+    } else if (warp < NOW) {
+        // =========================== output warps ===========================
+        Walk walk(a, nullptr);
+        uint32_t ai = 0;
+        while (walk.next(node, seg0, len)) {
+            for (int p0 = 0; p0 < len; p0 += pass_tiles * TILE) {
+                const int plen = min(len - p0, pass_tiles * TILE), tiles = (plen + TILE - 1) / TILE;
+                for (int run = 0; run < runs; ++run, ++ai) {
+                    const uint32_t buf = ai & 1;
+                    if (warp == 0) mbar_spin(bar_accfull + 8 * buf, (ai >> 1) & 1, a.status);
+                    asm volatile("bar.sync 1, %0;" ::"n"(NOW * 32) : "memory");
+                    tc_fence_after();
+                    for (int t = 0; t < tiles; t += 2) {
+                        const int le = (t + (lane >> 4)) * TILE + warp * 16 + (lane & 15);
+                        const bool ok = le < plen;
+                        if (!__any_sync(0xffffffffu, ok)) continue;
+                        const uint32_t td = tmem_base + ((uint32_t)(warp * 32) << 16) + buf * HALF + (uint32_t)((t >> 1) * nop * n_cols);
+                        edge_sums<NQ, DUAL>(a, td, td + (uint32_t)n_cols, seg0 + p0 + (ok ? le : 0), ok, run * NQ, run == 0, has_vx);
+                    }
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar_accfree + 8 * buf);
+                }
+            }
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    }
+}
+
+}  // namespace
+
+// Tables of the receiver direction's edge pass in moment form.
+void build_moment_edge(const sobek_plan* p, Direction& dir) {
+    constexpr int kSmem = 227 * 1024;
+    MomentEdge& T = dir.me;
+    T = MomentEdge{};
+    if (p->K > 16 || p->K < 2 || (dir.C_src & 7) || dir.paths.empty()) return;
+    struct Blk { int so, c, d; std::vector<std::pair<const DPath*, int>> paths; };
+    std::vector<Blk> blocks;
+    for (size_t gi = 0; gi < dir.groups.size(); ++gi)
+        for (int k = dir.groups[gi].path_begin; k < dir.groups[gi].path_end; ++k) {
+            const DPath& P = dir.paths[k];
+            if ((P.c_src & 7) || (P.src_off & 7)) return;
+            auto it = std::find_if(blocks.begin(), blocks.end(), [&](const Blk& b) { return b.so == P.src_off; });
+            if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
+            it->paths.push_back({&P, (int)gi});
+        }
+    std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
+    int max_comp = 0;
+    for (const Blk& B : blocks) {
+        int n = 0;
+        for (const auto& t : B.paths) n += t.first->d_dst;
+        max_comp = std::max(max_comp, n);
+    }
+    const int dsh = p->dim_sh;
+    // the longest run of radial indices whose Pbar and Zbar leave room for four entries of gathered rows
+    for (int nq : {8, 4, 2}) {
+        if (nq > 2 && p->K <= nq / 2) continue;
+        const int n_cols = (dsh * nq + 7) & ~7;
+        if (n_cols > 128) continue;                                    // the dual pass holds two accumulators in a TMEM half
+        T = MomentEdge{};
+        T.nq = nq; T.n_cols = n_cols;
+        for (const Blk& B : blocks) {
+            const int parts = (B.c + 63) / 64, per = ((B.c / 8 + parts - 1) / parts) * 8;
+            for (int u0 = 0; u0 < B.c; u0 += per) {
+                MEBlk M{};
+                M.src_off = B.so + u0; M.c = std::min(per, B.c - u0); M.c_row = B.c; M.d = B.d; M.ksteps = (M.c + 15) / 16;
+                M.comp_begin = (int)T.comps.size();
+                std::vector<int> first;
+                for (const auto& t : B.paths) {
+                    const DGroup& G = dir.groups[t.second];
+                    first.push_back((int)T.comps.size() - M.comp_begin);
+                    for (int o = 0; o < t.first->d_dst; ++o)
+                        T.comps.push_back(MEComp{G.z_off, (int64_t)o * G.D + t.first->koff + u0, G.d_dst * G.D, B.c});
+                }
+                M.ncomp = (int)T.comps.size() - M.comp_begin;
+                M.t_begin = (int)T.tptr.size();
+                for (int s = 0; s < B.d; ++s)
+                    for (int b = 0; b < dsh; ++b) {
+                        T.tptr.push_back((int)T.terms.size());
+                        for (size_t k = 0; k < B.paths.size(); ++k) {
+                            const DPath& P = *B.paths[k].first;
+                            if (b < P.sh_off || b >= P.sh_off + P.d_sh) continue;
+                            for (int o = 0; o < P.d_dst; ++o)
+                                for (int z = p->tab_ptr[P.tabM + s * P.d_dst + o]; z < p->tab_ptr[P.tabM + s * P.d_dst + o + 1]; ++z)
+                                    if (P.sh_off + p->tab_idx[z] == b) T.terms.push_back(MTerm{(uint32_t)((first[k] + o) * nq * 64), p->tab_coef[z]});
+                        }
+                    }
+                T.tptr.push_back((int)T.terms.size());
+                T.blks.push_back(M);
+            }
+        }
+        T.p_bytes = (2 * n_cols * 128 + 1023) & ~1023;
+        T.z_bytes = (max_comp * nq * 256 + 1023) & ~1023;
+        const int fixed = 1024 + NBAR * 8 + 16 + (int)(T.comps.size() * sizeof(MEComp) + T.blks.size() * sizeof(MEBlk) + T.terms.size() * sizeof(MTerm) + T.tptr.size() * 4 + 64);
+        for (int np = 3, nz = 2;;) {
+            const int left = kSmem - fixed - np * T.p_bytes - nz * T.z_bytes;
+            if (left >= 4 * 2 * SLAB) {
+                T.np = np; T.nz = nz; T.nx = std::min(MAXNX, left / (2 * SLAB));
+                T.smem_bytes = fixed + np * T.p_bytes + nz * T.z_bytes + T.nx * 2 * SLAB;
+                T.ok = true;
+                break;
+            }
+            if (nz == 2 && T.z_bytes > T.p_bytes) nz = 1;
+            else if (np == 3) np = 2;
+            else if (nz == 2) nz = 1;
+            else break;
+        }
+        if (T.ok) return;
+    }
+    T = MomentEdge{};
+}
+
+cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes, const SplitSrc& ss,
+                               const float* Y, const float* vY, const float* phi, const float* vphi, int dual, const float* zbar, float* gphi,
+                               float* gY, int phi_mode, int Y_mode, int* status, cudaStream_t s) {
+    const MomentEdge& T = dir.me;
+    if (!T.ok || !ss.h || !ss.l || ss.rvec) return cudaErrorInvalidValue;
+    if (n_nodes <= 0) return cudaSuccess;
+    MeArgs a{};
+    a.blks = T.d_blks; a.comps = T.d_comps; a.tptr = T.d_tptr; a.terms = T.d_terms;
+    a.n_blks = (int)T.blks.size(); a.n_comps = (int)T.comps.size(); a.n_tptr = (int)T.tptr.size(); a.n_terms = (int)T.terms.size();
+    a.row_ptr = ev.ptr; a.col = ev.col; a.node0 = node0; a.n_nodes = n_nodes; a.N = ev.N; a.E = ev.E;
+    a.oseg = ss.oseg ? ss.oseg + node0 : nullptr;
+    a.sh = (const __nv_bfloat16*)ss.h; a.sl = (const __nv_bfloat16*)ss.l;
+    a.vsh = dual ? (const __nv_bfloat16*)ss.vh : nullptr; a.vsl = dual ? (const __nv_bfloat16*)ss.vl : nullptr;
+    a.Y = Y; a.vY = vY; a.phi = phi; a.vphi = vphi; a.zbar = zbar; a.gphi = gphi; a.gY = gY;
+    a.phi_mode = phi_mode; a.Y_mode = Y_mode;
+    a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src; a.nq = T.nq; a.N_cols = T.n_cols; a.nx = T.nx; a.np = T.np; a.nz = T.nz;
+    a.p_bytes = T.p_bytes; a.z_bytes = T.z_bytes; a.status = status;
+    void (*kern)(const MeArgs) = T.nq == 8 ? (dual ? k_moment_edge<8, true> : k_moment_edge<8, false>)
+                                 : T.nq == 4 ? (dual ? k_moment_edge<4, true> : k_moment_edge<4, false>)
+                                             : (dual ? k_moment_edge<2, true> : k_moment_edge<2, false>);
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem_bytes);
+    if (e != cudaSuccess) return e;
+    KernelTimer kt(K_EDGE, s);
+    kern<<<(int)std::min<int64_t>(n_nodes, 148), TT, T.smem_bytes, s>>>(a);
+    count_launch();
+    return cudaGetLastError();
+}
+
+}  // namespace sobek

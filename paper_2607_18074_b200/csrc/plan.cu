@@ -463,6 +463,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
     build_stream_sets(p, p->fwd);
     build_stream_sets(p, p->tr);
     build_tc_edge_sets(p, p->fwd);
+    build_moment_edge(p, p->fwd);
     p->uvu_state = (flags & SOBEK_FLAG_UVU_STATE) != 0;
     build_uvu_direct(p, in, n_in, out, n_out);
     build_edge_tasks(p, p->fwd);
@@ -512,6 +513,12 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
         if (e == cudaSuccess) e = upload(d->fs_begin, &d->d_fs_begin);
         if (e == cudaSuccess) e = upload(d->fs_count, &d->d_fs_count);
         if (e == cudaSuccess) e = upload(d->fk_off, &d->d_fk_off);
+        if (d->me.ok) {
+            if (e == cudaSuccess) e = upload(d->me.blks, &d->me.d_blks);
+            if (e == cudaSuccess) e = upload(d->me.comps, &d->me.d_comps);
+            if (e == cudaSuccess) e = upload(d->me.tptr, &d->me.d_tptr);
+            if (e == cudaSuccess) e = upload(d->me.terms, &d->me.d_terms);
+        }
         for (MomentSets& t : d->ms) {
             if (!t.ok) continue;
             if (e == cudaSuccess) e = upload(t.sets, &t.d_sets);
@@ -572,6 +579,7 @@ extern "C" void sobek_plan_destroy(sobek_plan* p) {
         cudaFree(d->d_kn_off); cudaFree(d->d_nk_off); cudaFree(d->d_kn_ld); cudaFree(d->d_nk_ld); cudaFree(d->d_path_group);
         cudaFree(d->d_stasks); cudaFree(d->d_scomps); cudaFree(d->d_etasks); cudaFree(d->d_ecomps); cudaFree(d->d_zb_off);
         cudaFree(d->d_fstages); cudaFree(d->d_fs_begin); cudaFree(d->d_fs_count); cudaFree(d->d_fk_off);
+        cudaFree(d->me.d_blks); cudaFree(d->me.d_comps); cudaFree(d->me.d_tptr); cudaFree(d->me.d_terms);
         for (MomentSets& t : d->ms) {
             cudaFree(t.d_sets); cudaFree(t.d_grps); cudaFree(t.d_blks); cudaFree(t.d_units); cudaFree(t.d_terms); cudaFree(t.d_outs); cudaFree(t.d_rows);
         }
