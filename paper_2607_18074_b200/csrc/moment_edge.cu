@@ -38,8 +38,8 @@ using namespace ptx;
 
 constexpr int NOW = 4;                  // output warps (one per TMEM lane quarter)
 constexpr int NBW = 12;                 // builder warps
-constexpr int NXW = 4;                  // row warps
-constexpr int NZW = 2;                  // state warps
+constexpr int NXW = 3;                  // row warps
+constexpr int NZW = 4;                  // state warps
 constexpr int W_B = NOW, W_X = W_B + NBW, W_Z = W_X + NXW, W_M = W_Z + NZW;
 constexpr int TT = (W_M + 1) * 32;
 constexpr int TILE = 64;                // edges of a tile
@@ -274,23 +274,28 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
         }
     } else if (warp >= W_Z && warp < W_Z + NZW) {
         // =========================== state warps ===========================
-        const int lt = (warp - W_Z) * 32 + lane;
+        // A component's NQ rows by one warp, sixteen threads per row of 64 multiplicities (index arithmetic once per component:
+        // with it for every copy these warps held up all others, 42 us a node at 64 x (0..2) instead of 17).
+        const int me = warp - W_Z, j = lane & 15, rr = lane >> 4;
         Walk walk(a, nullptr);
         int zs = 0; uint32_t zr = 0;
         while (walk.next(node, seg0, len)) {
             for (int p0 = 0; p0 < len; p0 += pass_tiles * TILE)
             for (int run = 0; run < runs; ++run)
             for (int bi = 0; bi < a.n_blks; ++bi) {
-                const MEBlk B = sBlk[bi];
+                const int c4 = sBlk[bi].c >> 2, ncomp = sBlk[bi].ncomp;
+                const MEComp* cps = sComp + sBlk[bi].comp_begin;
                 if (zr > 0) mbar_spin(bar_zfree + 8 * zs, (zr & 1) ^ 1, a.status);
-                const uint32_t dst0 = smem_u32(sZ + (size_t)zs * a.z_bytes);
-                const int c4 = B.c >> 2, rows = B.ncomp * NQ, j = lt & 15, q0 = run * NQ;
-                for (int i = lt >> 4; i < rows; i += NZW * 2) {        // sixteen threads per row of 64 multiplicities
-                    const MEComp cp = sComp[B.comp_begin + i / NQ];
-                    const int q = q0 + i % NQ;
-                    const uint32_t ok = q < a.K && j < c4 ? 16u : 0u;
-                    const float* src = a.zbar + (ok ? a.n_nodes * cp.zoff + node * cp.b + cp.a + (int64_t)q * cp.c_row + 4 * j : 0);
-                    cp_async16_zfill(dst0 + (uint32_t)((i * 64 + 4 * j) * 4), src, ok);
+                uint32_t dst = smem_u32(sZ + (size_t)zs * a.z_bytes) + (uint32_t)(((me * NQ + rr) * 64 + 4 * j) * 4);
+                const int q0 = run * NQ + rr;
+                for (int i = me; i < ncomp; i += NZW, dst += NZW * NQ * 256) {
+                    const MEComp cp = cps[i];
+                    const float* src = a.zbar + (a.n_nodes * cp.zoff + node * cp.b + cp.a + q0 * cp.c_row + 4 * j);
+#pragma unroll
+                    for (int r = 0; r < NQ; r += 2, src += 2 * cp.c_row) {
+                        const bool ok = j < c4 && q0 + r < a.K;
+                        cp_async16_zfill(dst + (uint32_t)(r * 256), ok ? src : a.zbar, ok ? 16u : 0u);
+                    }
                 }
                 cp_async_arrive(bar_zfull + 8 * zs);
                 if (++zs == a.nz) { zs = 0; ++zr; }
