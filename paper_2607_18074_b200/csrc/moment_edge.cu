@@ -38,8 +38,8 @@ using namespace ptx;
 
 constexpr int NOW = 4;                  // output warps (one per TMEM lane quarter)
 constexpr int NBW = 12;                 // builder warps
-constexpr int NXW = 3;                  // row warps
-constexpr int NZW = 4;                  // state warps
+constexpr int NXW = 4;                  // row warps
+constexpr int NZW = 3;                  // state warps
 constexpr int W_B = NOW, W_X = W_B + NBW, W_Z = W_X + NXW, W_M = W_Z + NZW;
 constexpr int TT = (W_M + 1) * 32;
 constexpr int TILE = 64;                // edges of a tile
@@ -252,18 +252,21 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                             const __nv_bfloat16* bh = (op == 0 ? a.sh : a.vsh) + B.src_off + s * B.c_row;
                             const __nv_bfloat16* bl = (op == 0 ? a.sl : a.vsl) + B.src_off + s * B.c_row;
                             const int j = lane & 7, rmax = min(TILE, plen - t * TILE);
-#pragma unroll 2
-                            for (int r0 = 0; r0 < rmax; r0 += 4) {     // eight threads per row; rows past the edges are not read by anyone
-                                const int r = r0 + (lane >> 3);
-                                const int32_t ia = __shfl_sync(0xffffffffu, id0, r & 31), ib = __shfl_sync(0xffffffffu, id1, r & 31);
-                                const int64_t g = (int64_t)(r < 32 ? ia : ib) * a.C_src + 8 * j;
-                                const uint32_t ok = ((r < 32 ? m0 >> r : m1 >> (r - 32)) & 1u) && j < cpr ? 16u : 0u;
-                                const uint32_t d = dst0 + (uint32_t)(r * 128 + ((j ^ (r & 7)) << 4));
-                                if (j < pieces) {
-                                    cp_async16_zfill(d, bh + (ok ? g : 0), ok);
-                                    cp_async16_zfill(d + SLAB, bl + (ok ? g : 0), ok);
+                            if (j < pieces) {      // eight threads per row, four rows at a time; nobody reads the rows past the edges
+                                const uint32_t d0 = dst0 + (uint32_t)((lane >> 3) * 128);
+                                const uint32_t live = __activemask();
+#pragma unroll 4
+                                for (int r0 = 0; r0 < rmax; r0 += 4) {
+                                    const int r = (r0 & 31) + (lane >> 3);
+                                    const int32_t id = __shfl_sync(live, r0 < 32 ? id0 : id1, r);
+                                    const bool ok = (((r0 < 32 ? m0 : m1) >> r) & 1u) && j < cpr;
+                                    const int64_t g = (int64_t)id * a.C_src + 8 * j;
+                                    const uint32_t d = d0 + (uint32_t)(r0 * 128 + ((j ^ ((r0 + (lane >> 3)) & 7)) << 4));
+                                    cp_async16_zfill(d, bh + (j < cpr ? g : 0), ok ? 16u : 0u);
+                                    cp_async16_zfill(d + SLAB, bl + (j < cpr ? g : 0), ok ? 16u : 0u);
                                 }
                             }
+                            __syncwarp();
                             cp_async_arrive(bar_xfull + 8 * xs);
                         }
                         if (++turn == nw) turn = 0;
@@ -387,9 +390,15 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                                 const uint64_t dX = dX0 + __shfl_sync(0xffffffffu, (uint32_t)xs * (2u * SLAB >> 4), 0);
                                 const uint32_t dt = tm_u + buf * HALF + __shfl_sync(0xffffffffu, (uint32_t)((t >> 1) * nop + op) * uN + (uint32_t)((t & 1) * 16 << 16), 0);
                                 if (elect_one()) {
+                                    if (ks == 4) {
+#pragma unroll
+                                        for (uint32_t k = 0; k < 4; ++k)
+                                            tc_mma_bf16_x3(dt, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                    } else {
 #pragma unroll 1
-                                    for (uint32_t k = 0; k < ks; ++k)
-                                        tc_mma_bf16_x3(dt, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                        for (uint32_t k = 0; k < ks; ++k)
+                                            tc_mma_bf16_x3(dt, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                    }
                                     tc_commit(bar_xfree + 8 * xs);
                                     if (t + 1 == tiles && op + 1 == nop) {
                                         tc_commit(bar_pfree + 8 * ps);
