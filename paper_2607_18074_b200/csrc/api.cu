@@ -91,22 +91,22 @@ Workspace carve(const sobek_plan* p, int64_t N, int order, void* ws) {
             w.gbh = (uint16_t*)take((size_t)w.chunk * (size_t)p->fwd.gb_elems * 2);
             w.gbl = (uint16_t*)take((size_t)w.chunk * (size_t)p->fwd.gb_elems * 2);
         }
+        // the edge pass in moment form takes the adjoint state in fp32, in the place of both halves
+        if (p->use_tc_edge && p->fwd.me.ok) w.zf = (float*)w.zbh;
         if (p->use_tc_edge && p->fwd.etc[0].ok) {
             // the adjoint state of a chunk is made after the chunk's state has been consumed (by the mixing and
             // weight-adjoint contractions): the two share one buffer
             w.zqh = w.zbh;
             w.zql = w.zbl;
-            // (the edge pass in moment form takes it in fp32, in the place of both halves)
-            if (p->fwd.me.ok) w.zf = (float*)w.zbh;
-        } else {
+        } else if (!w.zf) {
             w.zbar = (float*)take((size_t)w.chunk * (size_t)p->fwd.state_floats * 4);
         }
     }
-    if (p->use_tc_stream || (p->use_tc_edge && p->fwd.etc[0].ok)) {
+    if (p->use_tc_stream || w.zqh || w.zf) {
         const size_t nx = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_x * 2, ny = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_y * 2;
-        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || (order >= 1 && w.zqh)) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
+        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || w.zqh || w.zf) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
         if (order >= 1 && (tc_stream_ok(p->tr, 0) || (order >= 2 && tc_stream_ok(p->tr, 1)))) { w.gsh = (uint16_t*)take(ny); w.gsl = (uint16_t*)take(ny); }
-        if (order >= 2 && (tc_stream_ok(p->fwd, 1) || (w.zqh && p->fwd.etc[1].ok))) { w.vsh = (uint16_t*)take(nx); w.vsl = (uint16_t*)take(nx); }
+        if (order >= 2 && (tc_stream_ok(p->fwd, 1) || (w.zqh && p->fwd.etc[1].ok) || w.zf)) { w.vsh = (uint16_t*)take(nx); w.vsl = (uint16_t*)take(nx); }
         // load balance of the persistent edge kernels: only where a CTA takes several nodes of a chunk
         if (w.chunk >= kOrderMinChunk && N >= kOrderMinChunk) {
             w.oseg_r = (int4*)take((size_t)N * sizeof(int4));
@@ -171,6 +171,20 @@ EdgeView receiver_view(const sobek_graph* g) {
 }
 EdgeView sender_view(const sobek_graph* g) {
     return EdgeView{g->src_ptr, g->src_perm, g->col, g->row_ptr, g->N, g->E, 1, g->src_recv};
+}
+
+// Edge pass: the moment form costs a node the building of its Pbar and an edge little, the form with the coupling left in costs by
+// the edge.  They meet at the mean degree below (calls of the backward at 2,000 nodes, time of the other form over that of the
+// moment form at degree 12 / 30 / 64, K = 8 and 16):
+//   32 x (0..2) 0.91 / 1.04 / 1.11, 0.90 / 1.04 / 1.21     64 x (0..2) 0.87 / 0.99 / 1.12, 0.84 / 0.95 / 1.09
+//   32 x (0..4) 0.85 / 1.04 / 1.30, 0.78 / 1.02 / 1.27     64 x (0..4) 0.82 / 0.97 / 1.19, 0.77 / 0.95 / 1.16
+//   32, 64 x (0..1) 0.82 - 0.92 / 0.93 - 0.99 / 0.96 - 1.06     128 x (0..3) 0.80 - 0.84 / 0.88 - 0.93 / 0.98 - 1.11
+// and with two operands an edge (the dual pass) at three quarters of it.  128/64/64 at degree 255: 4,342 against 2,950 us.
+bool moment_edge_pays(const sobek_plan* p, const sobek_graph* g, int dual) {
+    int c = 0, d = 0;
+    for (const DPath& P : p->fwd.paths) { c = std::max(c, P.c_src); d = std::max(d, P.d_src); }
+    const double deg = c > 64 ? 60 : d <= 3 ? 48 : c > 32 ? 36 : 28;
+    return (double)g->E >= (dual ? 0.75 : 1.0) * deg * (double)g->N;
 }
 
 bool has_uncovered(const Direction& d) {
@@ -411,7 +425,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
     if (geo) { xs = *geo; gs = *geo; gs.g_rvec = nullptr; }
     const bool g_edge = geo && geo->g_rvec;       // geometry mode: the edge pass writes the adjoint of the edge vectors
     if (g_edge) { gphi = geo->g_rvec; gY = geo->g_rvec; }      // (stand-ins: "wanted"; the kernel writes g_rvec only)
-    const bool tc_edge = w.zqh != nullptr;
+    const bool tc_edge = w.zqh != nullptr, me_edge = w.zf && !geo && (!tc_edge || moment_edge_pays(p, g, 0));
     const bool gx_direct = p->uvu && p->ud.ok && !p->uvu_state && !geo && g->src_recv;      // channelwise mode: no state for gx
     const bool gR_direct = gR && p->uvu && p->ud.ok && !p->uvu_state && !geo && !z_valid;   // nor for gR
     if (gR_direct) {
@@ -427,7 +441,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
         gs.oseg = w.oseg_s;
     }
     FeatureSplits fs;
-    if (w.xsh && (gR || ((gphi || gY) && tc_edge))) { fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl; }
+    if (w.xsh && (gR || ((gphi || gY) && (tc_edge || me_edge)))) { fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl; }
     if (w.gsh && gx && !w.fused_t && !gx_direct) { fs.add(gy, g->N, p->C_y, w.gsh, w.gsl); gs.h = w.gsh; gs.l = w.gsl; }
     CK(fs.flush(s));
     PackQueue pq(p);              // every operand layout of R this call needs, one launch
@@ -445,7 +459,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
                 CK(weight_grad(p, p->fwd, n0, nn, w.zbh, w.zbl, w.gbh, w.gbl, gy, w.gRp, w.part, w.splits, w.status, s));
             }
             if (gphi || gY) {
-                if (w.zf && !geo) {
+                if (me_edge) {
                     CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s));
                     CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xs, Y, nullptr, phi, nullptr, 0, w.zf, gphi, gY, gphi ? 1 : 0, gY ? 1 : 0, w.status, s));
                 } else if (tc_edge) {
@@ -525,13 +539,15 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
     SplitSrc xs{}, gs{};
     if (geo) { xs = *geo; gs = *geo; }
     const bool tc_edge_plain = w.zqh != nullptr, tc_edge_dual = tc_edge_plain && p->fwd.etc[1].ok && (!vx || w.vsh);
+    const bool me_edge_plain = w.zf && !geo && (!tc_edge_plain || moment_edge_pays(p, g, 0)),
+               me_edge_dual = w.zf && !geo && (!tc_edge_dual || moment_edge_pays(p, g, 1));
     if (w.oseg_r && (ggy || hR || hphi || hY)) { CK(launch_chunk_order(rv, w.chunk, kOrderPeriod, w.oseg_r, w.status, s)); xs.oseg = w.oseg_r; }
     if (w.oseg_s && hx && !w.fused_t) {
         CK(launch_chunk_order(sender_view(g), w.chunk, kOrderPeriod, w.oseg_s, w.status, s));
         gs.oseg = w.oseg_s;
     }
     FeatureSplits fs;
-    if (w.xsh && (ggy || hR || ((hphi || hY) && tc_edge_plain))) {
+    if (w.xsh && (ggy || hR || ((hphi || hY) && (tc_edge_plain || w.zf)))) {
         fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl;
         if (vx && w.vsh) { fs.add(vx, g->N, p->C_x, w.vsh, w.vsl); xs.vh = w.vsh; xs.vl = w.vsl; }
     }
@@ -589,7 +605,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                 int pm = 1, ym = 1;   // first writer overwrites, later ones accumulate
                 if (any_edge_dir) {
                     // the three direction terms that share Zbar = gy R^T, in one pass
-                    if (w.zf && !geo && (!vx || w.vsh)) {
+                    if (me_edge_dual) {
                         CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s));
                         CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xs, Y, vY, phi, vphi, 1, w.zf, hphi, hY, hphi ? pm : 0, hY ? ym : 0, w.status, s));
                     } else if (tc_edge_dual) {
@@ -605,7 +621,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                 }
                 if (vR) {   // the term through dZbar = gy vR^T
                     SplitSrc xp{}; xp.h = xs.h; xp.l = xs.l; xp.oseg = xs.oseg;
-                    if (w.zf && !geo) {
+                    if (me_edge_plain) {
                         CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.vfKNh, w.vfKNl, gy, vR, w.zf, w.status, s));
                         CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xp, Y, nullptr, phi, nullptr, 0, w.zf, hphi, hY, hphi ? pm : 0, hY ? ym : 0, w.status, s));
                     } else if (tc_edge_plain) {
