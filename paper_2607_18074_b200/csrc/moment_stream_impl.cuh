@@ -72,8 +72,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// ---- read-out: n consecutive columns of this thread's TMEM lane ----------------
-// R columns from each of two places, waited for
+// R consecutive columns of this thread's TMEM lane from each of two places, waited for
 template <int R>
 __device__ __forceinline__ void tm_ld_pair(uint32_t ta, uint32_t tb, float* p, float* q) {
     if constexpr (R == 4)
@@ -92,9 +91,9 @@ __device__ __forceinline__ void st_b32_if(uint32_t ok, void* p, uint32_t v) {
 
 // Read-out of a unit by one warp: every MS_NDT-th component of the state, R radial indices (columns) at a time.  The coupling
 // terms come from a table {column, coefficient} and are summed straight out of TMEM, which serves the repeated reads at a few
-// cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients the same sums ran at
-// 8 - 10 cycles an instruction, however many warps and independent chains there were: every warp streamed kilobytes of code
-// through the instruction cache for each radial index.)
+// cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients, a function for every
+// (source order, harmonic order), the kernel took 25.4 instead of 21.2 thousand cycles a node at 64 x (0..2), K = 16, degree 32,
+// and neither more warps nor two radial indices at a time changed that.)
 // FULL: every lane and radial index of the unit is wanted.
 template <int R, bool FULL>
 __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
@@ -253,8 +252,9 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
 
     if (warp >= W_LOAD && warp < W_LOAD + NLW) {
         // =========================== loader warps ===========================
-        // A slot is filled by one warp alone, the warps take turns: a warp spends most of its time on index arithmetic, a few cycles an instruction
-        // whatever the others do, so slots side by side go faster than warps side by side on one slot (2.3 against 0.8 us).
+        // A slot is filled by one warp alone, the warps take turns: a warp spends most of its time on index arithmetic, a few cycles
+        // an instruction whatever the others do.  (All four on one slot: 32 x (0..2) forward 312 instead of 294 us, 128/64/64
+        // backward at degree 255, which gathers for every unit, 6.8 instead of 4.9 ms.)
         const int me = warp - W_LOAD;
         const int le = lane & (TB - 1);
         MsWalk walk(a, nsub, a.status);

@@ -71,16 +71,17 @@ def test_double_backward(cases, name):
         assert rel_err(got, ref) <= BWD_TOL, nm
 
 
-# The moment form of the stream where its tables change shape: radial indices of one, of two and of more than one run per lane
-# half with and without padding, blocks cut into parts, orders split over units and groups, nodes whose edges fill one slot, all
-# slots and more than the ring holds.  (All sums are fp32 over split-bf16 products, 2^-17 per factor: the common tolerances.)
+# The moment forms of the stream and of the edge pass where their tables change shape: radial indices of one, of two and of more
+# than one run with and without padding, blocks cut into parts, orders split over units and groups, nodes whose edges fill one
+# slot, all slots and more than the ring holds, one tile, two, and more than the accumulators hold.  (All sums are fp32 over split-bf16 products, 2^-17 per factor: the common tolerances.)
 MOMENT = [("8x0e+8x1o", "8x0e+8x1o", 2, 1, 40, 15), ("16x0e+8x1o", "24x0e+16x1o", 2, 2, 40, 16), ("8x0e+64x1o", "8x0e+16x1o", 2, 5, 40, 17),
           ("72x0e+16x1o", "16x0e+136x1o", 1, 9, 30, 12), ("64x1o+64x2e", "32x0e+8x3o", 3, 8, 40, 33), ("16x3o+8x4e", "16x0e+8x1o+8x4e", 4, 7, 30, 20),
-          ("8x0e+8x1o+8x2e+8x3o", "8x0e+8x2e", 3, 16, 25, 9), ("8x0e+8x1o", "8x0e+8x1o", 1, 8, 260, 140), ("64x0e+64x2e", "64x2e", 2, 16, 160, 75)]
+          ("8x0e+8x1o+8x2e+8x3o", "8x0e+8x2e", 3, 16, 25, 9), ("8x0e+8x1o", "8x0e+8x1o", 1, 8, 260, 140), ("64x0e+64x2e", "64x2e", 2, 16, 160, 75), ("8x0e+8x1o", "8x0e+8x1o", 2, 8, 430, 400),
+          ("32x0e+32x1o+32x2e", "32x0e+32x2e", 2, 8, 120, 60), ("48x1o+32x3o", "16x0e+16x2e", 4, 12, 90, 40)]
 
 
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg", MOMENT)
-def test_moment_stream_shapes(ir_in, ir_out, l_max, K, N, deg):
+def test_moment_form_shapes(ir_in, ir_out, l_max, K, N, deg):
     L = 4.0 * (N / 60.0) ** (1 / 3)
     c = Case(synth.Workload("moment", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=17))
     assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
