@@ -329,6 +329,7 @@ struct sobek_plan {
     int32_t* d_tab_ptr = nullptr;
     int32_t* d_tab_idx = nullptr;
     float* d_tab_coef = nullptr;
+    void* d_tables = nullptr;    // the allocation that holds every device table of the plan
     int device = -1;
     bool use_tc_stream = true;   // edge stream on the tensor cores where the profile allows it
     bool use_tc_edge = true;     // edge pass on the tensor cores where the profile allows it

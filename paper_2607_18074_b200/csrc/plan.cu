@@ -256,14 +256,29 @@ bool invariant_tensors(const std::vector<int>& triples /* l1,l2,l3 ... */,
     return true;
 }
 
-template <class T>
-cudaError_t upload(const std::vector<T>& h, T** d) {
-    *d = nullptr;
-    if (h.empty()) return cudaSuccess;
-    cudaError_t e = cudaMalloc((void**)d, h.size() * sizeof(T));
-    if (e != cudaSuccess) return e;
-    return cudaMemcpy(*d, h.data(), h.size() * sizeof(T), cudaMemcpyHostToDevice);
-}
+// All device tables of a plan in one allocation and one copy: some sixty of each, one by one, took most of a small plan's
+// creation.
+struct TableArena {
+    std::vector<char> bytes;
+    std::vector<std::pair<void**, size_t>> places;       // pointers to set and the offsets of their tables
+    template <class T>
+    cudaError_t add(const std::vector<T>& h, T** d) {
+        *d = nullptr;
+        if (h.empty()) return cudaSuccess;
+        const size_t off = (bytes.size() + 255) & ~size_t(255);
+        bytes.resize(off + h.size() * sizeof(T));
+        memcpy(bytes.data() + off, h.data(), h.size() * sizeof(T));
+        places.push_back({reinterpret_cast<void**>(d), off});
+        return cudaSuccess;
+    }
+    cudaError_t place(void** base) {
+        if (bytes.empty()) return cudaSuccess;
+        cudaError_t e = cudaMalloc(base, bytes.size());
+        if (e == cudaSuccess) e = cudaMemcpy(*base, bytes.data(), bytes.size(), cudaMemcpyHostToDevice);
+        for (const auto& q : places) *q.first = e == cudaSuccess ? static_cast<char*>(*base) + q.second : nullptr;
+        return e;
+    }
+};
 
 // Build one traversal direction.  transposed = 0: groups are output irreps; 1: input irreps.
 void build_direction(sobek_plan* p, int transposed, Direction& dir) {
@@ -479,6 +494,8 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
         *plan = p;
         return SOBEK_OK;
     }
+    TableArena arena;
+    auto upload = [&](const auto& h, auto** d) { return arena.add(h, d); };
     if (e == cudaSuccess) e = upload(p->tab_ptr, &p->d_tab_ptr);
     if (e == cudaSuccess) e = upload(p->tab_idx, &p->d_tab_idx);
     if (e == cudaSuccess) e = upload(p->tab_coef, &p->d_tab_coef);
@@ -546,6 +563,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
             if (e == cudaSuccess) e = upload(t.comps, &t.d_comps);
         }
     }
+    if (e == cudaSuccess) e = arena.place(&p->d_tables);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();
         sobek_plan_destroy(p);
@@ -572,25 +590,7 @@ extern "C" void sobek_plan_destroy(sobek_plan* p) {
         if (p->ev_join[i]) cudaEventDestroy(p->ev_join[i]);
     }
     if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-    cudaFree(p->d_tab_ptr); cudaFree(p->d_tab_idx); cudaFree(p->d_tab_coef);
-    for (UvuDirectTables& T : p->ud.dir) { cudaFree(T.d_woff); cudaFree(T.d_ent); cudaFree(T.d_nz); }
-    cudaFree(p->d_in_blocks); cudaFree(p->d_out_blocks);
-    for (Direction* d : {&p->fwd, &p->tr}) {
-        cudaFree(d->d_paths); cudaFree(d->d_groups); cudaFree(d->d_wtasks);
-        cudaFree(d->d_kn_off); cudaFree(d->d_nk_off); cudaFree(d->d_kn_ld); cudaFree(d->d_nk_ld); cudaFree(d->d_path_group);
-        cudaFree(d->d_stasks); cudaFree(d->d_scomps); cudaFree(d->d_etasks); cudaFree(d->d_ecomps); cudaFree(d->d_zb_off);
-        cudaFree(d->d_fstages); cudaFree(d->d_fs_begin); cudaFree(d->d_fs_count); cudaFree(d->d_fk_off);
-        cudaFree(d->me.d_blks); cudaFree(d->me.d_comps); cudaFree(d->me.d_tptr); cudaFree(d->me.d_terms);
-        for (MomentSets& t : d->ms) {
-            cudaFree(t.d_sets); cudaFree(t.d_grps); cudaFree(t.d_blks); cudaFree(t.d_units); cudaFree(t.d_terms); cudaFree(t.d_outs); cudaFree(t.d_rows);
-        }
-        for (TcSets* tp : {&d->tc[0], &d->tc[1], &d->etc[0], &d->etc[1]}) {
-            TcSets& t = *tp;
-            cudaFree(t.d_inv_ptr); cudaFree(t.d_inv);
-            cudaFree(t.d_ents_s); cudaFree(t.d_nz); cudaFree(t.d_comps_s); cudaFree(t.d_slabs);
-            cudaFree(t.d_sets); cudaFree(t.d_units); cudaFree(t.d_blks); cudaFree(t.d_ents); cudaFree(t.d_comps);
-        }
-    }
+    cudaFree(p->d_tables);
     (void)cudaGetLastError();
     delete p;
 }
