@@ -252,21 +252,20 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                             const __nv_bfloat16* bh = (op == 0 ? a.sh : a.vsh) + B.src_off + s * B.c_row;
                             const __nv_bfloat16* bl = (op == 0 ? a.sl : a.vsl) + B.src_off + s * B.c_row;
                             const int j = lane & 7, rmax = min(TILE, plen - t * TILE);
-                            if (j < pieces) {      // eight threads per row, four rows at a time; nobody reads the rows past the edges
-                                const uint32_t d0 = dst0 + (uint32_t)((lane >> 3) * 128);
-                                const uint32_t live = __activemask();
+                            const uint32_t d0 = dst0 + (uint32_t)((lane >> 3) * 128);
+                            // eight threads per row, four rows at a time; nobody reads the rows past the edges
 #pragma unroll 4
-                                for (int r0 = 0; r0 < rmax; r0 += 4) {
-                                    const int r = (r0 & 31) + (lane >> 3);
-                                    const int32_t id = __shfl_sync(live, r0 < 32 ? id0 : id1, r);
-                                    const bool ok = (((r0 < 32 ? m0 : m1) >> r) & 1u) && j < cpr;
-                                    const int64_t g = (int64_t)id * a.C_src + 8 * j;
-                                    const uint32_t d = d0 + (uint32_t)(r0 * 128 + ((j ^ ((r0 + (lane >> 3)) & 7)) << 4));
+                            for (int r0 = 0; r0 < rmax; r0 += 4) {
+                                const int r = (r0 & 31) + (lane >> 3);
+                                const int32_t id = __shfl_sync(0xffffffffu, r0 < 32 ? id0 : id1, r);
+                                const bool ok = (((r0 < 32 ? m0 : m1) >> r) & 1u) && j < cpr;
+                                const int64_t g = (int64_t)id * a.C_src + 8 * j;
+                                const uint32_t d = d0 + (uint32_t)(r0 * 128 + ((j ^ ((r0 + (lane >> 3)) & 7)) << 4));
+                                if (j < pieces) {
                                     cp_async16_zfill(d, bh + (j < cpr ? g : 0), ok ? 16u : 0u);
                                     cp_async16_zfill(d + SLAB, bl + (j < cpr ? g : 0), ok ? 16u : 0u);
                                 }
                             }
-                            __syncwarp();
                             cp_async_arrive(bar_xfull + 8 * xs);
                         }
                         if (++turn == nw) turn = 0;
