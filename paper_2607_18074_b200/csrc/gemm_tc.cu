@@ -236,6 +236,30 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
                 *reinterpret_cast<float4*>(park + lane * P4 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
         }
         __syncwarp();
+        // fp32 output whose rows start on 16 bytes: 16 bytes per lane, 8, 16 or 32 lanes a row, the row offsets worked out by
+        // one lane each.  Bound by instructions per stored byte (a tile of one or two k-blocks is all epilogue): with 4 bytes a
+        // lane and the divisions in every row the fp32 adjoint state took longer to write than its bf16 halves do.  All node
+        // products of a call, before / after, us: 64 x (0..4), 5,000 nodes, all three orders 19,323 / 11,559; 128 x (0..3)
+        // second order 7,283 / 5,676; 128/64/64 backward 570 / 332; 32 x (0..2) forward 61.9 / 45.4.
+        const bool wide = !g.Ch && !(((uintptr_t)g.C & 15) | ((g.c_outer | g.c_inner | g.split_stride | g.N) & 3));
+        if (wide) {
+            const int64_t ml = (int64_t)m0 + q * 32 + lane;
+            const int64_t rb = (int64_t)bz * g.split_stride + (int64_t)((uint32_t)ml / (uint32_t)g.c_d) * g.c_outer + (int64_t)((uint32_t)ml % (uint32_t)g.c_d) * g.c_inner + n0;
+            const int sh = g.BN <= 32 ? 3 : g.BN <= 64 ? 4 : 5, cl = 4 * (lane & ((1 << sh) - 1));
+            const int left = (int)min((int64_t)32, g.M - m0 - q * 32), ncol = (int)min((int64_t)g.BN, g.N - n0);
+#pragma unroll 4
+            for (int i = 0; i < (1 << sh); ++i) {
+                const int r = (i << (5 - sh)) + (lane >> sh);
+                float* crow = g.C + __shfl_sync(0xffffffffu, rb, r);
+                if (r >= left) continue;
+                for (int c = cl; c < ncol; c += 128) {
+                    float4 v = num_kb > 0 ? *reinterpret_cast<const float4*>(park + r * P4 + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    float4* out = reinterpret_cast<float4*>(crow + c);
+                    if (g.accumulate) { const float4 o = *out; v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w; }
+                    *out = v;
+                }
+            }
+        } else
         for (int r = 0; r < 32; ++r) {
             const int64_t m = (int64_t)m0 + q * 32 + r;
             if (m >= g.M) break;
