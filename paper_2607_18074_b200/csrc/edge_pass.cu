@@ -329,7 +329,7 @@ cudaError_t launch_one(EdgeArgs a, int t_begin, int t_count, cudaStream_t s) {
     const size_t sh = (size_t)a.warp_floats * nw * sizeof(float);
     auto kern = k_edge_pass<CAP, KC, DS, DUAL>;
     if (sh > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+        cudaError_t e = allow_dynamic_smem(kern);
         if (e != cudaSuccess) return e;
     }
     const int grid = (int)std::min<int64_t>(a.n_nodes, 148 * 32);

@@ -873,10 +873,8 @@ cudaError_t launch_edge_pass_tc(const sobek_plan* p, const Direction& dir, const
         kern2 = k8 ? k_edge_tc<8, false, 8, 3, true, 2> : k_edge_tc<16, false, 8, 3, true, 2>;
         kern1 = k8 ? k_edge_tc<8, false, 8, 3, true, 1> : k_edge_tc<16, false, 8, 3, true, 1>;
     }
-    int max_smem = 0;
-    for (const auto& ep : T.epar) max_smem = std::max(max_smem, ep.smem);
-    cudaError_t e = cudaFuncSetAttribute(kern2, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern1, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+    cudaError_t e = allow_dynamic_smem(kern2);
+    if (e == cudaSuccess) e = allow_dynamic_smem(kern1);
     if (e != cudaSuccess) return e;
     // one launch per set of accumulator tiles: the first writes in the caller's mode, the others accumulate
     for (size_t si = 0; si < T.sets.size(); ++si) {

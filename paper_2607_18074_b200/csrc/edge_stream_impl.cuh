@@ -242,7 +242,7 @@ cudaError_t launch_one(StreamArgs a, int t_begin, int t_count, cudaStream_t s) {
     const size_t sh = (size_t)wf * SW * sizeof(float);
     auto kern = k_stream<CAP, KC, DS, DUAL>;
     if (sh > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+        cudaError_t e = allow_dynamic_smem(kern);
         if (e != cudaSuccess) return e;
     }
     const int64_t total = a.n_nodes * t_count;

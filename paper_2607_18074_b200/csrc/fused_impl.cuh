@@ -371,7 +371,7 @@ cudaError_t launch_fused_d(int D, const CUtensorMap& th, const CUtensorMap& tl, 
 #define SOBEK_FUSED_CASE(DD)                                                                                  \
     case DD: {                                                                                                \
         auto kern = k_fused<DD, KP, DUAL>;                                                                    \
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);     \
+        cudaError_t e = allow_dynamic_smem(kern);                                                             \
         if (e != cudaSuccess) return e;                                                                       \
         kern<<<grid, F_THREADS, sh, s>>>(th, tl, a);                                                          \
         return cudaGetLastError();                                                                            \

@@ -401,6 +401,15 @@ struct EdgeView {          // how a traversal walks the graph
     const int32_t* recv;   // transposed only, optional: receiver of the edge at each position (else searched)
 };
 
+// Lets a kernel be launched with any dynamic shared memory that the device has.  The limit belongs to the function, not to the
+// launch: set to one launch's size, it is too small for a larger launch that another host thread (with a plan of its own) is about
+// to make, and that launch is refused.  So it is always the same value.  (No kernel that uses it has static shared memory.)
+constexpr int kMaxDynSmem = 227 * 1024;
+template <class K>
+cudaError_t allow_dynamic_smem(K kern) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
+}
+
 cudaError_t launch_unpack_R(const sobek_plan* p, const Direction& dir, const float* Rp, float* R,
                             cudaStream_t s);
 void build_edge_tasks(const sobek_plan* p, Direction& dir);

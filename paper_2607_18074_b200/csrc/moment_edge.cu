@@ -552,7 +552,7 @@ cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const 
     void (*kern)(const MeArgs) = T.nq == 8 ? (dual ? k_moment_edge<8, true> : k_moment_edge<8, false>)
                                  : T.nq == 4 ? (dual ? k_moment_edge<4, true> : k_moment_edge<4, false>)
                                              : (dual ? k_moment_edge<2, true> : k_moment_edge<2, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem_bytes);
+    cudaError_t e = allow_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
     KernelTimer kt(K_EDGE, s);
     kern<<<(int)std::min<int64_t>(n_nodes, 148), TT, T.smem_bytes, s>>>(a);

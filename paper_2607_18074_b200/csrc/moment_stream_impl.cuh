@@ -604,7 +604,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
 
 template <bool DUAL>
 cudaError_t moment_stream_launch(const MsArgs& a, int grid, int smem, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_moment_stream<DUAL>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = allow_dynamic_smem(k_moment_stream<DUAL>);
     if (e != cudaSuccess) return e;
     k_moment_stream<DUAL><<<grid, MS_TT, smem, s>>>(a);
     return cudaGetLastError();

@@ -1026,7 +1026,7 @@ cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const Ed
     const bool k8 = p->K <= 8;
     void (*kern)(const TcArgs) = k8 ? (dual ? k_stream_tc<8, true> : k_stream_tc<8, false>)
                                     : (dual ? k_stream_tc<16, true> : k_stream_tc<16, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T.smem_bytes);
+    cudaError_t e = allow_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
     const int64_t total = n_nodes * a.nsets;
     const int grid = (int)std::min<int64_t>(total, (int64_t)148);

@@ -672,7 +672,7 @@ cudaError_t launch_ud(const UdArgs& a, size_t tables, int max_grid, int* grid_ou
     const size_t sh = ud_smem_bytes<L, KP>(a.C, tables);
     auto kern = a.part ? (a.H > 1 ? k_uvu_direct_wgrad<L, KP, true> : k_uvu_direct_wgrad<L, KP, false>)
                        : (a.H > 1 ? k_uvu_direct_fwd<L, KP, true> : k_uvu_direct_fwd<L, KP, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh);
+    cudaError_t e = allow_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, sh);

@@ -715,6 +715,41 @@ def test_bounded_wait_gives_up_and_reports():
     assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
 
 
+def test_two_host_threads_with_plans_of_their_own():
+    """The limit on a kernel's dynamic shared memory belongs to the kernel, not to a launch: two threads whose plans need
+    different amounts of it must not take it away from each other between setting it and launching."""
+    import threading
+    import torch
+    names = [("8x0e+8x1o", 8), ("64x0e+64x1o+64x2e", 16)]
+    cs = [Case(synth.Workload("threads", P(ir), P(ir), 2, K, 24, 4.0, 2.0, "bessel", seed=21)) for ir, K in names]
+    ref = [c.bwd() for c in cs]
+    errors, results = [], [None, None]
+
+    def work(k):
+        try:
+            c = cs[k]
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for n in range(1500):
+                    i = c.plan.info
+                    if n % 50 == 0:
+                        outs = [c._new(c.N, i.C_x), c._new(c.E, i.dim_sh), c._new(c.E, i.K), c._new(i.K, i.N_w)]
+                    c.sb.conv_bwd(c.plan, c.graph, c.x, c.Y, c.phi, c.R, c.gy, *outs, c.ws(1))
+                torch.cuda.current_stream().synchronize()
+                results[k] = [t.cpu().numpy() for t in outs]
+        except Exception as e:      # noqa: BLE001  (reported by the main thread)
+            errors.append((k, e))
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
+    for got, want in zip(results, ref):
+        for a, b in zip(got, want):
+            assert np.array_equal(a, b)
+
+
 # ---------------------------------------------------------------------------------------
 # randomised profiles: multiplicities, orders, parities, K, mode and graph drawn from a seed
 # ---------------------------------------------------------------------------------------
