@@ -583,7 +583,7 @@ __global__ void __launch_bounds__(256) k_uvu_direct_wgrad(const UdArgs a) {
 }  // namespace
 
 // Whether the plan's profile is  C x 0e + C x 1o + ... + C x L  on both sides with l_max = L <= 3, C a multiple of 16
-// that splits into slices of at most 256 / (thread shares) channels; fills the per-path and per-entry tables in the kernel's static path order and
+// that splits into slices of at most 256 / (thread shares) channels (whole warps where there are several shares); fills the per-path and per-entry tables in the kernel's static path order and
 // padded M_e layout.
 void build_uvu_direct(sobek_plan* p, const sobek_irrep* in, int n_in, const sobek_irrep* out, int n_out) {
     UvuDirect& D = p->ud;
@@ -594,6 +594,9 @@ void build_uvu_direct(sobek_plan* p, const sobek_irrep* in, int n_in, const sobe
     // a CTA takes C / H channels (a multiple of 16) so that its (channel, share) threads number at most 256
     const int H = (C * NG + 255) / 256;
     if (C < 16 || (C & 15) || NG > 4 || C % H != 0 || ((C / H) & 15)) return;
+    // The shares meet at CTA barriers from code of their own, so no warp may hold threads of two of them: a warp whose lanes
+    // reach different barrier instructions waits for ever.  (Multiplicities that are odd multiples of 16 take the state.)
+    if (NG > 1 && ((C / H) & 31)) return;
     for (int i = 0; i < n_in; ++i) {
         const int par = (i & 1) ? -1 : 1;
         if (in[i].l != i || out[i].l != i || in[i].mul != C || out[i].mul != C || in[i].parity != par || out[i].parity != par) return;

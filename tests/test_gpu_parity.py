@@ -628,6 +628,19 @@ def test_uvu_direct_and_state_route_agree(name):
         assert np.array_equal(b_direct[k], b_state[k])
 
 
+@pytest.mark.parametrize("C,K", [(16, 8), (16, 16), (48, 8), (48, 16), (80, 16), (96, 8), (96, 16)])
+def test_uvu_multiplicities_that_are_odd_multiples_of_16(C, K):
+    """Orders up to 3 need several thread shares per channel in the direct kernels; where a share (or a channel slice of it) is
+    no whole number of warps the state route must be taken."""
+    ir = P("+".join(f"{C}x{l}{'eo'[l % 2]}" for l in range(4)))
+    c = Case(synth.Workload("uvu_share", ir, ir, 3, K, 40, 4.0, 1.7, "bessel", seed=12, mode="uvu"))
+    assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
+    for got, ref in zip(c.bwd(), c.o_bwd()):
+        assert rel_err(got, ref) <= BWD_TOL
+    for got, ref in zip(c.dbwd(), c.o_dbwd()):
+        assert rel_err(got, ref) <= BWD_TOL
+
+
 def test_uvu_full_size_sampled():
     """The paper's 128/128/128 channelwise profile (K = 16) on 31 copies of its 128-node graph."""
     FULL["uvu_128x3_31"] = (synth.config("uvu_128x3_31"), 6, (0, 1, 2))
