@@ -98,7 +98,8 @@ Workspace carve(const sobek_plan* p, int64_t N, int order, void* ws) {
             // weight-adjoint contractions): the two share one buffer
             w.zqh = w.zbh;
             w.zql = w.zbl;
-        } else if (!w.zf) {
+        }
+        if (needs_zbar(p, order)) {
             w.zbar = (float*)take((size_t)w.chunk * (size_t)p->fwd.state_floats * 4);
         }
     }

@@ -359,6 +359,8 @@ constexpr size_t kHeaderBytes = 256;
 constexpr int64_t kMinChunkNodes = 512;
 
 int64_t chunk_nodes(const sobek_plan* p, int64_t N, int order);
+// a call of this order runs the FP32-pipe edge pass somewhere, which reads an fp32 adjoint state of its own
+bool needs_zbar(const sobek_plan* p, int order);
 
 void count_launch(int n = 1);
 

@@ -91,6 +91,17 @@ def test_moment_form_shapes(ir_in, ir_out, l_max, K, N, deg):
         assert rel_err(got, ref) <= BWD_TOL, nm
 
 
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K", [("96x2e+96x4e", "128x1o+24x2e+32x4e", 2, 1), ("112x2e+112x3o+112x4e", "16x0e+16x1o+16x2e+16x3o", 2, 10)])
+def test_double_backward_where_only_the_plain_edge_pass_fits(ir_in, ir_out, l_max, K):
+    """Wide blocks of high order: the tensor-core edge pass fits shared memory in its plain form and not in its dual one."""
+    c = Case(synth.Workload("no_dual", P(ir_in), P(ir_out), l_max, K, 24, 4.0, 2.0, "gaussian", seed=23))
+    for got, ref, nm in zip(c.bwd(), c.o_bwd(), ("gx", "gY", "gphi", "gR")):
+        assert rel_err(got, ref) <= BWD_TOL, nm
+    for dirs in ((True, True, True, True), (True, False, False, False), (False, False, False, True)):
+        for got, ref, nm in zip(c.dbwd(dirs=dirs), c.o_dbwd(dirs=dirs), ("ggy", "hx", "hY", "hphi", "hR")):
+            assert rel_err(got, ref) <= BWD_TOL if np.abs(ref).max() > 0 else np.all(got == 0), (dirs, nm)
+
+
 @pytest.mark.parametrize("dirs", [(1, 0, 0, 0), (0, 1, 0, 0), (0, 0, 1, 0), (0, 0, 0, 1), (0, 0, 0, 0), (1, 0, 1, 0)])
 def test_double_backward_null_directions(cases, dirs):
     c = get(cases, "cfg1")
