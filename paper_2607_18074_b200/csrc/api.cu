@@ -103,9 +103,9 @@ Workspace carve(const sobek_plan* p, int64_t N, int order, void* ws) {
             w.zbar = (float*)take((size_t)w.chunk * (size_t)p->fwd.state_floats * 4);
         }
     }
-    if (p->use_tc_stream || w.zqh || w.zf) {
+    if (p->use_tc_stream || w.zqh) {
         const size_t nx = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_x * 2, ny = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_y * 2;
-        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || w.zqh || w.zf) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
+        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || w.zqh) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
         if (order >= 1 && (tc_stream_ok(p->tr, 0) || (order >= 2 && tc_stream_ok(p->tr, 1)))) { w.gsh = (uint16_t*)take(ny); w.gsl = (uint16_t*)take(ny); }
         if (order >= 2 && (tc_stream_ok(p->fwd, 1) || (w.zqh && p->fwd.etc[1].ok) || w.zf)) { w.vsh = (uint16_t*)take(nx); w.vsl = (uint16_t*)take(nx); }
         // load balance of the persistent edge kernels: only where a CTA takes several nodes of a chunk
@@ -426,7 +426,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
     if (geo) { xs = *geo; gs = *geo; gs.g_rvec = nullptr; }
     const bool g_edge = geo && geo->g_rvec;       // geometry mode: the edge pass writes the adjoint of the edge vectors
     if (g_edge) { gphi = geo->g_rvec; gY = geo->g_rvec; }      // (stand-ins: "wanted"; the kernel writes g_rvec only)
-    const bool tc_edge = w.zqh != nullptr, me_edge = w.zf && !geo && (!tc_edge || moment_edge_pays(p, g, 0));
+    const bool tc_edge = w.zqh != nullptr, me_edge = w.zf && !geo && moment_edge_pays(p, g, 0);
     const bool gx_direct = p->uvu && p->ud.ok && !p->uvu_state && !geo && g->src_recv;      // channelwise mode: no state for gx
     const bool gR_direct = gR && p->uvu && p->ud.ok && !p->uvu_state && !geo && !z_valid;   // nor for gR
     if (gR_direct) {
@@ -442,7 +442,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
         gs.oseg = w.oseg_s;
     }
     FeatureSplits fs;
-    if (w.xsh && (gR || ((gphi || gY) && (tc_edge || me_edge)))) { fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl; }
+    if (w.xsh && (gR || ((gphi || gY) && tc_edge))) { fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl; }
     if (w.gsh && gx && !w.fused_t && !gx_direct) { fs.add(gy, g->N, p->C_y, w.gsh, w.gsl); gs.h = w.gsh; gs.l = w.gsl; }
     CK(fs.flush(s));
     PackQueue pq(p);              // every operand layout of R this call needs, one launch
@@ -540,7 +540,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
     SplitSrc xs{}, gs{};
     if (geo) { xs = *geo; gs = *geo; }
     const bool tc_edge_plain = w.zqh != nullptr, tc_edge_dual = tc_edge_plain && p->fwd.etc[1].ok && (!vx || w.vsh);
-    const bool me_edge_plain = w.zf && !geo && (!tc_edge_plain || moment_edge_pays(p, g, 0)),
+    const bool me_edge_plain = w.zf && !geo && moment_edge_pays(p, g, 0),
                me_edge_dual = w.zf && !geo && (!tc_edge_dual || moment_edge_pays(p, g, 1));
     if (w.oseg_r && (ggy || hR || hphi || hY)) { CK(launch_chunk_order(rv, w.chunk, kOrderPeriod, w.oseg_r, w.status, s)); xs.oseg = w.oseg_r; }
     if (w.oseg_s && hx && !w.fused_t) {
@@ -548,7 +548,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
         gs.oseg = w.oseg_s;
     }
     FeatureSplits fs;
-    if (w.xsh && (ggy || hR || ((hphi || hY) && (tc_edge_plain || w.zf)))) {
+    if (w.xsh && (ggy || hR || ((hphi || hY) && tc_edge_plain))) {
         fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl;
         if (vx && w.vsh) { fs.add(vx, g->N, p->C_x, w.vsh, w.vsl); xs.vh = w.vsh; xs.vl = w.vsl; }
     }

@@ -455,6 +455,10 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
     constexpr int kSmem = 227 * 1024;
     MomentEdge& T = dir.me;
     T = MomentEdge{};
+    // Only in the place of k_edge_tc: the FP32-pipe pass holds rows and adjoint state in 32 bits, this one as bf16 hi + lo, and a
+    // profile that runs that pass keeps its precision (error of gY, 2-norm against fp64: 1e-7 there, 5e-6 here in the channelwise
+    // mode; 4.5e-6 and 8e-6 behind the node products of the other mode).
+    if (!dir.etc[0].ok) return;
     if (p->K > 16 || p->K < 2 || (dir.C_src & 7) || dir.paths.empty()) return;
     struct Blk { int so, c, d; std::vector<std::pair<const DPath*, int>> paths; };
     std::vector<Blk> blocks;

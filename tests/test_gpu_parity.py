@@ -102,6 +102,22 @@ def test_double_backward_where_only_the_plain_edge_pass_fits(ir_in, ir_out, l_ma
             assert rel_err(got, ref) <= BWD_TOL if np.abs(ref).max() > 0 else np.all(got == 0), (dirs, nm)
 
 
+@pytest.mark.parametrize("mode,irreps", [("uvu", "24x0e+24x1o+24x2e"), ("uvw", "8x0e+24x1o"), ("uvw", "144x0e+16x1o")])
+def test_edge_outputs_keep_32_bits_off_the_16s(mode, irreps):
+    """Multiplicities that are no multiples of 16, or above 128: the edge pass runs on the FP32 pipes by default, and its outputs are
+    those of a plan that asks for it.  In the channelwise mode, whose adjoint state is plain fp32 products, their error is that of
+    32-bit sums: some hundred terms of both signs, 2^-24 each, bounded by 1e-6 of the largest output."""
+    ir = P(irreps)
+    w = synth.Workload("keep32", ir, ir, 2, 8, 60, 4.0, 2.8, "bessel", seed=25, mode=mode)
+    c = Case(w)
+    f = Case(w, inputs=c.d, tc_edge=False)
+    for a, b in zip(c.bwd()[1:3] + c.dbwd()[2:4], f.bwd()[1:3] + f.dbwd()[2:4]):
+        assert np.array_equal(a, b)
+    if mode == "uvu":
+        for got, ref in zip(c.bwd()[1:3] + c.dbwd()[2:4], c.o_bwd()[1:3] + c.o_dbwd()[2:4]):
+            assert rel_err(got, ref) <= 1e-6
+
+
 @pytest.mark.parametrize("dirs", [(1, 0, 0, 0), (0, 1, 0, 0), (0, 0, 1, 0), (0, 0, 0, 1), (0, 0, 0, 0), (1, 0, 1, 0)])
 def test_double_backward_null_directions(cases, dirs):
     c = get(cases, "cfg1")
