@@ -12,7 +12,7 @@ namespace {
 inline size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // the stream of a direction runs on the tensor cores, in one of its two forms
-bool tc_stream_ok(const Direction& d, int dual) { return d.ms[dual].ok || d.tc[dual].ok; }
+bool tc_stream_ok(const Direction& d, int dual) { return d.tc[dual].ok; }
 
 struct Workspace {
     int* status;

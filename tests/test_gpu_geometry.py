@@ -220,6 +220,15 @@ def test_partial_outputs_and_argument_errors():
     assert e.value.code == -2
 
 
+def test_blocks_above_128_are_refused():
+    """The geometry mode lives in the tensor-core kernels, which take blocks of up to 128: in the forward as in the backward."""
+    c = GeoCase(synth.Workload("wide", P("160x0e+160x1o"), P("16x0e+16x1o"), 1, 8, 20, 4.0, 2.0, "bessel", seed=27))
+    for call in (c.geo_fwd, c.geo_bwd):
+        with pytest.raises(c.sb.SobekError) as e:
+            call()
+        assert e.value.code == -2
+
+
 @pytest.mark.parametrize("name", ["uvu_16x3", "uvu_32x4_K16"])
 def test_channelwise_mode(name):
     """The geometry front end in the channelwise (uvu) mode: same edge kernels, elementwise node-side steps."""

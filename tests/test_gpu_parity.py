@@ -118,6 +118,15 @@ def test_edge_outputs_keep_32_bits_off_the_16s(mode, irreps):
             assert rel_err(got, ref) <= 1e-6
 
 
+def test_streams_keep_32_bits_above_128():
+    """Blocks of more than 128 multiplicities: the streams run on the FP32 pipes by default, with the bits of a plan that asks for it."""
+    w = synth.Workload("keep32", P("160x0e+16x1o"), P("136x0e+24x1o"), 2, 8, 50, 4.0, 2.4, "bessel", seed=26)
+    c = Case(w)
+    f = Case(w, inputs=c.d, tc_stream=False)
+    for a, b in zip([c.fwd()] + c.bwd() + c.dbwd(), [f.fwd()] + f.bwd() + f.dbwd()):
+        assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("dirs", [(1, 0, 0, 0), (0, 1, 0, 0), (0, 0, 1, 0), (0, 0, 0, 1), (0, 0, 0, 0), (1, 0, 1, 0)])
 def test_double_backward_null_directions(cases, dirs):
     c = get(cases, "cfg1")
