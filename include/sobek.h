@@ -84,6 +84,8 @@ enum { SOBEK_MAX_L = 4 };
 #define SOBEK_FLAG_FP32_STREAM 16u /* edge stream on the FP32 pipes even where the tensor-core kernel applies */
 #define SOBEK_FLAG_FP32_EDGE 32u   /* edge pass on the FP32 pipes even where the tensor-core kernel applies */
 #define SOBEK_FLAG_UVU_STATE 64u   /* channelwise mode: y and gx through the receiver state even where the direct kernel applies */
+#define SOBEK_FLAG_COUPLED_FORM 128u /* tensor-core edge kernels with the coupling in the operand / epilogue, whatever pays */
+#define SOBEK_FLAG_MOMENT_FORM 256u  /* tensor-core edge kernels in moment form wherever that form exists, whatever pays */
 /* scratch budget in MiB (1 .. 2^20 - 1) in bits 12..31 of the flags word; 0 = the default */
 #define SOBEK_FLAG_STATE_BUDGET_MIB(mb) (((uint32_t)(mb) & 0xFFFFFu) << 12)
 
@@ -113,7 +115,9 @@ enum { SOBEK_MAX_L = 4 };
  * GEMM schedule, which is the faster one at present.  In the default schedule the edge stream and the edge pass run
  * on the tensor cores where the profile allows it (multiplicities that are multiples of 8 / 16, at most 128,
  * K <= 16); SOBEK_FLAG_FP32_STREAM / SOBEK_FLAG_FP32_EDGE select the FP32-pipe kernels instead (same results
- * within the tolerances).
+ * within the tolerances).  On the tensor cores both exist in two forms, with the coupling inside the sum over the edges and
+ * in moment form with the coupling outside of it; a call takes the one that is faster at its graph's mean degree.
+ * SOBEK_FLAG_COUPLED_FORM / SOBEK_FLAG_MOMENT_FORM (not both) take one of them wherever it exists.
  * SOBEK_FLAG_STATE_BUDGET_MIB(mb) sets the scratch budget (section "Runtime scratch-budget policy"; the paper
  * measures with 128 MiB): the bytes of receiver (or sender) state held at once.  Nodes are processed in chunks that
  * fit the budget, but never fewer than 512 at a time; the results do not depend on the budget beyond the summation

@@ -182,6 +182,7 @@ EdgeView sender_view(const sobek_graph* g) {
 //   32, 64 x (0..1) 0.82 - 0.92 / 0.93 - 0.99 / 0.96 - 1.06     128 x (0..3) 0.80 - 0.84 / 0.88 - 0.93 / 0.98 - 1.11
 // and with two operands an edge (the dual pass) at three quarters of it.  128/64/64 at degree 255: 4,342 against 2,950 us.
 bool moment_edge_pays(const sobek_plan* p, const sobek_graph* g, int dual) {
+    if (p->form != kFormAuto) return p->form == kFormMoment;
     int c = 0, d = 0;
     for (const DPath& P : p->fwd.paths) { c = std::max(c, P.c_src); d = std::max(d, P.d_src); }
     const double deg = c > 64 ? 60 : d <= 3 ? 48 : c > 32 ? 36 : 28;

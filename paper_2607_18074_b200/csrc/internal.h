@@ -315,6 +315,9 @@ struct UvuDirect {
     UvuDirectTables dir[2];         // [0] y from x on the receiver view, [1] gx from gy on the sender view
 };
 
+// form of the tensor-core edge kernels: the faster one by measurement, or one of the two wherever it exists
+enum { kFormAuto = 0, kFormCoupled, kFormMoment };
+
 struct sobek_plan {
     std::vector<sobek_irrep> in, out;
     int l_max = 0, K = 0;
@@ -333,6 +336,7 @@ struct sobek_plan {
     int device = -1;
     bool use_tc_stream = true;   // edge stream on the tensor cores where the profile allows it
     bool use_tc_edge = true;     // edge pass on the tensor cores where the profile allows it
+    int form = kFormAuto;        // form of both on the tensor cores
     size_t state_budget = size_t(2048) << 20;   // bytes of receiver / sender state held at once (the scratch budget)
     int gemm_passes = 3;      // 3: split-bf16 node GEMMs (fp32-faithful); 1: plain bf16 GEMMs (SOBEK_FLAG_FAST_GEMM)
     bool mul_ir = false;      // node features cross the boundary in mul_ir order and are re-laid through the workspace

@@ -32,7 +32,7 @@ static void build_moment_set(const sobek_plan* p, Direction& dir, int dual);
 void build_stream_sets(const sobek_plan* p, Direction& dir) {
     for (int dual = 0; dual < 2; ++dual) {
         build_tc_sets(p, dir, dual);
-        if (dir.tc[dual].ok && moment_form_pays(p, dir, dual)) build_moment_set(p, dir, dual);
+        if (dir.tc[dual].ok && p->form != kFormCoupled && (p->form == kFormMoment || moment_form_pays(p, dir, dual))) build_moment_set(p, dir, dual);
     }
 }
 

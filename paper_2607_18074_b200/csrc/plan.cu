@@ -405,7 +405,8 @@ using namespace sobek;
 
 extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_irrep* out, int n_out,
                                  int l_max, int K, uint32_t flags, sobek_plan** plan) {
-    if (!in || !out || !plan || n_in < 1 || n_out < 1 || K < 1 || (flags & 0xFFFu & ~uint32_t(SOBEK_FLAG_UVU | SOBEK_FLAG_MUL_IR | SOBEK_FLAG_FAST_GEMM | SOBEK_FLAG_FUSED_FP32 | SOBEK_FLAG_FP32_STREAM | SOBEK_FLAG_FP32_EDGE | SOBEK_FLAG_UVU_STATE)) != 0 || l_max < 0)
+    if (!in || !out || !plan || n_in < 1 || n_out < 1 || K < 1 || (flags & 0xFFFu & ~uint32_t(SOBEK_FLAG_UVU | SOBEK_FLAG_MUL_IR | SOBEK_FLAG_FAST_GEMM | SOBEK_FLAG_FUSED_FP32 | SOBEK_FLAG_FP32_STREAM | SOBEK_FLAG_FP32_EDGE | SOBEK_FLAG_UVU_STATE | SOBEK_FLAG_COUPLED_FORM | SOBEK_FLAG_MOMENT_FORM)) != 0 ||
+        (flags & SOBEK_FLAG_COUPLED_FORM && flags & SOBEK_FLAG_MOMENT_FORM) || l_max < 0)
         return SOBEK_ERR_INVALID_ARG;
     *plan = nullptr;
     if (l_max > SOBEK_MAX_L) return SOBEK_ERR_UNSUPPORTED;
@@ -475,6 +476,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
     p->use_fused = (flags & SOBEK_FLAG_FUSED_FP32) != 0 && !p->uvu;   // the fused kernels contain the channel-mixing GEMM
     p->use_tc_stream = (flags & SOBEK_FLAG_FP32_STREAM) == 0;
     p->use_tc_edge = (flags & SOBEK_FLAG_FP32_EDGE) == 0;
+    p->form = flags & SOBEK_FLAG_COUPLED_FORM ? kFormCoupled : flags & SOBEK_FLAG_MOMENT_FORM ? kFormMoment : kFormAuto;
     if (const uint32_t mb = flags >> 12) p->state_budget = size_t(mb) << 20;
     build_direction(p, 0, p->fwd);
     build_direction(p, 1, p->tr);

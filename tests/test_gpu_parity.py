@@ -91,6 +91,33 @@ def test_moment_form_shapes(ir_in, ir_out, l_max, K, N, deg):
         assert rel_err(got, ref) <= BWD_TOL, nm
 
 
+# The same with multiplicities of 16, so that the edge pass has both forms too.
+MOMENT16 = [("16x0e+16x1o", "16x0e+16x1o", 2, 2, 40, 16), ("16x0e+64x1o", "16x0e+16x1o", 2, 5, 40, 17), ("80x0e+16x1o", "16x0e+128x1o", 1, 9, 30, 12),
+            ("16x3o+16x4e", "16x0e+16x1o+16x4e", 4, 7, 30, 20), ("16x0e+16x1o+16x2e+16x3o", "16x0e+16x2e", 3, 16, 25, 9),
+            ("16x0e+16x1o", "16x0e+16x1o", 1, 8, 260, 140), ("16x0e+16x1o", "16x0e+16x1o", 2, 8, 430, 400)]
+
+
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg", MOMENT + MOMENT16)
+def test_both_forms(ir_in, ir_out, l_max, K, N, deg):
+    """Both forms of the tensor-core edge kernels whatever the dispatch would take, all three orders against the oracle.  That each ran
+    its own kernels shows in the bits: they sum in different orders."""
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("forms", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=17)
+    c = Case(w, form="moment")
+    o = Case(w, inputs=c.d, form="coupled")
+    refs = [c.o_fwd()] + list(c.o_bwd()) + list(c.o_dbwd())
+    names = ("y", "gx", "gY", "gphi", "gR", "ggy", "hx", "hY", "hphi", "hR")
+    got = [[k.fwd()] + k.bwd() + k.dbwd() for k in (c, o)]
+    # (no output block above 128: the sender-owned streams exist on the tensor cores as well)
+    both = ["y", "gR", "ggy", "hR"] + (["gx", "hx"] if max(m for m, _, _ in w.irreps_out) <= 128 else [])
+    if K > 1 and all(m % 16 == 0 for m, _, _ in w.irreps_in):
+        both += ["gY", "gphi", "hY", "hphi"]
+    for a, b, ref, nm in zip(*got, refs, names):
+        tol = FWD_TOL if nm == "y" else BWD_TOL
+        assert rel_err(a, ref) <= tol and rel_err(b, ref) <= tol, nm
+        assert nm not in both or not np.array_equal(a, b), nm
+
+
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K", [("96x2e+96x4e", "128x1o+24x2e+32x4e", 2, 1), ("112x2e+112x3o+112x4e", "16x0e+16x1o+16x2e+16x3o", 2, 10)])
 def test_double_backward_where_only_the_plain_edge_pass_fits(ir_in, ir_out, l_max, K):
     """Wide blocks of high order: the tensor-core edge pass fits shared memory in its plain form and not in its dual one."""
