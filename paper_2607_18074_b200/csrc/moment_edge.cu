@@ -11,6 +11,12 @@
 // of which its epilogue reads twice: 1,840 against 144 at 64 x (0..2), K = 16.  What binds here is building Pbar (per node, not
 // per edge).  fp32 parity: coupling sums in fp32, split-bf16 product with fp32 accumulation in TMEM.
 //
+// The contraction is long (all multiplicities of all components of all blocks, 1,152 terms at 128 x (0..2); k_edge_tc adds its
+// components in fp32 instead), and an accumulation in tensor memory rounds towards zero.  So the small products of the split have an
+// accumulator of their own, in the lanes that a product of 64 rows leaves free, and the fourth of them, lo x lo, is taken along.
+// Error of gY against fp64 (2-norm), 128 x (0..2), K = 16, channelwise: 6.0e-6 with the three products in one accumulator,
+// 4.4e-6 in k_edge_tc, 3.4e-6 so; the pass takes 6 % longer up to degree 64 and 14 % above, where a TMEM half holds half as many edges.
+//
 // With DUAL the pass gives the second-order terms that share Zbar (Eq. streamed_operand_second_adjoints) from G (rows of x) and Gv
 // (rows of vx):   hphi[q] = sum_b Gv Y + G vY,     hY[b] = sum_q Gv phi + G vphi.
 //
@@ -19,9 +25,10 @@
 //   state warps    cp.async of the Zbar rows of one (block, run), fp32, into shared memory;
 //   builder warps  Pbar of one slab: a warp takes (harmonic b) x NQ rows, a lane two multiplicities; K-major, 128-byte swizzle;
 //   row warps      cp.async of the sender rows of one (slab, tile), taking turns;
-//   MMA warp       M = 64 edges, N = NQ x harmonics; even tiles in the lower 16 lanes of each TMEM lane quarter, odd ones in the
-//                  upper 16;
-//   output warps   the two sums, one thread per edge; the two TMEM halves alternate between products and read-out.
+//   MMA warp       M = 64 edges, N = NQ x harmonics; hi x hi in the lower 16 lanes of each TMEM lane quarter, the small products in
+//                  the upper 16;
+//   output warps   the two sums, two threads per edge (one per accumulator); the two TMEM halves alternate between products and
+//                  read-out.
 // Every wait is bounded.
 #include <cuda_bf16.h>
 
@@ -63,7 +70,7 @@ struct MeArgs {
     const float* zbar;
     float *gphi, *gY;
     int32_t phi_mode, Y_mode;   // 0 skip, 1 overwrite, 2 accumulate
-    int32_t K, dsh, C_src, nq, N_cols, nx, np, nz, p_bytes, z_bytes;
+    int32_t K, dsh, C_src, N_cols, nx, np, nz, p_bytes, z_bytes;
     int* status;
 };
 
@@ -118,9 +125,9 @@ struct Walk {
     }
 };
 
-// The two sums of one run of radial indices for the edge of this thread.
+// The two sums of one run of radial indices for the edge of this thread and of lane ^ 16, which has the other accumulator.
 template <int NQ, bool DUAL>
-__device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t tv, int64_t e, bool ok, int q0, bool first_run, bool has_vx) {
+__device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t tv, int64_t e, bool ok, int part, int q0, bool first_run, bool has_vx) {
     float f[NQ], vf[NQ], gp[NQ];
     const bool has_vY = DUAL && a.vY, has_vphi = DUAL && a.vphi;
 #pragma unroll
@@ -155,15 +162,18 @@ __device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t 
                 if (q0 + r < a.K) gy = fmaf(g[r], f[r], gy);
             }
         }
-        if (ok && a.Y_mode) {
+        gy += __shfl_xor_sync(0xffffffffu, gy, 16);
+        if (ok && a.Y_mode && (b & 1) == part) {
             float* d = a.gY + e * a.dsh + b;
             *d = (first_run && a.Y_mode == 1) ? gy : *d + gy;
         }
     }
+#pragma unroll
+    for (int r = 0; r < NQ; ++r) gp[r] += __shfl_xor_sync(0xffffffffu, gp[r], 16);
     if (ok && a.phi_mode) {
 #pragma unroll
         for (int r = 0; r < NQ; ++r)
-            if (q0 + r < a.K) {
+            if (q0 + r < a.K && (r & 1) == part) {
                 float* d = a.gphi + e * a.K + q0 + r;
                 *d = a.phi_mode == 1 ? gp[r] : *d + gp[r];
             }
@@ -191,7 +201,7 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
     const bool has_vx = DUAL && a.vsh != nullptr;
     const int nop = has_vx ? 2 : 1;                                    // operands: rows of x, of vx
     const int n_cols = a.N_cols, runs = (a.K + NQ - 1) / NQ;
-    const int pass_tiles = 2 * (HALF / (n_cols * nop));                // tiles that one accumulator holds
+    const int pass_tiles = HALF / (n_cols * nop);                      // tiles that one TMEM half holds
     if (tid == 0) {
         for (int s = 0; s < MAXNX; ++s) { mbar_init(bar_xfull + 8 * s, 32); mbar_init(bar_xfree + 8 * s, 1); }
         for (int s = 0; s < MAXNP; ++s) { mbar_init(bar_pfull + 8 * s, NBW * 32); mbar_init(bar_pfree + 8 * s, 1); }
@@ -387,16 +397,17 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                                 fence_async_smem();      // the gathered rows were written through the generic proxy
                                 tc_fence_after();
                                 const uint64_t dX = dX0 + __shfl_sync(0xffffffffu, (uint32_t)xs * (2u * SLAB >> 4), 0);
-                                const uint32_t dt = tm_u + buf * HALF + __shfl_sync(0xffffffffu, (uint32_t)((t >> 1) * nop + op) * uN + (uint32_t)((t & 1) * 16 << 16), 0);
+                                const uint32_t dt = tm_u + buf * HALF + __shfl_sync(0xffffffffu, (uint32_t)(t * nop + op) * uN, 0);
+                                constexpr uint32_t small = 16u << 16;      // lanes of the small products
                                 if (elect_one()) {
                                     if (ks == 4) {
 #pragma unroll
                                         for (uint32_t k = 0; k < 4; ++k)
-                                            tc_mma_bf16_x3(dt, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                            tc_mma_bf16_x4(dt, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
                                     } else {
 #pragma unroll 1
                                         for (uint32_t k = 0; k < ks; ++k)
-                                            tc_mma_bf16_x3(dt, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                            tc_mma_bf16_x4(dt, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
                                     }
                                     tc_commit(bar_xfree + 8 * xs);
                                     if (t + 1 == tiles && op + 1 == nop) {
@@ -425,12 +436,12 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                     if (warp == 0) mbar_spin(bar_accfull + 8 * buf, (ai >> 1) & 1, a.status);
                     asm volatile("bar.sync 1, %0;" ::"n"(NOW * 32) : "memory");
                     tc_fence_after();
-                    for (int t = 0; t < tiles; t += 2) {
-                        const int le = (t + (lane >> 4)) * TILE + warp * 16 + (lane & 15);
+                    for (int t = 0; t < tiles; ++t) {
+                        const int le = t * TILE + warp * 16 + (lane & 15);
                         const bool ok = le < plen;
                         if (!__any_sync(0xffffffffu, ok)) continue;
-                        const uint32_t td = tmem_base + ((uint32_t)(warp * 32) << 16) + buf * HALF + (uint32_t)((t >> 1) * nop * n_cols);
-                        edge_sums<NQ, DUAL>(a, td, td + (uint32_t)n_cols, seg0 + p0 + (ok ? le : 0), ok, run * NQ, run == 0, has_vx);
+                        const uint32_t td = tmem_base + ((uint32_t)(warp * 32) << 16) + buf * HALF + (uint32_t)(t * nop * n_cols);
+                        edge_sums<NQ, DUAL>(a, td, td + (uint32_t)n_cols, seg0 + p0 + (ok ? le : 0), ok, lane >> 4, run * NQ, run == 0, has_vx);
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -551,7 +562,7 @@ cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const 
     a.vsh = dual ? (const __nv_bfloat16*)ss.vh : nullptr; a.vsl = dual ? (const __nv_bfloat16*)ss.vl : nullptr;
     a.Y = Y; a.vY = vY; a.phi = phi; a.vphi = vphi; a.zbar = zbar; a.gphi = gphi; a.gY = gY;
     a.phi_mode = phi_mode; a.Y_mode = Y_mode;
-    a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src; a.nq = T.nq; a.N_cols = T.n_cols; a.nx = T.nx; a.np = T.np; a.nz = T.nz;
+    a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src; a.N_cols = T.n_cols; a.nx = T.nx; a.np = T.np; a.nz = T.nz;
     a.p_bytes = T.p_bytes; a.z_bytes = T.z_bytes; a.status = status;
     void (*kern)(const MeArgs) = T.nq == 8 ? (dual ? k_moment_edge<8, true> : k_moment_edge<8, false>)
                                  : T.nq == 4 ? (dual ? k_moment_edge<4, true> : k_moment_edge<4, false>)

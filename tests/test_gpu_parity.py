@@ -118,6 +118,21 @@ def test_both_forms(ir_in, ir_out, l_max, K, N, deg):
         assert nm not in both or not np.array_equal(a, b), nm
 
 
+@pytest.mark.parametrize("mode,irreps,l_max,K", [("uvw", "64x0e+64x1o+64x2e+64x3o+64x4e", 4, 8), ("uvw", "128x0e+64x1o+64x2e", 2, 16),
+                                                 ("uvu", "112x0e+112x1o+112x2e", 2, 10), ("uvu", "64x0e+64x1o+64x2e+64x3o", 3, 16)])
+def test_moment_edge_pass_is_as_exact_as_the_other_form(mode, irreps, l_max, K):
+    """The contraction of the moment form runs over all components of all blocks at once, k-step after k-step into one accumulator,
+    and must not lose by that.  (Both forms have the representation error of bf16 hi + lo; 3 % for the spread of a small graph.)"""
+    ir = P(irreps)
+    w = synth.Workload("exact", ir, ir, l_max, K, 24, 4.0, 2.4, "bessel", seed=29, mode=mode)
+    m = Case(w, form="moment")
+    o = Case(w, inputs=m.d, form="coupled")
+    norm2 = lambda got, ref: np.linalg.norm(got - ref) / np.linalg.norm(ref)
+    refs = list(m.o_bwd()[1:3]) + list(m.o_dbwd()[2:4])
+    for a, b, ref, nm in zip(m.bwd()[1:3] + m.dbwd()[2:4], o.bwd()[1:3] + o.dbwd()[2:4], refs, ("gY", "gphi", "hY", "hphi")):
+        assert norm2(a, ref) <= 1.03 * norm2(b, ref), nm
+
+
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K", [("96x2e+96x4e", "128x1o+24x2e+32x4e", 2, 1), ("112x2e+112x3o+112x4e", "16x0e+16x1o+16x2e+16x3o", 2, 10)])
 def test_double_backward_where_only_the_plain_edge_pass_fits(ir_in, ir_out, l_max, K):
     """Wide blocks of high order: the tensor-core edge pass fits shared memory in its plain form and not in its dual one."""
