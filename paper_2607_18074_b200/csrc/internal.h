@@ -161,6 +161,7 @@ struct TcSets {
     int32_t ring_stages = 2;          // stream: stages of the shared-memory ring (as many as fit)
     int32_t nbuf = 2;                 // stream: accumulator buffers in tensor memory (2, or 1 for wider sets)
     int32_t smem_bytes = 0, ctas_per_sm = 1;
+    double node_us = 0, slot_us = 0;      // streams with a moment form beside them: estimate (stream_costs) of a node, of 16 of its edges
 };
 
 // --- moment-form edge stream (moment_stream.cu) --------------------------------------------
@@ -213,6 +214,7 @@ struct MomentSets {
     MSet* d_sets = nullptr; MGrp* d_grps = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
     uint16_t* d_rows = nullptr;
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;
+    double node_us = 0, slot_us = 0, slot_again_us = 0;      // estimate (stream_costs): a node, 16 of its edges, the same gathered per unit
 };
 
 // --- moment-form edge pass (moment_edge.cu) ------------------------------------------------
@@ -468,6 +470,9 @@ cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const Ed
                              const float* vphi, int dual, void* zh, void* zl, int* status, cudaStream_t s);
 // --- moment_stream.cu -------------------------------------------------------------------
 void build_stream_sets(const sobek_plan* p, Direction& dir);
+// the moment form is taken for a stream over a graph of N nodes and E edges (operands: 2 in a dual stream with a source direction and
+// a direction of Y or phi, else 1)
+bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, int64_t N, int64_t E);
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
                                  const SplitSrc& ss, const float* Y, const float* vY, const float* phi, const float* vphi, int dual,
                                  void* zh, void* zl, int* status, cudaStream_t s);

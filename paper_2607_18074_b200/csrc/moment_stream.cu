@@ -1,39 +1,76 @@
-// Host side of the moment-form edge stream: sets, units and read-out tables of a direction, and the launch.
+// Host side of the moment-form edge stream: sets, units and read-out tables of a direction, the choice between the two forms of the
+// stream, and the launch.
 #include <algorithm>
+#include <cmath>
 
 #include "moment_stream.h"
 
 namespace sobek {
 
-// Where both forms of the stream apply, which one: measured on 2,000 nodes of degree 30 in whole calls, time of the other form over
-// that of this one, m x (0..L).
-//   forward   K = 8:  L = 1 1.26 - 1.37, L = 2 1.06 - 1.15, L = 3 1.04 - 1.17, L = 4 1.03 - 1.14   (m = 8 .. 64)
-//             K = 16: L = 1 1.04 - 1.12, L = 2 1.01 - 1.21, L = 3 0.91 - 1.06, L = 4 0.80 - 0.95
-//   second order (the dual stream and the plain one of the transposed direction)  1.01 - 1.25 throughout
-//   m = 96, cut into 48 + 48 of 64 rows: 0.76 - 1.13, mostly below one; m = 128: 0.94 - 1.26
-// The plain form loses where a run of radial indices has to be split over many narrow products: orders from three on with more
-// than eight radial indices; both lose where cutting a wide block leaves the products a quarter empty.
-static bool moment_form_pays(const sobek_plan* p, const Direction& dir, int dual) {
-    int d = 0, rows = 0, used = 0;
-    for (const DPath& P : dir.paths) {
-        d = std::max(d, P.d_src);
-        if (P.c_src > 64) { rows += P.d_src * 64 * ((P.c_src + 63) / 64); used += P.d_src * P.c_src; }
-    }
-    if (rows && used * 5 < rows * 4) return false;
-    return dual || p->K <= 8 || d <= 5;
-}
-
-// Sets, units and read-out tables of one direction, plain or dual stream.
 static void build_moment_set(const sobek_plan* p, Direction& dir, int dual);
+static void stream_costs(Direction& dir, int dual);
 
-// Which form each stream of a direction takes, and its tables.  The moment form only in the place of k_stream_tc: a profile that
-// neither fits keeps the FP32-pipe stream, whose rows and coupling values have 32 bits (error of gR, 2-norm against fp64, 192 x (0..3):
-// 4.5e-6 there, 6.4e-6 in either form on the tensor cores).
+// Both forms of each stream of a direction; a call takes one of them (moment_stream_pays).  The moment form only in the place of
+// k_stream_tc: a profile that k_stream_tc does not fit keeps the FP32-pipe stream, whose rows and coupling values have 32 bits (error
+// of gR, 2-norm against fp64, 192 x (0..3): 4.5e-6 there, 6.4e-6 in either form on the tensor cores).
 void build_stream_sets(const sobek_plan* p, Direction& dir) {
     for (int dual = 0; dual < 2; ++dual) {
         build_tc_sets(p, dir, dual);
-        if (dir.tc[dual].ok && p->form != kFormCoupled && (p->form == kFormMoment || moment_form_pays(p, dir, dual))) build_moment_set(p, dir, dual);
+        if (!dir.tc[dual].ok || p->form == kFormCoupled) continue;
+        build_moment_set(p, dir, dual);
+        if (dir.ms[dual].ok) stream_costs(dir, dual);
     }
+}
+
+// Microseconds that one SM spends on a node and on 16 of its edges in either form, from the counts of the forms' tables.  The
+// constants are least-squares fits (of relative errors, 10 - 13 % left) to the streams of 720 random layers, 8 to 128 multiplicities
+// of orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes, in both directions.  With them the slower form is taken where
+// the two are close: the chosen form takes 0.7 % longer than the faster one on average (0.5 % in the dual streams), 23 % (35 %) at
+// worst longer than the other.  (Rules on K, order and width alone, from graphs of degree 30: 6.2 % and 8.2 %, up to 2.8 times as
+// long.  Fixed forms: moment 8 %, coupled 26 to 36 %.)
+static void stream_costs(Direction& dir, int dual) {
+    TcSets& T = dir.tc[dual];
+    MomentSets& M = dir.ms[dual];
+    double cols = 0, slabs = 0, rows = 0;
+    for (const TSet& S : T.sets) {
+        slabs += S.nslab;
+        for (int u = 0; u < S.nunit; ++u) cols += (T.blks[T.units[S.unit_begin + u].blk].ncols + 31) & ~31;
+        for (int b = 0; b < S.nblk; ++b) rows += T.blks[S.blk_begin + b].d_src * ((T.blks[S.blk_begin + b].c_src + 63) / 64);
+    }
+    T.node_us = dual ? 0.0146 * cols : 0.0144 * cols;                                        // read-out of the accumulators
+    T.slot_us = dual ? 0.2 * slabs + 0.023 * rows + 1.04 * T.sets.size()                     // built operand; gathered rows; hand-over
+                     : 0.1375 * slabs + 0.04 * rows + 0.87 * T.sets.size();
+    double units = 0, outs = 0, vals = 0, terms = 0, kcycles = 0, w_once = 0, w_again = 0, rows_once = 0, rows_again = 0;
+    for (const MSet& S : M.sets) {
+        for (int b = 0; b < S.nblk; ++b) rows_once += M.blks[S.blk_begin + b].d_src;
+        for (int g = 0; g < S.ngrp; ++g) {
+            const MGrp& G = M.grps[S.grp_begin + g];
+            w_once += 2 * G.rows;
+            for (int u = 0; u < G.nunit; ++u) {
+                const MUnit& U = M.units[G.unit_begin + u];
+                units += 1;
+                kcycles += 6e-3 * U.d * std::max(41.0, U.N / 2.0);                           // six products per component, at least 41 cycles each
+                w_again += 2 * U.N;
+                for (int b = 0; b < U.nblk; ++b) rows_again += M.blks[S.blk_begin + U.blk0 + b].d_src;
+                for (int o = 0; o < U.n_out; ++o) {
+                    outs += U.nqs; vals += U.nqs * S.nq; terms += 0.5 * U.nqs * M.outs[U.out_begin + o].n;
+                }
+            }
+        }
+    }
+    M.node_us = dual ? 0.557 * units + 0.0416 * outs + 0.0068 * vals : 0.513 * units + 0.0406 * outs + 0.0057 * vals + 0.0053 * terms;
+    const double w = dual ? 0.0044 : 0.0031, r = dual ? 0.071 : 0.0535, c = (dual ? 0.133 : 0.171) * kcycles;
+    M.slot_us = c + w * w_once + r * rows_once;
+    M.slot_again_us = c + w * w_again + r * rows_again;                                      // rows and W anew for every unit
+}
+
+bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, int64_t N, int64_t E) {
+    const TcSets& T = dir.tc[dual];
+    const MomentSets& M = dir.ms[dual];
+    if (!M.ok || p->form != kFormAuto) return M.ok && p->form == kFormMoment;
+    const double deg = (double)E / (double)std::max<int64_t>(N, 1), slots = (deg / MS_TB + 0.5) * operands;
+    const bool resident = std::ceil(deg / MS_TB + 0.3) * operands <= std::min(M.ns, M.nw);   // (degrees spread around their mean)
+    return M.node_us + slots * (resident ? M.slot_us : M.slot_again_us) < T.node_us + slots * T.slot_us;
 }
 
 static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {

@@ -118,6 +118,21 @@ def test_both_forms(ir_in, ir_out, l_max, K, N, deg):
         assert nm not in both or not np.array_equal(a, b), nm
 
 
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg,output,form", [
+    ("8x0e+8x1o+8x2e", "8x0e+8x1o+8x2e", 2, 16, 400, 4, "y", "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "y", "moment"),
+    ("96x1o+96x2e", "96x0e", 2, 16, 200, 100, "y", "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "gx", "moment"),
+    ("96x1o+96x2e+96x3o", "96x0e", 3, 10, 160, 90, "ggy", "coupled"), ("64x0e+64x1o+64x2e", "64x0e+64x1o+64x2e", 2, 8, 160, 20, "ggy", "moment")])
+def test_stream_takes_the_form_that_pays(ir_in, ir_out, l_max, K, N, deg, output, form):
+    """Degrees and shapes at which one form of the stream takes at most 0.8 of the other's time: the default plan has its bits."""
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("pays", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=31)
+    c = Case(w)
+    run = lambda k: dict(y=lambda: k.fwd(), gx=lambda: k.bwd()[0], ggy=lambda: k.dbwd()[0])[output]()
+    got, other = run(c), "moment" if form == "coupled" else "coupled"
+    assert np.array_equal(got, run(Case(w, inputs=c.d, form=form)))
+    assert not np.array_equal(got, run(Case(w, inputs=c.d, form=other)))
+
+
 @pytest.mark.parametrize("mode,irreps,l_max,K", [("uvw", "64x0e+64x1o+64x2e+64x3o+64x4e", 4, 8), ("uvw", "128x0e+64x1o+64x2e", 2, 16),
                                                  ("uvu", "112x0e+112x1o+112x2e", 2, 10), ("uvu", "64x0e+64x1o+64x2e+64x3o", 3, 16)])
 def test_moment_edge_pass_is_as_exact_as_the_other_form(mode, irreps, l_max, K):
