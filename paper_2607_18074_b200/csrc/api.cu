@@ -174,21 +174,6 @@ EdgeView sender_view(const sobek_graph* g) {
     return EdgeView{g->src_ptr, g->src_perm, g->col, g->row_ptr, g->N, g->E, 1, g->src_recv};
 }
 
-// Edge pass: the moment form costs a node the building of its Pbar and an edge little, the form with the coupling left in costs by
-// the edge.  They meet at the mean degree below (calls of the backward at 2,000 nodes, time of the other form over that of the
-// moment form at degree 12 / 30 / 64, K = 8 and 16):
-//   32 x (0..2) 0.91 / 1.04 / 1.11, 0.90 / 1.04 / 1.21     64 x (0..2) 0.87 / 0.99 / 1.12, 0.84 / 0.95 / 1.09
-//   32 x (0..4) 0.85 / 1.04 / 1.30, 0.78 / 1.02 / 1.27     64 x (0..4) 0.82 / 0.97 / 1.19, 0.77 / 0.95 / 1.16
-//   32, 64 x (0..1) 0.82 - 0.92 / 0.93 - 0.99 / 0.96 - 1.06     128 x (0..3) 0.80 - 0.84 / 0.88 - 0.93 / 0.98 - 1.11
-// and with two operands an edge (the dual pass) at three quarters of it.  128/64/64 at degree 255: 4,342 against 2,950 us.
-bool moment_edge_pays(const sobek_plan* p, const sobek_graph* g, int dual) {
-    if (p->form != kFormAuto) return p->form == kFormMoment;
-    int c = 0, d = 0;
-    for (const DPath& P : p->fwd.paths) { c = std::max(c, P.c_src); d = std::max(d, P.d_src); }
-    const double deg = c > 64 ? 60 : d <= 3 ? 48 : c > 32 ? 36 : 28;
-    return (double)g->E >= (dual ? 0.75 : 1.0) * deg * (double)g->N;
-}
-
 bool has_uncovered(const Direction& d) {
     for (const DGroup& G : d.groups)
         if (G.path_end == G.path_begin) return true;
@@ -427,7 +412,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
     if (geo) { xs = *geo; gs = *geo; gs.g_rvec = nullptr; }
     const bool g_edge = geo && geo->g_rvec;       // geometry mode: the edge pass writes the adjoint of the edge vectors
     if (g_edge) { gphi = geo->g_rvec; gY = geo->g_rvec; }      // (stand-ins: "wanted"; the kernel writes g_rvec only)
-    const bool tc_edge = w.zqh != nullptr, me_edge = w.zf && !geo && moment_edge_pays(p, g, 0);
+    const bool tc_edge = w.zqh != nullptr, me_edge = w.zf && !geo && moment_edge_pays(p, 0, 1, g->N, g->E, w.chunk);
     const bool gx_direct = p->uvu && p->ud.ok && !p->uvu_state && !geo && g->src_recv;      // channelwise mode: no state for gx
     const bool gR_direct = gR && p->uvu && p->ud.ok && !p->uvu_state && !geo && !z_valid;   // nor for gR
     if (gR_direct) {
@@ -541,8 +526,8 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
     SplitSrc xs{}, gs{};
     if (geo) { xs = *geo; gs = *geo; }
     const bool tc_edge_plain = w.zqh != nullptr, tc_edge_dual = tc_edge_plain && p->fwd.etc[1].ok && (!vx || w.vsh);
-    const bool me_edge_plain = w.zf && !geo && moment_edge_pays(p, g, 0),
-               me_edge_dual = w.zf && !geo && (!tc_edge_dual || moment_edge_pays(p, g, 1));
+    const bool me_edge_plain = w.zf && !geo && moment_edge_pays(p, 0, 1, g->N, g->E, w.chunk),
+               me_edge_dual = w.zf && !geo && (!tc_edge_dual || moment_edge_pays(p, 1, vx ? 2 : 1, g->N, g->E, w.chunk));
     if (w.oseg_r && (ggy || hR || hphi || hY)) { CK(launch_chunk_order(rv, w.chunk, kOrderPeriod, w.oseg_r, w.status, s)); xs.oseg = w.oseg_r; }
     if (w.oseg_s && hx && !w.fused_t) {
         CK(launch_chunk_order(sender_view(g), w.chunk, kOrderPeriod, w.oseg_s, w.status, s));

@@ -237,6 +237,7 @@ struct MomentEdge {
     std::vector<MTerm> terms;         // {offset of the component in the staged Zbar, coefficient}
     MEBlk* d_blks = nullptr; MEComp* d_comps = nullptr; int32_t* d_tptr = nullptr; MTerm* d_terms = nullptr;
     int32_t nq = 0, n_cols = 0, nx = 0, np = 0, nz = 0, p_bytes = 0, z_bytes = 0, smem_bytes = 0;
+    int32_t slabs = 0, ksteps = 0;    // of all blocks
 };
 
 struct FStage {        // one 256-column stage of the fused kernel's contraction axis
@@ -479,6 +480,9 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
 
 // --- moment_edge.cu ---------------------------------------------------------------------
 void build_moment_edge(const sobek_plan* p, Direction& dir);
+// the moment form is taken for the edge pass over a graph of N nodes and E edges in chunks of `chunk` nodes (operands: rows of x, or
+// of x and vx)
+bool moment_edge_pays(const sobek_plan* p, int dual, int operands, int64_t N, int64_t E, int64_t chunk);
 cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes, const SplitSrc& ss,
                                const float* Y, const float* vY, const float* phi, const float* vphi, int dual, const float* zbar, float* gphi,
                                float* gY, int phi_mode, int Y_mode, int* status, cudaStream_t s);

@@ -524,6 +524,7 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
                     }
                 T.tptr.push_back((int)T.terms.size());
                 T.blks.push_back(M);
+                T.slabs += M.d; T.ksteps += M.d * M.ksteps;
             }
         }
         T.p_bytes = (2 * n_cols * 128 + 1023) & ~1023;
@@ -545,6 +546,35 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
         if (T.ok) return;
     }
     T = MomentEdge{};
+}
+
+// Microseconds per node that one SM spends in either form of the pass, the adjoint state's product with it (fp32 for one, bf16 hi + lo
+// for the other).  Least-squares fits (of relative errors, 11 % and 18 % left) to the passes of 531 random layers with
+// multiplicities of 16 (and 250 channelwise ones), orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes.  The chosen form takes 1.6 % longer than the
+// faster one on average (1.3 % in the dual pass), 37 % (50 %) at worst longer than the other.  (Lines at fixed degrees, drawn before
+// the fp32 products wrote 16 bytes a lane and the small products had an accumulator of their own: 8.3 % and 11 %, up to 2.2 and 2.7
+// times as long.)
+bool moment_edge_pays(const sobek_plan* p, int dual, int operands, int64_t N, int64_t E, int64_t chunk) {
+    const Direction& dir = p->fwd;
+    const MomentEdge& M = dir.me;
+    const TcSets& T = dir.etc[dual];
+    if (!M.ok || p->form != kFormAuto) return M.ok && p->form == kFormMoment;
+    const double deg = (double)E / (double)std::max<int64_t>(N, 1), per_sm = std::max(1.0, (double)std::min(N, chunk) / 148.0);
+    const double state = 1e-4 * (double)dir.state_floats;
+    const double fp32 = (dual ? 0.88 : 1.12) + (p->uvu ? 1.9 : 0.0);     // (the channelwise mode writes fp32 rows at 0.6 of the rate of its bf16 ones)
+    const double runs = (p->K + M.nq - 1) / M.nq, cap = TILE * (HALF / (M.n_cols * operands));           // edges of a pass
+    const double builds = runs * (deg > 0.6 * cap ? std::max(1.0, deg / cap + 0.4) : 1.0);
+    const double tiles = runs * (deg > 40 ? deg / TILE + 0.5 : 1.0) * operands;
+    const double build = dual ? 0.88 + 0.364 * M.slabs + M.nq * (0.00135 * M.terms.size() + 0.00154 * M.slabs * p->dim_sh)
+                              : 0.45 + 0.206 * M.slabs + M.nq * (0.00274 * M.terms.size() + 0.0006 * M.slabs * p->dim_sh);
+    const double moment = 27.0 / per_sm + builds * build + tiles * (M.ksteps * (dual ? 0.055 + 0.00063 * M.n_cols : 0.053 + 0.00083 * M.n_cols) +
+                          (dual ? 0.061 : 0.127) * p->dim_sh) + runs * operands * deg * 0.0035 * M.slabs + fp32 * state;
+    double coupled = (dual ? 2.46 : 2.48) * state;
+    for (const TcSets::ESetPar& e : T.epar) {
+        const double batches = std::max(1.0, deg / e.tb + 0.45);
+        coupled += 25.0 / per_sm + batches / e.ctas * (dual ? 5.97 + 0.0133 * e.acc_cols + 3.7e-5 * e.nnz * e.tb : 3.24 + 0.009 * e.acc_cols + 1.9e-5 * e.nnz * e.tb);
+    }
+    return moment < coupled;
 }
 
 cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes, const SplitSrc& ss,

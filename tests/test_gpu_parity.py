@@ -133,6 +133,20 @@ def test_stream_takes_the_form_that_pays(ir_in, ir_out, l_max, K, N, deg, output
     assert not np.array_equal(got, run(Case(w, inputs=c.d, form=other)))
 
 
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg,dual,form", [
+    ("64x0e+64x1o+64x2e", "64x0e+64x1o+64x2e", 2, 8, 1500, 10, 0, "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 16, 200, 60, 0, "moment"),
+    ("96x1o+96x2e+96x3o", "96x0e", 3, 10, 160, 70, 1, "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 16, 200, 60, 1, "moment")])
+def test_edge_pass_takes_the_form_that_pays(ir_in, ir_out, l_max, K, N, deg, dual, form):
+    """The same for the edge pass, plain and dual."""
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("pays", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=33)
+    c = Case(w)
+    run = lambda k: k.dbwd(dirs=(True, True, True, False))[3] if dual else k.bwd()[2]
+    got, other = run(c), "moment" if form == "coupled" else "coupled"
+    assert np.array_equal(got, run(Case(w, inputs=c.d, form=form)))
+    assert not np.array_equal(got, run(Case(w, inputs=c.d, form=other)))
+
+
 @pytest.mark.parametrize("mode,irreps,l_max,K", [("uvw", "64x0e+64x1o+64x2e+64x3o+64x4e", 4, 8), ("uvw", "128x0e+64x1o+64x2e", 2, 16),
                                                  ("uvu", "112x0e+112x1o+112x2e", 2, 10), ("uvu", "64x0e+64x1o+64x2e+64x3o", 3, 16)])
 def test_moment_edge_pass_is_as_exact_as_the_other_form(mode, irreps, l_max, K):
