@@ -99,13 +99,11 @@ Workspace carve(const sobek_plan* p, int64_t N, int order, void* ws) {
             w.zqh = w.zbh;
             w.zql = w.zbl;
         }
-        if (needs_zbar(p, order)) {
-            w.zbar = (float*)take((size_t)w.chunk * (size_t)p->fwd.state_floats * 4);
-        }
+        w.zbar = needs_zbar(p, order) ? (float*)take((size_t)w.chunk * (size_t)p->fwd.state_floats * 4) : w.zf;
     }
-    if (p->use_tc_stream || w.zqh) {
+    if (p->use_tc_stream || w.zqh || w.zf) {
         const size_t nx = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_x * 2, ny = (size_t)std::max<int64_t>(N, 0) * (size_t)p->C_y * 2;
-        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || w.zqh) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
+        if (tc_stream_ok(p->fwd, 0) || (order >= 2 && tc_stream_ok(p->fwd, 1)) || w.zqh || w.zf) { w.xsh = (uint16_t*)take(nx); w.xsl = (uint16_t*)take(nx); }
         if (order >= 1 && (tc_stream_ok(p->tr, 0) || (order >= 2 && tc_stream_ok(p->tr, 1)))) { w.gsh = (uint16_t*)take(ny); w.gsl = (uint16_t*)take(ny); }
         if (order >= 2 && (tc_stream_ok(p->fwd, 1) || (w.zqh && p->fwd.etc[1].ok) || w.zf)) { w.vsh = (uint16_t*)take(nx); w.vsl = (uint16_t*)take(nx); }
         // load balance of the persistent edge kernels: only where a CTA takes several nodes of a chunk
@@ -218,10 +216,11 @@ cudaError_t mix_tc(const sobek_plan* p, const Direction& dir, int64_t n0, int64_
 }
 
 // Zbar_g = gy_g * Rp_g^T       (Eq. receiver_adjoint)
-// With zqh / zql the result is written as bf16 (hi, lo) rows in the layout of the stream's state instead.
+// With zqh / zql the result is written as bf16 (hi, lo) rows in the layout of the stream's state instead; exact (fp32 result only):
+// four products instead of three, for the edge pass in moment form where it stands for the FP32-pipe pass.
 cudaError_t state_adjoint_tc(const sobek_plan* p, const Direction& dir, int64_t nn, const uint16_t* gh,
                              const uint16_t* gl, const uint16_t* knh, const uint16_t* knl, float* Zbar, int* status,
-                             cudaStream_t s, uint16_t* zqh = nullptr, uint16_t* zql = nullptr) {
+                             cudaStream_t s, uint16_t* zqh = nullptr, uint16_t* zql = nullptr, bool exact = false) {
     GemmBatch gb;
     for (size_t gi = 0; gi < dir.groups.size(); ++gi) {
         const DGroup& G = dir.groups[gi];
@@ -236,7 +235,7 @@ cudaError_t state_adjoint_tc(const sobek_plan* p, const Direction& dir, int64_t 
             e = gemm_tc_add(gb, gh + nn * dir.gb_off[gi], gl + nn * dir.gb_off[gi], dir.kn_ld[gi],
                             knh + dir.kn_off[gi], knl + dir.kn_off[gi], dir.kn_ld[gi],
                             Zbar + nn * G.z_off, G.D, 0, 1, nn * G.d_dst, G.D, G.c_dst, 0, 0, status, s, 1, 0, nullptr, nullptr,
-                            p->gemm_passes);
+                            p->gemm_passes == 3 && exact ? 4 : p->gemm_passes);
         if (e != cudaSuccess) return e;
     }
     return gemm_tc_flush(gb, s, p);
@@ -298,9 +297,9 @@ cudaError_t mix(const sobek_plan* p, const Direction& dir, int64_t n0, int64_t n
 cudaError_t state_adjoint(const sobek_plan* p, const Direction& dir, int64_t n0, int64_t nn, const uint16_t* gh,
                           const uint16_t* gl, const uint16_t* knh, const uint16_t* knl, const float* gy,
                           const float* Rraw, float* Zbar, int* status, cudaStream_t s, uint16_t* zqh = nullptr,
-                          uint16_t* zql = nullptr) {
+                          uint16_t* zql = nullptr, bool exact = false) {
     if (p->uvu) return launch_uvu_zbar(p, dir, n0, nn, gy, Rraw, Zbar, zqh, zql, s);
-    return state_adjoint_tc(p, dir, nn, gh, gl, knh, knl, Zbar, status, s, zqh, zql);
+    return state_adjoint_tc(p, dir, nn, gh, gl, knh, knl, Zbar, status, s, zqh, zql, exact);
 }
 cudaError_t weight_grad(const sobek_plan* p, const Direction& dir, int64_t n0, int64_t nn, const uint16_t* zh,
                         const uint16_t* zl, const uint16_t* gh, const uint16_t* gl, const float* gy, float* gRp,
@@ -428,7 +427,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
         gs.oseg = w.oseg_s;
     }
     FeatureSplits fs;
-    if (w.xsh && (gR || ((gphi || gY) && tc_edge))) { fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl; }
+    if (w.xsh && (gR || ((gphi || gY) && (tc_edge || me_edge)))) { fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl; }
     if (w.gsh && gx && !w.fused_t && !gx_direct) { fs.add(gy, g->N, p->C_y, w.gsh, w.gsl); gs.h = w.gsh; gs.l = w.gsl; }
     CK(fs.flush(s));
     PackQueue pq(p);              // every operand layout of R this call needs, one launch
@@ -447,7 +446,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
             }
             if (gphi || gY) {
                 if (me_edge) {
-                    CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s));
+                    CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s, nullptr, nullptr, p->fwd.me.exact));
                     CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xs, Y, nullptr, phi, nullptr, 0, w.zf, gphi, gY, gphi ? 1 : 0, gY ? 1 : 0, w.status, s));
                 } else if (tc_edge) {
                     CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, nullptr, w.status, s, w.zqh, w.zql));
@@ -527,14 +526,14 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
     if (geo) { xs = *geo; gs = *geo; }
     const bool tc_edge_plain = w.zqh != nullptr, tc_edge_dual = tc_edge_plain && p->fwd.etc[1].ok && (!vx || w.vsh);
     const bool me_edge_plain = w.zf && !geo && moment_edge_pays(p, 0, 1, g->N, g->E, w.chunk),
-               me_edge_dual = w.zf && !geo && (!tc_edge_dual || moment_edge_pays(p, 1, vx ? 2 : 1, g->N, g->E, w.chunk));
+               me_edge_dual = w.zf && !geo && moment_edge_pays(p, 1, vx ? 2 : 1, g->N, g->E, w.chunk);
     if (w.oseg_r && (ggy || hR || hphi || hY)) { CK(launch_chunk_order(rv, w.chunk, kOrderPeriod, w.oseg_r, w.status, s)); xs.oseg = w.oseg_r; }
     if (w.oseg_s && hx && !w.fused_t) {
         CK(launch_chunk_order(sender_view(g), w.chunk, kOrderPeriod, w.oseg_s, w.status, s));
         gs.oseg = w.oseg_s;
     }
     FeatureSplits fs;
-    if (w.xsh && (ggy || hR || ((hphi || hY) && tc_edge_plain))) {
+    if (w.xsh && (ggy || hR || ((hphi || hY) && (tc_edge_plain || me_edge_plain || me_edge_dual)))) {
         fs.add(x, g->N, p->C_x, w.xsh, w.xsl); xs.h = w.xsh; xs.l = w.xsl;
         if (vx && w.vsh) { fs.add(vx, g->N, p->C_x, w.vsh, w.vsl); xs.vh = w.vsh; xs.vl = w.vsl; }
     }
@@ -593,7 +592,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                 if (any_edge_dir) {
                     // the three direction terms that share Zbar = gy R^T, in one pass
                     if (me_edge_dual) {
-                        CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s));
+                        CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, w.zf, w.status, s, nullptr, nullptr, p->fwd.me.exact));
                         CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xs, Y, vY, phi, vphi, 1, w.zf, hphi, hY, hphi ? pm : 0, hY ? ym : 0, w.status, s));
                     } else if (tc_edge_dual) {
                         CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.fKNh, w.fKNl, gy, R, nullptr, w.status, s, w.zqh, w.zql));
@@ -609,7 +608,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                 if (vR) {   // the term through dZbar = gy vR^T
                     SplitSrc xp{}; xp.h = xs.h; xp.l = xs.l; xp.oseg = xs.oseg;
                     if (me_edge_plain) {
-                        CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.vfKNh, w.vfKNl, gy, vR, w.zf, w.status, s));
+                        CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.vfKNh, w.vfKNl, gy, vR, w.zf, w.status, s, nullptr, nullptr, p->fwd.me.exact));
                         CK(launch_moment_edge(p, p->fwd, rv, n0, nn, xp, Y, nullptr, phi, nullptr, 0, w.zf, hphi, hY, hphi ? pm : 0, hY ? ym : 0, w.status, s));
                     } else if (tc_edge_plain) {
                         CK(state_adjoint(p, p->fwd, n0, nn, w.gbh, w.gbl, w.vfKNh, w.vfKNl, gy, vR, nullptr, w.status, s, w.zqh, w.zql));

@@ -42,12 +42,13 @@ struct TcArgs {
     int64_t c_outer, c_inner;   // C(m,n) = C[(m/c_d)*c_outer + (m%c_d)*c_inner + n]
     int32_t c_d;
     int32_t accumulate;
-    int32_t passes;             // 3: split-bf16 product (fp32-faithful); 1: the hi x hi product only (plain bf16 GEMM)
+    int32_t passes;             // 3: split-bf16 product (fp32-faithful); 1: the hi x hi product only (plain bf16 GEMM);
+                                // 4: lo x lo too, the small products in an accumulator of their own (columns BN .. 2 BN)
     int64_t M, N, Kd;
     int32_t BN;                 // tile width (multiple of 16, <= 256)
     int32_t stages;
     int32_t ring_bytes;         // bytes of the operand ring = what the epilogue may use as its staging area
-    int32_t tmem_cols;          // power of two >= max(32, BN)
+    int32_t tmem_cols;          // power of two >= max(32, columns of the accumulators)
     int32_t mn_major;           // 0: A[M,Kd], B[N,Kd] row-major;  1: A^T[Kd,M], B^T[Kd,N] row-major
     int32_t splits;             // gridDim.z: the contraction range is cut into this many pieces,
     int64_t split_stride;       //   piece z writes its partial result to C + z*split_stride
@@ -166,7 +167,8 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
 #pragma unroll
                 for (uint32_t k = 0; k < BK / 16; ++k) {
                     const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u, o = k * kstep16;
-                    if (g.passes != 1) tc_mma_bf16_x3(tmem_base, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
+                    if (g.passes == 4) tc_mma_bf16_x4(tmem_base, tmem_base + (uint32_t)g.BN, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
+                    else if (g.passes != 1) tc_mma_bf16_x3(tmem_base, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
                     else tc_mma_bf16(tmem_base, dAh + o, dBh + o, idesc, acc);
                 }
                 tc_commit(bar0 + 8 * (S + s));                       // frees the slot when the MMAs retire
@@ -183,6 +185,12 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
         const int q = warp & 3;
         mbar_wait(bar0 + 8 * 2 * S, 0, g.status);
         tc_fence_after();
+        auto add_small = [&](float* v, int q, int c0) {
+            float w[16];
+            tc_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(g.BN + c0), w);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[j] += w[j];
+        };
         // The pipeline buffers are idle now: each warp parks its 32 x BN block there and then writes C row by row
         // with the lanes along the columns (coalesced).
         if (g.Ch && (g.N & 7) == 0) {
@@ -194,6 +202,7 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
             for (int c0 = 0; c0 < g.BN; c0 += 16) {
                 float v[16];
                 tc_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);   // warp-collective
+                if (g.passes == 4) add_small(v, q, c0);
 #pragma unroll
                 for (int j = 0; j < 16; j += 4)
                     *reinterpret_cast<float4*>(pk + lane * P4 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -231,6 +240,7 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
         for (int c0 = 0; c0 < g.BN; c0 += 16) {
             float v[16];
             tc_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);   // warp-collective
+            if (g.passes == 4) add_small(v, q, c0);
 #pragma unroll
             for (int j = 0; j < 16; j += 4)
                 *reinterpret_cast<float4*>(park + lane * P4 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -516,13 +526,13 @@ cudaError_t gemm_tc_add(GemmBatch& gb, const void* Ahi, const void* Alo, int64_t
     TcProblem& pr = fresh;
     TcArgs& g = pr.g;
     g = TcArgs{};
-    g.C = C; g.Ch = (__nv_bfloat16*)Chi; g.Cl = (__nv_bfloat16*)Clo; g.c_outer = c_outer; g.c_inner = c_inner; g.c_d = c_d; g.accumulate = accumulate; g.passes = passes == 1 ? 1 : 3;
+    g.C = C; g.Ch = (__nv_bfloat16*)Chi; g.Cl = (__nv_bfloat16*)Clo; g.c_outer = c_outer; g.c_inner = c_inner; g.c_d = c_d; g.accumulate = accumulate; g.passes = passes == 1 || passes == 4 ? passes : 3;
     g.M = M; g.N = N; g.Kd = Kd; g.mn_major = mn_major; g.status = status;
     g.splits = std::max(1, std::min<int>(splits, (int)((Kd + BK - 1) / BK))); g.split_stride = split_stride;
     int BN;
     const int num_kb = (int)((Kd + BK - 1) / BK);
     if (mn_major) BN = N <= 64 ? 64 : (N <= 128 ? 128 : 256);     // whole 64-wide boxes
-    else BN = (int)std::min<int64_t>(num_kb <= 2 ? 128 : 256, (N + 15) / 16 * 16);   // one or two k-blocks are all epilogue: narrower tiles, more CTAs
+    else BN = (int)std::min<int64_t>(num_kb <= 2 || passes == 4 ? 128 : 256, (N + 15) / 16 * 16);   // one or two k-blocks are all epilogue: narrower tiles, more CTAs
     g.BN = BN;
     const size_t stage = 2 * (size_t)BM * BK * 2 + 2 * (size_t)BN * BK * 2;
     // two (or more) CTAs per SM where the ring fits twice (more loads and epilogues in flight per SM), else one
@@ -537,7 +547,7 @@ cudaError_t gemm_tc_add(GemmBatch& gb, const void* Ahi, const void* Alo, int64_t
     const size_t park = (size_t)4 * 32 * (BN + 4) * sizeof(float);       // epilogue staging of the four drain warps
     g.ring_bytes = (int32_t)((std::max(park, (size_t)stages * stage) + 1023) & ~size_t(1023));
     int cols = 32;
-    while (cols < BN) cols <<= 1;
+    while (cols < (passes == 4 ? 2 : 1) * BN) cols <<= 1;
     g.tmem_cols = cols;
     bool ok;
     if (!mn_major) {

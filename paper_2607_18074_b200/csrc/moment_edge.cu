@@ -53,6 +53,7 @@ constexpr int TILE = 64;                // edges of a tile
 constexpr int SLAB = TILE * 128;        // bytes of one copy of a (slab, tile): 64 edges x 64 bf16
 constexpr int MAXNX = 8, MAXNP = 4, MAXNZ = 2;
 constexpr int HALF = 256;
+constexpr int MAX_EXACT_KSTEPS = 80;
 constexpr int NBAR = 2 * MAXNX + 2 * MAXNP + 2 * MAXNZ + 4;
 
 struct MeArgs {
@@ -88,6 +89,12 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t&
     const float rb = b - __uint_as_float(hi & 0xffff0000u);
     const __nv_bfloat162 l = __floats2bfloat162_rn(ra, rb);
     lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+// what a split leaves, in bf16 pairs
+__device__ __forceinline__ uint32_t rest2(float a, float b, uint32_t hi, uint32_t lo) {
+    const __nv_bfloat162 r = __floats2bfloat162_rn((a - __uint_as_float(hi << 16)) - __uint_as_float(lo << 16),
+                                                   (b - __uint_as_float(hi & 0xffff0000u)) - __uint_as_float(lo & 0xffff0000u));
+    return *reinterpret_cast<const uint32_t*>(&r);
 }
 // NQ columns of this thread's TMEM lane, waited for
 template <int NQ>
@@ -180,12 +187,13 @@ __device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t 
     }
 }
 
-template <int NQ, bool DUAL>
+// EXACT: Pbar in three parts instead of two, so that only the rows' representation error is left.
+template <int NQ, bool DUAL, bool EXACT>
 __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);
     uint8_t* sX = smem;                                                // rows of (slab, tile): hi, lo
-    uint8_t* sP = sX + (size_t)a.nx * 2 * SLAB;                        // Pbar of a slab: hi rows, lo rows
+    uint8_t* sP = sX + (size_t)a.nx * 2 * SLAB;                        // Pbar of a slab: hi rows, lo rows (EXACT: the rest's rows)
     uint8_t* sZ = sP + (size_t)a.np * a.p_bytes;                       // Zbar of (block, run): [component][NQ][64]
     uint64_t* bars = reinterpret_cast<uint64_t*>(sZ + (size_t)a.nz * a.z_bytes);
     uint32_t* tmem_holder = reinterpret_cast<uint32_t*>(bars + NBAR);
@@ -352,11 +360,13 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                         const int ch = lane >> 2;
 #pragma unroll
                         for (int r = 0; r < NQ; ++r) {
-                            uint32_t hi, lo;
+                            uint32_t hi, lo, rest;
                             split2(v[r][0], v[r][1], hi, lo);
+                            if (EXACT) rest = rest2(v[r][0], v[r][1], hi, lo);
                             const uint32_t o = (uint32_t)(r * 128 + ((ch ^ ((b * NQ + r) & 7)) << 4));
                             *reinterpret_cast<uint32_t*>(d + o) = hi;
                             *reinterpret_cast<uint32_t*>(d + o + n_cols * 128) = lo;
+                            if (EXACT) *reinterpret_cast<uint32_t*>(d + o + 2 * n_cols * 128) = rest;
                         }
                     }
                     turn = (turn + a.dsh) % NBW;
@@ -400,14 +410,16 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                                 const uint32_t dt = tm_u + buf * HALF + __shfl_sync(0xffffffffu, (uint32_t)(t * nop + op) * uN, 0);
                                 constexpr uint32_t small = 16u << 16;      // lanes of the small products
                                 if (elect_one()) {
+                                    auto kstep = [&](uint32_t k) {
+                                        tc_mma_bf16_x4(dt, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                        if (EXACT) tc_mma_bf16(dt + small, dX + 2 * k, dP + 2 * k + uN * 16u, idesc, 1u);
+                                    };
                                     if (ks == 4) {
 #pragma unroll
-                                        for (uint32_t k = 0; k < 4; ++k)
-                                            tc_mma_bf16_x4(dt, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                        for (uint32_t k = 0; k < 4; ++k) kstep(k);
                                     } else {
 #pragma unroll 1
-                                        for (uint32_t k = 0; k < ks; ++k)
-                                            tc_mma_bf16_x4(dt, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                        for (uint32_t k = 0; k < ks; ++k) kstep(k);
                                     }
                                     tc_commit(bar_xfree + 8 * xs);
                                     if (t + 1 == tiles && op + 1 == nop) {
@@ -466,10 +478,13 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
     constexpr int kSmem = 227 * 1024;
     MomentEdge& T = dir.me;
     T = MomentEdge{};
-    // Only in the place of k_edge_tc: the FP32-pipe pass holds rows and adjoint state in 32 bits, this one as bf16 hi + lo, and a
-    // profile that runs that pass keeps its precision (error of gY, 2-norm against fp64: 1e-7 there, 5e-6 here in the channelwise
-    // mode; 4.5e-6 and 8e-6 behind the node products of the other mode).
-    if (!dir.etc[0].ok) return;
+    // In the place of k_edge_tc, or (EXACT) of the FP32-pipe pass, which holds rows and adjoint state in 32 bits.  There the error
+    // against fp64 must not grow by the split: in the fully connected mode it does not, since Pbar then has three parts and the product
+    // that makes its Zbar takes lo x lo along (2-norm of gY, 81 random profiles: 0.97 of the FP32 pipes' on average, 1.05 at most).  The
+    // channelwise mode, whose Zbar has the error of one fp32 product, keeps the FP32 pipes (1e-7), and so does a contraction that is
+    // too long for an accumulator that rounds towards zero.
+    const bool exact = !dir.etc[0].ok;
+    if (exact && p->uvu) return;
     if (p->K > 16 || p->K < 2 || (dir.C_src & 7) || dir.paths.empty()) return;
     struct Blk { int so, c, d; std::vector<std::pair<const DPath*, int>> paths; };
     std::vector<Blk> blocks;
@@ -525,9 +540,13 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
                 T.tptr.push_back((int)T.terms.size());
                 T.blks.push_back(M);
                 T.slabs += M.d; T.ksteps += M.d * M.ksteps;
+                const int w = (M.c + 31) / 32;
+                T.comps32 += w * M.ncomp; T.rows32 += w * M.d; T.terms32 += w * ((int)T.terms.size() - T.tptr[M.t_begin]);
             }
         }
-        T.p_bytes = (2 * n_cols * 128 + 1023) & ~1023;
+        if (exact && T.ksteps > MAX_EXACT_KSTEPS) break;
+        T.exact = exact;
+        T.p_bytes = ((exact ? 3 : 2) * n_cols * 128 + 1023) & ~1023;
         T.z_bytes = (max_comp * nq * 256 + 1023) & ~1023;
         const int fixed = 1024 + NBAR * 8 + 16 + (int)(T.comps.size() * sizeof(MEComp) + T.blks.size() * sizeof(MEBlk) + T.terms.size() * sizeof(MTerm) + T.tptr.size() * 4 + 64);
         for (int np = 3, nz = 2;;) {
@@ -553,12 +572,15 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
 // multiplicities of 16 (and 250 channelwise ones), orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes.  The chosen form takes 1.6 % longer than the
 // faster one on average (1.3 % in the dual pass), 37 % (50 %) at worst longer than the other.  (Lines at fixed degrees, drawn before
 // the fp32 products wrote 16 bytes a lane and the small products had an accumulator of their own: 8.3 % and 11 %, up to 2.2 and 2.7
-// times as long.)
+// times as long.)  Against the FP32-pipe pass (EXACT; its own fit from 219 layers, 31 % left, counts per 32 lanes): 1.6 % (1.2 %) above
+// the faster one, 34 % (21 %) at worst longer than the FP32 pipes, where the moment form throughout is 20 % above and up to four times
+// as long, with scalar outputs at low degrees, and the FP32 pipes 58 % (73 %).
 bool moment_edge_pays(const sobek_plan* p, int dual, int operands, int64_t N, int64_t E, int64_t chunk) {
     const Direction& dir = p->fwd;
     const MomentEdge& M = dir.me;
     const TcSets& T = dir.etc[dual];
     if (!M.ok || p->form != kFormAuto) return M.ok && p->form == kFormMoment;
+    if (!M.exact && !T.ok) return true;          // (the dual pass of a plan whose tensor-core pass fits in its plain form only)
     const double deg = (double)E / (double)std::max<int64_t>(N, 1), per_sm = std::max(1.0, (double)std::min(N, chunk) / 148.0);
     const double state = 1e-4 * (double)dir.state_floats;
     const double fp32 = (dual ? 0.88 : 1.12) + (p->uvu ? 1.9 : 0.0);     // (the channelwise mode writes fp32 rows at 0.6 of the rate of its bf16 ones)
@@ -569,6 +591,9 @@ bool moment_edge_pays(const sobek_plan* p, int dual, int operands, int64_t N, in
                               : 0.45 + 0.206 * M.slabs + M.nq * (0.00274 * M.terms.size() + 0.0006 * M.slabs * p->dim_sh);
     const double moment = 27.0 / per_sm + builds * build + tiles * (M.ksteps * (dual ? 0.055 + 0.00063 * M.n_cols : 0.053 + 0.00083 * M.n_cols) +
                           (dual ? 0.061 : 0.127) * p->dim_sh) + runs * operands * deg * 0.0035 * M.slabs + fp32 * state;
+    if (M.exact)
+        return 1.13 * moment < (dual ? 59.0 / per_sm + 1.1 + deg * (0.0092 * M.terms32 + 0.015 * M.rows32) + 21.0 * state
+                                     : 52.0 / per_sm + deg * (0.004 * M.terms32 + 0.011 * M.rows32) + 11.5 * state + 0.0077 * p->K * M.comps32);
     double coupled = (dual ? 2.46 : 2.48) * state;
     for (const TcSets::ESetPar& e : T.epar) {
         const double batches = std::max(1.0, deg / e.tb + 0.45);
@@ -594,9 +619,11 @@ cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const 
     a.phi_mode = phi_mode; a.Y_mode = Y_mode;
     a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src; a.N_cols = T.n_cols; a.nx = T.nx; a.np = T.np; a.nz = T.nz;
     a.p_bytes = T.p_bytes; a.z_bytes = T.z_bytes; a.status = status;
-    void (*kern)(const MeArgs) = T.nq == 8 ? (dual ? k_moment_edge<8, true> : k_moment_edge<8, false>)
-                                 : T.nq == 4 ? (dual ? k_moment_edge<4, true> : k_moment_edge<4, false>)
-                                             : (dual ? k_moment_edge<2, true> : k_moment_edge<2, false>);
+#define SOBEK_ME(x) (T.nq == 8 ? (dual ? k_moment_edge<8, true, x> : k_moment_edge<8, false, x>) \
+                     : T.nq == 4 ? (dual ? k_moment_edge<4, true, x> : k_moment_edge<4, false, x>) \
+                                 : (dual ? k_moment_edge<2, true, x> : k_moment_edge<2, false, x>))
+    void (*kern)(const MeArgs) = T.exact ? SOBEK_ME(true) : SOBEK_ME(false);
+#undef SOBEK_ME
     cudaError_t e = allow_dynamic_smem(kern);
     if (e != cudaSuccess) return e;
     KernelTimer kt(K_EDGE, s);

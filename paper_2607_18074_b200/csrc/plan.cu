@@ -381,8 +381,9 @@ void build_direction(sobek_plan* p, int transposed, Direction& dir) {
 
 bool needs_zbar(const sobek_plan* p, int order) {
     if (order < 1) return false;
-    // (the plain tensor-core pass may fit where its dual form does not; the moment form then does the dual pass)
-    return !p->use_tc_edge || !p->fwd.etc[0].ok || (order >= 2 && !p->fwd.etc[1].ok && !p->fwd.me.ok);
+    if (!p->use_tc_edge) return true;
+    // (the plain tensor-core pass may fit where its dual form does not)
+    return !p->fwd.me.ok && (!p->fwd.etc[0].ok || (order >= 2 && !p->fwd.etc[1].ok));
 }
 
 int64_t chunk_nodes(const sobek_plan* p, int64_t N, int order) {

@@ -110,7 +110,7 @@ def test_both_forms(ir_in, ir_out, l_max, K, N, deg):
     got = [[k.fwd()] + k.bwd() + k.dbwd() for k in (c, o)]
     # (no output block above 128: the sender-owned streams exist on the tensor cores as well)
     both = ["y", "gR", "ggy", "hR"] + (["gx", "hx"] if max(m for m, _, _ in w.irreps_out) <= 128 else [])
-    if K > 1 and all(m % 16 == 0 for m, _, _ in w.irreps_in):
+    if K > 1:       # (without the coupled form off the 16s: the FP32-pipe pass beside the moment form)
         both += ["gY", "gphi", "hY", "hphi"]
     for a, b, ref, nm in zip(*got, refs, names):
         tol = FWD_TOL if nm == "y" else BWD_TOL
@@ -135,9 +135,10 @@ def test_stream_takes_the_form_that_pays(ir_in, ir_out, l_max, K, N, deg, output
 
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg,dual,form", [
     ("64x0e+64x1o+64x2e", "64x0e+64x1o+64x2e", 2, 8, 1500, 10, 0, "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 16, 200, 60, 0, "moment"),
-    ("96x1o+96x2e+96x3o", "96x0e", 3, 10, 160, 70, 1, "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 16, 200, 60, 1, "moment")])
+    ("8x0e+8x1o+8x2e", "8x0e", 2, 10, 1500, 8, 0, "coupled"), ("8x0e+8x1o", "8x0e+8x1o", 2, 8, 64, 17, 0, "moment"),
+    ("96x1o+96x2e+96x3o", "96x0e", 3, 10, 160, 70, 1, "coupled"), ("24x0e+24x1o", "24x0e+24x1o+24x2e", 2, 16, 300, 30, 1, "moment"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 16, 200, 60, 1, "moment")])
 def test_edge_pass_takes_the_form_that_pays(ir_in, ir_out, l_max, K, N, deg, dual, form):
-    """The same for the edge pass, plain and dual."""
+    """The same for the edge pass, plain and dual; off the 16s "coupled" leaves the FP32-pipe pass."""
     L = 4.0 * (N / 60.0) ** (1 / 3)
     w = synth.Workload("pays", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=33)
     c = Case(w)
@@ -173,20 +174,25 @@ def test_double_backward_where_only_the_plain_edge_pass_fits(ir_in, ir_out, l_ma
             assert rel_err(got, ref) <= BWD_TOL if np.abs(ref).max() > 0 else np.all(got == 0), (dirs, nm)
 
 
-@pytest.mark.parametrize("mode,irreps", [("uvu", "24x0e+24x1o+24x2e"), ("uvw", "8x0e+24x1o"), ("uvw", "144x0e+16x1o")])
-def test_edge_outputs_keep_32_bits_off_the_16s(mode, irreps):
-    """Multiplicities that are no multiples of 16, or above 128: the edge pass runs on the FP32 pipes by default, and its outputs are
-    those of a plan that asks for it.  In the channelwise mode, whose adjoint state is plain fp32 products, their error is that of
-    32-bit sums: some hundred terms of both signs, 2^-24 each, bounded by 1e-6 of the largest output."""
+@pytest.mark.parametrize("mode,irreps,l_max,K", [("uvu", "24x0e+24x1o+24x2e", 2, 8), ("uvw", "8x0e+24x1o", 2, 8), ("uvw", "144x0e+16x1o", 2, 16),
+                                                 ("uvw", "8x0e+40x1o+24x2e+40x3o", 3, 10), ("uvw", "40x0e+40x1o+40x2e+40x3o+40x4e", 4, 4),
+                                                 ("uvw", "24x0e+8x1o+24x2e+8x4e", 4, 16)])
+def test_edge_outputs_off_the_16s_are_as_exact_as_the_fp32_pipes(mode, irreps, l_max, K):
+    """Multiplicities that are no multiples of 16, or above 128, for which the edge pass with the coupling in its epilogue does not exist:
+    the moment form is no further from fp64 than the FP32-pipe pass (5 % for the spread of a small graph).  In the channelwise mode,
+    whose adjoint state is plain fp32 products, that pass runs, with the error of 32-bit sums: some hundred terms of both signs, 2^-24
+    each, bounded by 1e-6 of the largest output."""
     ir = P(irreps)
-    w = synth.Workload("keep32", ir, ir, 2, 8, 60, 4.0, 2.8, "bessel", seed=25, mode=mode)
-    c = Case(w)
+    w = synth.Workload("keep32", ir, ir, l_max, K, 40, 4.0, 2.8, "bessel", seed=25, mode=mode)
+    c = Case(w, form="moment")
     f = Case(w, inputs=c.d, tc_edge=False)
-    for a, b in zip(c.bwd()[1:3] + c.dbwd()[2:4], f.bwd()[1:3] + f.dbwd()[2:4]):
-        assert np.array_equal(a, b)
-    if mode == "uvu":
-        for got, ref in zip(c.bwd()[1:3] + c.dbwd()[2:4], c.o_bwd()[1:3] + c.o_dbwd()[2:4]):
-            assert rel_err(got, ref) <= 1e-6
+    norm2 = lambda got, ref: np.linalg.norm(got - ref) / np.linalg.norm(ref)
+    refs = list(c.o_bwd()[1:3]) + list(c.o_dbwd()[2:4])
+    for a, b, ref in zip(c.bwd()[1:3] + c.dbwd()[2:4], f.bwd()[1:3] + f.dbwd()[2:4], refs):
+        if mode == "uvu":
+            assert np.array_equal(a, b) and rel_err(a, ref) <= 1e-6
+        else:
+            assert not np.array_equal(a, b) and norm2(a, ref) <= 1.05 * norm2(b, ref)
 
 
 def test_streams_keep_32_bits_above_128():
