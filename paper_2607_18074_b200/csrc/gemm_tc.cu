@@ -167,7 +167,7 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
 #pragma unroll
                 for (uint32_t k = 0; k < BK / 16; ++k) {
                     const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u, o = k * kstep16;
-                    if (g.passes == 4) tc_mma_bf16_x4(tmem_base, tmem_base + (uint32_t)g.BN, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
+                    if (g.passes == 4) tc_mma_bf16_x4(tmem_base, tmem_base + (uint32_t)g.BN, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc, acc);
                     else if (g.passes != 1) tc_mma_bf16_x3(tmem_base, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
                     else tc_mma_bf16(tmem_base, dAh + o, dBh + o, idesc, acc);
                 }

@@ -239,6 +239,7 @@ struct MomentEdge {
     int32_t nq = 0, n_cols = 0, nx = 0, np = 0, nz = 0, p_bytes = 0, z_bytes = 0, smem_bytes = 0;
     int32_t slabs = 0, ksteps = 0;    // of all blocks
     int32_t comps32 = 0, rows32 = 0, terms32 = 0;      // state components, row components, coupling terms, each per 32 multiplicities
+    int32_t nacc = 1;                 // accumulators of the hi x hi products
     bool exact = false;               // in the place of the FP32-pipe pass: Pbar in three parts, four products in the one that makes Zbar
 };
 

@@ -53,7 +53,8 @@ constexpr int TILE = 64;                // edges of a tile
 constexpr int SLAB = TILE * 128;        // bytes of one copy of a (slab, tile): 64 edges x 64 bf16
 constexpr int MAXNX = 8, MAXNP = 4, MAXNZ = 2;
 constexpr int HALF = 256;
-constexpr int MAX_EXACT_KSTEPS = 80;
+constexpr int ACC_KSTEPS = 80;          // EXACT: k-steps that one accumulator takes (its rounding stays below the rows' representation error)
+constexpr int SET2 = HALF / 2;          // EXACT with more of them: first column of the accumulators of the second and the third run of k-steps
 constexpr int NBAR = 2 * MAXNX + 2 * MAXNP + 2 * MAXNZ + 4;
 
 struct MeArgs {
@@ -72,6 +73,7 @@ struct MeArgs {
     float *gphi, *gY;
     int32_t phi_mode, Y_mode;   // 0 skip, 1 overwrite, 2 accumulate
     int32_t K, dsh, C_src, N_cols, nx, np, nz, p_bytes, z_bytes;
+    int32_t nacc, acc_ksteps;   // EXACT: accumulators of the hi x hi products, k-steps of each
     int* status;
 };
 
@@ -133,7 +135,7 @@ struct Walk {
 };
 
 // The two sums of one run of radial indices for the edge of this thread and of lane ^ 16, which has the other accumulator.
-template <int NQ, bool DUAL>
+template <int NQ, bool DUAL, bool EXACT>
 __device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t tv, int64_t e, bool ok, int part, int q0, bool first_run, bool has_vx) {
     float f[NQ], vf[NQ], gp[NQ];
     const bool has_vY = DUAL && a.vY, has_vphi = DUAL && a.vphi;
@@ -148,11 +150,20 @@ __device__ __forceinline__ void edge_sums(const MeArgs& a, uint32_t t, uint32_t 
     for (int b = 0; b < a.dsh; ++b) {
         const float y = ok ? __ldg(a.Y + e * a.dsh + b) : 0.f, vy = ok && has_vY ? __ldg(a.vY + e * a.dsh + b) : 0.f;
         float g[NQ], gv[NQ];
-        tm_read<NQ>(t + (uint32_t)(b * NQ), g);
+        auto read = [&](uint32_t at, float* v) {
+            tm_read<NQ>(at, v);
+            if (EXACT && a.nacc > 1) {         // the second accumulator beside the first, the third (if any) beside the small products
+                float w[NQ];
+                tm_read<NQ>(at + SET2, w);
+#pragma unroll
+                for (int r = 0; r < NQ; ++r) v[r] += part == 0 || a.nacc > 2 ? w[r] : 0.f;
+            }
+        };
+        read(t + (uint32_t)(b * NQ), g);
         float gy = 0.f;
         if (DUAL) {
             if (has_vx) {
-                tm_read<NQ>(tv + (uint32_t)(b * NQ), gv);
+                read(tv + (uint32_t)(b * NQ), gv);
             } else {
 #pragma unroll
                 for (int r = 0; r < NQ; ++r) gv[r] = 0.f;
@@ -209,7 +220,7 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
     const bool has_vx = DUAL && a.vsh != nullptr;
     const int nop = has_vx ? 2 : 1;                                    // operands: rows of x, of vx
     const int n_cols = a.N_cols, runs = (a.K + NQ - 1) / NQ;
-    const int pass_tiles = HALF / (n_cols * nop);                      // tiles that one TMEM half holds
+    const int pass_tiles = (EXACT && a.nacc > 1 ? SET2 : HALF) / (n_cols * nop);      // tiles that one TMEM half holds
     if (tid == 0) {
         for (int s = 0; s < MAXNX; ++s) { mbar_init(bar_xfull + 8 * s, 32); mbar_init(bar_xfree + 8 * s, 1); }
         for (int s = 0; s < MAXNP; ++s) { mbar_init(bar_pfull + 8 * s, NBW * 32); mbar_init(bar_pfree + 8 * s, 1); }
@@ -394,6 +405,7 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                     const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0);
                     if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
                     tc_fence_after();
+                    int k_acc = 0, i_acc = 0;          // EXACT: k-steps in the accumulator at hand, its number
                     for (int bi = 0; bi < a.n_blks; ++bi) {
                         const int d = sBlk[bi].d;
                         const uint32_t ks = __shfl_sync(0xffffffffu, (uint32_t)sBlk[bi].ksteps, 0);
@@ -401,6 +413,13 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                             mbar_spin(bar_pfull + 8 * ps, pr & 1, a.status);
                             const uint64_t dP = dP0 + __shfl_sync(0xffffffffu, (uint32_t)ps * ((uint32_t)a.p_bytes >> 4), 0);
                             const uint32_t acc = __shfl_sync(0xffffffffu, bi + s > 0 ? 1u : 0u, 0);
+                            uint32_t acc_d = acc, main = 0;
+                            if (EXACT) {
+                                if (k_acc >= a.acc_ksteps && i_acc + 1 < a.nacc) { ++i_acc; k_acc = 0; }
+                                acc_d = __shfl_sync(0xffffffffu, k_acc > 0 ? 1u : 0u, 0);
+                                main = __shfl_sync(0xffffffffu, i_acc == 0 ? 0u : SET2 + (i_acc == 2 ? 16u << 16 : 0u), 0);
+                                k_acc += (int)ks;
+                            }
                             for (int t = 0; t < tiles; ++t)
                             for (int op = 0; op < nop; ++op) {
                                 mbar_spin(bar_xfull + 8 * xs, xr & 1, a.status);
@@ -411,7 +430,8 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                                 constexpr uint32_t small = 16u << 16;      // lanes of the small products
                                 if (elect_one()) {
                                     auto kstep = [&](uint32_t k) {
-                                        tc_mma_bf16_x4(dt, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc, k > 0 ? 1u : acc);
+                                        tc_mma_bf16_x4(dt + main, dt + small, dX + 2 * k, dX + 2 * k + (SLAB >> 4), dP + 2 * k, dP + 2 * k + uN * 8u, idesc,
+                                                       k > 0 ? 1u : acc_d, k > 0 ? 1u : acc);
                                         if (EXACT) tc_mma_bf16(dt + small, dX + 2 * k, dP + 2 * k + uN * 16u, idesc, 1u);
                                     };
                                     if (ks == 4) {
@@ -453,7 +473,7 @@ __global__ void __launch_bounds__(TT, 1) k_moment_edge(const MeArgs a) {
                         const bool ok = le < plen;
                         if (!__any_sync(0xffffffffu, ok)) continue;
                         const uint32_t td = tmem_base + ((uint32_t)(warp * 32) << 16) + buf * HALF + (uint32_t)(t * nop * n_cols);
-                        edge_sums<NQ, DUAL>(a, td, td + (uint32_t)n_cols, seg0 + p0 + (ok ? le : 0), ok, lane >> 4, run * NQ, run == 0, has_vx);
+                        edge_sums<NQ, DUAL, EXACT>(a, td, td + (uint32_t)n_cols, seg0 + p0 + (ok ? le : 0), ok, lane >> 4, run * NQ, run == 0, has_vx);
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -482,7 +502,7 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
     // against fp64 must not grow by the split: in the fully connected mode it does not, since Pbar then has three parts and the product
     // that makes its Zbar takes lo x lo along (2-norm of gY, 81 random profiles: 0.97 of the FP32 pipes' on average, 1.05 at most).  The
     // channelwise mode, whose Zbar has the error of one fp32 product, keeps the FP32 pipes (1e-7), and so does a contraction that is
-    // too long for an accumulator that rounds towards zero.
+    // too long for three accumulators (they round towards zero, a little with every k-step).
     const bool exact = !dir.etc[0].ok;
     if (exact && p->uvu) return;
     if (p->K > 16 || p->K < 2 || (dir.C_src & 7) || dir.paths.empty()) return;
@@ -544,8 +564,10 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
                 T.comps32 += w * M.ncomp; T.rows32 += w * M.d; T.terms32 += w * ((int)T.terms.size() - T.tptr[M.t_begin]);
             }
         }
-        if (exact && T.ksteps > MAX_EXACT_KSTEPS) break;
         T.exact = exact;
+        T.nacc = exact ? (T.ksteps + ACC_KSTEPS - 1) / ACC_KSTEPS : 1;
+        if (T.nacc > 3) break;
+        if (T.nacc > 1 && 2 * n_cols > SET2) continue;
         T.p_bytes = ((exact ? 3 : 2) * n_cols * 128 + 1023) & ~1023;
         T.z_bytes = (max_comp * nq * 256 + 1023) & ~1023;
         const int fixed = 1024 + NBAR * 8 + 16 + (int)(T.comps.size() * sizeof(MEComp) + T.blks.size() * sizeof(MEBlk) + T.terms.size() * sizeof(MTerm) + T.tptr.size() * 4 + 64);
@@ -584,7 +606,7 @@ bool moment_edge_pays(const sobek_plan* p, int dual, int operands, int64_t N, in
     const double deg = (double)E / (double)std::max<int64_t>(N, 1), per_sm = std::max(1.0, (double)std::min(N, chunk) / 148.0);
     const double state = 1e-4 * (double)dir.state_floats;
     const double fp32 = (dual ? 0.88 : 1.12) + (p->uvu ? 1.9 : 0.0);     // (the channelwise mode writes fp32 rows at 0.6 of the rate of its bf16 ones)
-    const double runs = (p->K + M.nq - 1) / M.nq, cap = TILE * (HALF / (M.n_cols * operands));           // edges of a pass
+    const double runs = (p->K + M.nq - 1) / M.nq, cap = TILE * ((M.nacc > 1 ? SET2 : HALF) / (M.n_cols * operands));      // edges of a pass
     const double builds = runs * (deg > 0.6 * cap ? std::max(1.0, deg / cap + 0.4) : 1.0);
     const double tiles = runs * (deg > 40 ? deg / TILE + 0.5 : 1.0) * operands;
     const double build = dual ? 0.88 + 0.364 * M.slabs + M.nq * (0.00135 * M.terms.size() + 0.00154 * M.slabs * p->dim_sh)
@@ -618,6 +640,7 @@ cudaError_t launch_moment_edge(const sobek_plan* p, const Direction& dir, const 
     a.Y = Y; a.vY = vY; a.phi = phi; a.vphi = vphi; a.zbar = zbar; a.gphi = gphi; a.gY = gY;
     a.phi_mode = phi_mode; a.Y_mode = Y_mode;
     a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src; a.N_cols = T.n_cols; a.nx = T.nx; a.np = T.np; a.nz = T.nz;
+    a.nacc = T.nacc; a.acc_ksteps = (T.ksteps + T.nacc - 1) / T.nacc;
     a.p_bytes = T.p_bytes; a.z_bytes = T.z_bytes; a.status = status;
 #define SOBEK_ME(x) (T.nq == 8 ? (dual ? k_moment_edge<8, true, x> : k_moment_edge<8, false, x>) \
                      : T.nq == 4 ? (dual ? k_moment_edge<4, true, x> : k_moment_edge<4, false, x>) \

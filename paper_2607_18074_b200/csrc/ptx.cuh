@@ -121,16 +121,17 @@ __device__ __forceinline__ void tc_mma_bf16_x3(uint32_t tmem_d, uint64_t da_hi, 
 // accumulation in tensor memory rounds towards zero, by up to an ulp of the accumulator whatever is added: the small products, which
 // are most of the additions, round a small accumulator here.
 __device__ __forceinline__ void tc_mma_bf16_x4(uint32_t tmem_d, uint32_t tmem_s, uint64_t da_hi, uint64_t da_lo, uint64_t db_hi, uint64_t db_lo,
-                                               uint32_t idesc, uint32_t acc) {
+                                               uint32_t idesc, uint32_t acc_d, uint32_t acc_s) {
     asm volatile(
-        "{\n\t.reg .pred p, t;\n\t"
+        "{\n\t.reg .pred p, s, t;\n\t"
         "setp.ne.b32 p, %7, 0;\n\t"
+        "setp.ne.b32 s, %8, 0;\n\t"
         "setp.eq.u32 t, 0, 0;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16 [%0], %2, %4, %6, p;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%1], %2, %5, %6, p;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%1], %2, %5, %6, s;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%1], %3, %4, %6, t;\n\t"
         "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], %3, %5, %6, t;\n\t}"
-        ::"r"(tmem_d), "r"(tmem_s), "l"(da_hi), "l"(da_lo), "l"(db_hi), "l"(db_lo), "r"(idesc), "r"(acc) : "memory");
+        ::"r"(tmem_d), "r"(tmem_s), "l"(da_hi), "l"(da_lo), "l"(db_hi), "l"(db_lo), "r"(idesc), "r"(acc_d), "r"(acc_s) : "memory");
 }
 // eight consecutive 32-bit columns of this thread's TMEM lane (lane = 32 * (warp % 4) + lane id)
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* r) {

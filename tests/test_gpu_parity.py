@@ -176,6 +176,7 @@ def test_double_backward_where_only_the_plain_edge_pass_fits(ir_in, ir_out, l_ma
 
 @pytest.mark.parametrize("mode,irreps,l_max,K", [("uvu", "24x0e+24x1o+24x2e", 2, 8), ("uvw", "8x0e+24x1o", 2, 8), ("uvw", "144x0e+16x1o", 2, 16),
                                                  ("uvw", "8x0e+40x1o+24x2e+40x3o", 3, 10), ("uvw", "40x0e+40x1o+40x2e+40x3o+40x4e", 4, 4),
+                                                 ("uvw", "96x0e+96x1o+96x2e+96x3o+96x4e", 4, 3), ("uvw", "104x1o+104x2e+104x3o+104x4e", 4, 5),
                                                  ("uvw", "24x0e+8x1o+24x2e+8x4e", 4, 16)])
 def test_edge_outputs_off_the_16s_are_as_exact_as_the_fp32_pipes(mode, irreps, l_max, K):
     """Multiplicities that are no multiples of 16, or above 128, for which the edge pass with the coupling in its epilogue does not exist:
