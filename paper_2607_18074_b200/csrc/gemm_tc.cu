@@ -414,20 +414,28 @@ __global__ void k_reduce_ranges(float* __restrict__ dst, const float* __restrict
 }  // namespace
 
 namespace {
-// Self-test of the bounded wait: one thread waits on an mbarrier that nothing ever completes; the wait gives up after
-// `limit_ns`, records SOBEK_ERR_DEVICE_TIMEOUT in the status word and the kernel returns normally.
+// Self-test of the bounded waits: one thread of two warps each waits on an mbarrier that nothing ever completes, one with the wait
+// that suspends, the other with the one that spins; each gives up after `limit_ns` and records SOBEK_ERR_DEVICE_TIMEOUT in a word of
+// its own.  If both did, so does the status word, and the kernel returns normally.
 __global__ void k_wait_selftest(int* status, uint64_t limit_ns) {
     __shared__ uint64_t bar;
+    __shared__ int word[2];
+    if (threadIdx.x < 2) word[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        mbar_wait(smem_u32(&bar), 0, status, limit_ns);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) mbar_wait(smem_u32(&bar), 0, word, limit_ns);
+    if (threadIdx.x == 32) mbar_spin(smem_u32(&bar), 0, word + 1, limit_ns);
+    __syncthreads();
+    if (threadIdx.x == 0 && word[0] == (int)SOBEK_ERR_DEVICE_TIMEOUT && word[1] == (int)SOBEK_ERR_DEVICE_TIMEOUT)
+        atomicExch(status, (int)SOBEK_ERR_DEVICE_TIMEOUT);
 }
 }  // namespace
 
 cudaError_t launch_wait_selftest(int* status, uint64_t limit_ns, cudaStream_t s) {
-    k_wait_selftest<<<1, 32, 0, s>>>(status, limit_ns);
+    k_wait_selftest<<<1, 64, 0, s>>>(status, limit_ns);
     count_launch();
     return cudaGetLastError();
 }
