@@ -64,7 +64,7 @@ cudaError_t launch_stream(const sobek_plan* p, const Direction& dir, const EdgeV
     // tensor-core stream when the profile allows it and the caller made the bf16 copies of the sources
     if (p->use_tc_stream && status && ss.h && ss.l && (!vsrc || (ss.vh && ss.vl))) {
         const int operands = dual && ss.vh && (ss.rvec ? ss.vrvec != nullptr : vY || vphi) ? 2 : 1;
-        if (moment_stream_pays(p, dir, dual ? 1 : 0, operands, ev.N, ev.E))
+        if (moment_stream_pays(p, dir, dual ? 1 : 0, operands, ss.rvec != nullptr, ev.N, ev.E))
             return launch_moment_stream(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
         if (dir.tc[dual ? 1 : 0].ok) return launch_stream_tc(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
     }

@@ -475,8 +475,8 @@ cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const Ed
 // --- moment_stream.cu -------------------------------------------------------------------
 void build_stream_sets(const sobek_plan* p, Direction& dir);
 // the moment form is taken for a stream over a graph of N nodes and E edges (operands: 2 in a dual stream with a source direction and
-// a direction of Y or phi, else 1)
-bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, int64_t N, int64_t E);
+// a direction of Y or phi, else 1; geo: Y and phi computed from edge vectors)
+bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, bool geo, int64_t N, int64_t E);
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
                                  const SplitSrc& ss, const float* Y, const float* vY, const float* phi, const float* vphi, int dual,
                                  void* zh, void* zl, int* status, cudaStream_t s);

@@ -64,13 +64,21 @@ static void stream_costs(Direction& dir, int dual) {
     M.slot_again_us = c + w * w_again + r * rows_again;                                      // rows and W anew for every unit
 }
 
-bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, int64_t N, int64_t E) {
+// With the edge inputs computed from vectors (geo) one warp of either kernel makes the rows of every slot, 1.7 us for 16 edges, and the
+// moment form needs them again for every unit of a node that is not resident.  (250 random layers, both directions: 1.5 % above the
+// faster form, at worst 1.2 times the coupled one; without it 2.0 %, 1.9 times, at degrees from 150 on.)
+bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, bool geo, int64_t N, int64_t E) {
     const TcSets& T = dir.tc[dual];
     const MomentSets& M = dir.ms[dual];
     if (!M.ok || p->form != kFormAuto) return M.ok && p->form == kFormMoment;
     const double deg = (double)E / (double)std::max<int64_t>(N, 1), slots = (deg / MS_TB + 0.5) * operands;
     const bool resident = std::ceil(deg / MS_TB + 0.3) * operands <= std::min(M.ns, M.nw);   // (degrees spread around their mean)
-    return M.node_us + slots * (resident ? M.slot_us : M.slot_again_us) < T.node_us + slots * T.slot_us;
+    double moment = M.node_us + slots * (resident ? M.slot_us : M.slot_again_us), coupled = T.node_us + slots * T.slot_us;
+    if (geo) {
+        moment = std::max(moment, 1.7 * slots * (double)(resident ? M.sets.size() : M.units.size()));
+        coupled = std::max(coupled, 1.7 * slots * (double)T.sets.size());
+    }
+    return moment < coupled;
 }
 
 static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {

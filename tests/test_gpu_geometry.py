@@ -220,6 +220,20 @@ def test_partial_outputs_and_argument_errors():
     assert e.value.code == -2
 
 
+@pytest.mark.parametrize("irreps,l_max,K,N,deg,form", [("32x0e+32x1o+32x2e+32x3o", 3, 16, 420, 380, "coupled"), ("32x0e+32x1o+32x2e", 2, 8, 200, 36, "moment")])
+def test_long_neighbourhoods_take_the_coupled_form(irreps, l_max, K, N, deg, form):
+    """The moment form computes the edge inputs of a node that its ring does not hold again for every unit: the default plan has the bits
+    of the form that does not pay for it."""
+    ir = P(irreps)
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("long", ir, ir, l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "bessel", seed=35)
+    c = GeoCase(w)
+    y = c.geo_fwd()
+    other = "moment" if form == "coupled" else "coupled"
+    assert np.array_equal(y, GeoCase(w, inputs=c.d, form=form).geo_fwd())
+    assert not np.array_equal(y, GeoCase(w, inputs=c.d, form=other).geo_fwd())
+
+
 def test_blocks_above_128_are_refused():
     """The geometry mode lives in the tensor-core kernels, which take blocks of up to 128: in the forward as in the backward."""
     c = GeoCase(synth.Workload("wide", P("160x0e+160x1o"), P("16x0e+16x1o"), 1, 8, 20, 4.0, 2.0, "bessel", seed=27))
