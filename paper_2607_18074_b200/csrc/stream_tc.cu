@@ -824,182 +824,180 @@ int smem_need(int KP, bool dual, int dsh, int ns, int b_cap, int max_ent, int n_
 }  // namespace
 
 // Units, passes ("sets") and entries of one direction, plain (0) or dual (1) stream.
-void build_tc_sets(const sobek_plan* p, Direction& dir, int only) {
+void build_tc_sets(const sobek_plan* p, Direction& dir, int dual) {
     const int KP = p->K <= 8 ? 8 : 16;
-    for (int dual = only; dual <= only; ++dual) {
-        TcSets& T = dir.tc[dual];
-        T = TcSets{};
-        if (p->K > 16) continue;
-        bool ok = true;
-        for (const DPath& P : dir.paths)
-            if ((P.c_src & 7) || P.c_src > 128 || (P.src_off & 7)) ok = false;
-        if (!ok || (dir.C_src & 7) || dir.paths.empty()) continue;
-        // distinct source blocks in order of appearance, with the components of all paths reading them
-        struct Blk { int so, c_src, d_src; std::vector<SComp> comps; };
-        std::vector<Blk> blocks;
-        for (size_t gi = 0; gi < dir.groups.size(); ++gi) {
-            const DGroup& G = dir.groups[gi];
-            for (int k = G.path_begin; k < G.path_end; ++k) {
-                const DPath& P = dir.paths[k];
-                auto it = std::find_if(blocks.begin(), blocks.end(), [&](const Blk& b) { return b.so == P.src_off; });
-                if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
-                for (int o = 0; o < G.d_dst; ++o)
-                    it->comps.push_back(SComp{P.tabM + o, G.d_dst, P.sh_off, (int)gi, o, P.koff, G.d_dst, 0});
-            }
+    TcSets& T = dir.tc[dual];
+    T = TcSets{};
+    if (p->K > 16) return;
+    bool ok = true;
+    for (const DPath& P : dir.paths)
+        if ((P.c_src & 7) || P.c_src > 128 || (P.src_off & 7)) ok = false;
+    if (!ok || (dir.C_src & 7) || dir.paths.empty()) return;
+    // distinct source blocks in order of appearance, with the components of all paths reading them
+    struct Blk { int so, c_src, d_src; std::vector<SComp> comps; };
+    std::vector<Blk> blocks;
+    for (size_t gi = 0; gi < dir.groups.size(); ++gi) {
+        const DGroup& G = dir.groups[gi];
+        for (int k = G.path_begin; k < G.path_end; ++k) {
+            const DPath& P = dir.paths[k];
+            auto it = std::find_if(blocks.begin(), blocks.end(), [&](const Blk& b) { return b.so == P.src_off; });
+            if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
+            for (int o = 0; o < G.d_dst; ++o)
+                it->comps.push_back(SComp{P.tabM + o, G.d_dst, P.sh_off, (int)gi, o, P.koff, G.d_dst, 0});
         }
-        std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
-        // candidate units: accumulator tiles of up to 128 / KP components of one source block, split evenly
-        struct Cand { int blk, c0, nc; };
-        std::vector<Cand> cands;
-        const int comps_per_tile = 128 / KP;
-        for (size_t b = 0; b < blocks.size(); ++b) {
-            const int nc = (int)blocks[b].comps.size();
-            const int ntile = (nc + comps_per_tile - 1) / comps_per_tile;
-            const int per = (nc + ntile - 1) / ntile;
-            for (int c0 = 0; c0 < nc; c0 += per) cands.push_back(Cand{(int)b, c0, std::min(per, nc - c0)});
-        }
-        auto blk_b = [&](int b) { return blocks[b].d_src * 2048 * ((blocks[b].c_src + 63) / 64); };
-        auto ncols = [&](int b) { return (blocks[b].c_src + 15) & ~15; };
-        auto cols32 = [&](int b) { return (ncols(b) + 31) & ~31; };
-        auto cand_nz = [&](const Cand& c) {
-            int n = 0;
-            for (int cl = 0; cl < c.nc; ++cl) {
-                const SComp& cp = blocks[c.blk].comps[c.c0 + cl];
-                for (int sdx = 0; sdx < blocks[c.blk].d_src; ++sdx) {
-                    const int t = cp.tab0 + sdx * cp.tstride;
-                    n += p->tab_ptr[t + 1] - p->tab_ptr[t];
-                }
-            }
-            return n;
-        };
-        int n_comps_total = 0, n_slab = 0;
-        for (const Blk& b : blocks) n_comps_total += (int)b.comps.size();
-        for (const Cand& c : cands) n_slab += blocks[c.blk].d_src;        // one slab per (tile, s)
-        // greedy packing of consecutive units into passes: the accumulator tiles of a pass fit one of the two TMEM
-        // buffers and its operand regions fit shared memory with at least two ring stages
-        const int budget = 227 * 1024;
-        // Two accumulator buffers (the drain of one receiver overlaps the MMAs of the next) when at least two of the
-        // widest tiles fit half of the accumulator columns; else one buffer over all of them: with 128-column tiles a
-        // half holds a single tile, a set then has one to nine slabs per batch and most builder groups idle, which
-        // costs more than the wait for the drain (measured: 128-wide profiles 10 - 17 % faster with one buffer, 32- and
-        // 64-wide ones 2 - 10 % slower).
-        int widest = 0;
-        for (const Cand& c : cands) widest = std::max(widest, cols32(c.blk));
-        T.nbuf = 2 * widest > ACC_BUDGET ? 1 : 2;
-        const int acc_budget = T.nbuf == 2 ? ACC_BUDGET : RING0;
-        bool fits = true;
-        size_t i = 0;
-        while (i < cands.size() && fits) {
-            int b_bytes = 0, cols = 0, nent = 0, nnz = 0, slabs_in = 0;
-            std::vector<int> set_blks;
-            size_t j = i;
-            for (; j < cands.size(); ++j) {
-                const Cand& c = cands[j];
-                const bool new_blk = std::find(set_blks.begin(), set_blks.end(), c.blk) == set_blks.end();
-                const int b2 = b_bytes + (new_blk ? blk_b(c.blk) : 0);
-                const int c2 = cols + cols32(c.blk), e2 = nent + c.nc * blocks[c.blk].d_src, n2 = nnz + cand_nz(c);
-                // the kernel sizes its regions by the maxima over all passes
-                const int bcap = std::max(T.b_cap, (b2 + 1023) & ~1023);
-                const int own2 = (slabs_in + blocks[c.blk].d_src + NBG - 1) / NBG;
-                const int need = smem_need(KP, dual, p->dim_sh, 2, bcap, std::max(T.max_ent, e2), (int)cands.size(), (int)cands.size(),
-                                           n_comps_total, std::max(T.max_nz, n2), n_slab, std::max(T.max_units, own2));
-                if (need > budget || c2 > acc_budget) break;
-                b_bytes = b2; cols = c2; nent = e2; nnz = n2; slabs_in += blocks[c.blk].d_src;
-                if (new_blk) set_blks.push_back(c.blk);
-            }
-            if (j == i) { fits = false; break; }
-            TSet S{};
-            S.unit_begin = (int)T.units.size(); S.blk_begin = (int)T.blks.size(); S.ent_begin = (int)T.ents.size();
-            int b_off = 0, col = 0, ent = 0;
-            std::vector<int> local_blk;   // block index -> index in T.blks
-            for (size_t k = i; k < j; ++k) {
-                const Cand& c = cands[k];
-                const Blk& Bk = blocks[c.blk];
-                int bi = -1;
-                for (size_t m = 0; m < local_blk.size(); ++m) if (local_blk[m] == c.blk) bi = S.blk_begin + (int)m;
-                if (bi < 0) {
-                    TBlk tb{};
-                    tb.src_off = Bk.so; tb.c_src = Bk.c_src; tb.d_src = Bk.d_src; tb.ncols = ncols(c.blk);
-                    tb.b_off = b_off; tb.slab_bytes = 2048 * ((Bk.c_src + 63) / 64); tb.atom_stride = 2048;
-                    b_off += blk_b(c.blk);
-                    bi = (int)T.blks.size();
-                    T.blks.push_back(tb);
-                    local_blk.push_back(c.blk);
-                }
-                TUnit U{};
-                U.blk = bi; U.comp_begin = (int)T.comps.size(); U.ncomp = c.nc;
-                U.a_off = ent;                 // first entry of the unit inside the pass: entry = a_off + cl * d_src + s
-                U.slab_stride = 0; U.tmem_col = col;
-                for (int cl = 0; cl < c.nc; ++cl) {
-                    const SComp& cp = Bk.comps[c.c0 + cl];
-                    T.comps.push_back(cp);
-                    for (int s = 0; s < Bk.d_src; ++s) T.ents.push_back(TEnt{cp.tab0 + s * cp.tstride, cp.sh_off, 0, 0});
-                }
-                ent += c.nc * Bk.d_src;
-                col += cols32(c.blk);
-                T.units.push_back(U);
-            }
-            S.nunit = (int)T.units.size() - S.unit_begin; S.nblk = (int)T.blks.size() - S.blk_begin;
-            S.nent = (int)T.ents.size() - S.ent_begin;
-            // build order of the pass's slabs: tile after tile in turn (s = 0 of every tile, then s = 1, ...), so that
-            // the builder groups (slab j mod NBG) and the MMA threads (tile mod NMW) find work at the same rate
-            S.sched_begin = (int)T.slabs.size() / 2;
-            std::vector<uint32_t> order;      // (tile << 8) | s
-            for (int sdx = 0, more = 1; more; ++sdx) {
-                more = 0;
-                for (int u = 0; u < S.nunit; ++u)
-                    if (sdx < T.blks[T.units[S.unit_begin + u].blk].d_src) { order.push_back(((uint32_t)u << 8) | (uint32_t)sdx); more = 1; }
-            }
-            S.nslab = (int)order.size();
-            S.mfirst = 0x00ffffff;
-            S.oddmask = 0;
-            for (int sl = 0; sl < NSLOT; ++sl)
-                if (((S.nslab - sl + NSLOT - 1) / NSLOT) & 1) S.oddmask |= 1 << sl;      // slots used an odd number of times per batch
-            for (int j = 0; j < S.nslab; ++j) {
-                const int u = (int)(order[j] >> 8), sdx = (int)(order[j] & 255u);
-                const TUnit& Uu = T.units[S.unit_begin + u];
-                const int d = T.blks[Uu.blk].d_src;
-                uint32_t next = 255;
-                for (int k = j + 1; k < S.nslab && next == 255; ++k)
-                    if ((int)(order[k] >> 8) % NMW == u % NMW) next = (uint32_t)k;
-                T.slabs.push_back((uint32_t)(Uu.a_off + sdx) | ((uint32_t)d << 16) | ((uint32_t)Uu.ncomp << 24));
-                T.slabs.push_back((uint32_t)u | ((uint32_t)sdx << 8) | (next << 16));
-                const int t = u % NMW;
-                if (((S.mfirst >> (8 * t)) & 255) == 255) S.mfirst = (S.mfirst & ~(255 << (8 * t))) | (j << (8 * t));
-            }
-            if (S.nslab > 254) fits = false;
-            T.max_units = std::max(T.max_units, (S.nslab + NBG - 1) / NBG);      // own slabs of a builder group at most
-            T.sets.push_back(S);
-            T.b_cap = std::max(T.b_cap, (b_off + 1023) & ~1023);
-            T.max_ent = std::max(T.max_ent, S.nent);
-            T.max_nz = std::max(T.max_nz, nnz);
-            T.acc_cols = std::max(T.acc_cols, col);
-            i = j;
-        }
-        if (!fits) { T = TcSets{}; continue; }
-        // as many ring stages as shared memory holds (the loaders run that many batches ahead)
-        int ns = 2;
-        while (ns < MAXNS && smem_need(KP, dual, p->dim_sh, ns + 1, T.b_cap, T.max_ent, (int)cands.size(), (int)cands.size(),
-                                       n_comps_total, T.max_nz, n_slab, T.max_units) <= budget) ++ns;
-        T.ctas_per_sm = 1;
-        T.ring_stages = ns;
-        T.tmem_cols = TMEM_COLS;
-        T.smem_bytes = smem_need(KP, dual, p->dim_sh, ns, T.b_cap, T.max_ent, (int)cands.size(), (int)cands.size(), n_comps_total, T.max_nz, n_slab, T.max_units);
-        // shared-memory images of the tables
-        for (TSet& S : T.sets) {
-            S.b_items = (int)T.nz.size();
-            for (int j = 0; j < S.nent; ++j) {
-                const TEnt& E = T.ents[S.ent_begin + j];
-                EntS es{0, (int)T.nz.size() - S.b_items, p->tab_ptr[E.tab + 1] - p->tab_ptr[E.tab], 0};
-                for (int k = p->tab_ptr[E.tab]; k < p->tab_ptr[E.tab + 1]; ++k) T.nz.push_back(NzS{E.sh_off + p->tab_idx[k], p->tab_coef[k]});
-                T.ents_s.push_back(es);
-            }
-            S.pad = (int)T.nz.size() - S.b_items;
-        }
-        for (const SComp& cp : T.comps)
-            T.comps_s.push_back(CompS{dir.zb_off[cp.group], dir.nk_ld[cp.group], cp.d_dst, cp.o, cp.koff, {0, 0}});
-        T.ok = true;
     }
+    std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
+    // candidate units: accumulator tiles of up to 128 / KP components of one source block, split evenly
+    struct Cand { int blk, c0, nc; };
+    std::vector<Cand> cands;
+    const int comps_per_tile = 128 / KP;
+    for (size_t b = 0; b < blocks.size(); ++b) {
+        const int nc = (int)blocks[b].comps.size();
+        const int ntile = (nc + comps_per_tile - 1) / comps_per_tile;
+        const int per = (nc + ntile - 1) / ntile;
+        for (int c0 = 0; c0 < nc; c0 += per) cands.push_back(Cand{(int)b, c0, std::min(per, nc - c0)});
+    }
+    auto blk_b = [&](int b) { return blocks[b].d_src * 2048 * ((blocks[b].c_src + 63) / 64); };
+    auto ncols = [&](int b) { return (blocks[b].c_src + 15) & ~15; };
+    auto cols32 = [&](int b) { return (ncols(b) + 31) & ~31; };
+    auto cand_nz = [&](const Cand& c) {
+        int n = 0;
+        for (int cl = 0; cl < c.nc; ++cl) {
+            const SComp& cp = blocks[c.blk].comps[c.c0 + cl];
+            for (int sdx = 0; sdx < blocks[c.blk].d_src; ++sdx) {
+                const int t = cp.tab0 + sdx * cp.tstride;
+                n += p->tab_ptr[t + 1] - p->tab_ptr[t];
+            }
+        }
+        return n;
+    };
+    int n_comps_total = 0, n_slab = 0;
+    for (const Blk& b : blocks) n_comps_total += (int)b.comps.size();
+    for (const Cand& c : cands) n_slab += blocks[c.blk].d_src;        // one slab per (tile, s)
+    // greedy packing of consecutive units into passes: the accumulator tiles of a pass fit one of the two TMEM
+    // buffers and its operand regions fit shared memory with at least two ring stages
+    const int budget = 227 * 1024;
+    // Two accumulator buffers (the drain of one receiver overlaps the MMAs of the next) when at least two of the
+    // widest tiles fit half of the accumulator columns; else one buffer over all of them: with 128-column tiles a
+    // half holds a single tile, a set then has one to nine slabs per batch and most builder groups idle, which
+    // costs more than the wait for the drain (measured: 128-wide profiles 10 - 17 % faster with one buffer, 32- and
+    // 64-wide ones 2 - 10 % slower).
+    int widest = 0;
+    for (const Cand& c : cands) widest = std::max(widest, cols32(c.blk));
+    T.nbuf = 2 * widest > ACC_BUDGET ? 1 : 2;
+    const int acc_budget = T.nbuf == 2 ? ACC_BUDGET : RING0;
+    bool fits = true;
+    size_t i = 0;
+    while (i < cands.size() && fits) {
+        int b_bytes = 0, cols = 0, nent = 0, nnz = 0, slabs_in = 0;
+        std::vector<int> set_blks;
+        size_t j = i;
+        for (; j < cands.size(); ++j) {
+            const Cand& c = cands[j];
+            const bool new_blk = std::find(set_blks.begin(), set_blks.end(), c.blk) == set_blks.end();
+            const int b2 = b_bytes + (new_blk ? blk_b(c.blk) : 0);
+            const int c2 = cols + cols32(c.blk), e2 = nent + c.nc * blocks[c.blk].d_src, n2 = nnz + cand_nz(c);
+            // the kernel sizes its regions by the maxima over all passes
+            const int bcap = std::max(T.b_cap, (b2 + 1023) & ~1023);
+            const int own2 = (slabs_in + blocks[c.blk].d_src + NBG - 1) / NBG;
+            const int need = smem_need(KP, dual, p->dim_sh, 2, bcap, std::max(T.max_ent, e2), (int)cands.size(), (int)cands.size(),
+                                       n_comps_total, std::max(T.max_nz, n2), n_slab, std::max(T.max_units, own2));
+            if (need > budget || c2 > acc_budget) break;
+            b_bytes = b2; cols = c2; nent = e2; nnz = n2; slabs_in += blocks[c.blk].d_src;
+            if (new_blk) set_blks.push_back(c.blk);
+        }
+        if (j == i) { fits = false; break; }
+        TSet S{};
+        S.unit_begin = (int)T.units.size(); S.blk_begin = (int)T.blks.size(); S.ent_begin = (int)T.ents.size();
+        int b_off = 0, col = 0, ent = 0;
+        std::vector<int> local_blk;   // block index -> index in T.blks
+        for (size_t k = i; k < j; ++k) {
+            const Cand& c = cands[k];
+            const Blk& Bk = blocks[c.blk];
+            int bi = -1;
+            for (size_t m = 0; m < local_blk.size(); ++m) if (local_blk[m] == c.blk) bi = S.blk_begin + (int)m;
+            if (bi < 0) {
+                TBlk tb{};
+                tb.src_off = Bk.so; tb.c_src = Bk.c_src; tb.d_src = Bk.d_src; tb.ncols = ncols(c.blk);
+                tb.b_off = b_off; tb.slab_bytes = 2048 * ((Bk.c_src + 63) / 64); tb.atom_stride = 2048;
+                b_off += blk_b(c.blk);
+                bi = (int)T.blks.size();
+                T.blks.push_back(tb);
+                local_blk.push_back(c.blk);
+            }
+            TUnit U{};
+            U.blk = bi; U.comp_begin = (int)T.comps.size(); U.ncomp = c.nc;
+            U.a_off = ent;                 // first entry of the unit inside the pass: entry = a_off + cl * d_src + s
+            U.slab_stride = 0; U.tmem_col = col;
+            for (int cl = 0; cl < c.nc; ++cl) {
+                const SComp& cp = Bk.comps[c.c0 + cl];
+                T.comps.push_back(cp);
+                for (int s = 0; s < Bk.d_src; ++s) T.ents.push_back(TEnt{cp.tab0 + s * cp.tstride, cp.sh_off, 0, 0});
+            }
+            ent += c.nc * Bk.d_src;
+            col += cols32(c.blk);
+            T.units.push_back(U);
+        }
+        S.nunit = (int)T.units.size() - S.unit_begin; S.nblk = (int)T.blks.size() - S.blk_begin;
+        S.nent = (int)T.ents.size() - S.ent_begin;
+        // build order of the pass's slabs: tile after tile in turn (s = 0 of every tile, then s = 1, ...), so that
+        // the builder groups (slab j mod NBG) and the MMA threads (tile mod NMW) find work at the same rate
+        S.sched_begin = (int)T.slabs.size() / 2;
+        std::vector<uint32_t> order;      // (tile << 8) | s
+        for (int sdx = 0, more = 1; more; ++sdx) {
+            more = 0;
+            for (int u = 0; u < S.nunit; ++u)
+                if (sdx < T.blks[T.units[S.unit_begin + u].blk].d_src) { order.push_back(((uint32_t)u << 8) | (uint32_t)sdx); more = 1; }
+        }
+        S.nslab = (int)order.size();
+        S.mfirst = 0x00ffffff;
+        S.oddmask = 0;
+        for (int sl = 0; sl < NSLOT; ++sl)
+            if (((S.nslab - sl + NSLOT - 1) / NSLOT) & 1) S.oddmask |= 1 << sl;      // slots used an odd number of times per batch
+        for (int j = 0; j < S.nslab; ++j) {
+            const int u = (int)(order[j] >> 8), sdx = (int)(order[j] & 255u);
+            const TUnit& Uu = T.units[S.unit_begin + u];
+            const int d = T.blks[Uu.blk].d_src;
+            uint32_t next = 255;
+            for (int k = j + 1; k < S.nslab && next == 255; ++k)
+                if ((int)(order[k] >> 8) % NMW == u % NMW) next = (uint32_t)k;
+            T.slabs.push_back((uint32_t)(Uu.a_off + sdx) | ((uint32_t)d << 16) | ((uint32_t)Uu.ncomp << 24));
+            T.slabs.push_back((uint32_t)u | ((uint32_t)sdx << 8) | (next << 16));
+            const int t = u % NMW;
+            if (((S.mfirst >> (8 * t)) & 255) == 255) S.mfirst = (S.mfirst & ~(255 << (8 * t))) | (j << (8 * t));
+        }
+        if (S.nslab > 254) fits = false;
+        T.max_units = std::max(T.max_units, (S.nslab + NBG - 1) / NBG);      // own slabs of a builder group at most
+        T.sets.push_back(S);
+        T.b_cap = std::max(T.b_cap, (b_off + 1023) & ~1023);
+        T.max_ent = std::max(T.max_ent, S.nent);
+        T.max_nz = std::max(T.max_nz, nnz);
+        T.acc_cols = std::max(T.acc_cols, col);
+        i = j;
+    }
+    if (!fits) { T = TcSets{}; return; }
+    // as many ring stages as shared memory holds (the loaders run that many batches ahead)
+    int ns = 2;
+    while (ns < MAXNS && smem_need(KP, dual, p->dim_sh, ns + 1, T.b_cap, T.max_ent, (int)cands.size(), (int)cands.size(),
+                                   n_comps_total, T.max_nz, n_slab, T.max_units) <= budget) ++ns;
+    T.ctas_per_sm = 1;
+    T.ring_stages = ns;
+    T.tmem_cols = TMEM_COLS;
+    T.smem_bytes = smem_need(KP, dual, p->dim_sh, ns, T.b_cap, T.max_ent, (int)cands.size(), (int)cands.size(), n_comps_total, T.max_nz, n_slab, T.max_units);
+    // shared-memory images of the tables
+    for (TSet& S : T.sets) {
+        S.b_items = (int)T.nz.size();
+        for (int j = 0; j < S.nent; ++j) {
+            const TEnt& E = T.ents[S.ent_begin + j];
+            EntS es{0, (int)T.nz.size() - S.b_items, p->tab_ptr[E.tab + 1] - p->tab_ptr[E.tab], 0};
+            for (int k = p->tab_ptr[E.tab]; k < p->tab_ptr[E.tab + 1]; ++k) T.nz.push_back(NzS{E.sh_off + p->tab_idx[k], p->tab_coef[k]});
+            T.ents_s.push_back(es);
+        }
+        S.pad = (int)T.nz.size() - S.b_items;
+    }
+    for (const SComp& cp : T.comps)
+        T.comps_s.push_back(CompS{dir.zb_off[cp.group], dir.nk_ld[cp.group], cp.d_dst, cp.o, cp.koff, {0, 0}});
+    T.ok = true;
 }
 
 cudaError_t launch_stream_tc(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
