@@ -71,6 +71,9 @@ struct TcBatch {
 };
 static_assert(sizeof(TcBatch) <= sizeof(GemmBatch::storage), "GemmBatch::storage holds a TcBatch");
 
+// FOUR: products of four passes (a kernel of its own: as a run-time branch the second accumulator cost the others 7 % of a call of
+// four small launches, 28.9 -> 30.7 us)
+template <bool FOUR>
 __global__ void __launch_bounds__(TC_THREADS, 2)
 k_gemm_tc(const __grid_constant__ TcBatch B) {
     int bi = 0;
@@ -167,7 +170,7 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
 #pragma unroll
                 for (uint32_t k = 0; k < BK / 16; ++k) {
                     const uint32_t acc = (kb > 0 || k > 0) ? 1u : 0u, o = k * kstep16;
-                    if (g.passes == 4) tc_mma_bf16_x4(tmem_base, tmem_base + (uint32_t)g.BN, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc, acc);
+                    if (FOUR) tc_mma_bf16_x4(tmem_base, tmem_base + (uint32_t)g.BN, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc, acc);
                     else if (g.passes != 1) tc_mma_bf16_x3(tmem_base, dAh + o, dAl + o, dBh + o, dBl + o, idesc, acc);
                     else tc_mma_bf16(tmem_base, dAh + o, dBh + o, idesc, acc);
                 }
@@ -202,7 +205,7 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
             for (int c0 = 0; c0 < g.BN; c0 += 16) {
                 float v[16];
                 tc_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);   // warp-collective
-                if (g.passes == 4) add_small(v, q, c0);
+                if (FOUR) add_small(v, q, c0);
 #pragma unroll
                 for (int j = 0; j < 16; j += 4)
                     *reinterpret_cast<float4*>(pk + lane * P4 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -240,7 +243,7 @@ k_gemm_tc(const __grid_constant__ TcBatch B) {
         for (int c0 = 0; c0 < g.BN; c0 += 16) {
             float v[16];
             tc_ld16(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);   // warp-collective
-            if (g.passes == 4) add_small(v, q, c0);
+            if (FOUR) add_small(v, q, c0);
 #pragma unroll
             for (int j = 0; j < 16; j += 4)
                 *reinterpret_cast<float4*>(park + lane * P4 + c0 + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -570,7 +573,7 @@ cudaError_t gemm_tc_add(GemmBatch& gb, const void* Ahi, const void* Alo, int64_t
     pr.gy = (uint32_t)((N + BN - 1) / BN);
     const uint64_t tiles = (uint64_t)pr.gx * pr.gy * (uint64_t)g.splits;
     const size_t sh = (size_t)g.ring_bytes + 1024 + 8 * (2 * g.stages + 1) + 16;
-    if (gb.n > 0 && (gb.n == TC_MAX_BATCH || tiles + B.tile0[gb.n] >= (uint64_t(1) << 31))) {
+    if (gb.n > 0 && (gb.n == TC_MAX_BATCH || (B.p[0].g.passes == 4) != (g.passes == 4) || tiles + B.tile0[gb.n] >= (uint64_t(1) << 31))) {
         cudaError_t e = gemm_tc_flush(gb, s, nullptr);
         if (e != cudaSuccess) return e;
     }
@@ -595,7 +598,8 @@ void launch_sub(const TcBatch& B, const int* q, int n, size_t sh, cudaStream_t s
         sub.tile0[i + 1] = sub.tile0[i] + sub.p[i].gx * sub.p[i].gy * (uint32_t)sub.p[i].g.splits;
     }
     KernelTimer kt(K_GEMM, s);
-    k_gemm_tc<<<sub.tile0[n], TC_THREADS, sh, s>>>(sub);
+    if (sub.p[0].g.passes == 4) k_gemm_tc<true><<<sub.tile0[n], TC_THREADS, sh, s>>>(sub);      // (one number of passes in a queue)
+    else k_gemm_tc<false><<<sub.tile0[n], TC_THREADS, sh, s>>>(sub);
     count_launch();
 }
 }  // namespace
@@ -611,7 +615,8 @@ cudaError_t gemm_tc_flush(GemmBatch& gb, cudaStream_t s, const sobek_plan* p) {
     TcBatch& B = *reinterpret_cast<TcBatch*>(gb.storage);
     static bool attr_set = false;
     if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+        cudaError_t e = allow_dynamic_smem(k_gemm_tc<false>);
+        if (e == cudaSuccess) e = allow_dynamic_smem(k_gemm_tc<true>);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
