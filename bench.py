@@ -37,12 +37,14 @@ DTYPE = "f32 storage; products as split bf16 x3 (hi*hi + lo*hi + hi*lo) with f32
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of an edge-kernel class, measured with
 # ncu on the named profile at 20,000 nodes and stored per edge of the launch (a launch of these classes processes
-# the edges of one node chunk once; its traffic grows in proportion to them).  At this profile the stream's figure is
-# the state of the chunk written once (0.92 MB per node as bf16 hi + lo, i.e. 23 KB per edge at 40 edges per node)
-# plus the gathered sender rows.
+# the edges of one node chunk once; its traffic grows in proportion to them), averaged over the launches of a step.  At
+# this profile the stream's figure is the state of the chunk written once (0.92 MB per node as bf16 hi + lo, i.e. 23 KB per
+# edge at 40 edges per node) plus the gathered sender rows, the edge pass's the fp32 adjoint state read once plus those rows.
 NCU_TRAFFIC_BYTES_PER_EDGE = {
-    ("cfg5", "edge_stream_state"): (719.4e6 + 2082.7e6) / 90891.0,     # k_stream_tc, two launches
-    ("cfg5", "edge_pass"): (359.0e6 + 15.3e6) / 90891.0,                # k_edge_tc, three launches
+    # k_moment_stream: five plain passes and two dual ones
+    ("cfg5", "edge_stream_state"): (5 * (353.3e6 + 2079.0e6) + 2 * (721.7e6 + 2081.7e6)) / 7 / 90891.0,
+    # k_moment_edge: two plain passes and a dual one
+    ("cfg5", "edge_pass"): (2 * (2667.4e6 + 16.2e6) + (4771.5e6 + 26.8e6)) / 3 / 90891.0,
 }
 STATE_BUDGET_MIB = None         # --state-budget-mib: the plan's scratch budget (None = the library's default, 2048)
 STREAM_CALLS_PER_STEP = 7      # edge-stream passes over all edges per step: 1 fwd + 2 bwd + 4 dbwd

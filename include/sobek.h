@@ -113,11 +113,16 @@ enum { SOBEK_MAX_L = 4 };
  * SOBEK_FLAG_FUSED_FP32 selects the fused schedule for y / gx / ggy / hx (FP32-pipe edge stream feeding the tensor
  * core inside one kernel, receiver state never written to memory); the default is the stream -> bounded state ->
  * GEMM schedule, which is the faster one at present.  In the default schedule the edge stream and the edge pass run
- * on the tensor cores where the profile allows it (multiplicities that are multiples of 8 / 16, at most 128,
- * K <= 16); SOBEK_FLAG_FP32_STREAM / SOBEK_FLAG_FP32_EDGE select the FP32-pipe kernels instead (same results
- * within the tolerances).  On the tensor cores both exist in two forms, with the coupling inside the sum over the edges and
- * in moment form with the coupling outside of it; a call takes the one that is faster at its graph's mean degree.
- * SOBEK_FLAG_COUPLED_FORM / SOBEK_FLAG_MOMENT_FORM (not both) take one of them wherever it exists.
+ * on the tensor cores where the profile allows it; SOBEK_FLAG_FP32_STREAM / SOBEK_FLAG_FP32_EDGE select the FP32-pipe
+ * kernels instead (same results within the tolerances).  On the tensor cores both exist in two forms, with the coupling
+ * inside the sum over the edges and in moment form with the coupling outside of it; a call takes the one that is estimated
+ * to be faster at its graph's mean degree.  K is at most 16 for all of them, and the gathered blocks are:
+ *   stream, either form          multiplicities that are multiples of 8, at most 128
+ *   edge pass, coupling inside   multiples of 16, at most 128
+ *   edge pass, moment form       the same; in the fully connected mode multiples of 8 of any size, K >= 2
+ * (some wide profiles of order 3 and 4 do not fit shared memory and run on the FP32 pipes all the same).
+ * SOBEK_FLAG_COUPLED_FORM / SOBEK_FLAG_MOMENT_FORM (not both) take one of the forms wherever it exists; where the
+ * coupled one does not, SOBEK_FLAG_COUPLED_FORM leaves the FP32-pipe kernel.
  * SOBEK_FLAG_STATE_BUDGET_MIB(mb) sets the scratch budget (section "Runtime scratch-budget policy"; the paper
  * measures with 128 MiB): the bytes of receiver (or sender) state held at once.  Nodes are processed in chunks that
  * fit the budget, but never fewer than 512 at a time; the results do not depend on the budget beyond the summation
@@ -261,8 +266,9 @@ int sobek_conv_dbwd(const sobek_plan* plan, const sobek_graph* g,
  *          SOBEK_BASIS_GAUSSIAN  exp(-(r - mu_q)^2 / (2 s^2)), mu_q = q s, s = r_cut / (K - 1), q = 0..K-1
  *                                (envelope_p is ignored).
  * Every r_e must be non-zero (an edge of length zero has no direction; nothing is checked).
- * Plans: fully connected or channelwise, ir_mul layout, l_max <= 4, the tensor-core edge kernels in use (the
- * default where the profile allows them: K <= 16, multiplicities multiples of 16 up to 128); otherwise UNSUPPORTED.
+ * Plans: fully connected or channelwise, ir_mul layout, l_max <= 4, the tensor-core edge kernels in use (the default
+ * where the profile allows them: K <= 16, multiplicities up to 128 that are multiples of 8 in the forward and, for the
+ * input features, of 16 in the backward and double backward); otherwise UNSUPPORTED.
  * Workspace: sobek_workspace_bytes(plan, N, E, 0) for the forward, (.., 1) for the backward, (.., 2) for the double
  * backward.  Errors as for sobek_conv_fwd / sobek_conv_bwd / sobek_conv_dbwd.
  *

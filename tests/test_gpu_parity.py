@@ -332,7 +332,7 @@ def test_stale_graph_arrays_are_reported_not_followed(name, fp32_pipe):
     access through the bad value.  One corrupted entry per array, positive and negative, all three orders."""
     import torch
     opts = dict(tc_stream=False, tc_edge=False) if fp32_pipe else {}
-    c = Case(CASES[name], **opts)          # cfg1: tensor-core stream + FP32-pipe edge pass; tc_K6_dense: both on tensor cores
+    c = Case(CASES[name], **opts)          # (without the option: streams and edge pass on the tensor cores)
     sb, i = c.sb, c.plan.info
     names = ("row_ptr", "col", "src_ptr", "src_perm", "src_recv")
     new = lambda *s: torch.full(s, float("nan"), dtype=torch.float32, device="cuda:0")
