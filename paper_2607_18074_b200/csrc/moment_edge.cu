@@ -500,7 +500,7 @@ void build_moment_edge(const sobek_plan* p, Direction& dir) {
     T = MomentEdge{};
     // In the place of k_edge_tc, or (EXACT) of the FP32-pipe pass, which holds rows and adjoint state in 32 bits.  There the error
     // against fp64 must not grow by the split: in the fully connected mode it does not, since Pbar then has three parts and the product
-    // that makes its Zbar takes lo x lo along (2-norm of gY, 81 random profiles: 0.97 of the FP32 pipes' on average, 1.05 at most).  The
+    // that makes its Zbar takes lo x lo along (2-norm of gY, 168 random profiles: 0.97 of the FP32 pipes' on average, 1.07 at most).  The
     // channelwise mode, whose Zbar has the error of one fp32 product, keeps the FP32 pipes (1e-7), and so does a contraction that is
     // too long for three accumulators (they round towards zero, a little with every k-step).
     const bool exact = !dir.etc[0].ok;
