@@ -280,10 +280,6 @@ cudaError_t weight_grad_tc(const sobek_plan* p, const Direction& dir, int64_t nn
 
 // ---- the node-side steps in either multiplicity mode: tensor-core GEMMs on the packed copies of R (uvw), or
 // the elementwise kernels on R itself (uvu, Eq. uvu_connection) --------------------------------------------
-cudaError_t pack_R(const sobek_plan* p, const Direction& dir, int transposed, int n_major, const float* R, void* hi,
-                   void* lo, cudaStream_t s) {
-    return p->uvu ? cudaSuccess : launch_pack_R_bf16(p, dir, transposed, n_major, R, hi, lo, s);
-}
 cudaError_t split_gy(const sobek_plan* p, const Direction& dir, int64_t n0, int64_t nn, const float* gdst,
                      uint16_t* gh, uint16_t* gl, cudaStream_t s) {
     return p->uvu ? cudaSuccess : split_adjoint(p, dir, n0, nn, gdst, gh, gl, s);
@@ -308,9 +304,9 @@ cudaError_t weight_grad(const sobek_plan* p, const Direction& dir, int64_t n0, i
     return weight_grad_tc(p, dir, nn, zh, zl, gh, gl, gRp, part, splits, status, s);
 }
 // the accumulated weight adjoint -> the caller's [K, N_w] array (already in that layout in the uvu mode)
-cudaError_t unpack_R(const sobek_plan* p, const Direction& dir, const float* Rp, float* R, cudaStream_t s) {
+cudaError_t unpack_R(const sobek_plan* p, const Direction& dir, const int32_t* zq, const float* Rp, float* R, cudaStream_t s) {
     if (p->uvu) return cudaMemcpyAsync(R, Rp, (size_t)p->K * (size_t)p->N_w * 4, cudaMemcpyDeviceToDevice, s);
-    return launch_unpack_R(p, dir, Rp, R, s);
+    return launch_unpack_R(p, dir, zq, Rp, R, s);
 }
 
 }  // namespace
@@ -372,11 +368,13 @@ int conv_fwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
         CK(launch_fused(p, p->fwd, rv, x, nullptr, Y, nullptr, phi, nullptr, 0, w.fFKh, w.fFKl, y, 0, w.status, s));
         return SOBEK_OK;
     }
-    CK(pack_R(p, p->fwd, 0, 1, R, w.fNKh, w.fNKl, s));
     SplitSrc xs{};
     if (geo) xs = *geo;
     if (w.oseg_r) { CK(launch_chunk_order(rv, w.chunk, kOrderPeriod, w.oseg_r, w.status, s)); xs.oseg = w.oseg_r; }
     if (w.xsh) { CK(split_features(x, g->N, p->C_x, w.xsh, w.xsl, s)); xs.h = w.xsh; xs.l = w.xsl; }
+    PackQueue pq(p);
+    pq.add(p->fwd, 0, 1, stream_order(p, p->fwd, rv, nullptr, xs, nullptr, nullptr, 0), R, w.fNKh, w.fNKl);
+    CK(pq.flush(s));
     for (int64_t n0 = 0; n0 < g->N; n0 += w.chunk) {
         const int64_t nn = std::min(w.chunk, g->N - n0);
         CK(launch_stream(p, p->fwd, rv, n0, nn, x, nullptr, xs, Y, nullptr, phi, nullptr, 0, w.zbh, w.zbl, w.status, s));
@@ -431,8 +429,9 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
     if (w.gsh && gx && !w.fused_t && !gx_direct) { fs.add(gy, g->N, p->C_y, w.gsh, w.gsl); gs.h = w.gsh; gs.l = w.gsl; }
     CK(fs.flush(s));
     PackQueue pq(p);              // every operand layout of R this call needs, one launch
-    if (gphi || gY) pq.add(p->fwd, 0, 0, R, w.fKNh, w.fKNl);
-    if (gx && !gx_direct && !w.fused_t) pq.add(p->tr, 1, 1, R, w.tNKh, w.tNKl);
+    if (gphi || gY) pq.add(p->fwd, 0, 0, nullptr, R, w.fKNh, w.fKNl);
+    if (gx && !gx_direct && !w.fused_t)
+        pq.add(p->tr, 1, 1, stream_order(p, p->tr, sender_view(g), nullptr, gs, nullptr, nullptr, 0), R, w.tNKh, w.tNKl);
     CK(pq.flush(s));
     if (gR || gphi || gY) {
         if (gR) CK(launch_fill_zero(w.gRp, KN, s));
@@ -459,7 +458,7 @@ int conv_bwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, con
                 }
             }
         }
-        if (gR) CK(unpack_R(p, p->fwd, w.gRp, gR, s));
+        if (gR) CK(unpack_R(p, p->fwd, stream_order(p, p->fwd, rv, nullptr, xs, nullptr, nullptr, 0), w.gRp, gR, s));
     }
     if (gx) {
         if (has_uncovered(p->tr)) CK(launch_fill_zero(gx, g->N * (int64_t)p->C_x, s));
@@ -539,17 +538,19 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
     }
     if (w.gsh && hx && !w.fused_t) { fs.add(gy, g->N, p->C_y, w.gsh, w.gsl); gs.h = w.gsh; gs.l = w.gsl; }
     CK(fs.flush(s));
+    const int32_t* const dz_order = stream_order(p, p->fwd, rv, vx, xs, vY, vphi, 1);
     {
         // every operand layout of R and vR this call needs, one launch (the fused schedule packs its own)
         const bool fuse_ggy = ggy && w.fused_f, fuse_dz = fuse_ggy && !hR;
         PackQueue pq(p);
-        if (ggy && any_edge_dir && !fuse_dz) pq.add(p->fwd, 0, 1, R, w.fNKh, w.fNKl);
-        if (ggy && vR && !fuse_ggy) pq.add(p->fwd, 0, 1, vR, w.vfNKh, w.vfNKl);
-        if ((hphi || hY) && any_edge_dir) pq.add(p->fwd, 0, 0, R, w.fKNh, w.fKNl);
-        if ((hphi || hY) && vR) pq.add(p->fwd, 0, 0, vR, w.vfKNh, w.vfKNl);
+        if (ggy && any_edge_dir && !fuse_dz) pq.add(p->fwd, 0, 1, dz_order, R, w.fNKh, w.fNKl);
+        if (ggy && vR && !fuse_ggy) pq.add(p->fwd, 0, 1, stream_order(p, p->fwd, rv, nullptr, xs, nullptr, nullptr, 0), vR, w.vfNKh, w.vfNKl);
+        if ((hphi || hY) && any_edge_dir) pq.add(p->fwd, 0, 0, nullptr, R, w.fKNh, w.fKNl);
+        if ((hphi || hY) && vR) pq.add(p->fwd, 0, 0, nullptr, vR, w.vfKNh, w.vfKNl);
         if (hx && !w.fused_t) {
-            if (vY || vphi) pq.add(p->tr, 1, 1, R, w.tNKh, w.tNKl);
-            if (vR) pq.add(p->tr, 1, 1, vR, w.vtNKh, w.vtNKl);
+            const EdgeView sv = sender_view(g);
+            if (vY || vphi) pq.add(p->tr, 1, 1, stream_order(p, p->tr, sv, nullptr, gs, vY, vphi, 1), R, w.tNKh, w.tNKl);
+            if (vR) pq.add(p->tr, 1, 1, stream_order(p, p->tr, sv, nullptr, gs, nullptr, nullptr, 0), vR, w.vtNKh, w.vtNKl);
         }
         CK(pq.flush(s));
     }
@@ -622,7 +623,7 @@ int conv_dbwd_core(const sobek_plan* p, const sobek_graph* g, const float* x, co
                 }
             }
         }
-        if (hR) CK(unpack_R(p, p->fwd, w.gRp, hR, s));
+        if (hR) CK(unpack_R(p, p->fwd, dz_order, w.gRp, hR, s));
     }
     if (hx) {
         if (has_uncovered(p->tr)) CK(launch_fill_zero(hx, g->N * (int64_t)p->C_x, s));

@@ -56,18 +56,29 @@ void build_stream_tasks(const sobek_plan* p, Direction& dir) {
     }
 }
 
+// tensor-core stream when the profile allows it and the caller made the bf16 copies of the sources
+static bool takes_tc(const sobek_plan* p, const float* vsrc, const SplitSrc& ss) {
+    return p->use_tc_stream && ss.h && ss.l && (!vsrc || (ss.vh && ss.vl));
+}
+static bool takes_moment(const sobek_plan* p, const Direction& dir, const EdgeView& ev, const float* vsrc, const SplitSrc& ss, const float* vY,
+                         const float* vphi, int dual) {
+    const int operands = dual && ss.vh && (ss.rvec ? ss.vrvec != nullptr : vY || vphi) ? 2 : 1;
+    return takes_tc(p, vsrc, ss) && moment_stream_pays(p, dir, dual ? 1 : 0, operands, ss.rvec != nullptr, ev.N, ev.E);
+}
+const int32_t* stream_order(const sobek_plan* p, const Direction& dir, const EdgeView& ev, const float* vsrc, const SplitSrc& ss, const float* vY,
+                            const float* vphi, int dual) {
+    return !p->uvu && takes_moment(p, dir, ev, vsrc, ss, vY, vphi, dual) ? dir.ms[dual ? 1 : 0].d_zq : nullptr;
+}
+
 cudaError_t launch_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
                           int64_t n_nodes, const float* src, const float* vsrc, const SplitSrc& ss, const float* Y,
                           const float* vY, const float* phi, const float* vphi, int dual, void* zh, void* zl,
                           int* status, cudaStream_t s) {
     if (n_nodes <= 0 || dir.stasks.empty()) return cudaSuccess;
-    // tensor-core stream when the profile allows it and the caller made the bf16 copies of the sources
-    if (p->use_tc_stream && status && ss.h && ss.l && (!vsrc || (ss.vh && ss.vl))) {
-        const int operands = dual && ss.vh && (ss.rvec ? ss.vrvec != nullptr : vY || vphi) ? 2 : 1;
-        if (moment_stream_pays(p, dir, dual ? 1 : 0, operands, ss.rvec != nullptr, ev.N, ev.E))
-            return launch_moment_stream(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
-        if (dir.tc[dual ? 1 : 0].ok) return launch_stream_tc(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
-    }
+    if (takes_moment(p, dir, ev, vsrc, ss, vY, vphi, dual))
+        return launch_moment_stream(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
+    if (takes_tc(p, vsrc, ss) && dir.tc[dual ? 1 : 0].ok)
+        return launch_stream_tc(p, dir, ev, node0, n_nodes, ss, Y, vY, phi, vphi, dual, zh, zl, status, s);
     if (ss.rvec) return cudaErrorNotSupported;      // the geometry mode exists in the tensor-core kernels only
     const int KC = p->K <= 8 ? 8 : 16;
     StreamArgsHost a{};

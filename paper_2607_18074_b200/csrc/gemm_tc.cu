@@ -25,6 +25,7 @@
 
 #include "internal.h"
 #include "ptx.cuh"
+#include "state_order.cuh"
 
 namespace sobek {
 namespace {
@@ -319,7 +320,10 @@ __global__ void k_split(const float* __restrict__ src, int64_t s_outer, int64_t 
     }
 }
 
-// several such packings (directions, layouts, R or its direction vR) in one launch: blockIdx.z picks the job
+// R[K, N_w] -> bf16 hi/lo GEMM operands of one direction, per group g:
+//   layout KN (n_major = 0): [k][c_dst] rows of length ldn_g      (B operand of Zbar = gy Rp^T)
+//   layout NK (n_major = 1): [c_dst][k] rows of length ldk_g      (B operand of y = Z Rp), k in the order of the state Z
+// Several such packings (directions, layouts, R or its direction vR) in one launch: blockIdx.z picks the job.
 struct PackJobsArg { PackJob j[kMaxPackJobs]; int K; int64_t N_w; };
 __global__ void k_pack_R_jobs(const PackJobsArg J) {
     const PackJob q = J.j[blockIdx.z];
@@ -328,7 +332,7 @@ __global__ void k_pack_R_jobs(const PackJobsArg J) {
     const int gi = q.path_group[blockIdx.y];
     const int64_t base = q.grp_off[gi];
     const int64_t ld = q.grp_ld[gi];
-    const int K = J.K;
+    const int K = J.K, zq = q.zq ? q.zq[blockIdx.y] : 1;
     __nv_bfloat16* hi = reinterpret_cast<__nv_bfloat16*>(q.hi);
     __nv_bfloat16* lo = reinterpret_cast<__nv_bfloat16*>(q.lo);
     const int64_t total = (int64_t)K * P.c_src * P.c_dst;
@@ -339,7 +343,7 @@ __global__ void k_pack_R_jobs(const PackJobsArg J) {
         const int us = (int)(r / K);
         const int u = q.transposed ? n : us, w = q.transposed ? us : n;
         const float v = q.R[(int64_t)k1 * J.N_w + P.w_off + (int64_t)u * P.c_out + w];
-        const int64_t k = (int64_t)P.koff + (int64_t)k1 * P.c_src + us;
+        const int64_t k = (int64_t)P.koff + state_pos(zq, K, P.c_src, k1, us);
         const int64_t o = q.n_major ? base + (int64_t)n * ld + k : base + k * ld + n;
         const __nv_bfloat16 h = __float2bfloat16_rn(v);
         hi[o] = h;
@@ -361,33 +365,6 @@ __global__ void k_split_jobs(const SplitJobs J) {
         const __nv_bfloat16 h = __float2bfloat16_rn(v);
         hi[r * q.ld + c] = h;
         lo[r * q.ld + c] = __float2bfloat16_rn(v - __bfloat162float(h));
-    }
-}
-
-// R[K, N_w] -> bf16 hi/lo GEMM operands of one direction, per group g:
-//   layout KN (n_major = 0): [k][c_dst] rows of length ldn_g      (B operand of Zbar = gy Rp^T)
-//   layout NK (n_major = 1): [c_dst][k] rows of length ldk_g      (B operand of y = Z Rp)
-__global__ void k_pack_R_bf16(const DPath* __restrict__ paths, const int64_t* __restrict__ grp_off,
-                              const int32_t* __restrict__ grp_ld, const int32_t* __restrict__ path_group,
-                              int transposed, int n_major, int K, int64_t N_w, const float* __restrict__ R,
-                              __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
-    const DPath P = paths[blockIdx.y];
-    const int gi = path_group[blockIdx.y];
-    const int64_t base = grp_off[gi];
-    const int64_t ld = grp_ld[gi];
-    const int64_t total = (int64_t)K * P.c_src * P.c_dst;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int n = (int)(i % P.c_dst);
-        const int64_t r = i / P.c_dst;
-        const int q = (int)(r % K);
-        const int us = (int)(r / K);
-        const int u = transposed ? n : us, w = transposed ? us : n;
-        const float v = R[(int64_t)q * N_w + P.w_off + (int64_t)u * P.c_out + w];
-        const int64_t k = (int64_t)P.koff + (int64_t)q * P.c_src + us;
-        const int64_t o = n_major ? base + (int64_t)n * ld + k : base + k * ld + n;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        hi[o] = h;
-        lo[o] = __float2bfloat16_rn(v - __bfloat162float(h));
     }
 }
 
@@ -452,10 +429,10 @@ cudaError_t launch_reduce_parts(float* dst, const float* part, int64_t n, int64_
     return cudaGetLastError();
 }
 
-void PackQueue::add(const Direction& dir, int transposed, int n_major, const float* R, void* hi, void* lo) {
+void PackQueue::add(const Direction& dir, int transposed, int n_major, const int32_t* zq, const float* R, void* hi, void* lo) {
     if (p->uvu || n >= kMaxPackJobs) { overflow = overflow || (!p->uvu && n >= kMaxPackJobs); return; }
     j[n++] = PackJob{dir.d_paths, n_major ? dir.d_nk_off : dir.d_kn_off, n_major ? dir.d_nk_ld : dir.d_kn_ld, dir.d_path_group,
-                     (int)dir.paths.size(), transposed, n_major, R, hi, lo};
+                     zq, (int)dir.paths.size(), transposed, n_major, R, hi, lo};
 }
 cudaError_t PackQueue::flush(cudaStream_t s) {
     if (overflow) return cudaErrorInvalidValue;
@@ -508,17 +485,6 @@ cudaError_t launch_split(const float* src, int64_t s_outer, int64_t s_inner, int
     const int blocks = (int)std::min<int64_t>((total + 255) / 256, 148 * 16);
     KernelTimer kt(K_PACK, s);
     k_split<<<blocks, 256, 0, s>>>(src, s_outer, s_inner, s_d, rows, cols, ld, (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
-    count_launch();
-    return cudaGetLastError();
-}
-
-cudaError_t launch_pack_R_bf16(const sobek_plan* p, const Direction& dir, int transposed, int n_major,
-                               const float* R, void* hi, void* lo, cudaStream_t s) {
-    dim3 grid(32, (unsigned)dir.paths.size());
-    KernelTimer kt(K_PACK, s);
-    k_pack_R_bf16<<<grid, 256, 0, s>>>(dir.d_paths, n_major ? dir.d_nk_off : dir.d_kn_off,
-                                       n_major ? dir.d_nk_ld : dir.d_kn_ld, dir.d_path_group, transposed, n_major,
-                                       p->K, p->N_w, R, (__nv_bfloat16*)hi, (__nv_bfloat16*)lo);
     count_launch();
     return cudaGetLastError();
 }

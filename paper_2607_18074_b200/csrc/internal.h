@@ -169,7 +169,7 @@ struct MSet {          // a run of source blocks whose gathered rows share the s
     int32_t blk_begin, nblk;
     int32_t grp_begin, ngrp;  // groups of radial indices, one after another
     int32_t nunit;            // units of all groups
-    int32_t nq;               // radial indices side by side in the columns (1, 2 or 4)
+    int32_t nq;               // radial indices side by side in the columns (1, 2, 4 or 8)
     int32_t pad[2];
 };
 struct MGrp {          // radial indices whose W is built at once, and the units that use it
@@ -191,15 +191,16 @@ struct MUnit {         // one accumulator: components of neighbouring blocks x r
     int32_t q0;               // first radial index
     int32_t c;                // multiplicities
     int32_t blk0, nblk;       // blocks, relative to the set's
-    int32_t out_begin, n_out; // state components
-    int32_t pad[4];
+    int32_t out_begin, n_out; // state components, two entries for every pair of them
+    int32_t n_pair, pair0;    // pairs, pairs in the units before it
+    int32_t pad[2];
 };
-struct MOut {          // a state component (path, o) and its coupling terms
-    int64_t a;                // state offset of radial index 0, multiplicity 0 for node 0, without the group's share:
-    int64_t zoff;             // state offset per node of the destination group
+struct alignas(16) MOut {          // a state component (path, o); c = 0: none, where a unit has an odd number of them
+    int64_t a;                // state offset of the path for node 0, without the group's share (n_nodes x zoff, added on the device)
     int32_t b;                // state elements from one node to the next
-    int32_t c_row;            // state elements from one radial index to the next
-    int32_t term, n;          // first term, terms (even)
+    int32_t c, u0;            // multiplicities of the source block, first one of this part
+    int32_t term, n;          // coupling terms of it and its neighbour in turn: the first (even), how many of each
+    int32_t zoff;             // state offset per node of the destination group
 };
 struct MTerm { uint32_t col; float coef; };      // column of the term's moment (radial index 0 of the unit), coefficient
 struct MomentSets {
@@ -211,8 +212,10 @@ struct MomentSets {
     std::vector<MOut> outs;
     std::vector<MTerm> terms;
     std::vector<uint16_t> rows;      // per row of W: radial index inside the group | harmonic << 8; padding rows repeat another
+    std::vector<int32_t> zq;         // per path: order of its state (state_pos)
     MSet* d_sets = nullptr; MGrp* d_grps = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
     uint16_t* d_rows = nullptr;
+    int32_t* d_zq = nullptr;
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;
     double node_us = 0, slot_us = 0, slot_again_us = 0;      // estimate (stream_costs): a node, 16 of its edges, the same gathered per unit
 };
@@ -422,7 +425,8 @@ cudaError_t allow_dynamic_smem(K kern) {
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
 }
 
-cudaError_t launch_unpack_R(const sobek_plan* p, const Direction& dir, const float* Rp, float* R,
+// zq: order of the state whose product with gy was accumulated (NULL: q-major)
+cudaError_t launch_unpack_R(const sobek_plan* p, const Direction& dir, const int32_t* zq, const float* Rp, float* R,
                             cudaStream_t s);
 void build_edge_tasks(const sobek_plan* p, Direction& dir);
 // receiver-owned edge pass: gphi_e = <Zbar, C_e>, gY_e = CG^T_Y(x, phi_e Zbar); with `dual` the
@@ -457,6 +461,9 @@ struct SplitSrc {
     // every chunk in the order its persistent CTAs take them (launch_chunk_order); NULL: index order
     const int4* oseg = nullptr;
 };
+// Order (state_pos, per path, on the device) of the state that launch_stream writes with these arguments; NULL: q-major
+const int32_t* stream_order(const sobek_plan* p, const Direction& dir, const EdgeView& ev, const float* vsrc, const SplitSrc& ss, const float* vY,
+                            const float* vphi, int dual);
 cudaError_t launch_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0,
                           int64_t n_nodes, const float* src, const float* vsrc, const SplitSrc& ss, const float* Y,
                           const float* vY, const float* phi, const float* vphi, int dual, void* zh, void* zl,
@@ -547,6 +554,7 @@ int64_t round8(int64_t v);
 // the packings of R (or of its direction vR) into GEMM operand layouts that one call needs, queued and run as one launch
 struct PackJob {
     const DPath* paths; const int64_t* grp_off; const int32_t* grp_ld; const int32_t* path_group;
+    const int32_t* zq;        // order of the state that the operand meets (state_pos, per path); NULL: q-major
     int n_paths, transposed, n_major;
     const float* R; void* hi; void* lo;
 };
@@ -557,9 +565,9 @@ struct PackQueue {
     int n = 0;
     bool overflow = false;
     explicit PackQueue(const sobek_plan* plan) : p(plan) {}
-    // n_major = 1: [c_dst][k] rows (B operand of y = Z Rp); 0: [k][c_dst] rows (B operand of Zbar = gy Rp^T); no-op in
-    // the channelwise mode, which has no operand copies
-    void add(const Direction& dir, int transposed, int n_major, const float* R, void* hi, void* lo);
+    // n_major = 1: [c_dst][k] rows (B operand of y = Z Rp) for a state of order zq; 0: [k][c_dst] rows (B operand of
+    // Zbar = gy Rp^T, q-major); no-op in the channelwise mode, which has no operand copies
+    void add(const Direction& dir, int transposed, int n_major, const int32_t* zq, const float* R, void* hi, void* lo);
     cudaError_t flush(cudaStream_t s);
 };
 // several fp32 -> (bf16 hi, lo) conversions with mapped source rows in one launch (see launch_split)
@@ -568,8 +576,6 @@ constexpr int kMaxSplitJobs = 8;
 cudaError_t launch_split_jobs(const SplitJob* jobs, int n, cudaStream_t s);
 cudaError_t launch_split(const float* src, int64_t s_outer, int64_t s_inner, int s_d, int64_t rows, int cols,
                          int64_t ld, void* hi, void* lo, cudaStream_t s);
-cudaError_t launch_pack_R_bf16(const sobek_plan* p, const Direction& dir, int transposed, int n_major,
-                               const float* R, void* hi, void* lo, cudaStream_t s);
 // a queue of tensor-core products that one launch runs (gemm_tc.cu); plain storage so that only gemm_tc.cu needs the
 // tensor-map type
 struct GemmBatch {

@@ -1,6 +1,6 @@
 // Device kernels of the streaming convolution (sm_100a).
 //
-//   k_pack_R<UNPACK>      : the accumulated R adjoint, kept per group as gRp_g[(pi,u,q), w],
+//   k_unpack_R            : the accumulated R adjoint, kept per group as gRp_g[(pi,u,q), w],
 //                           back into the layout of R[K, N_w]
 // (the edge stream lives in edge_stream*.cu, the receiver-owned edge pass in edge_pass.cu, the
 //  node-side contractions in gemm_tc.cu)
@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "state_order.cuh"
 
 namespace sobek {
 
@@ -120,26 +121,21 @@ __global__ void k_fill_zero(float* __restrict__ p, int64_t n) {
 }
 
 // ------------------------------------------------------------------------------------
-// R re-layout.  One blockIdx.y per path; element (us, q, n) of the path's slab:
-//   forward    : us = u (input mult.), n = w      Rp[rp_off + (koff + q*c_in  + u)*c_out + w]
-//   transposed : us = w (output mult.), n = u     Rt[rp_off + (koff + q*c_out + w)*c_in  + u]
-// both read/write R[q*N_w + w_off + u*c_out + w].
+// Packed adjoint of R back into the layout of R.  One blockIdx.y per path; element (u, q, w) of the path's slab:
+//   Rp[rp_off + (koff + state_pos(q, u))*c_out + w] -> R[q*N_w + w_off + u*c_out + w]
 // ------------------------------------------------------------------------------------
-template <bool UNPACK>
-__global__ void k_pack_R(const DPath* __restrict__ paths, int transposed, int K, int64_t N_w,
-                         const float* __restrict__ src, float* __restrict__ dst) {
+__global__ void k_unpack_R(const DPath* __restrict__ paths, const int32_t* __restrict__ zqs, int K, int64_t N_w,
+                           const float* __restrict__ src, float* __restrict__ dst) {
     const DPath P = paths[blockIdx.y];
+    const int zq = zqs ? zqs[blockIdx.y] : 1;
     const int64_t total = (int64_t)K * P.c_src * P.c_dst;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
          i += (int64_t)gridDim.x * blockDim.x) {
         const int n = (int)(i % P.c_dst);
         const int64_t r = i / P.c_dst;
         const int q = (int)(r % K);
-        const int us = (int)(r / K);
-        const int u = transposed ? n : us, w = transposed ? us : n;
-        const int64_t ri = (int64_t)q * N_w + P.w_off + (int64_t)u * P.c_out + w;
-        const int64_t pi = P.rp_off + ((int64_t)P.koff + (int64_t)q * P.c_src + us) * P.c_dst + n;
-        if (UNPACK) dst[ri] = src[pi]; else dst[pi] = src[ri];
+        const int u = (int)(r / K);
+        dst[(int64_t)q * N_w + P.w_off + (int64_t)u * P.c_out + n] = src[P.rp_off + ((int64_t)P.koff + state_pos(zq, K, P.c_src, q, u)) * P.c_dst + n];
     }
 }
 
@@ -186,11 +182,11 @@ cudaError_t launch_relayout(const float* src, float* dst, int64_t N, int C, cons
     return cudaGetLastError();
 }
 
-cudaError_t launch_unpack_R(const sobek_plan* p, const Direction& dir, const float* Rp, float* R,
+cudaError_t launch_unpack_R(const sobek_plan* p, const Direction& dir, const int32_t* zq, const float* Rp, float* R,
                             cudaStream_t s) {
     dim3 grid(32, (unsigned)dir.paths.size());
     KernelTimer kt(K_PACK, s);
-    k_pack_R<true><<<grid, 256, 0, s>>>(dir.d_paths, 0, p->K, p->N_w, Rp, R);
+    k_unpack_R<<<grid, 256, 0, s>>>(dir.d_paths, zq, p->K, p->N_w, Rp, R);
     count_launch();
     return cudaGetLastError();
 }

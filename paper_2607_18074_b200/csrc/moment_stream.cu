@@ -7,7 +7,7 @@
 
 namespace sobek {
 
-static void build_moment_set(const sobek_plan* p, Direction& dir, int dual);
+static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int& nq_max);
 static void stream_costs(Direction& dir, int dual);
 
 // Both forms of each stream of a direction; a call takes one of them (moment_stream_pays).  The moment form only in the place of
@@ -17,7 +17,7 @@ void build_stream_sets(const sobek_plan* p, Direction& dir) {
     for (int dual = 0; dual < 2; ++dual) {
         build_tc_sets(p, dir, dual);
         if (!dir.tc[dual].ok || p->form == kFormCoupled) continue;
-        build_moment_set(p, dir, dual);
+        for (int nq_max = 8; !build_moment_set(p, dir, dual, nq_max);) {}
         if (dir.ms[dual].ok) stream_costs(dir, dual);
     }
 }
@@ -81,13 +81,15 @@ bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int
     return moment < coupled;
 }
 
-static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
+// Sets, units and tables with at most nq_max radial indices side by side.  False where parts of one block came into sets with
+// different numbers of them (nq_max is then the smallest): the order of a path's state is one for all its multiplicities.
+static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int& nq_max) {
     constexpr int kSmem = 227 * 1024;
     constexpr int kSlotBytes = 37 * 1024;      // gathered rows of a slot, hi and lo, beyond which a block starts a set of its own
     constexpr int kWRows = 224;                // rows of W at a time at most (both lane halves)
     MomentSets& T = dir.ms[dual];
     T = MomentSets{};
-    if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) return;
+    if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) return true;
     bool ok = true;
     struct Pth { const DPath* P; int lb, group; };
     struct Blk { int so, c, d; std::vector<Pth> paths; };
@@ -100,7 +102,7 @@ static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
             if (it == blocks.end()) { blocks.push_back(Blk{P.src_off, P.c_src, P.d_src, {}}); it = blocks.end() - 1; }
             it->paths.push_back(Pth{&P, (P.d_sh - 1) / 2, (int)gi});
         }
-    if (!ok) return;
+    if (!ok) return true;
     std::sort(blocks.begin(), blocks.end(), [](const Blk& x, const Blk& y) { return x.so < y.so; });
     const int raw = ((dual ? 2 : 1) * (p->K + p->dim_sh) * MS_PS * 4 + 1023) & ~1023;
     // blocks of more than 64 multiplicities are cut into equal parts
@@ -133,7 +135,8 @@ static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
         const int KH = (p->K + 1) / 2;
         struct Seg { int l0, l1, row, rows; };
         std::vector<Seg> segs;
-        int nq = KH >= 3 ? 4 : KH, rows_q = 0;
+        // (eight at a time only where they fill the run: 13 radial indices or more)
+        int nq = std::min(nq_max, KH >= 7 ? 8 : KH >= 3 ? 4 : KH), rows_q = 0;
         for (; nq >= 1; nq >>= 1) {
             segs.clear(); rows_q = 0;
             bool fits = true;
@@ -204,8 +207,10 @@ static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
                 }
         }
         // read-out tables (the same for every group)
+        int pairs = 0;
         for (MUnit& U : us) {
-            U.out_begin = (int)T.outs.size();
+            struct Comp { MOut e; std::vector<MTerm> t; };
+            std::vector<Comp> comps;
             int s0 = 0;
             for (int k = 0; k < U.nblk; ++k) {
                 const Part& Pt = parts[i + U.blk0 + k];
@@ -215,32 +220,55 @@ static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
                         if (t.lb < segs[g].l0 || t.lb > segs[g].l1) continue;
                         for (int o = 0; o < t.P->d_dst; ++o) {
                             const int ld = dir.nk_ld[t.group];
-                            MOut e{(int64_t)o * ld + t.P->koff + Pt.u0, dir.zb_off[t.group], t.P->d_dst * ld, B.c, (int)T.terms.size(), 0};
+                            Comp C{MOut{(int64_t)o * ld + t.P->koff, t.P->d_dst * ld, B.c, Pt.u0, 0, 0, (int)dir.zb_off[t.group]}, {}};
                             const int col0 = segs[g].row - segs[U.pad[0]].row + (t.lb * t.lb - segs[g].l0 * segs[g].l0) * nq;
                             for (int sc = 0; sc < B.d; ++sc)
                                 for (int z = p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o]; z < p->tab_ptr[t.P->tabM + sc * t.P->d_dst + o + 1]; ++z)
-                                    T.terms.push_back(MTerm{(uint32_t)((s0 + sc) * U.N + col0 + p->tab_idx[z] * nq), p->tab_coef[z]});
-                            if ((int)T.terms.size() == e.term) T.terms.push_back(MTerm{(uint32_t)col0, 0.f});
-                            if ((T.terms.size() - e.term) & 1) T.terms.push_back(MTerm{T.terms.back().col, 0.f});
-                            e.n = (int)T.terms.size() - e.term;
-                            T.outs.push_back(e);
+                                    C.t.push_back(MTerm{(uint32_t)((s0 + sc) * U.N + col0 + p->tab_idx[z] * nq), p->tab_coef[z]});
+                            if (C.t.empty()) C.t.push_back(MTerm{(uint32_t)col0, 0.f});
+                            comps.push_back(C);
                         }
                     }
                 s0 += B.d;
             }
-            U.n_out = (int)T.outs.size() - U.out_begin;
+            // pairs of about equally many terms; the shorter one reads its last column again, times zero
+            std::stable_sort(comps.begin(), comps.end(), [](const Comp& x, const Comp& y) { return x.t.size() > y.t.size(); });
+            U.out_begin = (int)T.outs.size();
+            U.n_out = (int)comps.size();
+            U.n_pair = (U.n_out + 1) / 2;
+            U.pair0 = pairs;
+            pairs += U.n_pair;
+            for (size_t k = 0; k < comps.size(); k += 2) {
+                const Comp& A = comps[k];
+                Comp N = k + 1 < comps.size() ? comps[k + 1] : Comp{MOut{A.e.a, A.e.b, 0, 0, 0, 0, A.e.zoff}, {MTerm{A.t[0].col, 0.f}}};
+                const int first = (int)T.terms.size(), n = (int)A.t.size();
+                while (N.t.size() < A.t.size()) N.t.push_back(MTerm{N.t.back().col, 0.f});
+                for (int z = 0; z < n; ++z) { T.terms.push_back(A.t[z]); T.terms.push_back(N.t[z]); }
+                for (MOut e : {A.e, N.e}) { e.term = first; e.n = n; T.outs.push_back(e); }
+            }
         }
         for (int g = 0; g < ngrp; ++g) {
             MGrp G{};
             G.q0 = 2 * g * nqs_g * nq; G.rows = rows_h; G.row_begin = row_begin; G.unit_begin = (int)T.units.size(); G.nunit = (int)us.size();
-            for (MUnit U : us) { U.q0 += G.q0; T.units.push_back(U); }
+            for (MUnit U : us) { U.q0 += G.q0; U.pair0 += g * pairs; T.units.push_back(U); }
             T.grps.push_back(G);
         }
         S.nunit = ngrp * (int)us.size();
         T.sets.push_back(S);
         i = j;
     }
-    if (!ok) { T = MomentSets{}; return; }
+    if (!ok) { T = MomentSets{}; return true; }
+    T.zq.assign(dir.paths.size(), 0);
+    for (const MSet& S : T.sets)
+        for (int b = 0; b < S.nblk; ++b) {
+            const MBlk& B = T.blks[S.blk_begin + b];
+            for (size_t k = 0; k < dir.paths.size(); ++k) {
+                const DPath& P = dir.paths[k];
+                if (B.src_off < P.src_off || B.src_off >= P.src_off + P.c_src) continue;
+                if (T.zq[k] && T.zq[k] != S.nq) { nq_max = std::min(T.zq[k], S.nq); T = MomentSets{}; return false; }
+                T.zq[k] = S.nq;
+            }
+        }
     const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + T.sets.size() * sizeof(MSet) + T.grps.size() * sizeof(MGrp) +
                              T.blks.size() * sizeof(MBlk) + T.units.size() * sizeof(MUnit) + T.rows.size() * 2 + 64);
     const int fixed = 1024 + MS_NBAR * 8 + 16 + tables;
@@ -251,6 +279,7 @@ static void build_moment_set(const sobek_plan* p, Direction& dir, int dual) {
     if (fixed + T.ns * (T.slot_bytes + T.w_bytes) + T.w_bytes <= kSmem && T.nw < MS_MAXNW) ++T.nw;
     T.smem_bytes = fixed + T.ns * T.slot_bytes + T.nw * T.w_bytes;
     T.ok = T.ns >= 2;
+    return true;
 }
 
 cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, const EdgeView& ev, int64_t node0, int64_t n_nodes,
@@ -273,6 +302,7 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
     a.zh = (__nv_bfloat16*)zh; a.zl = (__nv_bfloat16*)zl;
     a.K = p->K; a.dsh = p->dim_sh; a.C_src = dir.C_src;
     a.x_cap = T.x_cap; a.slot_bytes = T.slot_bytes; a.ns = T.ns; a.w_bytes = T.w_bytes; a.nw = T.nw;
+    a.interleaved = p->uvu ? 0 : 1;      // (the channelwise node-side kernels read the state q-major)
     a.status = status;
     const int grid = (int)std::min<int64_t>(n_nodes * a.nsets, (int64_t)148);
     KernelTimer kt(K_STATE, s);

@@ -11,7 +11,7 @@ constexpr int MS_NDT = 4;               // drain teams (four warps each, one per
 constexpr int MS_NDW = 4 * MS_NDT;
 constexpr int MS_NLW = 4;               // loader warps
 constexpr int MS_NBW = 4;               // builder warps
-constexpr int MS_TT = (MS_NDW + MS_NLW + MS_NBW + 2) * 32;      // plus the MMA warp and the geometry warp
+constexpr int MS_TT = (MS_NDW + MS_NLW + MS_NBW + 3) * 32;      // plus the two MMA warps and the geometry warp
 constexpr int MS_MAXNS = 8;             // ring slots at most
 constexpr int MS_MAXNW = 8;             // entries of the W ring at most
 constexpr int MS_HALF = 256;            // columns of one TMEM half
@@ -47,6 +47,7 @@ struct MsArgs {
     __nv_bfloat16* zl;
     int32_t K, dsh, C_src;
     int32_t x_cap, slot_bytes, ns, w_bytes, nw;
+    int32_t interleaved;        // the state's order has zq = MSet::nq (state_pos); 0: q-major
     int* status;
 };
 

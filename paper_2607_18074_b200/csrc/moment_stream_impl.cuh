@@ -24,11 +24,14 @@
 // unit.
 //   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
 //   builder warps  W of one (group, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
-//   MMA warp       one elected lane issues the three products per component and lane half;
+//   MMA warps      one per TMEM half, each with every second unit: one elected lane issues the three products per component and lane
+//                  half.  (The steps around a slot's products take a warp about as long as the products themselves.)
 //   drain warps    four teams of four warps (one per TMEM lane quarter) that share the state components of a unit: a lane holds one
 //                  multiplicity, sums the coupling terms and writes bf16 hi / lo.  All of them work on one accumulator while the
 //                  other is filled: with a group of its own for each, the read-out took twice as long as the products and both
 //                  waited a third of the time.
+// All waits suspend their warp: polling ones took half of the issued instructions (64 x (0..2), K = 16, degree 32: 43.6 thousand
+// a node), and without them the kernel is 5 to 9 % faster.
 // With DUAL the kernel produces the directional state of the double backward (Eq. receiver_double_adjoint)
 //     dP = sum_e (vphi Y + phi vY)[q,b] x[s,u] + (phi Y)[q,b] vx[s,u]
 // as two slots per batch of edges.  The same kernel runs the sender-owned transposed traversal.  Every wait is bounded.
@@ -62,116 +65,170 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, 
 __device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
+// Two floats side by side in a register pair: one instruction works on both (each result rounded as the scalar one's).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
 // (hi, lo) bf16 split of two floats: hi pair, lo pair (element 0 in the low half)
-__device__ __forceinline__ void split2(float a, float b, uint32_t& hi, uint32_t& lo) {
+__device__ __forceinline__ void split2(uint64_t v, uint32_t& hi, uint32_t& lo) {
+    float a, b;
+    unpack2(v, a, b);
     const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
     hi = *reinterpret_cast<const uint32_t*>(&h);
-    const float ra = a - __uint_as_float(hi << 16);
-    const float rb = b - __uint_as_float(hi & 0xffff0000u);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(ra, rb);
+    unpack2(fma2(pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pack2(-1.f, -1.f), v), a, b);      // (exact)
+    const __nv_bfloat162 l = __floats2bfloat162_rn(a, b);
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// R consecutive columns of this thread's TMEM lane from each of two places, waited for
+// R consecutive columns of this thread's TMEM lane, not waited for
 template <int R>
-__device__ __forceinline__ void tm_ld_pair(uint32_t ta, uint32_t tb, float* p, float* q) {
-    if constexpr (R == 4)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%8];\n\ttcgen05.ld.sync.aligned.32x32b.x4.b32 {%4,%5,%6,%7}, [%9];\n\ttcgen05.wait::ld.sync.aligned;"
-                     : "=f"(p[0]), "=f"(p[1]), "=f"(p[2]), "=f"(p[3]), "=f"(q[0]), "=f"(q[1]), "=f"(q[2]), "=f"(q[3]) : "r"(ta), "r"(tb) : "memory");
+__device__ __forceinline__ void tm_ld(uint32_t t, float* p) {
+    if constexpr (R == 8)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=f"(p[0]), "=f"(p[1]), "=f"(p[2]), "=f"(p[3]), "=f"(p[4]), "=f"(p[5]), "=f"(p[6]), "=f"(p[7]) : "r"(t) : "memory");
+    else if constexpr (R == 4)
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=f"(p[0]), "=f"(p[1]), "=f"(p[2]), "=f"(p[3]) : "r"(t) : "memory");
     else if constexpr (R == 2)
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%4];\n\ttcgen05.ld.sync.aligned.32x32b.x2.b32 {%2,%3}, [%5];\n\ttcgen05.wait::ld.sync.aligned;"
-                     : "=f"(p[0]), "=f"(p[1]), "=f"(q[0]), "=f"(q[1]) : "r"(ta), "r"(tb) : "memory");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x2.b32 {%0,%1}, [%2];" : "=f"(p[0]), "=f"(p[1]) : "r"(t) : "memory");
     else
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%2];\n\ttcgen05.ld.sync.aligned.32x32b.x1.b32 {%1}, [%3];\n\ttcgen05.wait::ld.sync.aligned;"
-                     : "=f"(p[0]), "=f"(q[0]) : "r"(ta), "r"(tb) : "memory");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=f"(p[0]) : "r"(t) : "memory");
+}
+// acc0 and acc1 += S steps of the coupling terms at tp, {column, coefficient} of either, summed straight out of TMEM
+template <int R, int S>
+__device__ __forceinline__ void add_terms(uint32_t t, const uint4* tp, float* acc0, float* acc1) {
+    uint4 c[S];
+    float p[2 * S][R];
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+        c[s] = tp[s];
+        tm_ld<R>(t + c[s].x, p[2 * s]);
+        tm_ld<R>(t + c[s].z, p[2 * s + 1]);
+    }
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int s = 0; s < 2 * S; ++s) {
+        float* const acc = s & 1 ? acc1 : acc0;
+        const float k = __uint_as_float(s & 1 ? c[s / 2].w : c[s / 2].y);
+#pragma unroll
+        for (int r = 0; r < R; ++r) asm volatile("" : "+f"(p[s][r]));      // (no use of a loaded value moves above the wait)
+        if constexpr (R == 1) acc[0] = fmaf(k, p[s][0], acc[0]);
+        else
+#pragma unroll
+            for (int r = 0; r < R; r += 2) unpack2(fma2(pack2(k, k), pack2(p[s][r], p[s][r + 1]), pack2(acc[r], acc[r + 1])), acc[r], acc[r + 1]);
+    }
 }
 __device__ __forceinline__ void st_b32_if(uint32_t ok, void* p, uint32_t v) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p st.global.b32 [%0], %1;\n\t}" ::"l"(p), "r"(v), "r"(ok) : "memory");
 }
-
-// Read-out of a unit by one warp: every MS_NDT-th component of the state, R radial indices (columns) at a time.  The coupling
-// terms come from a table {column, coefficient} and are summed straight out of TMEM, which serves the repeated reads at a few
-// cycles each: the loop is a few dozen instructions.  (Unrolled over the terms with immediate coefficients, a function for every
-// (source order, harmonic order), the kernel took 25.4 instead of 21.2 thousand cycles a node at 64 x (0..2), K = 16, degree 32,
-// and neither more warps nor two radial indices at a time changed that.)
-// FULL: every lane and radial index of the unit is wanted.
-template <int R, bool FULL>
-__device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int64_t nl,
-                                         int team, int u, int qh) {
-    const int q0 = U.q0 + qh, n_out = U.n_out, nqs = U.nqs, rows_q = U.rows_q, Kq = FULL ? 0 : (u < U.c ? a.K : 0);
-    const uint32_t sel = u & 1 ? 0x1054u : 0x7632u;
-    __nv_bfloat16* const z0 = u & 1 ? a.zl + u - 1 : a.zh + u;
-    outs += U.out_begin;
-#pragma unroll 1
-    for (int o = team; o < n_out; o += MS_NDT) {
-        const MOut e = outs[o];
-        const uint4* const tp = reinterpret_cast<const uint4*>(terms + e.term);        // two terms per 16 bytes
-        const uint32_t step = (uint32_t)e.c_row;         // words from one radial index of this lane to the next
-        uint32_t* z = reinterpret_cast<uint32_t*>(z0 + (e.a + nl * e.b + (uint32_t)(q0 * e.c_row)));
-        const int n = full ? e.n >> 1 : 0;
-        uint32_t t = t0;
-        int q = q0;
-#pragma unroll 1
-        for (int qc = 0; qc < nqs; ++qc, t += (uint32_t)rows_q) {
-            float acc[R];
+// One component, one run of radial indices from q0 on, into the state.  A whole run of 2 R radial indices leaves in the order that a
+// lane holds it (state_pos with zq = R): 4 R bytes, one store each for the hi and the lo parts.
+template <int R>
+__device__ __forceinline__ void put_state(const MsArgs& a, const MOut& e, const float* acc, int nl, int q0, int u, int qh, bool ok) {
+    const int64_t zr = e.a + (int64_t)nl * e.b + q0 * e.c;
+    if (R > 1 && a.interleaved && q0 + 2 * R <= a.K) {
+        constexpr int W = R > 1 ? R / 2 : 1;
+        uint32_t hi[W], lo[W];
 #pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] = 0.f;
-#pragma unroll 1
-            for (int k = 0; k < n; ++k) {
-                float p0[R], p1[R];
-                const uint4 c = tp[k];
-                tm_ld_pair<R>(t + c.x, t + c.z, p0, p1);
-#pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c.y), p0[r], acc[r]);
-#pragma unroll
-                for (int r = 0; r < R; ++r) acc[r] = fmaf(__uint_as_float(c.w), p1[r], acc[r]);
+        for (int r = 0; r + 1 < R; r += 2) split2(pack2(acc[r], acc[r + 1]), hi[r / 2], lo[r / 2]);
+        const int64_t z = zr + (qh * e.c + e.u0 + u) * R;
+        if (ok) {
+            if constexpr (R == 8) {
+                *reinterpret_cast<uint4*>(a.zh + z) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                *reinterpret_cast<uint4*>(a.zl + z) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            } else if constexpr (R == 4) {
+                *reinterpret_cast<uint2*>(a.zh + z) = make_uint2(hi[0], hi[1]);
+                *reinterpret_cast<uint2*>(a.zl + z) = make_uint2(lo[0], lo[1]);
+            } else {
+                *reinterpret_cast<uint32_t*>(a.zh + z) = hi[0];
+                *reinterpret_cast<uint32_t*>(a.zl + z) = lo[0];
             }
-            // Two neighbouring lanes swap halves: the even one writes the hi, the odd one the lo parts of both multiplicities.
+        }
+    } else {
+        // q-major.  Two neighbouring lanes swap halves: the even one writes the hi, the odd one the lo parts of both multiplicities.
+        const uint32_t sel = u & 1 ? 0x1054u : 0x7632u;
+        __nv_bfloat16* z = (u & 1 ? a.zl + u - 1 : a.zh + u) + zr + e.u0 + qh * e.c;
 #pragma unroll
-            for (int r = 0; r < R; ++r) {
-                uint32_t w, x;             // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
-                asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
-                const uint32_t y = __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel);
-                if (FULL) *z = y;
-                else { st_b32_if(q < Kq, z, y); q += 2; }
-                z += step;
-            }
+        for (int r = 0; r < R; ++r) {
+            uint32_t w, x;         // the value's bf16 in the high half, zero below: its fp32 pattern; then hi and lo together
+            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(w) : "f"(acc[r]), "f"(0.f));
+            asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(x) : "f"(acc[r]), "f"(acc[r] - __uint_as_float(w)));
+            st_b32_if(ok && q0 + 2 * r + qh < a.K, z, __byte_perm(x, __shfl_xor_sync(0xffffffffu, x, 1), sel));
+            z += 2 * e.c;
         }
     }
 }
 
-// Wait of a role of several warps: its first warp polls, the others sleep at the role's barrier (25 polling warps took half of
-// the issue slots).
-__device__ __forceinline__ void role_wait(bool leader, int id, int threads, uint32_t bar, uint32_t parity, int* status) {
-    if (leader) mbar_spin(bar, parity, status);
-    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+// Read-out of a unit by one warp: every MS_NDT-th pair of components of the state, R radial indices (columns) at a time.  The coupling
+// terms come from a table; TMEM serves the repeated reads at some ten cycles each.  A warp spends its time in the latency of one
+// table entry, one TMEM read, one sum and one split after another (450 cycles a component with the terms and the stores left out), so
+// two components go side by side.  (Unrolled over the terms with immediate coefficients, a function for every (source order, harmonic
+// order), the kernel took 25.4 instead of 21.2 thousand cycles a node at 64 x (0..2), K = 16, degree 32.)
+template <int R>
+__device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int nl,
+                                         int first, int u, int qh) {
+    const int n_pair = U.n_pair, nqs = U.nqs, rows_q = U.rows_q;
+    const bool lane_ok = u < U.c;
+    outs += U.out_begin;
+#pragma unroll 1
+    for (int o = first; o < n_pair; o += MS_NDT) {
+        const MOut* const e = outs + 2 * o;
+        uint32_t t = t0;
+        int q0 = U.q0;
+#pragma unroll 1
+        for (int qc = 0; qc < nqs; ++qc, t += (uint32_t)rows_q, q0 += 2 * R) {
+            float acc0[R], acc1[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) acc0[r] = acc1[r] = 0.f;
+            const uint4* tp = reinterpret_cast<const uint4*>(terms + e->term);
+            int n = full ? e->n : 0;
+            constexpr int S = R == 8 ? 1 : 2;
+#pragma unroll 1
+            for (; n >= S; n -= S, tp += S) add_terms<R, S>(t, tp, acc0, acc1);
+            if (S > 1 && n) add_terms<R, 1>(t, tp, acc0, acc1);
+            put_state<R>(a, e[0], acc0, nl, q0, u, qh, lane_ok);
+            put_state<R>(a, e[1], acc1, nl, q0, u, qh, lane_ok && e[1].c);
+        }
+    }
 }
 
 // Every role walks the same items; the next item's bounds are requested one item ahead.
-struct MsItem { int set; int64_t nl, seg0; int len, nslot; bool resident; };
+struct MsItem { int set, nl, seg0, len, nslot; bool resident; };        // (node counts and edge counts are below 2^31)
 struct MsWalk {
     const MsArgs& a;
-    int64_t v, nl, s0, s1;
-    int set, nsub;
+    uint32_t v;
+    int nl, s0, s1, set, nsub;
     int* st;
     __device__ MsWalk(const MsArgs& a_, int nsub_, int* st_) : a(a_), nl(0), s0(0), s1(0), nsub(nsub_), st(st_) {
-        v = blockIdx.x % a.n_nodes; set = (int)(blockIdx.x / a.n_nodes);
+        v = blockIdx.x % (uint32_t)a.n_nodes; set = (int)(blockIdx.x / (uint32_t)a.n_nodes);
         fetch();
     }
     __device__ void fetch() {
         if (set >= a.nsets) return;
         if (a.oseg) { const int4 q = __ldg(a.oseg + v); nl = q.x; s0 = q.y; s1 = q.z; return; }
-        seg_bounds(a.ev.ptr, a.node0 + v, a.ev.E, st, s0, s1);
-        nl = v;
+        int64_t b, e;
+        seg_bounds(a.ev.ptr, a.node0 + v, a.ev.E, st, b, e);
+        nl = (int)v; s0 = (int)b; s1 = (int)e;
     }
     __device__ bool next(MsItem& it) {
         if (set >= a.nsets) return false;
-        it.set = set; it.nl = nl; it.seg0 = s0; it.len = nsub ? (int)(s1 - s0) : 0;
+        it.set = set; it.nl = nl; it.seg0 = s0; it.len = nsub ? s1 - s0 : 0;
         it.nslot = ((it.len + MS_TB - 1) / MS_TB) * nsub;
         it.resident = it.nslot <= min(a.ns, a.nw);
         v += gridDim.x;
-        while (v >= a.n_nodes && set < a.nsets) { v -= a.n_nodes; ++set; }
+        while (v >= (uint32_t)a.n_nodes && set < a.nsets) { v -= (uint32_t)a.n_nodes; ++set; }
         fetch();
         return true;
     }
@@ -195,7 +252,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);       // (keeps the pointer in the shared address space)
     constexpr int TB = MS_TB, PS = MS_PS, SLAB = MS_SLAB, HALF = MS_HALF;
-    constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_GEO = W_MMA + 1;
+    constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_GEO = W_MMA + 2;
     const int NS = a.ns, NW = a.nw;
     uint8_t* sRing = smem;                                            // slots: x hi, x lo, raw phi / Y (+ directions)
     uint8_t* sW = sRing + (size_t)NS * a.slot_bytes;                  // W ring: hi rows, lo rows
@@ -220,8 +277,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     const int nsub = (has_a1 ? 1 : 0) + (has_a2 ? 1 : 0);
 
     if (tid == 0) {
-        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 1); }
-        for (int s = 0; s < MS_MAXNW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 1); }
+        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 2); }
+        for (int s = 0; s < MS_MAXNW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 2); }
         for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, 4 * MS_NDT); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -238,7 +295,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     table(sBlk, a.blks, a.n_blks * (int)sizeof(MBlk)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit)); table(sRow, a.rows, a.n_rows * 2);
     for (int i = tid; i < a.n_outs; i += MS_TT) {
         MOut e = a.outs[i];
-        e.a += a.n_nodes * e.zoff;         // the groups of a chunk's state lie one after another
+        e.a += a.n_nodes * (int64_t)e.zoff;         // the groups of a chunk's state lie one after another
         sOut[i] = e;
     }
     if (warp == 0) {
@@ -254,7 +311,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // =========================== loader warps ===========================
         // A slot is filled by one warp alone, the warps take turns: a warp spends most of its time on index arithmetic, a few cycles
         // an instruction whatever the others do.  (All four on one slot: 32 x (0..2) forward 312 instead of 294 us, 128/64/64
-        // backward at degree 255, which gathers for every unit, 6.8 instead of 4.9 ms.)
+        // backward at degree 255, which gathers for every unit, 6.8 instead of 4.9 ms.  TMA gathers of four rows: 3 to 20 % slower.)
         const int me = warp - W_LOAD;
         const int le = lane & (TB - 1);
         MsWalk walk(a, nsub, a.status);
@@ -279,24 +336,24 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // Lane e < 16 holds edge e of the batch.  The ids of the next batch are requested one batch ahead and not looked at before
         // their turn: bit e of msk then says that the edge exists and that its ids are in range (an id that is not turns the
         // edge's copies into zero fills and is reported in the status word).
-        struct Ids { int64_t eid; int64_t v; bool in; };
+        struct Ids { int eid, v; bool in; };
         auto request = [&]() -> Ids {
             Ids d{0, 0, b0 + lane < it.len && lane < TB};
             if (d.in) {
-                const int64_t pos = it.seg0 + b0 + lane;
-                d.eid = a.ev.perm ? (int64_t)a.ev.perm[pos] : pos;
-                if (!a.ev.transposed) d.v = (int64_t)a.ev.col[pos];
-                else if (a.ev.recv) d.v = (int64_t)a.ev.recv[pos];
+                const int pos = it.seg0 + b0 + lane;
+                d.eid = a.ev.perm ? a.ev.perm[pos] : pos;
+                if (!a.ev.transposed) d.v = a.ev.col[pos];
+                else if (a.ev.recv) d.v = a.ev.recv[pos];
             }
             return d;
         };
-        auto settle = [&](const Ids& d, int64_t& eid, int32_t& sn) -> uint32_t {
+        auto settle = [&](const Ids& d, int& eid, int32_t& sn) -> uint32_t {
             bool ok = d.in && id_ok(d.eid, a.ev.E, a.status);
             eid = ok ? d.eid : 0; sn = 0;
             if (ok) {
-                const int64_t v = a.ev.transposed && !a.ev.recv ? owner_of(a.ev.row_ptr, a.ev.N, eid) : d.v;
+                const int v = a.ev.transposed && !a.ev.recv ? (int)owner_of(a.ev.row_ptr, a.ev.N, eid) : d.v;
                 ok = id_ok(v, a.ev.N, a.status);
-                sn = ok ? (int32_t)v : 0;
+                sn = ok ? v : 0;
             }
             return __ballot_sync(0xffffffffu, ok);
         };
@@ -326,11 +383,11 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 blk0 += U.blk0; nblk = U.nblk;
             }
             const int op = has_a1 ? sub : 1;
-            int64_t eid; int32_t sn;
+            int eid; int32_t sn;
             const uint32_t msk = settle(ids, eid, sn);
             have = to_mine(false);
             if (have) ids = request();
-            if (round_now > 0) mbar_spin(bar_sfree + 8 * st_now, (round_now & 1) ^ 1, a.status);
+            if (round_now > 0) mbar_wait(bar_sfree + 8 * st_now, (round_now & 1) ^ 1, a.status);
             const uint32_t slot_u = smem_u32(sRing + (size_t)st_now * a.slot_bytes);
             const uint32_t raw_u = slot_u + (uint32_t)(2 * a.x_cap);
             if (!a.rvec) {
@@ -394,7 +451,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 for (int b0 = 0; b0 < it.len; b0 += TB) {
                     bool okb = b0 + le < it.len;
                     int64_t ee = 0;
-                    if (okb) { const int64_t pos = it.seg0 + b0 + le; ee = a.ev.perm ? (int64_t)a.ev.perm[pos] : pos; okb = ee >= 0 && ee < a.ev.E; }
+                    if (okb) { const int pos = it.seg0 + b0 + le; ee = a.ev.perm ? a.ev.perm[pos] : pos; okb = ee >= 0 && ee < a.ev.E; }
                     float rx = 0.f, ry = 0.f, rz = 1.f;
                     if (okb) { const float* rp = a.rvec + ee * 3; rx = __ldg(rp); ry = __ldg(rp + 1); rz = __ldg(rp + 2); }
                     const float r = sqrtf(rx * rx + ry * ry + rz * rz), ir = 1.f / r;
@@ -409,7 +466,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                         tx = (vx_ - ux * uv) * ir; ty = (vy_ - uy * uv) * ir; tz = (vz_ - uz * uv) * ir;
                     }
                     for (int sub = 0; sub < nsub; ++sub) {       // the slots of the operand pairs need the same rows
-                        if (round > 0) mbar_spin(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
+                        if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
                         float* F = reinterpret_cast<float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
                         float* Yt = F + a.K * PS;
                         const int dv = (a.K + a.dsh) * PS, dsh = a.dsh;
@@ -456,8 +513,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 for (int j = 0; j < it.nslot; ++j) {
                     const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
                     if (warp == W_BUILD) {
-                        mbar_spin(bar_full + 8 * st, rd & 1, a.status);
-                        if (wr > 0) mbar_spin(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
+                        mbar_wait(bar_full + 8 * st, rd & 1, a.status);
+                        if (wr > 0) mbar_wait(bar_wfree + 8 * ws, (wr & 1) ^ 1, a.status);
                     }
                     asm volatile("bar.sync 3, %0;" ::"n"(MS_NBW * 32) : "memory");
                     const float* F = reinterpret_cast<const float*>(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap);
@@ -468,34 +525,34 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                         const int m = ((i >> 4) << 3) | (i & 7), h = (i >> 3) & 1, n = m < n_lo ? lo + m : hi + m - n_lo;
                         const uint32_t qb = rt[n];
                         const int q = min(q_first + (int)(qb & 255u), a.K - 1), b = (int)(qb >> 8);   // (indices past K: any value)
-                        float f[8], y[8], v[8];
-                        *reinterpret_cast<float4*>(f) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h);
-                        *reinterpret_cast<float4*>(f + 4) = *reinterpret_cast<const float4*>(F + q * PS + 8 * h + 4);
-                        *reinterpret_cast<float4*>(y) = *reinterpret_cast<const float4*>(Yt + b * PS + 8 * h);
-                        *reinterpret_cast<float4*>(y + 4) = *reinterpret_cast<const float4*>(Yt + b * PS + 8 * h + 4);
+                        uint64_t f[4], y[4], v[4];                 // pairs of edges
+                        auto row = [&](uint64_t* r, const float* p) {
+                            const ulonglong2 p0 = *reinterpret_cast<const ulonglong2*>(p), p1 = *reinterpret_cast<const ulonglong2*>(p + 4);
+                            r[0] = p0.x; r[1] = p0.y; r[2] = p1.x; r[3] = p1.y;
+                        };
+                        row(f, F + q * PS + 8 * h);
+                        row(y, Yt + b * PS + 8 * h);
                         if (DUAL && op == 0) {
-                            float vf[8], vy[8];
-                            *reinterpret_cast<float4*>(vf) = *reinterpret_cast<const float4*>(F + dv + q * PS + 8 * h);
-                            *reinterpret_cast<float4*>(vf + 4) = *reinterpret_cast<const float4*>(F + dv + q * PS + 8 * h + 4);
-                            *reinterpret_cast<float4*>(vy) = *reinterpret_cast<const float4*>(Yt + dv + b * PS + 8 * h);
-                            *reinterpret_cast<float4*>(vy + 4) = *reinterpret_cast<const float4*>(Yt + dv + b * PS + 8 * h + 4);
+                            uint64_t vf[4], vy[4];
+                            row(vf, F + dv + q * PS + 8 * h);
+                            row(vy, Yt + dv + b * PS + 8 * h);
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = fmaf(vf[e], y[e], f[e] * vy[e]);
+                            for (int e = 0; e < 4; ++e) v[e] = fma2(vf[e], y[e], mul2(f[e], vy[e]));
                         } else {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) v[e] = f[e] * y[e];
+                            for (int e = 0; e < 4; ++e) v[e] = mul2(f[e], y[e]);
                         }
                         uint4 hi, lo;
-                        split2(v[0], v[1], hi.x, lo.x); split2(v[2], v[3], hi.y, lo.y);
-                        split2(v[4], v[5], hi.z, lo.z); split2(v[6], v[7], hi.w, lo.w);
+                        split2(v[0], hi.x, lo.x); split2(v[1], hi.y, lo.y); split2(v[2], hi.z, lo.z); split2(v[3], hi.w, lo.w);
                         uint8_t* d = w + (n >> 3) * 256 + h * 128 + (n & 7) * 16;
                         *reinterpret_cast<uint4*>(d) = hi;
                         *reinterpret_cast<uint4*>(d + rows * 32) = lo;
                     };
                     int i = bt;
 #pragma unroll 1
-                    for (; i + NBW * 32 < 2 * (n_lo + n_hi); i += 2 * NBW * 32) { build(i); build(i + NBW * 32); }
-                    if (i < 2 * (n_lo + n_hi)) build(i);
+                    for (; !DUAL && i + NBW * 32 < 2 * (n_lo + n_hi); i += 2 * NBW * 32) { build(i); build(i + NBW * 32); }
+#pragma unroll 1
+                    for (; i < 2 * (n_lo + n_hi); i += NBW * 32) build(i);
                     fence_async_smem();
                     mbar_arrive(bar_wfull + 8 * ws);
                     if (++ws == NW) { ws = 0; ++wr; }
@@ -504,13 +561,16 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             }
             st0 = st; r0 = rd;
         }
-    } else if (warp == W_MMA) {
-        // =========================== MMA warp ===========================
+    } else if (warp == W_MMA || warp == W_MMA + 1) {
+        // =========================== MMA warps: one for each TMEM half, the units go to them in turn ===========================
+        // Both follow every slot and every entry of W: each of these is free when both have passed it, and neither arrives there a
+        // second time before it is full again.
+        const uint32_t me = __shfl_sync(0xffffffffu, (uint32_t)(warp - W_MMA), 0);
         MsWalk walk(a, nsub, nullptr);
         MsItem it{};
         int st0 = 0; uint32_t r0 = 0;
         int ws = 0; uint32_t wr = 0, ai = 0;
-        const uint32_t tm_u = __shfl_sync(0xffffffffu, tmem_base, 0);
+        const uint32_t d0 = __shfl_sync(0xffffffffu, tmem_base, 0) + me * HALF;
         const uint64_t dX0 = make_desc(smem_u32(sRing), SLAB, 1024);          // 64 multiplicities per row
         const uint64_t dW0 = make_desc_plain(smem_u32(sW), 128, 256);
         const uint32_t slot16 = (uint32_t)a.slot_bytes >> 4, w16 = (uint32_t)a.w_bytes >> 4, xlo16 = (uint32_t)a.x_cap >> 4;
@@ -519,24 +579,27 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             const int g0 = sSet[it.set].grp_begin, g1 = g0 + sSet[it.set].ngrp;
             int st = st0; uint32_t rd = r0;
             for (int gi = g0; gi < g1; ++gi) {
-                const int ws0 = ws; const uint32_t wr0 = wr;
                 const int nu = sGrp[gi].nunit, u_begin = sGrp[gi].unit_begin;
                 const uint32_t grows = __shfl_sync(0xffffffffu, (uint32_t)sGrp[gi].rows, 0);
+                // resident slots: my units of the group, one after another over the same slots and entries of W
+                const int ws0 = ws; const uint32_t wr0 = wr;
+                bool first = true;
                 for (int ui = 0; ui < nu; ++ui, ++ai) {
+                    const bool mine = (ai & 1) == me, last = it.resident ? ui + 2 >= nu : true;       // (of mine)
+                    // a unit of the other warp: its slots pass by, unless the next one is mine and finds them
+                    if (!mine && it.resident && (!first || ui + 1 < nu)) continue;
                     if (it.resident) { st = st0; rd = r0; ws = ws0; wr = wr0; }
                     const MUnit& U = sUnit[u_begin + ui];
-                    const uint32_t buf = __shfl_sync(0xffffffffu, ai & 1, 0), uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0),
-                                   ud = __shfl_sync(0xffffffffu, (uint32_t)U.d, 0),
+                    const bool xlast = last && (gi + 1 == g1 || !it.resident);
+                    const uint32_t uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0), ud = __shfl_sync(0xffffffffu, (uint32_t)U.d, 0),
                                    x0 = __shfl_sync(0xffffffffu, (uint32_t)U.slab0 * (SLAB >> 4), 0), w0 = __shfl_sync(0xffffffffu, (uint32_t)U.row0 * 2u, 0);
                     // D = F32, A = B = BF16, A MN-major, B K-major, M = 64
                     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | (4u << 24);
-                    if (ai >= 2) mbar_spin(bar_accfree + 8 * buf, ((ai >> 1) & 1) ^ 1, a.status);
-                    const uint32_t d0 = tm_u + buf * HALF;
-                    const bool wlast = ui + 1 == nu || !it.resident, xlast = (wlast && gi + 1 == g1) || !it.resident;
+                    if (mine && ai >= 2) mbar_wait(bar_accfree + 8 * me, ((ai >> 1) & 1) ^ 1, a.status);
                     for (int j = 0; j < it.nslot; ++j) {
-                        if (ui == 0 || !it.resident) {       // (later units of a group find the slot's rows and W in place)
-                            mbar_spin(bar_full + 8 * st, rd & 1, a.status);
-                            mbar_spin(bar_wfull + 8 * ws, wr & 1, a.status);
+                        if (first || !it.resident) {         // (later units of a group find the slot's rows and W in place)
+                            mbar_wait(bar_full + 8 * st, rd & 1, a.status);
+                            mbar_wait(bar_wfull + 8 * ws, wr & 1, a.status);
                             fence_async_smem();      // the gathered rows were written through the generic proxy
                         }
                         tc_fence_after();
@@ -544,16 +607,21 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                         const uint64_t dX = dX0 + (x0 + __shfl_sync(0xffffffffu, (uint32_t)st * slot16, 0)),
                                        dW = dW0 + (w0 + __shfl_sync(0xffffffffu, (uint32_t)ws * w16, 0));
                         if (elect_one()) {
-                            const uint32_t acc = j > 0 ? 1u : 0u;
-                            ms_issue(ud, d0, dX, xlo16, dW, grows * 4u, grows * 2u, uN, idesc, acc);
-                            if (wlast) tc_commit(bar_wfree + 8 * ws);
-                            if (xlast) tc_commit(bar_sfree + 8 * st);
-                            if (j + 1 == it.nslot) tc_commit(bar_accfull + 8 * buf);
+                            if (mine) {
+                                ms_issue(ud, d0, dX, xlo16, dW, grows * 4u, grows * 2u, uN, idesc, j > 0 ? 1u : 0u);
+                                if (last) tc_commit(bar_wfree + 8 * ws);
+                                if (xlast) tc_commit(bar_sfree + 8 * st);
+                                if (j + 1 == it.nslot) tc_commit(bar_accfull + 8 * me);
+                            } else {
+                                mbar_arrive(bar_wfree + 8 * ws);
+                                if (xlast) mbar_arrive(bar_sfree + 8 * st);
+                            }
                         }
                         __syncwarp();
                         if (++ws == NW) { ws = 0; ++wr; }
                         if (++st == NS) { st = 0; ++rd; }
                     }
+                    first = false;
                 }
             }
             st0 = st; r0 = rd;
@@ -572,15 +640,16 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 if (full) ++ai;
                 const MUnit& U = sUnit[u_begin + ui];
                 if (full) {
-                    role_wait(warp == 0, 1, NDW * 32, bar_accfull + 8 * buf, par, a.status);
+                    mbar_wait(bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
                 if (quarter * 16 < U.c) {
                     const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
                     const int u = quarter * 16 + (lane & 15), qh = lane >> 4;
-                    const bool all = quarter * 16 + 16 <= U.c && U.q0 + 2 * R * U.nqs <= a.K;
-#define SOBEK_READ(r) (all ? read_out<r, true>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh) : read_out<r, false>(a, U, sOut, sTerm, t0, full, it.nl, team, u, qh))
-                    if (R == 4) SOBEK_READ(4);
+                    const int first = (team - U.pair0) & (MS_NDT - 1);       // the set's pairs go to the teams in turn, across its units
+#define SOBEK_READ(r) read_out<r>(a, U, sOut, sTerm, t0, full, it.nl, first, u, qh)
+                    if (R == 8) SOBEK_READ(8);
+                    else if (R == 4) SOBEK_READ(4);
                     else if (R == 2) SOBEK_READ(2);
                     else SOBEK_READ(1);
 #undef SOBEK_READ

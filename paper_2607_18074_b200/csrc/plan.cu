@@ -553,6 +553,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
             if (e == cudaSuccess) e = upload(t.terms, &t.d_terms);
             if (e == cudaSuccess) e = upload(t.outs, &t.d_outs);
             if (e == cudaSuccess) e = upload(t.rows, &t.d_rows);
+            if (e == cudaSuccess) e = upload(t.zq, &t.d_zq);
         }
         for (TcSets* tp : {&d->tc[0], &d->tc[1], &d->etc[0], &d->etc[1]}) {
             TcSets& t = *tp;

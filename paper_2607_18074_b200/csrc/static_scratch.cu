@@ -93,7 +93,9 @@ extern "C" int sobek_conv_fwd_static(const sobek_plan* p, const sobek_graph* g, 
     for (const DGroup& G : p->fwd.groups) uncovered = uncovered || (G.path_end == G.path_begin);
     if (g->E == 0 || uncovered) CKS(launch_fill_zero(y, g->N * (int64_t)p->C_y, s));
     if (g->E == 0) return SOBEK_OK;
-    CKS(launch_pack_R_bf16(p, p->fwd, 0, 1, R, nkh, nkl, s));
+    PackQueue pq(p);
+    pq.add(p->fwd, 0, 1, nullptr, R, nkh, nkl);
+    CKS(pq.flush(s));
     const EdgeView rv{g->row_ptr, nullptr, g->col, g->row_ptr, g->N, g->E, 0};
     const Direction& dir = p->fwd;
     for (int64_t n0 = 0; n0 < g->N; n0 += chunk) {

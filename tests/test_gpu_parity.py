@@ -118,6 +118,20 @@ def test_both_forms(ir_in, ir_out, l_max, K, N, deg):
         assert nm not in both or not np.array_equal(a, b), nm
 
 
+# Orders of the state in moment form: radial indices in runs of 1 to 8 per lane, whole runs (one store a lane) and the remainder of one
+# (q-major), on multiplicities of one part and of two, of one lane quarter and of four; an odd number of state components in a unit.
+@pytest.mark.parametrize("K", [2, 3, 4, 6, 8, 10, 13, 14, 15, 16])
+@pytest.mark.parametrize("ir_in,ir_out,l_max", [("8x0e+72x1o", "64x0e+8x1o", 1), ("64x0e+24x2e", "16x0e+8x2e", 2)])
+def test_state_orders(ir_in, ir_out, l_max, K):
+    N, deg = 24, 8
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("order", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=19)
+    c = Case(w, form="moment")
+    assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
+    for got, ref, nm in zip(c.bwd() + c.dbwd(), list(c.o_bwd()) + list(c.o_dbwd()), ("gx", "gY", "gphi", "gR", "ggy", "hx", "hY", "hphi", "hR")):
+        assert rel_err(got, ref) <= BWD_TOL, nm
+
+
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg,output,form", [
     ("8x0e+8x1o+8x2e", "8x0e+8x1o+8x2e", 2, 16, 400, 4, "y", "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "y", "moment"),
     ("96x1o+96x2e", "96x0e", 2, 16, 200, 100, "y", "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "gx", "moment"),
