@@ -170,7 +170,7 @@ struct MSet {          // a run of source blocks whose gathered rows share the s
     int32_t grp_begin, ngrp;  // groups of radial indices, one after another
     int32_t nunit;            // units of all groups
     int32_t nq;               // radial indices side by side in the columns (1, 2, 4 or 8)
-    int32_t pad[2];
+    int32_t gpass, npass;     // passes over the edges of a node whose slots do not stay: two units each, of one group / of all groups
 };
 struct MGrp {          // radial indices whose W is built at once, and the units that use it
     int32_t q0, rows;         // first radial index; rows of W per lane half

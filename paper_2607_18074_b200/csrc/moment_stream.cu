@@ -254,6 +254,7 @@ static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int&
             T.grps.push_back(G);
         }
         S.nunit = ngrp * (int)us.size();
+        S.gpass = ((int)us.size() + 1) / 2; S.npass = ngrp * S.gpass;
         T.sets.push_back(S);
         i = j;
     }

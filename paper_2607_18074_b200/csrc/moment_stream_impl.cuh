@@ -21,7 +21,7 @@
 // each 32-lane quarter: the even radial indices go to the lower 16, the odd ones to the upper 16, and every lane has work in the
 // read-out.  (M = 128 for wider blocks has half the products but needs slots twice as large: 128 x (0..2) ran 3 to 17 % slower.)
 // When the slots of a node's edges all fit the rings they stay there for all units; longer segments are gathered again for every
-// unit.
+// two units, whose accumulators then fill both TMEM halves side by side (the products of such a segment outlast the read-out).
 //   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
 //   builder warps  W of one (group, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
 //   MMA warps      one per TMEM half, each with every second unit: one elected lane issues the three products per component and lane
@@ -65,34 +65,6 @@ __device__ __forceinline__ void cp_async16_zfill(uint32_t dst, const void* src, 
 __device__ __forceinline__ void cp_async4_zfill(uint32_t dst, const void* src, uint32_t bytes) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
-// Two floats side by side in a register pair: one instruction works on both (each result rounded as the scalar one's).
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-    uint64_t r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-    uint64_t r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-    uint64_t r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-// (hi, lo) bf16 split of two floats: hi pair, lo pair (element 0 in the low half)
-__device__ __forceinline__ void split2(uint64_t v, uint32_t& hi, uint32_t& lo) {
-    float a, b;
-    unpack2(v, a, b);
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    hi = *reinterpret_cast<const uint32_t*>(&h);
-    unpack2(fma2(pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pack2(-1.f, -1.f), v), a, b);      // (exact)
-    const __nv_bfloat162 l = __floats2bfloat162_rn(a, b);
-    lo = *reinterpret_cast<const uint32_t*>(&l);
-}
-
 // R consecutive columns of this thread's TMEM lane, not waited for
 template <int R>
 __device__ __forceinline__ void tm_ld(uint32_t t, float* p) {
@@ -329,7 +301,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             for (;;) {
                 if (!walk.next(it)) return false;
                 if (it.len == 0) continue;
-                rep = 0; b0 = 0; sub = 0; nrep = it.resident ? 1 : sSet[it.set].nunit;
+                rep = 0; b0 = 0; sub = 0; nrep = it.resident ? 1 : sSet[it.set].npass;
                 return true;
             }
         };
@@ -378,9 +350,12 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         while (have) {
             const int st_now = st; const uint32_t round_now = round;
             int blk0 = sSet[it.set].blk_begin, nblk = sSet[it.set].nblk;
-            if (!it.resident) {          // a unit's turn: its blocks only
-                const MUnit& U = sUnit[sGrp[sSet[it.set].grp_begin].unit_begin + rep];
-                blk0 += U.blk0; nblk = U.nblk;
+            if (!it.resident) {          // two units' turn: their blocks only (the same for every group)
+                const MGrp& G = sGrp[sSet[it.set].grp_begin];
+                const int u0 = 2 * (rep % sSet[it.set].gpass), u1 = min(u0 + 1, G.nunit - 1);
+                const MUnit& U = sUnit[G.unit_begin + u0];
+                const MUnit& V = sUnit[G.unit_begin + u1];
+                blk0 += U.blk0; nblk = V.blk0 + V.nblk - U.blk0;
             }
             const int op = has_a1 ? sub : 1;
             int eid; int32_t sn;
@@ -446,7 +421,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             int st = 0; uint32_t round = 0;
             while (walk.next(it)) {
                 if (it.len == 0) continue;
-                const int nrep = it.resident ? 1 : sSet[it.set].nunit;
+                const int nrep = it.resident ? 1 : sSet[it.set].npass;
                 for (int rep = 0; rep < nrep; ++rep)
                 for (int b0 = 0; b0 < it.len; b0 += TB) {
                     bool okb = b0 + le < it.len;
@@ -500,15 +475,17 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             const int g0 = sSet[it.set].grp_begin, g1 = g0 + sSet[it.set].ngrp;
             int st = st0; uint32_t rd = r0;
             for (int gi = g0; gi < g1; ++gi)
-            for (int ui = 0; ui < (it.resident ? 1 : sGrp[gi].nunit); ++ui) {          // resident: one W for the units of the group
+            for (int ps = 0; ps < (it.resident ? 1 : sSet[it.set].gpass); ++ps) {      // resident: one W for the units of the group
                 if (it.resident) { st = st0; rd = r0; }
                 const MGrp& G = sGrp[gi];
                 const uint16_t* rt = sRow + G.row_begin;
                 const int rows = 2 * G.rows, q_first = G.q0;
                 int lo = 0, n_lo = rows, hi = 0, n_hi = 0;                             // rows [lo, lo + n_lo) and [hi, hi + n_hi)
                 if (!it.resident) {
-                    const MUnit& U = sUnit[G.unit_begin + ui];
-                    lo = U.row0; hi = U.row0 + G.rows; n_lo = n_hi = U.N;
+                    const MUnit& U = sUnit[G.unit_begin + 2 * ps];
+                    const MUnit& V = sUnit[G.unit_begin + min(2 * ps + 1, G.nunit - 1)];
+                    lo = min(U.row0, V.row0); hi = lo + G.rows;
+                    n_lo = n_hi = max(U.row0 + U.N, V.row0 + V.N) - lo;
                 }
                 for (int j = 0; j < it.nslot; ++j) {
                     const int op = has_a1 ? (nsub == 2 ? (j & 1) : 0) : 1;
@@ -584,18 +561,20 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 // resident slots: my units of the group, one after another over the same slots and entries of W
                 const int ws0 = ws; const uint32_t wr0 = wr;
                 bool first = true;
-                for (int ui = 0; ui < nu; ++ui, ++ai) {
-                    const bool mine = (ai & 1) == me, last = it.resident ? ui + 2 >= nu : true;       // (of mine)
+                for (int ui = 0, n; ui < nu; ui += n, ai += n) {
+                    n = it.resident ? 1 : min(2, nu - ui);             // slots that do not stay: one pass for two units, one of them mine
+                    const uint32_t k = (ai ^ me) & 1, my = ai + k;
+                    const bool mine = (int)k < n, last = it.resident ? ui + 2 >= nu : true;           // (of mine)
                     // a unit of the other warp: its slots pass by, unless the next one is mine and finds them
                     if (!mine && it.resident && (!first || ui + 1 < nu)) continue;
                     if (it.resident) { st = st0; rd = r0; ws = ws0; wr = wr0; }
-                    const MUnit& U = sUnit[u_begin + ui];
+                    const MUnit& U = sUnit[u_begin + ui + (mine ? (int)k : 0)];
                     const bool xlast = last && (gi + 1 == g1 || !it.resident);
                     const uint32_t uN = __shfl_sync(0xffffffffu, (uint32_t)U.N, 0), ud = __shfl_sync(0xffffffffu, (uint32_t)U.d, 0),
                                    x0 = __shfl_sync(0xffffffffu, (uint32_t)U.slab0 * (SLAB >> 4), 0), w0 = __shfl_sync(0xffffffffu, (uint32_t)U.row0 * 2u, 0);
                     // D = F32, A = B = BF16, A MN-major, B K-major, M = 64
                     const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uN >> 3) << 17) | (4u << 24);
-                    if (mine && ai >= 2) mbar_wait(bar_accfree + 8 * me, ((ai >> 1) & 1) ^ 1, a.status);
+                    if (mine && my >= 2) mbar_wait(bar_accfree + 8 * me, ((my >> 1) & 1) ^ 1, a.status);
                     for (int j = 0; j < it.nslot; ++j) {
                         if (first || !it.resident) {         // (later units of a group find the slot's rows and W in place)
                             mbar_wait(bar_full + 8 * st, rd & 1, a.status);

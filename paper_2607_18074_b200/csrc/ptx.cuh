@@ -3,6 +3,7 @@
 // shared-memory operand descriptor.
 #pragma once
 #include <cuda.h>
+#include <cuda_bf16.h>
 #include <stdint.h>
 
 #include "sobek.h"
@@ -135,6 +136,34 @@ __device__ __forceinline__ void tc_mma_bf16_x4(uint32_t tmem_d, uint32_t tmem_s,
         "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%1], %3, %5, %6, t;\n\t}"
         ::"r"(tmem_d), "r"(tmem_s), "l"(da_hi), "l"(da_lo), "l"(db_hi), "l"(db_lo), "r"(idesc), "r"(acc_d), "r"(acc_s) : "memory");
 }
+// Two floats side by side in a register pair: one instruction works on both (each result rounded as the scalar one's).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& a, float& b) { asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+// (hi, lo) bf16 split of two floats: hi pair, lo pair (element 0 in the low half)
+__device__ __forceinline__ void split2(uint64_t v, uint32_t& hi, uint32_t& lo) {
+    float a, b;
+    unpack2(v, a, b);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    unpack2(fma2(pack2(__uint_as_float(hi << 16), __uint_as_float(hi & 0xffff0000u)), pack2(-1.f, -1.f), v), a, b);      // (exact)
+    const __nv_bfloat162 l = __floats2bfloat162_rn(a, b);
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
 // eight consecutive 32-bit columns of this thread's TMEM lane (lane = 32 * (warp % 4) + lane id)
 __device__ __forceinline__ void tc_st8(uint32_t taddr, const uint32_t* r) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
