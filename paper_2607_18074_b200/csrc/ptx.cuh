@@ -52,8 +52,7 @@ __device__ __forceinline__ void mbar_wait(uint32_t bar, uint32_t parity, int* st
     atomicExch(status, (int)SOBEK_ERR_DEVICE_TIMEOUT);
 }
 // The same without suspending the thread between polls, for waits on the critical path.  Polling warps take issue slots from the
-// others: where a role has more than a few warps one of them polls and the others sleep at a barrier (role_wait of the moment stream,
-// in which 25 polling warps took half of the slots; the edge pass in moment form lets its warps poll, each behind entries of its own).
+// others: a single warp of a kernel at most (the MMA warp of the edge pass in moment form).
 __device__ __forceinline__ void mbar_spin(uint32_t bar, uint32_t parity, int* status, uint64_t limit_ns = 2000000000ull) {
     uint64_t t0 = 0;
     for (uint32_t it = 0;; ++it) {
