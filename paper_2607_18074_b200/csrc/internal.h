@@ -170,6 +170,7 @@ struct MSet {          // a run of source blocks whose gathered rows share the s
     int32_t grp_begin, ngrp;  // groups of radial indices, one after another
     int32_t nunit;            // units of all groups
     int32_t nq;               // radial indices side by side in the columns (1, 2, 4 or 8)
+    int32_t slab_begin, nslab;   // gathered rows of an edge, one per component of a block (MSlab)
     int32_t gpass, npass;     // passes over the edges of a node whose slots do not stay: two units each, of one group / of all groups
 };
 struct MGrp {          // radial indices whose W is built at once, and the units that use it
@@ -183,6 +184,11 @@ struct MBlk {          // (part of) a source block: at most 64 multiplicities
     int32_t c_row, d_src;     // elements between consecutive components, components
     int32_t slab0;            // first slab of the block in a slot (one per component)
     int32_t pad[3];
+};
+struct MSlab {         // one component of a block: what the loaders copy of it per edge
+    int32_t off;              // first element inside a source feature row
+    int32_t chunks, mask;     // pieces of eight multiplicities; piece j of the slab's eight is piece j & mask of the row, where there is one
+    int32_t pad;
 };
 struct MUnit {         // one accumulator: components of neighbouring blocks x rows of W
     int32_t slab0, d;         // first slab, components
@@ -207,13 +213,14 @@ struct MomentSets {
     bool ok = false;
     std::vector<MSet> sets;
     std::vector<MGrp> grps;
-    std::vector<MBlk> blks;
+    std::vector<MBlk> blks;          // (host only)
+    std::vector<MSlab> slabs;
     std::vector<MUnit> units;
     std::vector<MOut> outs;
     std::vector<MTerm> terms;
     std::vector<uint16_t> rows;      // per row of W: radial index inside the group | harmonic << 8; padding rows repeat another
     std::vector<int32_t> zq;         // per path: order of its state (state_pos)
-    MSet* d_sets = nullptr; MGrp* d_grps = nullptr; MBlk* d_blks = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
+    MSet* d_sets = nullptr; MGrp* d_grps = nullptr; MSlab* d_slabs = nullptr; MUnit* d_units = nullptr; MOut* d_outs = nullptr; MTerm* d_terms = nullptr;
     uint16_t* d_rows = nullptr;
     int32_t* d_zq = nullptr;
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;

@@ -128,6 +128,13 @@ static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int&
             dmax = std::max(dmax, B.d);
         }
         S.nblk = (int)T.blks.size() - S.blk_begin;
+        // a slab has room for 64 multiplicities: rows of up to 32 (16) go in twice (four times)
+        S.slab_begin = (int)T.slabs.size(); S.nslab = slabs;
+        for (int b = S.blk_begin; b < (int)T.blks.size(); ++b)
+            for (int k = 0; k < T.blks[b].d_src; ++k) {
+                const int chunks = (T.blks[b].c + 7) / 8;
+                T.slabs.push_back(MSlab{T.blks[b].src_off + k * T.blks[b].c_row, chunks, chunks > 4 ? 7 : (chunks > 2 ? 3 : 1), 0});
+            }
         x_cap = std::max(x_cap, slabs * MS_SLAB);
         // Rows of W: runs of nq radial indices (those of one lane half), per run the harmonics order by order, the radial
         // index fastest, so that one read-out instruction takes nq of them.  The orders are cut into segments of whole
@@ -271,7 +278,7 @@ static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int&
             }
         }
     const int tables = (int)(T.outs.size() * sizeof(MOut) + T.terms.size() * sizeof(MTerm) + T.sets.size() * sizeof(MSet) + T.grps.size() * sizeof(MGrp) +
-                             T.blks.size() * sizeof(MBlk) + T.units.size() * sizeof(MUnit) + T.rows.size() * 2 + 64);
+                             T.slabs.size() * sizeof(MSlab) + T.units.size() * sizeof(MUnit) + T.rows.size() * 2 + 64);
     const int fixed = 1024 + MS_NBAR * 8 + 16 + tables;
     T.x_cap = x_cap;
     T.slot_bytes = 2 * x_cap + raw;
@@ -290,8 +297,8 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
     if (!T.ok || !ss.h || !ss.l) return cudaErrorInvalidValue;
     if (n_nodes <= 0) return cudaSuccess;
     MsArgs a{};
-    a.sets = T.d_sets; a.grps = T.d_grps; a.blks = T.d_blks; a.units = T.d_units; a.outs = T.d_outs; a.terms = T.d_terms; a.rows = T.d_rows;
-    a.nsets = (int)T.sets.size(); a.n_grps = (int)T.grps.size(); a.n_blks = (int)T.blks.size(); a.n_units = (int)T.units.size(); a.n_terms = (int)T.terms.size();
+    a.sets = T.d_sets; a.grps = T.d_grps; a.slabs = T.d_slabs; a.units = T.d_units; a.outs = T.d_outs; a.terms = T.d_terms; a.rows = T.d_rows;
+    a.nsets = (int)T.sets.size(); a.n_grps = (int)T.grps.size(); a.n_slabs = (int)T.slabs.size(); a.n_units = (int)T.units.size(); a.n_terms = (int)T.terms.size();
     a.n_outs = (int)T.outs.size(); a.n_rows = (int)T.rows.size();
     a.ev = ev; a.node0 = node0; a.n_nodes = n_nodes;
     a.oseg = ss.oseg ? ss.oseg + node0 : nullptr;

@@ -11,7 +11,7 @@ constexpr int MS_NDT = 4;               // drain teams (four warps each, one per
 constexpr int MS_NDW = 4 * MS_NDT;
 constexpr int MS_NLW = 4;               // loader warps
 constexpr int MS_NBW = 4;               // builder warps
-constexpr int MS_TT = (MS_NDW + MS_NLW + MS_NBW + 3) * 32;      // plus the two MMA warps and the geometry warp
+constexpr int MS_TT = (MS_NDW + MS_NLW + MS_NBW + 3) * 32;      // plus the two MMA warps and the edge warp
 constexpr int MS_MAXNS = 8;             // ring slots at most
 constexpr int MS_MAXNW = 8;             // entries of the W ring at most
 constexpr int MS_HALF = 256;            // columns of one TMEM half
@@ -22,12 +22,12 @@ constexpr int MS_NBAR = 2 * MS_MAXNS + 2 * MS_MAXNW + 4;
 struct MsArgs {
     const MSet* sets;
     const MGrp* grps;
-    const MBlk* blks;
+    const MSlab* slabs;
     const MUnit* units;
     const MOut* outs;
     const MTerm* terms;
     const uint16_t* rows;
-    int32_t nsets, n_grps, n_blks, n_units, n_outs, n_terms, n_rows;
+    int32_t nsets, n_grps, n_slabs, n_units, n_outs, n_terms, n_rows;
     EdgeView ev;
     int64_t node0, n_nodes;
     const int4* oseg;           // the chunk's nodes in processing order {local node, segment begin, end} or NULL

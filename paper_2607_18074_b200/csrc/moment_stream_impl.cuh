@@ -22,12 +22,14 @@
 // read-out.  (M = 128 for wider blocks has half the products but needs slots twice as large: 128 x (0..2) ran 3 to 17 % slower.)
 // When the slots of a node's edges all fit the rings they stay there for all units; longer segments are gathered again for every
 // two units, whose accumulators then fill both TMEM halves side by side (the products of such a segment outlast the read-out).
-//   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle), phi and Y (transposed) into the ring;
+//   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle) into the ring;
+//   edge warp      phi and Y (transposed) into the ring, from memory or computed from the edge vectors;
 //   builder warps  W of one (group, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
 //   MMA warps      one per TMEM half, each with every second unit: one elected lane issues the three products per component and lane
 //                  half.  (The steps around a slot's products take a warp about as long as the products themselves.)
 //   drain warps    four teams of four warps (one per TMEM lane quarter) that share the state components of a unit: a lane holds one
-//                  multiplicity, sums the coupling terms and writes bf16 hi / lo.  All of them work on one accumulator while the
+//                  multiplicity, sums the coupling terms and writes bf16 hi / lo.  Rows of up to 32 multiplicities are gathered twice
+//                  (up to 16: four times) side by side, so that no lane quarter is left without work.  All of them work on one accumulator while the
 //                  other is filled: with a group of its own for each, the read-out took twice as long as the products and both
 //                  waited a third of the time.
 // All waits suspend their warp: polling ones took half of the issued instructions (64 x (0..2), K = 16, degree 32: 43.6 thousand
@@ -143,19 +145,19 @@ __device__ __forceinline__ void put_state(const MsArgs& a, const MOut& e, const 
     }
 }
 
-// Read-out of a unit by one warp: every MS_NDT-th pair of components of the state, R radial indices (columns) at a time.  The coupling
+// Read-out of a unit by one warp: every n_team-th pair of components of the state, R radial indices (columns) at a time.  The coupling
 // terms come from a table; TMEM serves the repeated reads at some ten cycles each.  A warp spends its time in the latency of one
 // table entry, one TMEM read, one sum and one split after another (450 cycles a component with the terms and the stores left out), so
 // two components go side by side.  (Unrolled over the terms with immediate coefficients, a function for every (source order, harmonic
 // order), the kernel took 25.4 instead of 21.2 thousand cycles a node at 64 x (0..2), K = 16, degree 32.)
 template <int R>
 __device__ __forceinline__ void read_out(const MsArgs& a, const MUnit& U, const MOut* outs, const MTerm* terms, uint32_t t0, bool full, int nl,
-                                         int first, int u, int qh) {
+                                         int first, int n_team, int u, int qh) {
     const int n_pair = U.n_pair, nqs = U.nqs, rows_q = U.rows_q;
     const bool lane_ok = u < U.c;
     outs += U.out_begin;
 #pragma unroll 1
-    for (int o = first; o < n_pair; o += MS_NDT) {
+    for (int o = first; o < n_pair; o += n_team) {
         const MOut* const e = outs + 2 * o;
         uint32_t t = t0;
         int q0 = U.q0;
@@ -206,6 +208,30 @@ struct MsWalk {
     }
 };
 
+// The slots in the order in which the roles meet them: for every item its passes over the edges, for every batch its operands.
+struct MsSlots {
+    MsWalk walk;
+    MsItem it{};
+    const MSet* sets;
+    int nsub, rep = 0, nrep = 0, b0 = 0, sub = 0;
+    __device__ MsSlots(const MsArgs& a, const MSet* s, int n, int* st) : walk(a, n, st), sets(s), nsub(n) {}
+    __device__ bool first() {
+        for (;;) {
+            if (!walk.next(it)) return false;
+            if (it.len == 0) continue;
+            rep = 0; b0 = 0; sub = 0; nrep = it.resident ? 1 : sets[it.set].npass;
+            return true;
+        }
+    }
+    __device__ bool next() {
+        if (++sub < nsub) return true;
+        sub = 0; b0 += MS_TB;
+        if (b0 < it.len) return true;
+        b0 = 0;
+        return ++rep < nrep || first();
+    }
+};
+
 // The products of one slot: x_hi W_hi, x_hi W_lo, x_lo W_hi per component and lane half.  (x_hi stays in the collector for two
 // products of one lane half; a product into the other half does not find it there.)
 __device__ __forceinline__ void ms_issue(uint32_t d, uint32_t d0, uint64_t dX, uint32_t xlo16, uint64_t dW, uint32_t wlo16, uint32_t whalf16, uint32_t N,
@@ -224,7 +250,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);       // (keeps the pointer in the shared address space)
     constexpr int TB = MS_TB, PS = MS_PS, SLAB = MS_SLAB, HALF = MS_HALF;
-    constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_GEO = W_MMA + 2;
+    constexpr int NLW = MS_NLW, NBW = MS_NBW, NDW = MS_NDW, W_LOAD = NDW, W_BUILD = W_LOAD + NLW, W_MMA = W_BUILD + NBW, W_EDGE = W_MMA + 2;
     const int NS = a.ns, NW = a.nw;
     uint8_t* sRing = smem;                                            // slots: x hi, x lo, raw phi / Y (+ directions)
     uint8_t* sW = sRing + (size_t)NS * a.slot_bytes;                  // W ring: hi rows, lo rows
@@ -234,8 +260,8 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     MOut* sOut = reinterpret_cast<MOut*>(sTerm + a.n_terms);
     MSet* sSet = reinterpret_cast<MSet*>(sOut + a.n_outs);
     MGrp* sGrp = reinterpret_cast<MGrp*>(sSet + a.nsets);
-    MBlk* sBlk = reinterpret_cast<MBlk*>(sGrp + a.n_grps);
-    MUnit* sUnit = reinterpret_cast<MUnit*>(sBlk + a.n_blks);
+    MSlab* sSlab = reinterpret_cast<MSlab*>(sGrp + a.n_grps);
+    MUnit* sUnit = reinterpret_cast<MUnit*>(sSlab + a.n_slabs);
     uint16_t* sRow = reinterpret_cast<uint16_t*>(sUnit + a.n_units);
     const uint32_t bar0 = smem_u32(bars);
     const uint32_t bar_full = bar0, bar_sfree = bar0 + 8 * MS_MAXNS, bar_wfull = bar0 + 16 * MS_MAXNS, bar_wfree = bar_wfull + 8 * MS_MAXNW,
@@ -249,7 +275,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     const int nsub = (has_a1 ? 1 : 0) + (has_a2 ? 1 : 0);
 
     if (tid == 0) {
-        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, 32 + (a.rvec ? 32 : 0)); mbar_init(bar_sfree + 8 * s, 2); }
+        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, 64); mbar_init(bar_sfree + 8 * s, 2); }
         for (int s = 0; s < MS_MAXNW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 2); }
         for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, 4 * MS_NDT); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -264,7 +290,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     };
     table(sTerm, a.terms, a.n_terms * (int)sizeof(MTerm)); table(sSet, a.sets, a.nsets * (int)sizeof(MSet));
     table(sGrp, a.grps, a.n_grps * (int)sizeof(MGrp));
-    table(sBlk, a.blks, a.n_blks * (int)sizeof(MBlk)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit)); table(sRow, a.rows, a.n_rows * 2);
+    table(sSlab, a.slabs, a.n_slabs * (int)sizeof(MSlab)); table(sUnit, a.units, a.n_units * (int)sizeof(MUnit)); table(sRow, a.rows, a.n_rows * 2);
     for (int i = tid; i < a.n_outs; i += MS_TT) {
         MOut e = a.outs[i];
         e.a += a.n_nodes * (int64_t)e.zoff;         // the groups of a chunk's state lie one after another
@@ -285,49 +311,18 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // an instruction whatever the others do.  (All four on one slot: 32 x (0..2) forward 312 instead of 294 us, 128/64/64
         // backward at degree 255, which gathers for every unit, 6.8 instead of 4.9 ms.  TMA gathers of four rows: 3 to 20 % slower.)
         const int me = warp - W_LOAD;
-        const int le = lane & (TB - 1);
-        MsWalk walk(a, nsub, a.status);
-        MsItem it{};
-        int rep = 0, nrep = 0, b0 = 0, sub = 0;
-        // position of the next slot's batch; false at the end
-        auto advance = [&](bool first) -> bool {
-            if (!first) {
-                if (++sub < nsub) return true;
-                sub = 0; b0 += TB;
-                if (b0 < it.len) return true;
-                b0 = 0;
-                if (++rep < nrep) return true;
-            }
-            for (;;) {
-                if (!walk.next(it)) return false;
-                if (it.len == 0) continue;
-                rep = 0; b0 = 0; sub = 0; nrep = it.resident ? 1 : sSet[it.set].npass;
-                return true;
-            }
-        };
+        MsSlots at(a, sSet, nsub, a.status);
         // Lane e < 16 holds edge e of the batch.  The ids of the next batch are requested one batch ahead and not looked at before
-        // their turn: bit e of msk then says that the edge exists and that its ids are in range (an id that is not turns the
-        // edge's copies into zero fills and is reported in the status word).
-        struct Ids { int eid, v; bool in; };
+        // their turn (an id out of range turns the edge's copies into zero fills and is reported in the status word).
+        struct Ids { int v; bool in; };
         auto request = [&]() -> Ids {
-            Ids d{0, 0, b0 + lane < it.len && lane < TB};
+            Ids d{0, at.b0 + lane < at.it.len && lane < TB};
             if (d.in) {
-                const int pos = it.seg0 + b0 + lane;
-                d.eid = a.ev.perm ? a.ev.perm[pos] : pos;
+                const int pos = at.it.seg0 + at.b0 + lane;
                 if (!a.ev.transposed) d.v = a.ev.col[pos];
-                else if (a.ev.recv) d.v = a.ev.recv[pos];
+                else d.v = a.ev.recv ? a.ev.recv[pos] : a.ev.perm[pos];
             }
             return d;
-        };
-        auto settle = [&](const Ids& d, int& eid, int32_t& sn) -> uint32_t {
-            bool ok = d.in && id_ok(d.eid, a.ev.E, a.status);
-            eid = ok ? d.eid : 0; sn = 0;
-            if (ok) {
-                const int v = a.ev.transposed && !a.ev.recv ? (int)owner_of(a.ev.row_ptr, a.ev.N, eid) : d.v;
-                ok = id_ok(v, a.ev.N, a.status);
-                sn = ok ? v : 0;
-            }
-            return __ballot_sync(0xffffffffu, ok);
         };
         int st = 0; uint32_t round = 0;      // of the slot at hand
         // its index mod the number of warps that take part: no more than slots, so that the free barrier of a slot is never waited
@@ -335,85 +330,113 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         const int nlw = min(NLW, NS);
         int turn = 0;
         auto to_mine = [&](bool first) -> bool {
-            bool more = advance(first);
+            bool more = first ? at.first() : at.next();
             if (!first) { if (++st == NS) { st = 0; ++round; } if (++turn == nlw) turn = 0; }
             while (more && turn != me) {
-                more = advance(false);
+                more = at.next();
                 if (++st == NS) { st = 0; ++round; }
                 if (++turn == nlw) turn = 0;
             }
             return more;
         };
+        // 16 bytes = 8 multiplicities per copy: lane <-> piece j of eight rows' pieces; its four edges are lane / 8 + 0, 4, 8, 12
+        const int j = lane & 7, e0 = lane >> 3;
         bool have = me < nlw && to_mine(true);
-        Ids ids{0, 0, false};
+        Ids ids{0, false};
         if (have) ids = request();
         while (have) {
             const int st_now = st; const uint32_t round_now = round;
-            int blk0 = sSet[it.set].blk_begin, nblk = sSet[it.set].nblk;
-            if (!it.resident) {          // two units' turn: their blocks only (the same for every group)
-                const MGrp& G = sGrp[sSet[it.set].grp_begin];
-                const int u0 = 2 * (rep % sSet[it.set].gpass), u1 = min(u0 + 1, G.nunit - 1);
+            const MSet& S = sSet[at.it.set];
+            int slab0 = 0, slab1 = S.nslab;
+            if (!at.it.resident) {          // two units' turn: their slabs only (the same for every group)
+                const MGrp& G = sGrp[S.grp_begin];
+                const int u0 = 2 * (at.rep % S.gpass);
                 const MUnit& U = sUnit[G.unit_begin + u0];
-                const MUnit& V = sUnit[G.unit_begin + u1];
-                blk0 += U.blk0; nblk = V.blk0 + V.nblk - U.blk0;
+                const MUnit& V = sUnit[G.unit_begin + min(u0 + 1, G.nunit - 1)];
+                slab0 = U.slab0; slab1 = V.slab0 + V.d;
             }
-            const int op = has_a1 ? sub : 1;
-            int eid; int32_t sn;
-            const uint32_t msk = settle(ids, eid, sn);
+            const MSlab* const slabs = sSlab + S.slab_begin;
+            const int op = has_a1 ? at.sub : 1;
+            bool ok = ids.in;
+            int sn = ids.v;
+            if (ok && a.ev.transposed && !a.ev.recv) {
+                ok = id_ok(sn, a.ev.E, a.status);
+                if (ok) sn = (int)owner_of(a.ev.row_ptr, a.ev.N, sn);
+            }
+            ok = ok && id_ok(sn, a.ev.N, a.status);
+            if (!ok) sn = 0;
+            const uint32_t msk = __ballot_sync(0xffffffffu, ok);
             have = to_mine(false);
             if (have) ids = request();
             if (round_now > 0) mbar_wait(bar_sfree + 8 * st_now, (round_now & 1) ^ 1, a.status);
-            const uint32_t slot_u = smem_u32(sRing + (size_t)st_now * a.slot_bytes);
-            const uint32_t raw_u = slot_u + (uint32_t)(2 * a.x_cap);
-            if (!a.rvec) {
-                // phi and Y, transposed: thread <-> (edge le, every second radial index / harmonic)
-                const int64_t ee = __shfl_sync(0xffffffffu, eid, le);
-                const uint32_t ok = ((msk >> le) & 1u) * 4u;
-                for (int q = lane >> 4; q < a.K; q += 32 / TB) {
-                    cp_async4_zfill(raw_u + (uint32_t)(q * PS + le) * 4, a.phi + ee * a.K + q, ok);
-                    if (has_vphi) cp_async4_zfill(raw_u + (uint32_t)((a.K + a.dsh + q) * PS + le) * 4, a.vphi + ee * a.K + q, ok);
-                }
-                for (int b = lane >> 4; b < a.dsh; b += 32 / TB) {
-                    cp_async4_zfill(raw_u + (uint32_t)((a.K + b) * PS + le) * 4, a.Y + ee * a.dsh + b, ok);
-                    if (has_vY) cp_async4_zfill(raw_u + (uint32_t)((2 * a.K + a.dsh + b) * PS + le) * 4, a.vY + ee * a.dsh + b, ok);
-                }
+            const __nv_bfloat16* const baseh = op == 0 ? a.sh : a.vsh;
+            const int64_t to_lo = (op == 0 ? a.sl : a.vsl) - baseh;
+            const __nv_bfloat16* row[4];
+            uint32_t n[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                row[i] = baseh + (int64_t)__shfl_sync(0xffffffffu, sn, e0 + 4 * i) * a.C_src;
+                n[i] = ((msk >> (e0 + 4 * i)) & 1u) * 16u;
             }
-            // sender rows, hi and lo, 16 bytes = 8 multiplicities per copy: two to eight consecutive threads per row
-            const __nv_bfloat16* baseh = op == 0 ? a.sh : a.vsh;
-            const __nv_bfloat16* basel = op == 0 ? a.sl : a.vsl;
-            for (int bi = blk0; bi < blk0 + nblk; ++bi) {
-                const MBlk B = sBlk[bi];
-                const int cpr = (B.c + 7) >> 3;
-                const int lgp = cpr > 4 ? 3 : (cpr > 2 ? 2 : 1);
-                const int j = lane & ((1 << lgp) - 1), rows = 32 >> lgp;
-                const int64_t g0 = B.src_off + 8 * j;
-                const uint32_t d0 = slot_u + (uint32_t)(B.slab0 * SLAB);
+            uint32_t dst = smem_u32(sRing + (size_t)st_now * a.slot_bytes) + (uint32_t)(slab0 * SLAB + e0 * 128 + ((j ^ e0) << 4));
 #pragma unroll 1
-                for (int re0 = 0; re0 < TB; re0 += rows) {
-                    const int re = re0 + (lane >> lgp);
-                    const int32_t sne = __shfl_sync(0xffffffffu, sn, re);
-                    if (j < cpr) {
-                        const uint32_t ok = ((msk >> re) & 1u) * 16u;
-                        const int64_t g = (int64_t)sne * a.C_src + g0;
-                        uint32_t dst = d0 + (uint32_t)(re * 128 + ((j ^ (re & 7)) << 4));
-                        const __nv_bfloat16* ph = baseh + g;
-                        const __nv_bfloat16* pl = basel + g;
-#pragma unroll 3
-                        for (int s = 0; s < B.d_src; ++s) {
-                            cp_async16_zfill(dst, ph, ok);
-                            cp_async16_zfill(dst + (uint32_t)a.x_cap, pl, ok);
-                            dst += (uint32_t)SLAB; ph += B.c_row; pl += B.c_row;
-                        }
+            for (int k = slab0; k < slab1; ++k, dst += (uint32_t)SLAB) {
+                const MSlab B = slabs[k];
+                const int js = j & B.mask;
+                if (js < B.chunks) {
+                    const int off = B.off + 8 * js;
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const uint32_t d = (i & 1 ? dst ^ 64u : dst) + (uint32_t)(i * 512);
+                        cp_async16_zfill(d, row[i] + off, n[i]);
+                        cp_async16_zfill(d + (uint32_t)a.x_cap, row[i] + off + to_lo, n[i]);
                     }
                 }
             }
             // this thread's arrival on the slot's barrier fires when all its copies above have landed
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st_now) : "memory");
         }
-    } else if (warp == W_GEO) {
-        // =========================== geometry warp ===========================
-        // Walks the same slots as the loaders and fills their phi and Y rows from the edge vectors (lane <-> edge lane & 15, half
-        // of the radial indices / components each).
+    } else if (warp == W_EDGE) {
+        // =========================== edge warp ===========================
+        // Walks the same slots as the loaders and fills their phi and Y rows, transposed: from memory, or computed from the edge vectors
+        // (lane <-> edge lane & 15, half of the radial indices / harmonics each).
+        if (a.rvec == nullptr) {
+            MsSlots at(a, sSet, nsub, nullptr);
+            const int le = lane & (TB - 1), hf = lane >> 4;
+            int st = 0; uint32_t round = 0;
+            auto request = [&](bool have, bool& in) -> int {       // one slot ahead
+                in = have && at.b0 + le < at.it.len;
+                const int pos = at.it.seg0 + at.b0 + le;
+                return in && a.ev.perm ? a.ev.perm[pos] : pos;
+            };
+            bool have = at.first(), in;
+            int e = request(have, in);
+            while (have) {
+                const bool ok = in && id_ok(e, a.ev.E, a.status);
+                const int64_t ee = ok ? e : 0;
+                const uint32_t n = ok ? 4u : 0u;
+                have = at.next();
+                e = request(have, in);
+                if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
+                uint32_t d = smem_u32(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap) + (uint32_t)((hf * PS + le) * 4);
+                const uint32_t dv = (uint32_t)((a.K + a.dsh) * PS * 4);
+                const float* p = a.phi + ee * a.K;
+                const float* pv = has_vphi ? a.vphi + ee * a.K : p;
+                for (int q = hf; q < a.K; q += 2, d += 2 * PS * 4) {
+                    cp_async4_zfill(d, p + q, n);
+                    if (has_vphi) cp_async4_zfill(d + dv, pv + q, n);
+                }
+                d = smem_u32(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap) + (uint32_t)(((a.K + hf) * PS + le) * 4);
+                p = a.Y + ee * a.dsh;
+                pv = has_vY ? a.vY + ee * a.dsh : p;
+                for (int b = hf; b < a.dsh; b += 2, d += 2 * PS * 4) {
+                    cp_async4_zfill(d, p + b, n);
+                    if (has_vY) cp_async4_zfill(d + dv, pv + b, n);
+                }
+                asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st) : "memory");
+                if (++st == NS) { st = 0; ++round; }
+            }
+        }
         if (a.rvec != nullptr) {
             MsWalk walk(a, nsub, nullptr);
             MsItem it{};
@@ -622,11 +645,13 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                     mbar_wait(bar_accfull + 8 * buf, par, a.status);
                     tc_fence_after();
                 }
-                if (quarter * 16 < U.c) {
+                // rows of at most 32 (16) multiplicities lie in the slots twice (four times), and so in the lanes: twice (four times) the teams
+                const int lgq = U.c > 32 ? 2 : (U.c > 16 ? 1 : 0), lgt = 2 - lgq, qc = quarter & ((1 << lgq) - 1);
+                if (qc * 16 < U.c) {
                     const uint32_t t0 = tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * HALF;
-                    const int u = quarter * 16 + (lane & 15), qh = lane >> 4;
-                    const int first = (team - U.pair0) & (MS_NDT - 1);       // the set's pairs go to the teams in turn, across its units
-#define SOBEK_READ(r) read_out<r>(a, U, sOut, sTerm, t0, full, it.nl, first, u, qh)
+                    const int u = qc * 16 + (lane & 15), qh = lane >> 4, n_team = MS_NDT << lgt;
+                    const int first = ((team << lgt) + (quarter >> lgq) - U.pair0) & (n_team - 1);       // the set's pairs go to the teams in turn, across its units
+#define SOBEK_READ(r) read_out<r>(a, U, sOut, sTerm, t0, full, it.nl, first, n_team, u, qh)
                     if (R == 8) SOBEK_READ(8);
                     else if (R == 4) SOBEK_READ(4);
                     else if (R == 2) SOBEK_READ(2);

@@ -548,7 +548,7 @@ extern "C" int sobek_plan_create(const sobek_irrep* in, int n_in, const sobek_ir
             if (!t.ok) continue;
             if (e == cudaSuccess) e = upload(t.sets, &t.d_sets);
             if (e == cudaSuccess) e = upload(t.grps, &t.d_grps);
-            if (e == cudaSuccess) e = upload(t.blks, &t.d_blks);
+            if (e == cudaSuccess) e = upload(t.slabs, &t.d_slabs);
             if (e == cudaSuccess) e = upload(t.units, &t.d_units);
             if (e == cudaSuccess) e = upload(t.terms, &t.d_terms);
             if (e == cudaSuccess) e = upload(t.outs, &t.d_outs);
