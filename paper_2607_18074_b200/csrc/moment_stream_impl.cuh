@@ -449,7 +449,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 for (int b0 = 0; b0 < it.len; b0 += TB) {
                     bool okb = b0 + le < it.len;
                     int64_t ee = 0;
-                    if (okb) { const int pos = it.seg0 + b0 + le; ee = a.ev.perm ? a.ev.perm[pos] : pos; okb = ee >= 0 && ee < a.ev.E; }
+                    if (okb) { const int pos = it.seg0 + b0 + le; ee = a.ev.perm ? a.ev.perm[pos] : pos; okb = id_ok(ee, a.ev.E, a.status); }
                     float rx = 0.f, ry = 0.f, rz = 1.f;
                     if (okb) { const float* rp = a.rvec + ee * 3; rx = __ldg(rp); ry = __ldg(rp + 1); rz = __ldg(rp + 2); }
                     const float r = sqrtf(rx * rx + ry * ry + rz * rz), ir = 1.f / r;

@@ -89,6 +89,27 @@ def test_backward_and_position_gradient(name):
     assert all(np.array_equal(a, b) for a, b in zip((gx, g_rv, gR), again))
 
 
+@pytest.mark.parametrize("form", ["moment", "coupled"])
+@pytest.mark.parametrize("with_recv", [True, False])
+def test_stale_edge_order_is_reported(form, with_recv):
+    """A src_perm entry that is out of range when the sender-owned stream reads it ends in SOBEK_ERR_GRAPH, with the receivers of the
+    sender-sorted edges given or looked up, in the backward and in the double backward; the edge counts as none."""
+    import torch
+    c = GeoCase(CASES["cfg2_N200"], form=form)
+    sb, i = c.sb, c.plan.info
+    v_rvec = torch.from_numpy(np.random.default_rng(3).standard_normal((c.E, 3)).astype(np.float32)).to("cuda:0")
+    for pos, bad, status in ((3, c.E + 5, -4), (c.E - 1, -7, -4), (0, int(c.src_perm[0]), 0)):
+        perm = c.src_perm.clone()
+        perm[pos] = bad
+        g = sb.make_graph(c.row_ptr, c.col, c.src_ptr, perm, c.src_recv if with_recv else None)
+        gx, hx = c._new(c.N, i.C_x), c._new(c.N, i.C_x)
+        sb.conv_geo_bwd(c.plan, g, c.rvec, c.basis, c.w.r_c, 6, c.x, c.R, c.gy, gx, None, None, c.ws(1))
+        assert sb.last_device_status(c.ws(1)) == status, (pos, bad)
+        sb.conv_geo_dbwd(c.plan, g, c.rvec, c.basis, c.w.r_c, 6, c.x, c.R, c.gy, None, v_rvec, None, None, hx, None, c.ws(2))
+        assert sb.last_device_status(c.ws(2)) == status, (pos, bad)
+        assert torch.isfinite(gx).all() and torch.isfinite(hx).all()
+
+
 FULL = {"cfg3": (synth.config("cfg3"), 6), "cfg4_1e6": (synth.config("cfg4", edges=1e6), 8), "cfg5": (synth.config("cfg5"), 3)}
 
 
