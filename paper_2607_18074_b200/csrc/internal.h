@@ -161,7 +161,8 @@ struct TcSets {
     int32_t ring_stages = 2;          // stream: stages of the shared-memory ring (as many as fit)
     int32_t nbuf = 2;                 // stream: accumulator buffers in tensor memory (2, or 1 for wider sets)
     int32_t smem_bytes = 0, ctas_per_sm = 1;
-    double node_us = 0, slot_us = 0;      // streams with a moment form beside them: estimate (stream_costs) of a node, of 16 of its edges
+    // streams with a moment form beside them: estimate (stream_costs) of a node, of 16 of its edges, of the same for a second operand
+    double node_us = 0, slot_us = 0, slot2_us = 0;
 };
 
 // --- moment-form edge stream (moment_stream.cu) --------------------------------------------
@@ -224,7 +225,8 @@ struct MomentSets {
     uint16_t* d_rows = nullptr;
     int32_t* d_zq = nullptr;
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;
-    double node_us = 0, slot_us = 0, slot_again_us = 0;      // estimate (stream_costs): a node, 16 of its edges, the same gathered per unit
+    // estimate (stream_costs): a node; 16 of its edges, and the passes over them, where its slots stay / where they do not
+    double node_us = 0, slot_us[2] = {0, 0}, passes[2] = {0, 0};
 };
 
 // --- moment-form edge pass (moment_edge.cu) ------------------------------------------------

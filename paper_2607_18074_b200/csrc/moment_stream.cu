@@ -8,7 +8,7 @@
 namespace sobek {
 
 static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int& nq_max);
-static void stream_costs(Direction& dir, int dual);
+static void stream_costs(const sobek_plan* p, Direction& dir, int dual);
 
 // Both forms of each stream of a direction; a call takes one of them (moment_stream_pays).  The moment form only in the place of
 // k_stream_tc: a profile that k_stream_tc does not fit keeps the FP32-pipe stream, whose rows and coupling values have 32 bits (error
@@ -18,65 +18,95 @@ void build_stream_sets(const sobek_plan* p, Direction& dir) {
         build_tc_sets(p, dir, dual);
         if (!dir.tc[dual].ok || p->form == kFormCoupled) continue;
         for (int nq_max = 8; !build_moment_set(p, dir, dual, nq_max);) {}
-        if (dir.ms[dual].ok) stream_costs(dir, dual);
+        if (dir.ms[dual].ok) stream_costs(p, dir, dual);
     }
 }
 
-// Microseconds that one SM spends on a node and on 16 of its edges in either form, from the counts of the forms' tables.  The
-// constants are least-squares fits (of relative errors, 10 - 13 % left) to the streams of 720 random layers, 8 to 128 multiplicities
-// of orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes, in both directions.  With them the slower form is taken where
-// the two are close: the chosen form takes 0.7 % longer than the faster one on average (0.5 % in the dual streams), 23 % (35 %) at
-// worst longer than the other.  (Rules on K, order and width alone, from graphs of degree 30: 6.2 % and 8.2 %, up to 2.8 times as
-// long.  Fixed forms: moment 8 %, coupled 26 to 36 %.)
-static void stream_costs(Direction& dir, int dual) {
+// Microseconds of either form, from the counts of the forms' tables: a launch, and on one SM a node and 16 of its edges, which the roles
+// work at side by side: (a^p + b^p)^(1/p).  The constants are least-squares fits (of relative errors; 10 and 13 % left, dual 11 and 14 %)
+// to the streams of 7,288 random layers, 8 to 128 multiplicities of orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes, in
+// both directions.  On the half of the layers that a fit to the other half did not see the form taken is 0.4 % above the faster one on
+// average (dual streams: 0.2 %), at worst 1.5 times the coupled one; fixed forms: moment 4.6 % (2.3 %), coupled 44 % (64 %).
+struct StreamFit {
+    double launch, p;                                         // moment form
+    double unit, pair, val, part, set;                        //   node: units, pairs of components per team and run, their radial indices, those of runs not whole
+    double kcycle, w, row, pass, slot_unit;                   //   slot: products, rows of W, gathered slabs, passes, units
+    double c_launch, c_p;                                     // coupled form (1: with one accumulator buffer, on top)
+    double c_col, c_col1, c_node_set;                         //   node: accumulator columns, sets
+    double c_slab, c_row, c_set, c_slab1, c_set1;             //   batch: built operand, gathered rows, hand-over
+    double c2_slab, c2_row, c2_set, c2_set1;                  //   its second operand
+    double geo[5], c_geo[5];                                  // phi and Y of a slot from edge vectors: constant, per radial index, per harmonic; p; launch
+};
+constexpr StreamFit kFit[2] = {
+    {9.87, 1.47, 0.554, 0.401, 0.0257, 0.0503, 0.341, 0.171, 0.00214, 0.0197, 0.221, 0.143,
+     14.6, 1.87, 0.0203, 0.00446, 0.342, 0.182, 0.0459, 0.9, 0.0318, 0.187, 0, 0, 0, 0, {1.2, 0.0477, 0, 4.78, 7.86}, {1.1, 0.0651, 0.00335, 12.5, 8.79}},
+    {10.8, 1.35, 0.561, 0.389, 0.0395, 0.0472, 0.329, 0.172, 0.00289, 0.0104, 0.332, 0.0798,
+     15.5, 1.47, 0.0187, 0.00483, 0.465, 0.268, 0.0263, 1.1, 0.0267, 0.0754, 0.159, 0.049, 1.01, 0.155, {1.67, 0.18, 0.00331, 1.48, 4.43}, {1.53, 0.14, 0.0324, 3.95, 12.7}}};
+static double side_by_side(double a, double b, double p) { return std::pow(std::pow(a, p) + std::pow(b, p), 1 / p); }
+
+static void stream_costs(const sobek_plan* p, Direction& dir, int dual) {
+    const StreamFit& F = kFit[dual];
     TcSets& T = dir.tc[dual];
     MomentSets& M = dir.ms[dual];
     double cols = 0, slabs = 0, rows = 0;
+    const double sets = (double)T.sets.size(), one = T.nbuf == 1 ? 1 : 0;
     for (const TSet& S : T.sets) {
         slabs += S.nslab;
         for (int u = 0; u < S.nunit; ++u) cols += (T.blks[T.units[S.unit_begin + u].blk].ncols + 31) & ~31;
         for (int b = 0; b < S.nblk; ++b) rows += T.blks[S.blk_begin + b].d_src * ((T.blks[S.blk_begin + b].c_src + 63) / 64);
     }
-    T.node_us = dual ? 0.0146 * cols : 0.0144 * cols;                                        // read-out of the accumulators
-    T.slot_us = dual ? 0.2 * slabs + 0.023 * rows + 1.04 * T.sets.size()                     // built operand; gathered rows; hand-over
-                     : 0.1375 * slabs + 0.04 * rows + 0.87 * T.sets.size();
-    double units = 0, outs = 0, vals = 0, terms = 0, kcycles = 0, w_once = 0, w_again = 0, rows_once = 0, rows_again = 0;
+    T.node_us = (F.c_col + one * F.c_col1) * cols + F.c_node_set * sets;
+    T.slot_us = (F.c_slab + one * F.c_slab1) * slabs + F.c_row * rows + (F.c_set + one * F.c_set1) * sets;
+    T.slot2_us = F.c2_slab * slabs + F.c2_row * rows + (F.c2_set + one * F.c2_set1) * sets;
+    double units = 0, pairs = 0, vals = 0, part = 0, kcycles = 0, w[2] = {0, 0}, gathered[2] = {0, 0}, passes[2] = {0, 0};      // [1]: slots that do not stay
     for (const MSet& S : M.sets) {
-        for (int b = 0; b < S.nblk; ++b) rows_once += M.blks[S.blk_begin + b].d_src;
+        gathered[0] += S.nslab; passes[0] += 1; passes[1] += S.npass;
         for (int g = 0; g < S.ngrp; ++g) {
             const MGrp& G = M.grps[S.grp_begin + g];
-            w_once += 2 * G.rows;
+            w[0] += 2 * G.rows;
             for (int u = 0; u < G.nunit; ++u) {
                 const MUnit& U = M.units[G.unit_begin + u];
-                units += 1;
-                kcycles += 6e-3 * U.d * std::max(41.0, U.N / 2.0);                           // six products per component, at least 41 cycles each
-                w_again += 2 * U.N;
-                for (int b = 0; b < U.nblk; ++b) rows_again += M.blks[S.blk_begin + U.blk0 + b].d_src;
-                for (int o = 0; o < U.n_out; ++o) {
-                    outs += U.nqs; vals += U.nqs * S.nq; terms += 0.5 * U.nqs * M.outs[U.out_begin + o].n;
-                }
+                const double team = (double)U.n_pair / (U.c > 32 ? MS_NDT : U.c > 16 ? 2 * MS_NDT : 4 * MS_NDT);
+                units += 1; pairs += U.nqs * team; vals += U.nqs * S.nq * team;
+                for (int r = 1; r <= U.nqs; ++r)
+                    if (U.q0 + 2 * S.nq * r > p->K) part += S.nq * team;
+                kcycles += 6e-3 * U.d * std::max(41.0, U.N / 2.0);           // six products per component, at least 41 cycles each
+                if (u & 1) continue;
+                const MUnit& V = M.units[G.unit_begin + std::min(u + 1, G.nunit - 1)];               // two units' pass
+                w[1] += 2 * (std::max(U.row0 + U.N, V.row0 + V.N) - std::min(U.row0, V.row0));
+                gathered[1] += V.slab0 + V.d - U.slab0;
             }
         }
     }
-    M.node_us = dual ? 0.557 * units + 0.0416 * outs + 0.0068 * vals : 0.513 * units + 0.0406 * outs + 0.0057 * vals + 0.0053 * terms;
-    const double w = dual ? 0.0044 : 0.0031, r = dual ? 0.071 : 0.0535, c = (dual ? 0.133 : 0.171) * kcycles;
-    M.slot_us = c + w * w_once + r * rows_once;
-    M.slot_again_us = c + w * w_again + r * rows_again;                                      // rows and W anew for every unit
+    M.node_us = F.unit * units + F.pair * pairs + F.val * vals + F.part * part + F.set * M.sets.size();
+    for (int k = 0; k < 2; ++k) {
+        M.slot_us[k] = F.kcycle * kcycles + F.w * w[k] + F.row * gathered[k] + F.pass * passes[k] + F.slot_unit * units;
+        M.passes[k] = passes[k];
+    }
 }
 
-// With the edge inputs computed from vectors (geo) one warp of either kernel makes the rows of every slot, 1.7 us for 16 edges, and the
-// moment form needs them again for every unit of a node that is not resident.  (250 random layers, both directions: 1.5 % above the
-// faster form, at worst 1.2 times the coupled one; without it 2.0 %, 1.9 times, at degrees from 150 on.)
+// The slots of a node stay for all its units where they all fit the rings; the rows of the others are gathered, and their W built, for
+// every two units.  Degrees spread around their mean: the share of the latter falls from all to none where the longest node that stays
+// has 0.7 to 1.5 times the mean.  Below four nodes per SM the longest ones decide.  With the edge inputs computed from vectors (geo) one
+// warp of either kernel makes the rows of every slot in every pass, a bound of its own.  (Of such layers that the fit did not see: 0.5 %
+// above the faster form on average, dual streams 1.0 %, at worst 1.4 and 2.0 times the coupled one; moment throughout 7 % and 31 %.)
 bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, bool geo, int64_t N, int64_t E) {
+    const StreamFit& F = kFit[dual];
     const TcSets& T = dir.tc[dual];
     const MomentSets& M = dir.ms[dual];
     if (!M.ok || p->form != kFormAuto) return M.ok && p->form == kFormMoment;
-    const double deg = (double)E / (double)std::max<int64_t>(N, 1), slots = (deg / MS_TB + 0.5) * operands;
-    const bool resident = std::ceil(deg / MS_TB + 0.3) * operands <= std::min(M.ns, M.nw);   // (degrees spread around their mean)
-    double moment = M.node_us + slots * (resident ? M.slot_us : M.slot_again_us), coupled = T.node_us + slots * T.slot_us;
+    const double mean = (double)E / (double)std::max<int64_t>(N, 1), per_sm = std::max(1.0, (double)N / 148.0);
+    const bool few = per_sm < 4;
+    const double batches = (few ? 1.3 : 1.0) * mean / MS_TB + 0.5, slots = batches * operands;
+    const double longest = MS_TB * (double)(std::min(M.ns, M.nw) / operands), over = 1.5 * mean - longest;
+    const double again = few ? (over > 0 ? 1 : 0) : std::min(1.0, std::max(0.0, over / (0.8 * mean)));
+    auto mix = [&](const double* v) { return v[0] + again * (v[1] - v[0]); };
+    double moment = F.launch + per_sm * side_by_side(M.node_us, slots * mix(M.slot_us), F.p),
+           coupled = F.c_launch + per_sm * side_by_side(T.node_us, batches * (T.slot_us + (operands - 1) * T.slot2_us), F.c_p);
     if (geo) {
-        moment = std::max(moment, 1.7 * slots * (double)(resident ? M.sets.size() : M.units.size()));
-        coupled = std::max(coupled, 1.7 * slots * (double)T.sets.size());
+        auto rows = [&](const double* g, double passes) { return g[4] + per_sm * slots * passes * (g[0] + g[1] * p->K + g[2] * p->dim_sh); };
+        moment = side_by_side(moment, rows(F.geo, mix(M.passes)), F.geo[3]);
+        coupled = side_by_side(coupled, rows(F.c_geo, (double)T.sets.size()), F.c_geo[3]);
     }
     return moment < coupled;
 }

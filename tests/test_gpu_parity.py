@@ -133,11 +133,16 @@ def test_state_orders(ir_in, ir_out, l_max, K):
 
 
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg,output,form", [
-    ("8x0e+8x1o+8x2e", "8x0e+8x1o+8x2e", 2, 16, 400, 4, "y", "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "y", "moment"),
-    ("96x1o+96x2e", "96x0e", 2, 16, 200, 100, "y", "coupled"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "gx", "moment"),
-    ("96x1o+96x2e+96x3o", "96x0e", 3, 10, 160, 90, "ggy", "coupled"), ("64x0e+64x1o+64x2e", "64x0e+64x1o+64x2e", 2, 8, 160, 20, "ggy", "moment")])
+    ("8x0e+8x1o+8x2e", "8x0e+8x1o+8x2e", 2, 16, 400, 4, "y", "moment"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "y", "moment"),
+    ("96x1o+96x2e", "96x0e", 2, 16, 200, 100, "y", "moment"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "gx", "moment"),
+    ("96x1o+96x2e+96x3o", "96x0e", 3, 10, 160, 90, "ggy", "coupled"), ("64x0e+64x1o+64x2e", "64x0e+64x1o+64x2e", 2, 8, 160, 20, "ggy", "moment"),
+    ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 9, 123, 60, "y", "moment"), ("128x0e+128x1o+128x2e", "128x0e+128x1o+128x2e", 2, 8, 198, 99, "ggy", "moment"),
+    ("80x0e+80x1o+80x2e+80x3o+80x4e", "80x0e+80x1o+80x2e+80x3o+80x4e", 4, 13, 92, 7, "y", "coupled"), ("80x2e", "80x0e+80x4e", 4, 16, 146, 73, "gx", "coupled"),
+    ("128x0e+128x1o+128x2e+128x3o", "128x1o", 4, 10, 160, 80, "ggy", "coupled")])
 def test_stream_takes_the_form_that_pays(ir_in, ir_out, l_max, K, N, deg, output, form):
-    """Degrees and shapes at which one form of the stream takes at most 0.8 of the other's time: the default plan has its bits."""
+    """Degrees and shapes at which one form of the stream takes at most 0.8 of the other's time (96 x (1..3) -> 96 x 0: 0.88): the default
+    plan has its bits.  Microseconds of the moment form / of the coupled one, in this order: 21 / 33, 19 / 32, 44 / 67, 19 / 32, 169 / 149,
+    24 / 42, 25 / 45, 84 / 156, 122 / 67, 135 / 71, 320 / 160."""
     L = 4.0 * (N / 60.0) ** (1 / 3)
     w = synth.Workload("pays", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=31)
     c = Case(w)
