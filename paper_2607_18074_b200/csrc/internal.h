@@ -225,6 +225,7 @@ struct MomentSets {
     uint16_t* d_rows = nullptr;
     int32_t* d_zq = nullptr;
     int32_t x_cap = 0, slot_bytes = 0, ns = 0, nw = 0, w_bytes = 0, smem_bytes = 0;
+    bool loaders_edge = false;       // phi and Y by the loader warps
     // estimate (stream_costs): a node; 16 of its edges, and the passes over them, where its slots stay / where they do not
     double node_us = 0, slot_us[2] = {0, 0}, passes[2] = {0, 0};
 };

@@ -316,6 +316,11 @@ static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int&
     T.ns = T.nw = std::min(std::min(MS_MAXNS, MS_MAXNW), (kSmem - fixed) / (T.slot_bytes + T.w_bytes));
     if (fixed + T.ns * (T.slot_bytes + T.w_bytes) + T.w_bytes <= kSmem && T.nw < MS_MAXNW) ++T.nw;
     T.smem_bytes = fixed + T.ns * T.slot_bytes + T.nw * T.w_bytes;
+    // Where the loaders are to copy phi and Y: at most twelve state components a set.  (2,000 random layers of 600 nodes and more, loaders
+    // against edge warp: 1.5 to 15 % faster up to twelve; 21 to 30 components 0.2 to 0.5 % slower, above 30 0.5 to 1.4 %.)
+    int n_out = 0;
+    for (const MUnit& U : T.units) n_out += U.n_out;
+    T.loaders_edge = n_out <= 12 * (int)T.sets.size();
     T.ok = T.ns >= 2;
     return true;
 }
@@ -344,7 +349,8 @@ cudaError_t launch_moment_stream(const sobek_plan* p, const Direction& dir, cons
     a.status = status;
     const int grid = (int)std::min<int64_t>(n_nodes * a.nsets, (int64_t)148);
     KernelTimer kt(K_STATE, s);
-    const cudaError_t e = dual ? moment_stream_dual(a, grid, T.smem_bytes, s) : moment_stream_plain(a, grid, T.smem_bytes, s);
+    const bool le = T.loaders_edge && !a.rvec && n_nodes >= 4 * 148;      // (a node or two per SM: two warps side by side, 26.7 against 27.8 us a call at 64 nodes)
+    const cudaError_t e = dual ? moment_stream_dual(a, grid, T.smem_bytes, le, s) : moment_stream_plain(a, grid, T.smem_bytes, le, s);
     count_launch();
     return e;
 }

@@ -51,7 +51,7 @@ struct MsArgs {
     int* status;
 };
 
-cudaError_t moment_stream_plain(const MsArgs& a, int grid, int smem, cudaStream_t s);
-cudaError_t moment_stream_dual(const MsArgs& a, int grid, int smem, cudaStream_t s);
+cudaError_t moment_stream_plain(const MsArgs& a, int grid, int smem, bool loaders_edge, cudaStream_t s);
+cudaError_t moment_stream_dual(const MsArgs& a, int grid, int smem, bool loaders_edge, cudaStream_t s);
 
 }  // namespace sobek

@@ -23,7 +23,7 @@
 // When the slots of a node's edges all fit the rings they stay there for all units; longer segments are gathered again for every
 // two units, whose accumulators then fill both TMEM halves side by side (the products of such a segment outlast the read-out).
 //   loader warps   cp.async of the sender rows (MN-major, 128-byte swizzle) into the ring;
-//   edge warp      phi and Y (transposed) into the ring, from memory or computed from the edge vectors;
+//   edge warp      phi and Y (transposed) into the ring, from memory or computed from the edge vectors (LE: the loader warps, from memory);
 //   builder warps  W of one (group, slot): thread <-> (row (q,b), eight edges), bf16 hi / lo, K-major;
 //   MMA warps      one per TMEM half, each with every second unit: one elected lane issues the three products per component and lane
 //                  half.  (The steps around a slot's products take a warp about as long as the products themselves.)
@@ -245,7 +245,30 @@ __device__ __forceinline__ void ms_issue(uint32_t d, uint32_t d0, uint64_t dX, u
         }
 }
 
+// phi and Y (and their directions) of edge ee into a slot's transposed rows, every second radial index and harmonic from hf on
 template <bool DUAL>
+__device__ __forceinline__ void ms_edge_rows(const MsArgs& a, uint32_t raw, int64_t ee, uint32_t n, bool has_vphi, bool has_vY, int le, int hf) {
+    uint32_t d = raw + (uint32_t)((hf * MS_PS + le) * 4);
+    const uint32_t dv = (uint32_t)((a.K + a.dsh) * MS_PS * 4);
+    const float* p = a.phi + ee * a.K;
+    const float* pv = DUAL && has_vphi ? a.vphi + ee * a.K : p;
+    for (int q = hf; q < a.K; q += 2, d += 2 * MS_PS * 4) {
+        cp_async4_zfill(d, p + q, n);
+        if (DUAL && has_vphi) cp_async4_zfill(d + dv, pv + q, n);
+    }
+    d = raw + (uint32_t)(((a.K + hf) * MS_PS + le) * 4);
+    p = a.Y + ee * a.dsh;
+    pv = DUAL && has_vY ? a.vY + ee * a.dsh : p;
+    for (int b = hf; b < a.dsh; b += 2, d += 2 * MS_PS * 4) {
+        cp_async4_zfill(d, p + b, n);
+        if (DUAL && has_vY) cp_async4_zfill(d + dv, pv + b, n);
+    }
+}
+
+// LE: the loader warps copy phi and Y as well (stored edge inputs only).  One warp for the edge rows of every slot bounds the nodes whose
+// read-out is short, four share them among the loaders (64 x 0 -> 64 x 0, K = 8, 5,206 nodes of degree 11: 64 -> 52 us; 128 x 0 -> 128 x (0, 2),
+// K = 16, degree 6, dual: 119 -> 97 us); behind a long read-out the loaders are the longer chain (64 x (0..2), K = 16: 171 -> 176 us).
+template <bool DUAL, bool LE>
 __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = smem_raw + ((0u - smem_u32(smem_raw)) & 1023u);       // (keeps the pointer in the shared address space)
@@ -275,7 +298,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     const int nsub = (has_a1 ? 1 : 0) + (has_a2 ? 1 : 0);
 
     if (tid == 0) {
-        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, 64); mbar_init(bar_sfree + 8 * s, 2); }
+        for (int s = 0; s < MS_MAXNS; ++s) { mbar_init(bar_full + 8 * s, LE ? 32 : 64); mbar_init(bar_sfree + 8 * s, 2); }
         for (int s = 0; s < MS_MAXNW; ++s) { mbar_init(bar_wfull + 8 * s, NBW * 32); mbar_init(bar_wfree + 8 * s, 2); }
         for (int t = 0; t < 2; ++t) { mbar_init(bar_accfull + 8 * t, 1); mbar_init(bar_accfree + 8 * t, 4 * MS_NDT); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -314,13 +337,14 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         MsSlots at(a, sSet, nsub, a.status);
         // Lane e < 16 holds edge e of the batch.  The ids of the next batch are requested one batch ahead and not looked at before
         // their turn (an id out of range turns the edge's copies into zero fills and is reported in the status word).
-        struct Ids { int v; bool in; };
+        struct Ids { int v, e; bool in; };
         auto request = [&]() -> Ids {
-            Ids d{0, at.b0 + lane < at.it.len && lane < TB};
+            Ids d{0, 0, at.b0 + lane < at.it.len && lane < TB};
             if (d.in) {
                 const int pos = at.it.seg0 + at.b0 + lane;
                 if (!a.ev.transposed) d.v = a.ev.col[pos];
                 else d.v = a.ev.recv ? a.ev.recv[pos] : a.ev.perm[pos];
+                if (LE) d.e = a.ev.perm ? a.ev.perm[pos] : pos;
             }
             return d;
         };
@@ -342,7 +366,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // 16 bytes = 8 multiplicities per copy: lane <-> piece j of eight rows' pieces; its four edges are lane / 8 + 0, 4, 8, 12
         const int j = lane & 7, e0 = lane >> 3;
         bool have = me < nlw && to_mine(true);
-        Ids ids{0, false};
+        Ids ids{0, 0, false};
         if (have) ids = request();
         while (have) {
             const int st_now = st; const uint32_t round_now = round;
@@ -366,9 +390,15 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             ok = ok && id_ok(sn, a.ev.N, a.status);
             if (!ok) sn = 0;
             const uint32_t msk = __ballot_sync(0xffffffffu, ok);
+            const int eid = LE && ids.in && id_ok(ids.e, a.ev.E, a.status) ? ids.e : -1;
             have = to_mine(false);
             if (have) ids = request();
             if (round_now > 0) mbar_wait(bar_sfree + 8 * st_now, (round_now & 1) ^ 1, a.status);
+            if (LE) {
+                const int ee = __shfl_sync(0xffffffffu, eid, lane & (TB - 1));
+                ms_edge_rows<DUAL>(a, smem_u32(sRing + (size_t)st_now * a.slot_bytes + (size_t)2 * a.x_cap), ee < 0 ? 0 : ee, ee < 0 ? 0u : 4u, has_vphi, has_vY,
+                                   lane & (TB - 1), lane >> 4);
+            }
             const __nv_bfloat16* const baseh = op == 0 ? a.sh : a.vsh;
             const int64_t to_lo = (op == 0 ? a.sl : a.vsl) - baseh;
             const __nv_bfloat16* row[4];
@@ -396,7 +426,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
             // this thread's arrival on the slot's barrier fires when all its copies above have landed
             asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st_now) : "memory");
         }
-    } else if (warp == W_EDGE) {
+    } else if (!LE && warp == W_EDGE) {
         // =========================== edge warp ===========================
         // Walks the same slots as the loaders and fills their phi and Y rows, transposed: from memory, or computed from the edge vectors
         // (lane <-> edge lane & 15, half of the radial indices / harmonics each).
@@ -418,21 +448,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
                 have = at.next();
                 e = request(have, in);
                 if (round > 0) mbar_wait(bar_sfree + 8 * st, (round & 1) ^ 1, a.status);
-                uint32_t d = smem_u32(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap) + (uint32_t)((hf * PS + le) * 4);
-                const uint32_t dv = (uint32_t)((a.K + a.dsh) * PS * 4);
-                const float* p = a.phi + ee * a.K;
-                const float* pv = has_vphi ? a.vphi + ee * a.K : p;
-                for (int q = hf; q < a.K; q += 2, d += 2 * PS * 4) {
-                    cp_async4_zfill(d, p + q, n);
-                    if (has_vphi) cp_async4_zfill(d + dv, pv + q, n);
-                }
-                d = smem_u32(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap) + (uint32_t)(((a.K + hf) * PS + le) * 4);
-                p = a.Y + ee * a.dsh;
-                pv = has_vY ? a.vY + ee * a.dsh : p;
-                for (int b = hf; b < a.dsh; b += 2, d += 2 * PS * 4) {
-                    cp_async4_zfill(d, p + b, n);
-                    if (has_vY) cp_async4_zfill(d + dv, pv + b, n);
-                }
+                ms_edge_rows<DUAL>(a, smem_u32(sRing + (size_t)st * a.slot_bytes + (size_t)2 * a.x_cap), ee, n, has_vphi, has_vY, le, hf);
                 asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar_full + 8 * st) : "memory");
                 if (++st == NS) { st = 0; ++round; }
             }
@@ -675,11 +691,11 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
     }
 }
 
-template <bool DUAL>
+template <bool DUAL, bool LE>
 cudaError_t moment_stream_launch(const MsArgs& a, int grid, int smem, cudaStream_t s) {
-    cudaError_t e = allow_dynamic_smem(k_moment_stream<DUAL>);
+    cudaError_t e = allow_dynamic_smem(k_moment_stream<DUAL, LE>);
     if (e != cudaSuccess) return e;
-    k_moment_stream<DUAL><<<grid, MS_TT, smem, s>>>(a);
+    k_moment_stream<DUAL, LE><<<grid, MS_TT, smem, s>>>(a);
     return cudaGetLastError();
 }
 

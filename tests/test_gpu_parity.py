@@ -132,6 +132,42 @@ def test_state_orders(ir_in, ir_out, l_max, K):
         assert rel_err(got, ref) <= BWD_TOL, nm
 
 
+# The orders where the runs of one block come from sets of different lengths (128 x 1o beside 64 x 2e has one part in either: both take
+# the shorter), and on nodes whose edges are gathered again for every two units, of which there is an odd number.
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg", [("64x2e+128x1o", "64x2e+128x1o", 3, 16, 24, 8), ("64x0e+24x2e", "16x0e+8x2e", 2, 16, 150, 140),
+                                                       ("64x0e+24x2e", "16x0e+8x2e", 2, 13, 150, 140), ("8x0e+72x1o", "64x0e+8x1o", 1, 16, 150, 140)])
+def test_state_orders_of_sets_and_passes(ir_in, ir_out, l_max, K, N, deg):
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("order", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=41)
+    c = Case(w, form="moment")
+    assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
+    for got, ref, nm in zip(c.bwd() + c.dbwd(), list(c.o_bwd()) + list(c.o_dbwd()), ("gx", "gY", "gphi", "gR", "ggy", "hx", "hY", "hphi", "hR")):
+        assert rel_err(got, ref) <= BWD_TOL, nm
+
+
+# Streams with at most twelve state components a set, whose loader warps copy phi and Y too from 592 nodes on: K and harmonics that are odd
+# and even, one slot a node, several and more than the rings hold, the receivers of the sender view given or looked up.
+@pytest.mark.parametrize("with_recv", [True, False])
+@pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg", [("32x0e+40x3o", "32x0e", 1, 16, 592, 12), ("40x1o", "96x0e", 2, 9, 700, 2), ("8x0e+8x1o", "8x0e+8x1o", 2, 7, 600, 150),
+                                                       ("64x2e", "64x0e", 2, 16, 592, 140), ("128x0e", "128x0e+128x2e", 2, 1, 620, 33), ("40x1o", "96x0e", 2, 9, 591, 2)])
+def test_loaders_copy_the_edge_rows(ir_in, ir_out, l_max, K, N, deg, with_recv):
+    L = 4.0 * (N / 60.0) ** (1 / 3)
+    w = synth.Workload("loaders", P(ir_in), P(ir_out), l_max, K, N, L, float(synth.cutoff_for_edges(N, deg * N, L)), "gaussian", seed=37)
+    c = Case(w, form="moment")
+    if not with_recv:
+        c.graph = c.sb.make_graph(c.row_ptr, c.col, c.src_ptr, c.src_perm)
+    assert rel_err(c.fwd(), c.o_fwd()) <= FWD_TOL
+    for got, ref, nm in zip(c.bwd() + c.dbwd(), list(c.o_bwd()) + list(c.o_dbwd()), ("gx", "gY", "gphi", "gR", "ggy", "hx", "hY", "hphi", "hR")):
+        assert rel_err(got, ref) <= BWD_TOL, nm
+    # and they look at the edge indices of the sender view
+    perm = c.src_perm.clone()
+    perm[3] = c.E + 5
+    gx = c._new(c.N, c.plan.info.C_x)
+    g = c.sb.make_graph(c.row_ptr, c.col, c.src_ptr, perm, c.src_recv if with_recv else None)
+    c.sb.conv_bwd(c.plan, g, c.x, c.Y, c.phi, c.R, c.gy, gx, None, None, None, c.ws(1))
+    assert c.sb.last_device_status(c.ws(1)) == -4
+
+
 @pytest.mark.parametrize("ir_in,ir_out,l_max,K,N,deg,output,form", [
     ("8x0e+8x1o+8x2e", "8x0e+8x1o+8x2e", 2, 16, 400, 4, "y", "moment"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "y", "moment"),
     ("96x1o+96x2e", "96x0e", 2, 16, 200, 100, "y", "moment"), ("32x0e+32x1o+32x2e", "32x0e+32x1o+32x2e", 2, 8, 200, 30, "gx", "moment"),
