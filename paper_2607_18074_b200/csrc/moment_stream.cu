@@ -23,25 +23,25 @@ void build_stream_sets(const sobek_plan* p, Direction& dir) {
 }
 
 // Microseconds of either form, from the counts of the forms' tables: a launch, and on one SM a node and 16 of its edges, which the roles
-// work at side by side: (a^p + b^p)^(1/p).  The constants are least-squares fits (of relative errors; 10 and 13 % left, dual 11 and 14 %)
-// to the streams of 7,288 random layers, 8 to 128 multiplicities of orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes, in
-// both directions.  On the half of the layers that a fit to the other half did not see the form taken is 0.4 % above the faster one on
-// average (dual streams: 0.2 %), at worst 1.5 times the coupled one; fixed forms: moment 4.6 % (2.3 %), coupled 44 % (64 %).
+// work at side by side: (a^p + b^p)^(1/p).  The constants are least-squares fits (of relative errors; 8 and 10 % left, dual 9 and 11 %)
+// to the streams of 9,082 random layers, 8 to 128 multiplicities of orders up to 4, K = 1 .. 16, degrees 2 to 400, 64 to 8,000 nodes, in
+// both directions.  On the half of the layers that a fit to the other half did not see the form taken is 0.2 % above the faster one on
+// average (dual streams: 0.2 %), at worst 1.4 (1.3) times the coupled one; fixed forms: moment 4.8 % (2.5 %), coupled 44 % (64 %).
 struct StreamFit {
     double launch, p;                                         // moment form
     double unit, pair, val, part, set;                        //   node: units, pairs of components per team and run, their radial indices, those of runs not whole
     double kcycle, w, row, pass, slot_unit;                   //   slot: products, rows of W, gathered slabs, passes, units
     double c_launch, c_p;                                     // coupled form (1: with one accumulator buffer, on top)
     double c_col, c_col1, c_node_set;                         //   node: accumulator columns, sets
-    double c_slab, c_row, c_set, c_slab1, c_set1;             //   batch: built operand, gathered rows, hand-over
+    double c_slab, c_row, c_set, c_slab1;                     //   batch: built operand, gathered rows, hand-over
     double c2_slab, c2_row, c2_set, c2_set1;                  //   its second operand
     double geo[5], c_geo[5];                                  // phi and Y of a slot from edge vectors: constant, per radial index, per harmonic; p; launch
 };
 constexpr StreamFit kFit[2] = {
-    {9.87, 1.47, 0.554, 0.401, 0.0257, 0.0503, 0.341, 0.171, 0.00214, 0.0197, 0.221, 0.143,
-     14.6, 1.87, 0.0203, 0.00446, 0.342, 0.182, 0.0459, 0.9, 0.0318, 0.187, 0, 0, 0, 0, {1.2, 0.0477, 0, 4.78, 7.86}, {1.1, 0.0651, 0.00335, 12.5, 8.79}},
-    {10.8, 1.35, 0.561, 0.389, 0.0395, 0.0472, 0.329, 0.172, 0.00289, 0.0104, 0.332, 0.0798,
-     15.5, 1.47, 0.0187, 0.00483, 0.465, 0.268, 0.0263, 1.1, 0.0267, 0.0754, 0.159, 0.049, 1.01, 0.155, {1.67, 0.18, 0.00331, 1.48, 4.43}, {1.53, 0.14, 0.0324, 3.95, 12.7}}};
+    {9.89, 1.26, 0.517, 0.398, 0.0255, 0.0437, 0.0989, 0.226, 0.00195, 0.0139, 0.259, 0.0568,
+     14.6, 1.65, 0.0194, 0.00377, 0.182, 0.186, 0.0487, 0.789, 0.0515, 0, 0, 0, 0, {1.17, 0.0476, 0, 4.37, 7.59}, {1.02, 0.0633, 0.00452, 11.1, 7.54}},
+    {10.9, 1.21, 0.553, 0.39, 0.0369, 0.0406, 0, 0.219, 0.00282, 0.0095, 0.352, 0,
+     15.5, 1.36, 0.0176, 0.00402, 0.295, 0.274, 0.03, 1, 0.0395, 0.167, 0.061, 0.855, 0.093, {1.66, 0.182, 0.0134, 1.59, 5.18}, {1.09, 0.148, 0.0545, 3.94, 13.1}}};
 static double side_by_side(double a, double b, double p) { return std::pow(std::pow(a, p) + std::pow(b, p), 1 / p); }
 
 static void stream_costs(const sobek_plan* p, Direction& dir, int dual) {
@@ -56,7 +56,7 @@ static void stream_costs(const sobek_plan* p, Direction& dir, int dual) {
         for (int b = 0; b < S.nblk; ++b) rows += T.blks[S.blk_begin + b].d_src * ((T.blks[S.blk_begin + b].c_src + 63) / 64);
     }
     T.node_us = (F.c_col + one * F.c_col1) * cols + F.c_node_set * sets;
-    T.slot_us = (F.c_slab + one * F.c_slab1) * slabs + F.c_row * rows + (F.c_set + one * F.c_set1) * sets;
+    T.slot_us = (F.c_slab + one * F.c_slab1) * slabs + F.c_row * rows + F.c_set * sets;
     T.slot2_us = F.c2_slab * slabs + F.c2_row * rows + (F.c2_set + one * F.c2_set1) * sets;
     double units = 0, pairs = 0, vals = 0, part = 0, kcycles = 0, w[2] = {0, 0}, gathered[2] = {0, 0}, passes[2] = {0, 0};      // [1]: slots that do not stay
     for (const MSet& S : M.sets) {
@@ -85,28 +85,30 @@ static void stream_costs(const sobek_plan* p, Direction& dir, int dual) {
     }
 }
 
-// The slots of a node stay for all its units where they all fit the rings; the rows of the others are gathered, and their W built, for
-// every two units.  Degrees spread around their mean: the share of the latter falls from all to none where the longest node that stays
-// has 0.7 to 1.5 times the mean.  Below four nodes per SM the longest ones decide.  With the edge inputs computed from vectors (geo) one
-// warp of either kernel makes the rows of every slot in every pass, a bound of its own.  (Of such layers that the fit did not see: 0.5 %
-// above the faster form on average, dual streams 1.0 %, at worst 1.4 and 2.0 times the coupled one; moment throughout 7 % and 31 %.)
+// The busiest SM counts: items are (set, node), dealt to 148 of them.  The slots of a node stay for all its units where they all fit the
+// rings; the rows of the others are gathered, and their W built, for every two units.  Degrees spread around their mean: the share of the
+// latter falls from all to none where the longest node that stays has 0.7 to 1.5 times the mean.  Below four nodes per SM the longest ones
+// decide.  With the edge inputs computed from vectors (geo) one warp of either kernel makes the rows of every slot in every pass, a bound of
+// its own.  (Of such layers that the fit did not see: 0.4 % above the faster form on average, dual streams 0.9 %, at worst 1.4 and 2.0 times
+// the coupled one; moment throughout 7 % and 31 %.)
 bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int operands, bool geo, int64_t N, int64_t E) {
     const StreamFit& F = kFit[dual];
     const TcSets& T = dir.tc[dual];
     const MomentSets& M = dir.ms[dual];
     if (!M.ok || p->form != kFormAuto) return M.ok && p->form == kFormMoment;
-    const double mean = (double)E / (double)std::max<int64_t>(N, 1), per_sm = std::max(1.0, (double)N / 148.0);
-    const bool few = per_sm < 4;
-    const double batches = (few ? 1.3 : 1.0) * mean / MS_TB + 0.5, slots = batches * operands;
+    const double mean = (double)E / (double)std::max<int64_t>(N, 1), sets = (double)M.sets.size(), c_sets = (double)T.sets.size();
+    const double per_sm = std::ceil((double)N * sets / 148) / sets, c_per_sm = std::ceil((double)N * c_sets / 148) / c_sets;
+    const bool few = N < 4 * 148;
+    const double batches = (few ? 1.15 : 1.0) * mean / MS_TB + 0.5, slots = batches * operands;
     const double longest = MS_TB * (double)(std::min(M.ns, M.nw) / operands), over = 1.5 * mean - longest;
     const double again = few ? (over > 0 ? 1 : 0) : std::min(1.0, std::max(0.0, over / (0.8 * mean)));
     auto mix = [&](const double* v) { return v[0] + again * (v[1] - v[0]); };
     double moment = F.launch + per_sm * side_by_side(M.node_us, slots * mix(M.slot_us), F.p),
-           coupled = F.c_launch + per_sm * side_by_side(T.node_us, batches * (T.slot_us + (operands - 1) * T.slot2_us), F.c_p);
+           coupled = F.c_launch + c_per_sm * side_by_side(T.node_us, batches * (T.slot_us + (operands - 1) * T.slot2_us), F.c_p);
     if (geo) {
-        auto rows = [&](const double* g, double passes) { return g[4] + per_sm * slots * passes * (g[0] + g[1] * p->K + g[2] * p->dim_sh); };
-        moment = side_by_side(moment, rows(F.geo, mix(M.passes)), F.geo[3]);
-        coupled = side_by_side(coupled, rows(F.c_geo, (double)T.sets.size()), F.c_geo[3]);
+        auto rows = [&](const double* g, double passes) { return g[4] + slots * passes * (g[0] + g[1] * p->K + g[2] * p->dim_sh); };
+        moment = side_by_side(moment, rows(F.geo, per_sm * mix(M.passes)), F.geo[3]);
+        coupled = side_by_side(coupled, rows(F.c_geo, c_per_sm * c_sets), F.c_geo[3]);
     }
     return moment < coupled;
 }
