@@ -42,9 +42,9 @@ DTYPE = "f32 storage; products as split bf16 x3 (hi*hi + lo*hi + hi*lo) with f32
 # edge at 40 edges per node) plus the gathered sender rows, the edge pass's the fp32 adjoint state read once plus those rows.
 NCU_TRAFFIC_BYTES_PER_EDGE = {
     # k_moment_stream: five plain passes and two dual ones
-    ("cfg5", "edge_stream_state"): (5 * (353.3e6 + 2079.0e6) + 2 * (721.7e6 + 2081.7e6)) / 7 / 90891.0,
+    ("cfg5", "edge_stream_state"): (5 * (357.2e6 + 2078.6e6) + 2 * (722.5e6 + 2081.0e6)) / 7 / 90891.0,
     # k_moment_edge: two plain passes and a dual one
-    ("cfg5", "edge_pass"): (2 * (2667.4e6 + 16.2e6) + (4771.5e6 + 26.8e6)) / 3 / 90891.0,
+    ("cfg5", "edge_pass"): (2 * (2658.4e6 + 16.6e6) + (4638.0e6 + 31.2e6)) / 3 / 90891.0,
 }
 STATE_BUDGET_MIB = None         # --state-budget-mib: the plan's scratch budget (None = the library's default, 2048)
 STREAM_CALLS_PER_STEP = 7      # edge-stream passes over all edges per step: 1 fwd + 2 bwd + 4 dbwd

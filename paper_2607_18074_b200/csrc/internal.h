@@ -29,7 +29,7 @@ struct DPath {
     int32_t d_sh;      // 2 l_sh + 1
     int32_t d_dst;     // 2 l_dst + 1
     int32_t c_dst;     // destination multiplicity
-    int32_t koff;      // offset in the group's contraction axis; k = koff + q*c_src + u
+    int32_t koff;      // offset in the group's contraction axis; k = koff + state_pos(q, u), q*c_src + u unless the moment stream wrote the state
     int32_t m_off;     // offset of M[s][o] inside the group's per-edge M area
     int32_t tabM;      // index into tab_ptr: entry (s*d_dst+o) -> terms (b, coef)
     int32_t tabY;      // index into tab_ptr: b -> terms (s*d_dst+o, coef)   (adjoint wrt Y)

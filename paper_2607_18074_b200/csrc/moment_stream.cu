@@ -118,7 +118,7 @@ bool moment_stream_pays(const sobek_plan* p, const Direction& dir, int dual, int
 static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int& nq_max) {
     constexpr int kSmem = 227 * 1024;
     constexpr int kSlotBytes = 37 * 1024;      // gathered rows of a slot, hi and lo, beyond which a block starts a set of its own
-    constexpr int kWRows = 224;                // rows of W at a time at most (both lane halves)
+    constexpr int kWRows = 224;                // rows of W at a time (both lane halves) that several runs share; a single run may have more
     MomentSets& T = dir.ms[dual];
     T = MomentSets{};
     if (p->K > 16 || (dir.C_src & 7) || dir.paths.empty()) return true;
@@ -174,7 +174,10 @@ static bool build_moment_set(const sobek_plan* p, Direction& dir, int dual, int&
         const int KH = (p->K + 1) / 2;
         struct Seg { int l0, l1, row, rows; };
         std::vector<Seg> segs;
-        // (eight at a time only where they fill the run: 13 radial indices or more)
+        // Eight at a time from 13 radial indices on.  At 16, where the run is whole, four at a time are 3 to 13 % slower (dual: 0 to 10 %);
+        // at 13 to 15 within 2 % either way, one-order harmonics with long neighbourhoods 20 % slower.  At l_max 3 and 4 the run has 256 and
+        // 400 rows of W, which take ring slots: four at a time are 12 to 30 % slower at 64 and 128 multiplicities and degrees to 30, and
+        // 6 to 12 % faster in the dual streams of orders 0 and 1 at degree 120.
         int nq = std::min(nq_max, KH >= 7 ? 8 : KH >= 3 ? 4 : KH), rows_q = 0;
         for (; nq >= 1; nq >>= 1) {
             segs.clear(); rows_q = 0;

@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(MS_TT, 1) k_moment_stream(const MsArgs a) {
         // =========================== loader warps ===========================
         // A slot is filled by one warp alone, the warps take turns: a warp spends most of its time on index arithmetic, a few cycles
         // an instruction whatever the others do.  (All four on one slot: 32 x (0..2) forward 312 instead of 294 us, 128/64/64
-        // backward at degree 255, which gathers for every unit, 6.8 instead of 4.9 ms.  TMA gathers of four rows: 3 to 20 % slower.)
+        // backward at degree 255, whose slots did not stay, 6.8 instead of 4.9 ms.  TMA gathers of four rows: 3 to 20 % slower.)
         const int me = warp - W_LOAD;
         MsSlots at(a, sSet, nsub, a.status);
         // Lane e < 16 holds edge e of the batch.  The ids of the next batch are requested one batch ahead and not looked at before
